@@ -134,6 +134,12 @@ struct Plan {
     uint32_t *hv = nullptr, *hv2 = nullptr, *keep = nullptr, *kscan = nullptr;
     int grid = 304;
     int sort_grid = 608;
+    // short merge: bucket counts and drop bits, each bucket's first place
+    uint32_t *tail = nullptr, *bbase = nullptr;
+    float bscale = 0.0f;
+    // more raw hits than the short merge takes: the radix sort and the scans (as
+    // a search of this plan found; the look-back test switch needs that sort too)
+    bool long_tail = false;
     // execution
     cudaStream_t st = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
@@ -227,8 +233,39 @@ struct Plan {
     void enqueue(cudaStream_t s) {
         const tms_params &p = prm;
         const int prec = p.precision, fl = p.face_level;
+    // merge of the raw hits, at most kTailMax of them
+    void enqueue_short_tail(cudaStream_t s) {
+        mark(13, s);
+        TailArgs ta;
+        ta.key = hk; ta.slot = kscan; ta.tail = tail; ta.bbase = bbase; ta.bkey = hk2; ta.bidx = hv2;
+        ta.skey = okeys; ta.order = keep; ta.raw = hits; ta.meshes = d_meshes; ta.pairs = d_pairs;
+        ta.ctr = d_ctr; ta.raw_cap = hit_cap; ta.out = (tms_hit *)dHits;
+        ta.out_cap = (unsigned long long)hitCap; ta.offsets = dOffsets; ta.n_pairs = nPairs;
+        ta.tri_bits = tri_bits; ta.tau = prm.tau; ta.bscale = bscale;
+        launch_tail(ta, grid / 2, s);
+        kernels += 3;
+    }
+
+    // sort and merge of any number of raw hits
+    void enqueue_long_tail(cudaStream_t s) {
+        DedupArgs da;
+        da.raw = hits;
+        da.meshes = d_meshes; da.pairs = d_pairs; da.ctr = d_ctr; da.raw_cap = hit_cap;
+        da.keep = keep; da.keep_scan = kscan; da.partials = partials;
+        da.out = (tms_hit *)dHits; da.out_cap = (unsigned long long)hitCap; da.out_keys = okeys;
+        da.offsets = dOffsets; da.n_pairs = nPairs; da.tri_bits = tri_bits; da.tau = prm.tau;
+        const int bits = 2 * tri_bits + pair_bits;
+        const bool halt = radix_sort(hk, hv, hk2, hv2, sort_scratch, &d_ctr->raw_hits, hit_cap, bits, sort_grid,
+                                     &d_ctr->status, (unsigned long long)prm.spin_limit,
+                                     (prm.inject & 16u) ? 1 : 0, s);
+        kernels += 2 + (bits + kRadixBits - 1) / kRadixBits;
+        mark(13, s);
+        da.keys = halt ? hk2 : hk; da.vals = halt ? hv2 : hv;
+        launch_dedup(da, grid, s);
+        kernels += 5 + (dOffsets ? 1 : 0);
+    }
+
         const int block = (p.block_faces == 64 || p.block_faces == 256) ? p.block_faces : 128;
-        const int sort_passes_h = (2 * tri_bits + pair_bits + kRadixBits - 1) / kRadixBits;
         kernels = 0;
         mark(0, s);
         // the occupancy filter runs at the face level only: patches are few, and
@@ -236,7 +273,7 @@ struct Plan {
         const bool filter = p.cell_filter && !patch;
         launch_search_init(d_bounds, n_meshes, d_ctr, filter ? bmA : nullptr,
                            (unsigned long long)1 << bmA_bits, filter ? bmH : nullptr,
-                           (unsigned long long)1 << bmH_bits, grid, s);
+                           (unsigned long long)1 << bmH_bits, long_tail ? nullptr : tail, grid, s);
         GroupArgs ga;
         ga.ent_key = ek; ga.ent_face = ev; ga.d_n = &d_ctr->entries; ga.cap = ent_cap;
         ga.ent_slot = eslot; ga.ent_rank = erank;
@@ -342,25 +379,12 @@ struct Plan {
         na.meshes = d_meshes; na.pairs = d_pairs;
         na.ctr = d_ctr; na.hits = hits; na.hit_key = hk; na.hit_val = hv; na.hit_cap = hit_cap;
         na.tau = p.tau; na.tri_bits = tri_bits; na.fp32_filter = p.narrow_filter;
-        launch_narrow(na, fl, grid / 2, grid * 4, s);
-        kernels += 2;
+        na.tail = long_tail ? nullptr : tail; na.hit_slot = kscan; na.bscale = bscale;
+        launch_narrow(na, fl, grid / 2, s);
+        kernels += fl == 1 && p.narrow_filter ? 3 : 2;
         mark(12, s);
-
-        DedupArgs da;
-        da.raw = hits;
-        da.meshes = d_meshes; da.pairs = d_pairs; da.ctr = d_ctr; da.raw_cap = hit_cap;
-        da.keep = keep; da.keep_scan = kscan; da.partials = partials;
-        da.out = (tms_hit *)dHits; da.out_cap = (unsigned long long)hitCap; da.out_keys = okeys;
-        da.offsets = dOffsets; da.n_pairs = nPairs; da.tri_bits = tri_bits; da.tau = p.tau;
-        // the raw hits are few: a small grid keeps the per-pass fixed cost low
-        const bool halt = radix_sort(hk, hv, hk2, hv2, sort_scratch, &d_ctr->raw_hits, hit_cap,
-                                     2 * tri_bits + pair_bits, sort_grid, &d_ctr->status,
-                                     (unsigned long long)p.spin_limit, (p.inject & 16u) ? 1 : 0, s);
-        kernels += 2 + sort_passes_h;
-        mark(13, s);
-        da.keys = halt ? hk2 : hk; da.vals = halt ? hv2 : hv;
-        launch_dedup(da, grid, s);
-        kernels += 5 + (dOffsets ? 1 : 0);
+        if (long_tail) enqueue_long_tail(s);
+        else enqueue_short_tail(s);
         mark(14, s);
 
         cudaMemcpyAsync(h_ctr, d_ctr, kReadback, cudaMemcpyDeviceToHost, s);
@@ -494,10 +518,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     std::vector<PassEntry> pall, pa, pb;
     unsigned long long max_tri = 1;
     for (int i = 0; i < nPairs; ++i) {
-        int ia = (int)meshes.size();
-        meshes.push_back(A[i]->dev);
-        int ib = (int)meshes.size();
-        meshes.push_back(B[i]->dev);
+        const int ia = row(A[i]), ib = row(B[i]);
         pairs.push_back(make_int2(ia, ib));
         const unsigned long long fpq = prm.face_level == 0 ? 2 : 1;
         auto cells_of = [&](const MeshDev &d) -> unsigned long long {
@@ -629,6 +650,13 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
 
     const unsigned long long faces = P->facesA + P->facesB;
     unsigned long long ent = prm.entry_capacity > 0 ? (unsigned long long)prm.entry_capacity
+    TMS_PCK(dalloc(&P->tail, kTailBuckets + kTailMax / 32));
+    TMS_PCK(dalloc(&P->bbase, kTailBuckets + 1));
+    // the range of (pair, triA), over which the buckets are spread
+    P->bscale = (float)((double)kTailBuckets /
+                        (nPairs == 1 ? 2.0 * A[0]->dev.N * A[0]->dev.nqk
+                                     : (double)nPairs * (double)(1ULL << P->tri_bits)));
+    P->long_tail = (prm.inject & 16u) != 0;
                              : patch ? 4 * faces + (1 << 16)
                              : (prm.cell_filter ? std::max<unsigned long long>(1 << 16, faces / 2)
                                                 : 4 * faces + (1 << 16));
@@ -792,6 +820,10 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     st.fp32_solves = (long long)c.fp32;
     st.sat_tests = (long long)c.sat;
     st.quad_tests = (long long)c.quad;
+        if (!P->long_tail && c.raw_hits > kTailMax) {
+            P->long_tail = true;
+            grow = true;
+        }
     st.patch_pairs = (long long)c.ppairs;
     st.patch_tests = (long long)c.ptests;
     st.quad_kept = (long long)c.qkeep;

@@ -161,8 +161,20 @@ struct Counters {
     unsigned long long raw_hits;
     unsigned long long out;
     unsigned int status;
-    unsigned int pad;
+    unsigned int dropped;          // raw hits merged into another record (short tail)
 };
+
+// The short merge (k_tail_*, up to kTailMax raw hits): the hits are counted into
+// kTailBuckets buckets of increasing key as the FP64 solve lists them.
+constexpr unsigned kTailMax = 32768;
+constexpr unsigned kTailBuckets = 8192;
+
+// The bucket of a hit: its (pair, triA) scaled to the buckets, monotone in the
+// key (the conversion and the product round monotonically).
+__device__ __forceinline__ unsigned tail_bucket(uint64_t key, int tri_bits, float scale) {
+    const unsigned b = (unsigned)(__ull2float_rz(key >> tri_bits) * scale);
+    return b < kTailBuckets ? b : kTailBuckets - 1;
+}
 
 constexpr unsigned long long kHashEmpty = 0;   // free slot of the cell table (keys are stored + 1)
 constexpr uint32_t kNoCell = 0xFFFFFFFFu;
@@ -439,8 +451,9 @@ void launch_face_pass(const FacePassArgs &a, int precision, int face_level, int 
 cudaError_t configure_face_pass();
 // counters zeroed, bounds reset, bitmaps cleared (NULL: not cleared); word
 // counts are multiples of four
+// (tail: the short merge's bucket counts and drop bits, or NULL)
 void launch_search_init(Bounds *b, int n, Counters *ctr, uint32_t *bmA, unsigned long long n32a,
-                        uint32_t *bmH, unsigned long long n32h, int grid, cudaStream_t st);
+                        uint32_t *bmH, unsigned long long n32h, uint32_t *tail, int grid, cudaStream_t st);
 // cm_pair: per-pair cell multipliers (device, n_pairs), or NULL for cell_mult
 void launch_grid_params(const Bounds *b, const int2 *pairs, int n_pairs, Grid *g,
                         float cell_mult, cudaStream_t st, const float *cm_pair = nullptr);
@@ -564,10 +577,13 @@ struct NarrowArgs {
     double tau;
     int tri_bits;
     int fp32_filter;
+    uint32_t *tail;                // bucket counts of the short merge (NULL: not kept)
+    uint32_t *hit_slot;            // [hit_cap] the hit's place in its bucket
+    float bscale;                  // tail_bucket's scale
 };
 // the quad-level test over all candidates (quad faces), then the filter on what it
-// left as one wave of resident blocks on `sms` SMs, the FP64 solve on `grid` blocks
-void launch_narrow(const NarrowArgs &a, int face_level, int sms, int grid, cudaStream_t st);
+// left as one wave of resident blocks on `sms` SMs, then the FP64 solve
+void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st);
 void configure_narrow();
 
 // FP32 split of a double: hi = RN32(x), lo = RN32(x - hi), integer operations
@@ -644,6 +660,33 @@ struct DedupArgs {
     double tau;
 };
 void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st);
+
+// The merge of at most kTailMax raw hits in three launches, instead of the radix
+// sort and launch_dedup (nothing is written when there are more: the host takes
+// that path then).
+struct TailArgs {
+    const uint64_t *key;           // raw hits' keys, in the order they were found
+    const uint32_t *slot;          // and their places in their buckets
+    uint32_t *tail;                // bucket counts [kTailBuckets], then drop bits [kTailMax / 32]
+    uint32_t *bbase;               // [kTailBuckets + 1] each bucket's first place
+    uint64_t *bkey;                // [raw_cap] keys by bucket
+    uint32_t *bidx;                // [raw_cap] raw-hit indices by bucket
+    uint64_t *skey;                // [raw_cap] sorted keys
+    uint32_t *order;               // [raw_cap] raw-hit index by rank | shared-feature flag << 31
+    const tms_hit *raw;
+    const MeshDev *meshes;
+    const int2 *pairs;
+    Counters *ctr;
+    unsigned long long raw_cap;
+    tms_hit *out;
+    unsigned long long out_cap;
+    long long *offsets;            // nPairs + 1 (may be null)
+    int n_pairs;
+    int tri_bits;
+    double tau;
+    float bscale;
+};
+void launch_tail(const TailArgs &a, int sms, cudaStream_t st);
 
 
 struct AdjointArgs {

@@ -903,7 +903,8 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_cell_pass(FacePassArgs a, i
 // reset, and the two occupancy bitmaps cleared (n32a and n32h words, each a
 // multiple of four).
 __global__ void k_search_init(Bounds *b, int n, Counters *ctr, uint32_t *bmA,
-                              unsigned long long n32a, uint32_t *bmH, unsigned long long n32h) {
+                              unsigned long long n32a, uint32_t *bmH, unsigned long long n32h,
+                              uint32_t *tail) {
     const unsigned long long tid = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     if (tid == 0) memset(ctr, 0, sizeof(Counters));
@@ -915,6 +916,9 @@ __global__ void k_search_init(Bounds *b, int n, Counters *ctr, uint32_t *bmA,
         m.faces = 0;
     }
     const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+    if (tail)
+        for (unsigned long long i = tid; i < (kTailBuckets + kTailMax / 32) / 4; i += stride)
+            reinterpret_cast<uint4 *>(tail)[i] = z;
     if (bmA)
         for (unsigned long long i = tid; i < n32a / 4; i += stride) reinterpret_cast<uint4 *>(bmA)[i] = z;
     if (bmH)
@@ -1040,8 +1044,8 @@ void launch_face_pass(const FacePassArgs &a, int precision, int face_level, int 
 }
 
 void launch_search_init(Bounds *b, int n, Counters *ctr, uint32_t *bmA, unsigned long long n32a,
-                        uint32_t *bmH, unsigned long long n32h, int grid, cudaStream_t st) {
-    k_search_init<<<grid, 256, 0, st>>>(b, n, ctr, bmA, n32a, bmH, n32h);
+                        uint32_t *bmH, unsigned long long n32h, uint32_t *tail, int grid, cudaStream_t st) {
+    k_search_init<<<grid, 256, 0, st>>>(b, n, ctr, bmA, n32a, bmH, n32h, tail);
 }
 
 void launch_grid_params(const Bounds *b, const int2 *pairs, int n_pairs, Grid *g,

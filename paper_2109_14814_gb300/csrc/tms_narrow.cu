@@ -911,9 +911,11 @@ __global__ void __launch_bounds__(256) k_narrow_fp64(NarrowArgs a) {
         if (hit && pos < a.hit_cap) {
             h.pair = s.pair;
             a.hits[pos] = h;
-            a.hit_key[pos] = ((uint64_t)s.pair << (2 * a.tri_bits)) |
-                             ((uint64_t)s.faceA << a.tri_bits) | (uint64_t)s.faceB;
-            a.hit_val[pos] = (uint32_t)pos;
+            const uint64_t key = ((uint64_t)s.pair << (2 * a.tri_bits)) |
+                                 ((uint64_t)s.faceA << a.tri_bits) | (uint64_t)s.faceB;
+            a.hit_key[pos] = key;
+            if (a.tail) a.hit_slot[pos] = atomicAdd(a.tail + tail_bucket(key, a.tri_bits, a.bscale), 1u);
+            else a.hit_val[pos] = (uint32_t)pos;
         }
     }
 }
@@ -1069,6 +1071,164 @@ __global__ void k_offsets(const uint64_t *out_keys, const unsigned long long *d_
 }
 
 // ---------------------------------------------------------------------------
+// short merge: up to kTailMax raw hits
+// ---------------------------------------------------------------------------
+// Latency, not work, bounds the merge of a few thousand hits (a radix pass over
+// six tiles is 7 us of loads, ranking and look-back, and the sort and merge took
+// 15 launches), so it is three launches here.  The FP64 solve counts the hits into
+// buckets of increasing key; k_tail_bucket scans the counts (every block for
+// itself: 32 KB from L2) and lists the hits bucket by bucket; k_tail_rank compares
+// a hit with its bucket (about one at 8192 buckets; however unevenly the hits
+// fall, at most kTailMax compares) and decides whether it is a duplicate;
+// k_tail_out writes the records kept.
+__device__ __forceinline__ bool tail_count(const TailArgs &a, unsigned &n) {
+    const unsigned long long raw = a.ctr->raw_hits;
+    n = (unsigned)raw;
+    return raw <= a.raw_cap && raw <= kTailMax;
+}
+
+constexpr int kBucketBlock = 1024;
+__global__ void __launch_bounds__(kBucketBlock) k_tail_bucket(TailArgs a) {
+    constexpr int kPer = kTailBuckets / kBucketBlock;
+    static_assert(kPer == 8, "two 16-byte loads a thread");
+    __shared__ uint32_t base[kTailBuckets];
+    __shared__ uint32_t wsum[kBucketBlock / 32];
+    unsigned n;
+    if (!tail_count(a, n)) return;
+    const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const unsigned first = blockIdx.x * kBucketBlock;
+    if (blockIdx.x > 0 && first >= n) return;      // block 0 writes the buckets' places
+    const uint4 lo = reinterpret_cast<const uint4 *>(a.tail)[2 * t], hi = reinterpret_cast<const uint4 *>(a.tail)[2 * t + 1];
+    const uint32_t c[kPer] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+    uint32_t sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) sum += c[k];
+    uint32_t incl = sum;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t y = __shfl_up_sync(FULL, incl, off);
+        if (lane >= off) incl += y;
+    }
+    if (lane == 31) wsum[warp] = incl;
+    __syncthreads();
+    uint32_t before = __reduce_add_sync(FULL, lane < warp ? wsum[lane] : 0u) + incl - sum;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+        base[kPer * t + k] = before;
+        if (blockIdx.x == 0) a.bbase[kPer * t + k] = before;
+        before += c[k];
+    }
+    if (blockIdx.x == 0 && t == kBucketBlock - 1) a.bbase[kTailBuckets] = before;
+    __syncthreads();
+    for (unsigned i = first + t; i < n; i += gridDim.x * kBucketBlock) {
+        const uint64_t key = a.key[i];
+        const unsigned pos = base[tail_bucket(key, a.tri_bits, a.bscale)] + a.slot[i];
+        a.bkey[pos] = key;
+        a.bidx[pos] = i;
+    }
+}
+
+// whether the point with weights (u, v) lies inside its triangle (feature_of's code 0)
+__device__ __forceinline__ bool inside(double u, double v, double tau) {
+    return !(fabs(u) < tau || fabs(1.0 - u - v) < tau || fabs(v) < tau);
+}
+
+// true when an earlier record of the sorted list finds the same point on the
+// same features (k_dedup_flags' rule)
+__device__ __noinline__ bool tail_duplicate(const TailArgs &a, const tms_hit &h, uint64_t key) {
+    const int2 pr = a.pairs[h.pair];
+    const MeshDev &ma = a.meshes[pr.x], &mb = a.meshes[pr.y];
+    uint32_t incA[6], incB[6], t1[6], t2[6];
+    int nA, nB, n1, n2;
+    const uint32_t fA = feature_of(ma, h.triA, h.a, h.b, a.tau, incA, nA);
+    const uint32_t fB = feature_of(mb, h.triB, h.c, h.d, a.tau, incB, nB);
+    for (int p = 0; p < nA; ++p) {
+        for (int q = 0; q < nB; ++q) {
+            const uint64_t k2 = ((uint64_t)h.pair << (2 * a.tri_bits)) | ((uint64_t)incA[p] << a.tri_bits) |
+                                (uint64_t)incB[q];
+            if (k2 >= key) continue;
+            const unsigned b = tail_bucket(k2, a.tri_bits, a.bscale);
+            for (uint32_t e = a.bbase[b]; e < a.bbase[b + 1]; ++e) {
+                if (a.bkey[e] != k2) continue;
+                const tms_hit &o = a.raw[a.bidx[e]];
+                if (feature_of(ma, o.triA, o.a, o.b, a.tau, t1, n1) == fA &&
+                    feature_of(mb, o.triB, o.c, o.d, a.tau, t2, n2) == fB)
+                    return true;
+            }
+        }
+    }
+    return false;
+}
+
+constexpr int kRankBlock = 128;
+__global__ void __launch_bounds__(kRankBlock) k_tail_rank(TailArgs a) {
+    unsigned n;
+    if (!tail_count(a, n)) return;
+    for (unsigned e = blockIdx.x * kRankBlock + threadIdx.x; e < n; e += gridDim.x * kRankBlock) {
+        const uint64_t key = a.bkey[e];
+        const uint32_t idx = a.bidx[e];
+        const unsigned b = tail_bucket(key, a.tri_bits, a.bscale);
+        const uint32_t lo = a.bbase[b], hi = a.bbase[b + 1];
+        uint32_t rank = lo;
+        for (uint32_t j = lo; j < hi; ++j) rank += a.bkey[j] < key;
+        const tms_hit &h = a.raw[idx];
+        const bool shared = !(inside(h.a, h.b, a.tau) && inside(h.c, h.d, a.tau));
+        if (shared && tail_duplicate(a, h, key)) {
+            atomicOr(a.tail + kTailBuckets + (rank >> 5), 1u << (rank & 31));
+            atomicAdd(&a.ctr->dropped, 1u);
+        }
+        a.skey[rank] = key;
+        a.order[rank] = idx | (shared ? 0x80000000u : 0u);
+    }
+}
+
+// eight lanes a record, 16 bytes each
+__global__ void __launch_bounds__(256) k_tail_out(TailArgs a) {
+    unsigned n;
+    if (!tail_count(a, n)) return;
+    const uint32_t *drop = a.tail + kTailBuckets;
+    const unsigned dropped = a.ctr->dropped;
+    const unsigned tid = blockIdx.x * 256 + threadIdx.x, l = tid & 7;
+    // records dropped before rank r, counted by the record's eight lanes (every
+    // lane of the warp calls it together)
+    auto before = [&](unsigned r) {
+        if (dropped == 0) return 0u;
+        unsigned s = 0;
+        for (unsigned w = l; w < (r >> 5); w += 8) s += __popc(drop[w]);
+        s += __shfl_xor_sync(FULL, s, 1);
+        s += __shfl_xor_sync(FULL, s, 2);
+        s += __shfl_xor_sync(FULL, s, 4);
+        return s + ((r & 31) ? __popc(drop[r >> 5] & ((1u << (r & 31)) - 1u)) : 0);
+    };
+    const unsigned lanes = gridDim.x * 256;
+    for (unsigned g0 = tid & ~31u; g0 < 8 * n; g0 += lanes) {
+        const unsigned r = (g0 + (tid & 31)) >> 3;
+        const unsigned pos = r - before(r < n ? r : 0);
+        if (r >= n || ((drop[r >> 5] >> (r & 31)) & 1u)) continue;
+        const uint32_t o = a.order[r];
+        uint4 v = reinterpret_cast<const uint4 *>(a.raw + (o & 0x7FFFFFFFu))[l];
+        if (l == 0 && (o >> 31)) v.w |= 2u;        // flags
+        if (pos < a.out_cap) reinterpret_cast<uint4 *>(a.out + pos)[l] = v;
+    }
+    if (tid == 0) a.ctr->out = n - dropped;
+    // offsets: the records kept of earlier pairs, one pair per eight lanes
+    if (a.offsets) {
+        for (unsigned g0 = tid & ~31u; g0 < 8u * (a.n_pairs + 1); g0 += lanes) {
+            const unsigned p = (g0 + (tid & 31)) >> 3;
+            const uint64_t k = (uint64_t)p << (2 * a.tri_bits);
+            unsigned lo = 0, hi = n;
+            if (p >= (unsigned)a.n_pairs) lo = n;
+            while (lo < hi) {
+                const unsigned mid = (lo + hi) >> 1;
+                if (a.skey[mid] < k) lo = mid + 1; else hi = mid;
+            }
+            const unsigned d = before(lo);
+            if (l == 0 && p <= (unsigned)a.n_pairs) a.offsets[p] = (long long)(lo - d);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
 // adjoint of the hit outputs
 // ---------------------------------------------------------------------------
 __global__ void k_adjoint(AdjointArgs a) {
@@ -1160,14 +1320,14 @@ void configure_narrow() {
     filter_resident<1>();
 }
 
-void launch_narrow(const NarrowArgs &a, int face_level, int sms, int grid, cudaStream_t st) {
+void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st) {
     if (face_level == 0) {
         k_narrow_filter<0><<<sms * filter_resident<0>(), 256, 0, st>>>(a);
     } else {
         if (a.fp32_filter) k_quad_filter<<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
         k_narrow_filter<1><<<sms * filter_resident<1>(), 256, 0, st>>>(a);
     }
-    k_narrow_fp64<<<grid, 256, 0, st>>>(a);
+    k_narrow_fp64<<<sms * 8, 256, 0, st>>>(a);
 }
 
 void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st) {
@@ -1177,6 +1337,12 @@ void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st) {
     if (a.offsets)
         k_offsets<<<(a.n_pairs + 256) / 256, 256, 0, st>>>(a.out_keys, &a.ctr->out, a.raw_cap,
                                                             a.n_pairs, a.tri_bits, a.offsets);
+}
+
+void launch_tail(const TailArgs &a, int sms, cudaStream_t st) {
+    k_tail_bucket<<<kTailMax / kBucketBlock, kBucketBlock, 0, st>>>(a);
+    k_tail_rank<<<kTailMax / kRankBlock, kRankBlock, 0, st>>>(a);
+    k_tail_out<<<2 * sms, 256, 0, st>>>(a);
 }
 
 void launch_adjoint(const AdjointArgs &a, cudaStream_t st) {

@@ -287,7 +287,7 @@ extern "C" tms_status tms_search_noalloc(tms_mesh A, tms_mesh B, const tms_param
 
     // the launch sequence of tms_search, on the static buffers
     launch_search_init(b.bounds, 2, b.ctr, p.cell_filter ? b.bmA : nullptr, 1ull << kBmAWordBits,
-                       p.cell_filter ? b.bmH : nullptr, 1ull << kBmHWordBits, grid, s);
+                       p.cell_filter ? b.bmH : nullptr, 1ull << kBmHWordBits, nullptr, grid, s);
     GroupArgs ga;
     ga.ent_key = b.ek; ga.ent_face = b.ev; ga.d_n = &b.ctr->entries; ga.cap = kEntCap;
     ga.ent_slot = b.eslot; ga.ent_rank = b.erank;
@@ -342,7 +342,8 @@ extern "C" tms_status tms_search_noalloc(tms_mesh A, tms_mesh B, const tms_param
     na.meshes = b.tables->meshes; na.pairs = b.tables->pairs; na.ctr = b.ctr; na.hits = b.hits;
     na.hit_key = b.hk; na.hit_val = b.hv; na.hit_cap = kRawHitCap; na.tau = p.tau;
     na.tri_bits = tri_bits; na.fp32_filter = p.narrow_filter;
-    launch_narrow(na, p.face_level, grid / 2, grid * 4, s);
+    na.tail = nullptr; na.hit_slot = nullptr; na.bscale = 0.0f;
+    launch_narrow(na, p.face_level, grid / 2, s);
     const bool halt = radix_sort(b.hk, b.hv, b.hk2, b.hv2, b.sort_scratch, &b.ctr->raw_hits, kRawHitCap,
                                  2 * tri_bits, 2 * grid, &b.ctr->status,
                                  (unsigned long long)p.spin_limit, (p.inject & 16u) ? 1 : 0, s);
