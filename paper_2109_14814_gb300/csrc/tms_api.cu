@@ -81,6 +81,7 @@ struct Plan {
     int n_meshes = 0;
     MeshDev *d_meshes = nullptr;
     std::vector<MeshDev> h_meshes;    // host copy of the mesh table
+    int2 pair0 = {0, 0};              // pair 0's meshes in it
     // patch level: the patch views (one "face" per patch, its box in pbox),
     // which the cell passes and the grid emission read instead of the meshes
     bool patch = false;
@@ -98,9 +99,10 @@ struct Plan {
     Cand *psurv = nullptr;           // patch pairs left by the quarter test
     unsigned long long ppair_cap = 0;
     int2 *d_pairs = nullptr;
-    PassEntry *d_pass_all = nullptr, *d_pass_A = nullptr, *d_pass_B = nullptr;
-    int n_pass_all = 0, n_pass_A = 0, n_pass_B = 0;
-    long long tiles_all = 0, tiles_A = 0, tiles_B = 0;
+    // the bounds pass takes every mesh once, the cell passes every pair's two sides
+    PassEntry *d_pass_bounds = nullptr, *d_pass_all = nullptr, *d_pass_A = nullptr, *d_pass_B = nullptr;
+    int n_pass_bounds = 0, n_pass_all = 0, n_pass_A = 0, n_pass_B = 0;
+    long long tiles_all = 0;
     long long fslots_all = 0, fslots_A = 0, fslots_B = 0;   // padded face slots per pass
     unsigned long long facesA = 0, facesB = 0;
     int tri_bits = 0, pair_bits = 0;
@@ -132,14 +134,14 @@ struct Plan {
     tms_hit *hits = nullptr;
     uint64_t *hk = nullptr, *hk2 = nullptr, *okeys = nullptr;
     uint32_t *hv = nullptr, *hv2 = nullptr, *keep = nullptr, *kscan = nullptr;
-    int grid = 304;
-    int sort_grid = 608;
     // short merge: bucket counts and drop bits, each bucket's first place
     uint32_t *tail = nullptr, *bbase = nullptr;
     float bscale = 0.0f;
     // more raw hits than the short merge takes: the radix sort and the scans (as
     // a search of this plan found; the look-back test switch needs that sort too)
     bool long_tail = false;
+    int grid = 304;
+    int sort_grid = 608;
     // execution
     cudaStream_t st = nullptr;
     cudaEvent_t ev_in = nullptr, ev_out = nullptr;
@@ -168,8 +170,9 @@ struct Plan {
     ~Plan() {
         if (st) cudaStreamSynchronize(st);
         free_scratch();
-        void *ptrs[] = {d_meshes, d_pairs, d_pass_all, d_pass_A, d_pass_B, d_bounds,
-                        d_ctr, partials, split, fbox, d_pmeshes, pbox, qbox, pframe, d_cm_pair};
+        void *ptrs[] = {d_meshes, d_pairs, d_pass_bounds, d_pass_all, d_pass_A, d_pass_B, d_bounds,
+                        d_ctr, partials, split, fbox, d_pmeshes, pbox, qbox, pframe, d_cm_pair,
+                        tail, bbase};
         for (void *p : ptrs)
             if (p) cudaFree(p);
         if (h_ctr) cudaFreeHost(h_ctr);
@@ -230,9 +233,6 @@ struct Plan {
         else cudaEventRecord(tev[i], s);
     }
 
-    void enqueue(cudaStream_t s) {
-        const tms_params &p = prm;
-        const int prec = p.precision, fl = p.face_level;
     // merge of the raw hits, at most kTailMax of them
     void enqueue_short_tail(cudaStream_t s) {
         mark(13, s);
@@ -265,6 +265,9 @@ struct Plan {
         kernels += 5 + (dOffsets ? 1 : 0);
     }
 
+    void enqueue(cudaStream_t s) {
+        const tms_params &p = prm;
+        const int prec = p.precision, fl = p.face_level;
         const int block = (p.block_faces == 64 || p.block_faces == 256) ? p.block_faces : 128;
         kernels = 0;
         mark(0, s);
@@ -298,7 +301,7 @@ struct Plan {
         fa.ctr = d_ctr;
         fa.ent_cap = ent_cap;
 
-        fa.entries = d_pass_all; fa.n_entries = n_pass_all; fa.total_tiles = tiles_all;
+        fa.entries = d_pass_bounds; fa.n_entries = n_pass_bounds; fa.total_tiles = tiles_all;
         fa.mode = MODE_BOUNDS;
         fa.patch = patch ? 1 : 0;
         fa.frames = frames ? 1 : 0;
@@ -515,8 +518,23 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
 
     std::vector<MeshDev> meshes;
     std::vector<int2> pairs;
-    std::vector<PassEntry> pall, pa, pb;
+    std::vector<PassEntry> pbounds, pall, pa, pb;
     unsigned long long max_tri = 1;
+    const int fl = prm.face_level;
+    // a mesh that is in several pairs has one row of the mesh table and one bounds
+    // pass (a layer sweep takes every half-layer in four pairs: 387 -> 98 us of its
+    // bounds pass at the paper's shapes)
+    std::map<long long, int> row_of;
+    auto row = [&](tms_mesh m) {
+        auto it = row_of.find(m->id);
+        if (it != row_of.end()) return it->second;
+        const int r = (int)meshes.size();
+        meshes.push_back(m->dev);
+        row_of[m->id] = r;
+        long long unused = 0;
+        fill_pass(pbounds, P->tiles_all, unused, m, r, 0, 0, block, rows, fl, patch);
+        return r;
+    };
     for (int i = 0; i < nPairs; ++i) {
         const int ia = row(A[i]), ib = row(B[i]);
         pairs.push_back(make_int2(ia, ib));
@@ -531,12 +549,12 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         max_tri = std::max(max_tri, 2ULL * A[i]->dev.N * A[i]->dev.nqk);
         max_tri = std::max(max_tri, 2ULL * B[i]->dev.N * B[i]->dev.nqk);
     }
-    const int fl = prm.face_level;
+    long long unused = 0;
     for (int i = 0; i < nPairs; ++i) {
-        fill_pass(pall, P->tiles_all, P->fslots_all, A[i], pairs[i].x, i, 0, block, rows, fl, patch);
-        fill_pass(pall, P->tiles_all, P->fslots_all, B[i], pairs[i].y, i, 1, block, rows, fl, patch);
-        fill_pass(pa, P->tiles_A, P->fslots_A, A[i], pairs[i].x, i, 0, block, rows, fl, patch);
-        fill_pass(pb, P->tiles_B, P->fslots_B, B[i], pairs[i].y, i, 1, block, rows, fl, patch);
+        fill_pass(pall, unused, P->fslots_all, A[i], pairs[i].x, i, 0, block, rows, fl, patch);
+        fill_pass(pall, unused, P->fslots_all, B[i], pairs[i].y, i, 1, block, rows, fl, patch);
+        fill_pass(pa, unused, P->fslots_A, A[i], pairs[i].x, i, 0, block, rows, fl, patch);
+        fill_pass(pb, unused, P->fslots_B, B[i], pairs[i].y, i, 1, block, rows, fl, patch);
     }
     // FP32 split vertex copies (32 bytes per view vertex) and face boxes (32 or
     // 64 bytes per face slot), written by the bounds pass
@@ -592,6 +610,8 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     }
     P->n_meshes = (int)meshes.size();
     P->h_meshes = meshes;
+    P->pair0 = pairs[0];
+    P->n_pass_bounds = (int)pbounds.size();
     P->n_pass_all = (int)pall.size();
     P->n_pass_A = (int)pa.size();
     P->n_pass_B = (int)pb.size();
@@ -617,6 +637,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
                            cudaMemcpyHostToDevice));
     }
     TMS_PCK(dalloc(&P->d_pairs, pairs.size()));
+    TMS_PCK(dalloc(&P->d_pass_bounds, pbounds.size()));
     TMS_PCK(dalloc(&P->d_pass_all, pall.size()));
     TMS_PCK(dalloc(&P->d_pass_A, pa.size()));
     TMS_PCK(dalloc(&P->d_pass_B, pb.size()));
@@ -629,6 +650,13 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         P->d_grids = reinterpret_cast<Grid *>(blk + kGridOffset);
     }
     TMS_PCK(dalloc(&P->partials, 5 * 1024));
+    TMS_PCK(dalloc(&P->tail, kTailBuckets + kTailMax / 32));
+    TMS_PCK(dalloc(&P->bbase, kTailBuckets + 1));
+    // the range of (pair, triA), over which the buckets are spread
+    P->bscale = (float)((double)kTailBuckets /
+                        (nPairs == 1 ? 2.0 * A[0]->dev.N * A[0]->dev.nqk
+                                     : (double)nPairs * (double)(1ULL << P->tri_bits)));
+    P->long_tail = (prm.inject & 16u) != 0;
     {
         unsigned char *hb = nullptr;
         TMS_PCK(cudaMallocHost((void **)&hb, kReadback));
@@ -638,6 +666,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     TMS_PCK(cudaMemcpy(P->d_meshes, meshes.data(), meshes.size() * sizeof(MeshDev), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pmeshes, pmeshes.data(), pmeshes.size() * sizeof(MeshDev), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pairs, pairs.data(), pairs.size() * sizeof(int2), cudaMemcpyHostToDevice));
+    TMS_PCK(cudaMemcpy(P->d_pass_bounds, pbounds.data(), pbounds.size() * sizeof(PassEntry), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pass_all, pall.data(), pall.size() * sizeof(PassEntry), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pass_A, pa.data(), pa.size() * sizeof(PassEntry), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pass_B, pb.data(), pb.size() * sizeof(PassEntry), cudaMemcpyHostToDevice));
@@ -650,13 +679,6 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
 
     const unsigned long long faces = P->facesA + P->facesB;
     unsigned long long ent = prm.entry_capacity > 0 ? (unsigned long long)prm.entry_capacity
-    TMS_PCK(dalloc(&P->tail, kTailBuckets + kTailMax / 32));
-    TMS_PCK(dalloc(&P->bbase, kTailBuckets + 1));
-    // the range of (pair, triA), over which the buckets are spread
-    P->bscale = (float)((double)kTailBuckets /
-                        (nPairs == 1 ? 2.0 * A[0]->dev.N * A[0]->dev.nqk
-                                     : (double)nPairs * (double)(1ULL << P->tri_bits)));
-    P->long_tail = (prm.inject & 16u) != 0;
                              : patch ? 4 * faces + (1 << 16)
                              : (prm.cell_filter ? std::max<unsigned long long>(1 << 16, faces / 2)
                                                 : 4 * faces + (1 << 16));
@@ -798,6 +820,10 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
             P->hit_cap = c.raw_hits + c.raw_hits / 4 + 1024;
             grow = true;
         }
+        if (!P->long_tail && c.raw_hits > kTailMax) {
+            P->long_tail = true;
+            grow = true;
+        }
         if (!grow) break;
         ++P->retries;
         TMS_CK(cudaStreamSynchronize(P->st));
@@ -820,10 +846,6 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     st.fp32_solves = (long long)c.fp32;
     st.sat_tests = (long long)c.sat;
     st.quad_tests = (long long)c.quad;
-        if (!P->long_tail && c.raw_hits > kTailMax) {
-            P->long_tail = true;
-            grow = true;
-        }
     st.patch_pairs = (long long)c.ppairs;
     st.patch_tests = (long long)c.ptests;
     st.quad_kept = (long long)c.qkeep;
@@ -1151,8 +1173,8 @@ tms_status tms_last_patch_frames(void *stream, int side, float *host_out, long l
     Plan *P = nullptr;
     for (Plan *Q : g_plans)
         if (Q->user == (cudaStream_t)stream && (!P || Q->last_use > P->last_use)) P = Q;
-    if (!P || !P->frames || (int)P->h_meshes.size() < 2) return TMS_ERR_STATE;
-    const MeshDev &md = P->h_meshes[side];
+    if (!P || !P->frames) return TMS_ERR_STATE;
+    const MeshDev &md = P->h_meshes[side == 0 ? P->pair0.x : P->pair0.y];
     const long long n = (long long)md.npi * md.npk;
     if (n_patches) *n_patches = n;
     if (npi) *npi = md.npi;
