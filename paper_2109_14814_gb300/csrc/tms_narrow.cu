@@ -617,7 +617,7 @@ __device__ __forceinline__ void tri_params(const MeshDev &m, uint32_t t, double 
                                            double &th, double &sv) {
     uint32_t q = t >> 1;
     int tau = t & 1;
-    int i = (int)(q % (uint32_t)m.N), k = (int)(q / (uint32_t)m.N);
+    const int k = (int)__umul64hi((unsigned long long)q, m.nmagic), i = (int)(q - (uint32_t)k * (uint32_t)m.N);
     double dth = kTwoPi / m.N;
     double th_i = i * dth, th_ip = th_i + dth;
     double s_k = m.s[k], s_kp = m.s[k + 1];
@@ -628,7 +628,9 @@ __device__ __forceinline__ void tri_params(const MeshDev &m, uint32_t t, double 
         th = u * th_i + (1.0 - u) * th_ip;
         sv = v * s_k + (1.0 - v) * s_kp;
     }
-    th = fmod(th, kTwoPi);
+    // fmod(th, 2 pi): the weights of a hit lie in [-1, 2] (tau < 1) and dth <= pi, so
+    // -2 pi < th < 4 pi, where one subtraction is exact
+    if (th >= kTwoPi) th -= kTwoPi;
     if (th < 0) th += kTwoPi;
 }
 
@@ -889,8 +891,12 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
     if (lane == 0 && n_quad) atomicAdd(&a.ctr->quad, n_quad);
 }
 
-// Stage 2: the FP64 solve for the survivors
-__global__ void __launch_bounds__(256) k_narrow_fp64(NarrowArgs a) {
+// Stage 2: the FP64 solve for the survivors, one lane each.  Bound by the FP64
+// pipe, which takes 16 cycles an SM for a warp's instruction (two lanes a clock)
+// and by the solve's dependent chain; blocks of one warp, so that a few thousand
+// solves spread over every SM (in blocks of 256, 12,000 of them sat on 48 SMs).
+constexpr int kSolveBlock = 32;
+__global__ void __launch_bounds__(kSolveBlock) k_narrow_fp64(NarrowArgs a) {
     if (a.ctr->cand > a.cand_cap || a.ctr->fp64 > a.surv_cap) return;
     const unsigned long long n = a.ctr->fp64;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -1231,62 +1237,88 @@ __global__ void __launch_bounds__(256) k_tail_out(TailArgs a) {
 // ---------------------------------------------------------------------------
 // adjoint of the hit outputs
 // ---------------------------------------------------------------------------
-__global__ void k_adjoint(AdjointArgs a) {
-    for (long long h = blockIdx.x * (long long)blockDim.x + threadIdx.x; h < a.n;
-         h += (long long)gridDim.x * blockDim.x) {
-        const tms_hit hit = a.hits[h];
+// Two lanes a hit: the first solves A z = r (the hit's weights) while the second
+// solves A^T w = zbar, then the first takes mesh A's gradients and the second mesh
+// B's.  A few hundred hits leave the chip nearly idle, so the time is one chain of
+// loads and dependent FP64 instructions (16 cycles a warp on an SM's FP64 pipe, which
+// eight warps of a 256-thread block shared): blocks of one warp put every warp on an
+// SM of its own, and the two solves run side by side.
+constexpr int kAdjointHits = 16;       // per block of one warp
+__global__ void __launch_bounds__(2 * kAdjointHits) k_adjoint(const __grid_constant__ AdjointArgs a) {
+    const int role = threadIdx.x & 1;
+    const long long step = (long long)gridDim.x * kAdjointHits;
+    for (long long h0 = (long long)blockIdx.x * kAdjointHits; h0 < a.n; h0 += step) {
+        const long long h = h0 + (threadIdx.x >> 1);
+        const bool live = h < a.n;
+        const tms_hit *hit = a.hits + (live ? h : a.n - 1);
+        const uint32_t triA = hit->triA, triB = hit->triB;
         double x[3][4], y[3][4];
-        gather_tri(a.A, hit.triA, x);
-        gather_tri(a.B, hit.triB, y);
-        double M[4][4], Mt[4][4], r[4];
+        gather_tri(a.A, triA, x);
+        gather_tri(a.B, triB, y);
+        // this lane's mesh: vertex offsets, and the alpha derivatives, read ahead of
+        // the solve
+        const MeshDev &m = role ? a.B : a.A;
+        const double *const *dv = role ? a.dB : a.dA;
+        int ii[3], kk[3];
+        tri_ij(m, role ? triB : triA, ii, kk);
+        size_t off[3];
+        double d[3][4];
 #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            M[c][0] = x[0][c] - x[1][c];
-            M[c][1] = x[2][c] - x[1][c];
-            M[c][2] = y[1][c] - y[0][c];
-            M[c][3] = y[1][c] - y[2][c];
-            r[c] = y[1][c] - x[1][c];
+        for (int j = 0; j < 3; ++j) {
+            off[j] = (size_t)kk[j] * m.N + ii[j];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) d[j][c] = dv[c] ? __ldg(dv[c] + off[j]) : 0.0;
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) Mt[i][j] = M[j][i];
         double gP[4] = {0, 0, 0, 0}, zbar[4] = {0, 0, 0, 0};
-        if (a.gP) for (int c = 0; c < 4; ++c) gP[c] = a.gP[4 * h + c];
-        if (a.gZ) for (int c = 0; c < 4; ++c) zbar[c] = a.gZ[4 * h + c];
+        const long long hr = live ? h : a.n - 1;
+        if (a.gP) for (int c = 0; c < 4; ++c) gP[c] = a.gP[4 * hr + c];
+        if (a.gZ) for (int c = 0; c < 4; ++c) zbar[c] = a.gZ[4 * hr + c];
+        double M[4][4], rhs[4];
+        {
+            double F[4][4], r[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                F[c][0] = x[0][c] - x[1][c];
+                F[c][1] = x[2][c] - x[1][c];
+                F[c][2] = y[1][c] - y[0][c];
+                F[c][3] = y[1][c] - y[2][c];
+                r[c] = y[1][c] - x[1][c];
+                zbar[0] += F[c][0] * gP[c];
+                zbar[1] += F[c][1] * gP[c];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) M[i][j] = role ? F[j][i] : F[i][j];
+                rhs[i] = role ? zbar[i] : r[i];
+            }
+        }
+        double s[4], det;
+        bool ok = solve4_gepp<double>(M, rhs, s, det);
+        ok &= __shfl_xor_sync(FULL, (int)ok, 1) != 0;
+        double z[4], w[4];
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            zbar[0] += M[c][0] * gP[c];
-            zbar[1] += M[c][1] * gP[c];
+            const double o = __shfl_xor_sync(FULL, s[c], 1);
+            z[c] = role ? o : s[c];
+            w[c] = role ? s[c] : o;
         }
-        double z[4], det, w[4], det2;
-        const bool ok1 = solve4_gepp<double>(M, r, z, det);
-        const bool ok2 = solve4_gepp<double>(Mt, zbar, w, det2);
-        if (!(ok1 && ok2)) {
-            if (a.galpha) a.galpha[h] = 0.0;
-            continue;
-        }
-        const double beta[3] = {z[0], 1.0 - z[0] - z[1], z[1]};
-        const double gam[3] = {z[2], 1.0 - z[2] - z[3], z[3]};
-        int iA[3], kA[3], iB[3], kB[3];
-        tri_ij(a.A, hit.triA, iA, kA);
-        tri_ij(a.B, hit.triB, iB, kB);
+        // weights of this lane's triangle, and its share of the gradient
+        const double u = role ? z[2] : z[0], v = role ? z[3] : z[1];
+        const double wt[3] = {u, 1.0 - u - v, v};
+        double *const *g = role ? a.gB : a.gA;
         double ga = 0.0;
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
-            const size_t oa = (size_t)kA[j] * a.A.N + iA[j];
-            const size_t ob = (size_t)kB[j] * a.B.N + iB[j];
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
-                const double gx = beta[j] * (gP[c] - w[c]);
-                const double gy = gam[j] * w[c];
-                if (a.gA[c]) atomicAdd(a.gA[c] + oa, gx);
-                if (a.gB[c]) atomicAdd(a.gB[c] + ob, gy);
-                if (a.dA[c]) ga += gx * a.dA[c][oa];
-                if (a.dB[c]) ga += gy * a.dB[c][ob];
+                const double gv = wt[j] * (role ? w[c] : gP[c] - w[c]);
+                if (live && ok && g[c]) atomicAdd(g[c] + off[j], gv);
+                ga += gv * d[j][c];
             }
         }
-        if (a.galpha) a.galpha[h] = ga;
+        ga += __shfl_xor_sync(FULL, ga, 1);
+        if (a.galpha && live && role == 0) a.galpha[h] = ok ? ga : 0.0;
     }
 }
 
@@ -1327,7 +1359,7 @@ void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st
         if (a.fp32_filter) k_quad_filter<<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
         k_narrow_filter<1><<<sms * filter_resident<1>(), 256, 0, st>>>(a);
     }
-    k_narrow_fp64<<<sms * 8, 256, 0, st>>>(a);
+    k_narrow_fp64<<<sms * 16, kSolveBlock, 0, st>>>(a);
 }
 
 void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st) {
@@ -1347,9 +1379,8 @@ void launch_tail(const TailArgs &a, int sms, cudaStream_t st) {
 
 void launch_adjoint(const AdjointArgs &a, cudaStream_t st) {
     if (a.n <= 0) return;
-    int grid = (int)((a.n + 255) / 256);
-    if (grid > 4096) grid = 4096;
-    k_adjoint<<<grid, 256, 0, st>>>(a);
+    const long long blocks = (a.n + kAdjointHits - 1) / kAdjointHits;
+    k_adjoint<<<(unsigned)(blocks < (1 << 16) ? blocks : (1 << 16)), 2 * kAdjointHits, 0, st>>>(a);
 }
 
 }  // namespace tms
