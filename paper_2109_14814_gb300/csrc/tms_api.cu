@@ -126,10 +126,8 @@ struct Plan {
     unsigned long long *partials = nullptr;
     Cand *cand = nullptr, *surv = nullptr;
     uint32_t *qsurv = nullptr;        // candidates left by the quad-level test
-    float4 *split = nullptr;          // FP32 split vertex copies of all meshes
-    unsigned long long split_total = 0;
-    std::vector<unsigned long long> split_off;
-    unsigned char *fbox = nullptr;    // face boxes of all meshes
+    float4 *vlo = nullptr;            // vertices of all meshes rounded down to FP32
+    unsigned char *fbox = nullptr;    // face boxes of all meshes (face level)
     unsigned long long surv_cap = 0;
     tms_hit *hits = nullptr;
     uint64_t *hk = nullptr, *hk2 = nullptr, *okeys = nullptr;
@@ -171,7 +169,7 @@ struct Plan {
         if (st) cudaStreamSynchronize(st);
         free_scratch();
         void *ptrs[] = {d_meshes, d_pairs, d_pass_bounds, d_pass_all, d_pass_A, d_pass_B, d_bounds,
-                        d_ctr, partials, split, fbox, d_pmeshes, pbox, qbox, pframe, d_cm_pair,
+                        d_ctr, partials, vlo, fbox, d_pmeshes, pbox, qbox, pframe, d_cm_pair,
                         tail, bbase};
         for (void *p : ptrs)
             if (p) cudaFree(p);
@@ -384,7 +382,7 @@ struct Plan {
         na.tau = p.tau; na.tri_bits = tri_bits; na.fp32_filter = p.narrow_filter;
         na.tail = long_tail ? nullptr : tail; na.hit_slot = kscan; na.bscale = bscale;
         launch_narrow(na, fl, grid / 2, s);
-        kernels += fl == 1 && p.narrow_filter ? 3 : 2;
+        kernels += p.narrow_filter ? 3 : 2;
         mark(12, s);
         if (long_tail) enqueue_long_tail(s);
         else enqueue_short_tail(s);
@@ -556,16 +554,20 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         fill_pass(pa, unused, P->fslots_A, A[i], pairs[i].x, i, 0, block, rows, fl, patch);
         fill_pass(pb, unused, P->fslots_B, B[i], pairs[i].y, i, 1, block, rows, fl, patch);
     }
-    // FP32 split vertex copies (32 bytes per view vertex) and face boxes (32 or
-    // 64 bytes per face slot), written by the bounds pass
+    // written by the bounds pass: the vertices rounded down to FP32 (16 bytes each;
+    // the plain precision without the FP32 filters reads none) and, at the face
+    // level, the face boxes (32 or 64 bytes per face slot)
+    const bool keep_vlo = prm.precision == 1 || prm.narrow_filter != 0;
+    std::vector<unsigned long long> vlo_off;
+    unsigned long long vlo_total = 0;
     const unsigned long long box_bytes = prm.precision == 1 ? 32 : 64;
     std::vector<unsigned long long> fbox_off, pbox_off, pframe_off;
     unsigned long long fbox_total = 0, pbox_total = 0, pframe_total = 0;
     for (auto &md : meshes) {
-        P->split_off.push_back(P->split_total);
-        P->split_total += 2ULL * (unsigned long long)md.N * (unsigned long long)md.M;
+        vlo_off.push_back(vlo_total);
+        if (keep_vlo) vlo_total += (unsigned long long)md.N * (unsigned long long)md.M;
         fbox_off.push_back(fbox_total);
-        fbox_total += (face_slots(md, fl) * box_bytes + 255) / 256 * 256;
+        if (!patch) fbox_total += (face_slots(md, fl) * box_bytes + 255) / 256 * 256;
         md.npi = patch ? (md.nqi + kPatchI - 1) / kPatchI : 0;
         md.npk = patch ? (md.nqk + kPatchK - 1) / kPatchK : 0;
         md.pmagic = recip64((unsigned long long)md.npi);
@@ -579,15 +581,15 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     }
     std::vector<MeshDev> pmeshes;
     {
-        cudaError_t se = dalloc(&P->split, P->split_total);
-        if (se == cudaSuccess) se = dalloc(&P->fbox, fbox_total);
+        cudaError_t se = dalloc(&P->vlo, vlo_total);
+        if (se == cudaSuccess && !patch) se = dalloc(&P->fbox, fbox_total);
         if (se == cudaSuccess && patch) se = dalloc(&P->pbox, pbox_total);
         if (se == cudaSuccess && patch) se = dalloc(&P->qbox, 4 * pbox_total);
         if (se == cudaSuccess && P->frames) se = dalloc(&P->pframe, pframe_total);
         if (se != cudaSuccess) { g_err = cudaGetErrorString(se); delete P; return TMS_ERR_CUDA; }
         for (size_t i = 0; i < meshes.size(); ++i) {
-            meshes[i].split = P->split + P->split_off[i];
-            meshes[i].fbox = P->fbox + fbox_off[i];
+            meshes[i].vlo = keep_vlo ? P->vlo + vlo_off[i] : nullptr;
+            meshes[i].fbox = patch ? nullptr : P->fbox + fbox_off[i];
             if (patch) {
                 meshes[i].pbox = P->pbox + pbox_off[i];
                 meshes[i].qbox = P->qbox + 4 * pbox_off[i];
@@ -603,7 +605,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
             v.nqi = md.npi;
             v.nqk = md.npk;
             v.fbox = md.pbox;
-            v.split = nullptr;
+            v.vlo = nullptr;
             v.pframe = nullptr;
             pmeshes.push_back(v);
         }

@@ -49,14 +49,15 @@ enum StatusBits : unsigned int {
 struct MeshDev {
     const double *c[4];   // x, y, px, py, offset to the first view column
     const double *s;      // s values of the view (M entries), device
-    float4 *split;        // plan scratch: the FP32 split of every view vertex
-                          // (k*N + i): hi = RN32(x) at [k*N + i], lo = RN32(x - hi)
-                          // at [N*M + k*N + i] (hi and lo in separate halves, so a
-                          // gather of the hi parts alone reads dense 16-byte rows),
-                          // written by the bounds pass, gathered by the narrow filters
-    void *fbox;           // plan scratch: per face slot its box, written by the
-                          // bounds pass (mixed precision: float4 lo, float4 hi,
-                          // rounded outward; plain: 8 doubles lo[4], hi[4]);
+    float4 *vlo;          // plan scratch: every view vertex (k*N + i) rounded
+                          // down to FP32, written by the bounds pass; the boxes
+                          // of the quads at the patch level and the quad-level
+                          // narrow test are made from it (NULL: the plain
+                          // precision without the FP32 filters has no use for it)
+    void *fbox;           // plan scratch, face level only: per face slot its box,
+                          // written by the bounds pass (mixed precision: float4
+                          // lo, float4 hi, rounded outward; plain: 8 doubles
+                          // lo[4], hi[4]);
                           // slot = face id (quad k*N + i, or triangle 2(k*N + i) + t)
     int N;                // theta samples
     int M;                // vertex rows in the view
@@ -351,21 +352,25 @@ __device__ __forceinline__ float f32_special(unsigned long long b, int e32, int 
     if (dir < 0) return neg ? -1.17549435e-38f : 0.0f;
     return neg ? -0.0f : 1.17549435e-38f;
 }
+// round down.  In the FP32 normal range the bits of |x| shifted right by 29, less the
+// exponents' difference, are the truncated FP32 magnitude
 __device__ __forceinline__ float f32_rd(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int e32 = (int)((b >> 52) & 0x7ff) - 896;
-    if (e32 <= 0 || e32 >= 255) return f32_special(b, e32, -1);
-    unsigned f = f32_bits_trunc(b, e32);
-    f += (unsigned)(b >> 63) & (unsigned)((b & 0x1FFFFFFFULL) != 0);   // negative, inexact
-    return __uint_as_float(f);
+    const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
+    const unsigned mag = h & 0x7fffffffu;
+    if (mag - (897u << 20) >= (254u << 20))
+        return f32_special((unsigned long long)__double_as_longlong(x), (int)(mag >> 20) - 896, -1);
+    unsigned f = __funnelshift_r(l, mag, 29) - (896u << 23);
+    if ((int)h < 0 && (l & 0x1FFFFFFFu) != 0u) ++f;                    // negative, inexact
+    return __uint_as_float(f | (h & 0x80000000u));
 }
-__device__ __forceinline__ float f32_ru(double x) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int e32 = (int)((b >> 52) & 0x7ff) - 896;
-    if (e32 <= 0 || e32 >= 255) return f32_special(b, e32, +1);
-    unsigned f = f32_bits_trunc(b, e32);
-    f += ((unsigned)(b >> 63) ^ 1u) & (unsigned)((b & 0x1FFFFFFFULL) != 0);  // positive, inexact
-    return __uint_as_float(f);
+// an upper bound of every x with f32_rd(x) = f: the next FP32 number; outside the
+// normal range as f32_special rounds (an exact x is over by one place too, so that
+// the value rounded down is all a vertex has to keep)
+__device__ __forceinline__ float f32_above(float f) {
+    const int b = __float_as_int(f);
+    const float up = __int_as_float(b + (b >= 0 ? 1 : -1));
+    const float least = 1.17549435e-38f;
+    return f <= 0.0f && f >= -least ? (f < 0.0f ? 0.0f : least) : up;
 }
 __device__ __forceinline__ float f32_rn(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
@@ -606,38 +611,6 @@ __device__ __forceinline__ void split_f32(double x, float &hi, float &lo) {
     // outside that range lo is 0 and the caller's error bound carries an absolute
     // term for coordinates below 2^-74
     lo = (b >> 63) ? -l : l;
-}
-
-// All four FP32 roundings the bounds pass needs from one decomposition of x:
-// rd / ru the FP32 numbers just below and above x (outward box bounds) and the
-// split hi = RN32(x), lo = RN32(x - hi); identical to f32_rd, f32_ru and
-// split_f32, which take the special cases (zero, subnormal, huge, NaN).
-__device__ __forceinline__ void f32_all(double x, float &rd, float &ru, float &hi, float &lo) {
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7ff);
-    const int e32 = e - 896;
-    if (e32 <= 0 || e32 >= 255) {
-        rd = f32_rd(x);
-        ru = f32_ru(x);
-        split_f32(x, hi, lo);
-        return;
-    }
-    const unsigned long long m = b & 0xFFFFFFFFFFFFFULL;
-    const unsigned mag = ((unsigned)e32 << 23) | (unsigned)(m >> 29);   // truncated |x|
-    const unsigned rem = (unsigned)(m & 0x1FFFFFFFULL);               // the 29 bits dropped
-    const unsigned neg = (unsigned)(b >> 63);
-    const unsigned sgn = neg << 31;
-    const unsigned inexact = rem != 0u;
-    rd = __uint_as_float(sgn | (mag + (neg & inexact)));
-    ru = __uint_as_float(sgn | (mag + ((neg ^ 1u) & inexact)));
-    const unsigned up = (unsigned)(rem > 0x10000000u) | ((unsigned)(rem == 0x10000000u) & (mag & 1u));
-    hi = __uint_as_float(sgn | (mag + up));
-    // x - hi = (rem - up 2^29) ulp, ulp = 2^(e - 1075)
-    const int r = up ? (int)rem - (1 << 29) : (int)rem;
-    const int ex = e - 1075 + 127;
-    float l = 0.0f;
-    if (ex >= 1) l = __int2float_rn(r) * __uint_as_float((unsigned)ex << 23);
-    lo = neg ? -l : l;
 }
 
 struct DedupArgs {

@@ -4,8 +4,9 @@
 //   bounds pass      (one read of every vertex) per-mesh world bounds, widest
 //                    face extent per coordinate (the grid rule of Sec. 6.2.1:
 //                    cell edge > widest face), a finiteness check of every
-//                    vertex, the box of every face (Sec. 6.2.2) and the FP32
-//                    split copy of the vertices for the narrow filter;
+//                    vertex, the vertices rounded down to FP32, and the box of
+//                    every face (Sec. 6.2.2; at the patch level the boxes of the
+//                    patches and their quarters);
 //   cell passes      (one read of every face box) the cells each face covers:
 //     MODE_MARK        occupancy bits of the cells covered by mesh A's faces;
 //     MODE_PROBE_MARK  mesh B: one entry per face-cell incidence in a cell that
@@ -20,8 +21,8 @@
 //
 // Bounds pass tiling: a block owns a tile of TI quads along theta x TK quad
 // rows.  All (TI+1) x (TK+1) vertices of the tile are loaded once, coalesced
-// along theta, into shared memory (converted to FP32 lower/upper bounds in the
-// mixed precision mode), then each thread builds the boxes of its quads' faces.
+// along theta, into shared memory (rounded down to FP32 in the mixed precision
+// mode), then each thread builds the boxes of its quads' faces.
 //
 // Cell passes: one thread per face slot; a warp expands its 32 faces' cell
 // ranges into one list of (face, cell) items and works through it 32 items at
@@ -41,96 +42,69 @@ namespace {
 
 constexpr unsigned FULL = 0xffffffffu;
 
+// A vertex as the boxes need it: its coordinates rounded down to FP32 (mixed
+// precision; every exact coordinate then lies in [v, f32_above(v)], so the box of a
+// set of vertices is [min v, f32_above(max v)] and one value a coordinate does), or
+// as they are (plain).
 template <int PREC>
-struct Vtx;
-
-// mixed precision: a vertex as FP32 lower and upper bounds of its coordinates
+struct Num;
 template <>
-struct Vtx<1> {
-    float lo[4], hi[4];
+struct Num<1> {
+    typedef float T;
+    static __device__ __forceinline__ float of(double x) { return f32_rd(x); }
+    static __device__ __forceinline__ float above(float v) { return f32_above(v); }
+    static __device__ __forceinline__ float inf() { return __int_as_float(0x7f800000); }
 };
-
-// plain FP64
 template <>
-struct Vtx<0> {
-    double v[4];
+struct Num<0> {
+    typedef double T;
+    static __device__ __forceinline__ double of(double x) { return x; }
+    static __device__ __forceinline__ double above(double v) { return v; }
+    static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000LL); }
 };
 
 template <int PREC>
-struct BoxT;
-template <>
-struct BoxT<1> {
-    float lo[4], hi[4];
-};
-template <>
-struct BoxT<0> {
-    double lo[4], hi[4];
+struct __align__(16) Vtx {
+    typename Num<PREC>::T v[4];
 };
 
-__device__ __forceinline__ void box_init(BoxT<1> &b, const Vtx<1> &v) {
-#pragma unroll
-    for (int d = 0; d < 4; ++d) { b.lo[d] = v.lo[d]; b.hi[d] = v.hi[d]; }
-}
-__device__ __forceinline__ void box_add(BoxT<1> &b, const Vtx<1> &v) {
-#pragma unroll
-    for (int d = 0; d < 4; ++d) { b.lo[d] = fminf(b.lo[d], v.lo[d]); b.hi[d] = fmaxf(b.hi[d], v.hi[d]); }
-}
-__device__ __forceinline__ void box_init(BoxT<0> &b, const Vtx<0> &v) {
+// lo: the least, hi: the largest vertex value (closed() makes it the box)
+template <int PREC>
+struct BoxT {
+    typename Num<PREC>::T lo[4], hi[4];
+};
+
+template <int PREC>
+__device__ __forceinline__ void box_init(BoxT<PREC> &b, const Vtx<PREC> &v) {
 #pragma unroll
     for (int d = 0; d < 4; ++d) { b.lo[d] = v.v[d]; b.hi[d] = v.v[d]; }
 }
-__device__ __forceinline__ void box_add(BoxT<0> &b, const Vtx<0> &v) {
-#pragma unroll
-    for (int d = 0; d < 4; ++d) { b.lo[d] = fmin(b.lo[d], v.v[d]); b.hi[d] = fmax(b.hi[d], v.v[d]); }
-}
-
-__device__ __forceinline__ void to_vtx(const double x[4], Vtx<1> &v) {
-#pragma unroll
-    for (int d = 0; d < 4; ++d) {
-        v.lo[d] = f32_rd(x[d]);
-        v.hi[d] = f32_ru(x[d]);
-    }
-}
-__device__ __forceinline__ void to_vtx(const double x[4], Vtx<0> &v) {
-#pragma unroll
-    for (int d = 0; d < 4; ++d) v.v[d] = x[d];
-}
-
-// FP32 split copy of a vertex (hi and lo float4), gathered later by the FP32
-// narrow filter: one 32-byte record per vertex instead of four 8-byte loads
-__device__ __forceinline__ void write_split(const MeshDev &m, size_t idx, const double x[4]) {
-    float4 hi, lo;
-    split_f32(x[0], hi.x, lo.x);
-    split_f32(x[1], hi.y, lo.y);
-    split_f32(x[2], hi.z, lo.z);
-    split_f32(x[3], hi.w, lo.w);
-    m.split[idx] = hi;
-    m.split[(size_t)m.N * m.M + idx] = lo;
-}
-
-// The tile's own vertex: its FP32 bounds for the boxes and its split copy,
-// from one decomposition per coordinate in the mixed mode.
 template <int PREC>
-__device__ __forceinline__ void vtx_and_split(const double x[4], Vtx<PREC> &out, const MeshDev &m,
-                                              size_t idx);
-template <>
-__device__ __forceinline__ void vtx_and_split<1>(const double x[4], Vtx<1> &out, const MeshDev &m,
-                                                 size_t idx) {
-    Vtx<1> v;
-    float4 hi, lo;
-    f32_all(x[0], v.lo[0], v.hi[0], hi.x, lo.x);
-    f32_all(x[1], v.lo[1], v.hi[1], hi.y, lo.y);
-    f32_all(x[2], v.lo[2], v.hi[2], hi.z, lo.z);
-    f32_all(x[3], v.lo[3], v.hi[3], hi.w, lo.w);
-    out = v;
-    m.split[idx] = hi;
-    m.split[(size_t)m.N * m.M + idx] = lo;
+__device__ __forceinline__ void box_add(BoxT<PREC> &b, const Vtx<PREC> &v) {
+#pragma unroll
+    for (int d = 0; d < 4; ++d) { b.lo[d] = min(b.lo[d], v.v[d]); b.hi[d] = max(b.hi[d], v.v[d]); }
 }
-template <>
-__device__ __forceinline__ void vtx_and_split<0>(const double x[4], Vtx<0> &out, const MeshDev &m,
-                                                 size_t idx) {
-    to_vtx(x, out);
-    write_split(m, idx, x);
+template <int PREC>
+__device__ __forceinline__ BoxT<PREC> closed(BoxT<PREC> b) {
+#pragma unroll
+    for (int d = 0; d < 4; ++d) b.hi[d] = Num<PREC>::above(b.hi[d]);
+    return b;
+}
+
+template <int PREC>
+__device__ __forceinline__ Vtx<PREC> to_vtx(const double x[4]) {
+    Vtx<PREC> v;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) v.v[d] = Num<PREC>::of(x[d]);
+    return v;
+}
+
+// the rounded vertex, gathered later (MeshDev::vlo)
+__device__ __forceinline__ void write_vlo(const MeshDev &m, size_t idx, const Vtx<1> &v) {
+    m.vlo[idx] = make_float4(v.v[0], v.v[1], v.v[2], v.v[3]);
+}
+__device__ __forceinline__ void write_vlo(const MeshDev &m, size_t idx, const Vtx<0> &v) {
+    if (m.vlo) m.vlo[idx] = make_float4(f32_rd(v.v[0]), f32_rd(v.v[1]), f32_rd(v.v[2]), f32_rd(v.v[3]));
 }
 
 template <int PREC>
@@ -154,7 +128,7 @@ struct GridView<0> {
     }
 };
 
-// the box of a face (or patch) into slot `face` of a box array
+// the (closed) box of a face or patch into slot `face` of a box array
 template <int PREC>
 __device__ __forceinline__ void write_box(void *arr, uint32_t face, const BoxT<PREC> &b);
 template <>
@@ -173,17 +147,14 @@ __device__ __forceinline__ void write_box<0>(void *arr, uint32_t face, const Box
 }
 template <int PREC>
 __device__ __forceinline__ void write_fbox(const MeshDev &m, uint32_t face, const BoxT<PREC> &b) {
-    write_box<PREC>(m.fbox, face, b);
+    write_box<PREC>(m.fbox, face, closed<PREC>(b));
 }
 
 // a box that contains nothing (identity of the union)
-__device__ __forceinline__ void box_empty(BoxT<1> &b) {
+template <int PREC>
+__device__ __forceinline__ void box_empty(BoxT<PREC> &b) {
 #pragma unroll
-    for (int d = 0; d < 4; ++d) { b.lo[d] = __int_as_float(0x7f800000); b.hi[d] = -b.lo[d]; }
-}
-__device__ __forceinline__ void box_empty(BoxT<0> &b) {
-#pragma unroll
-    for (int d = 0; d < 4; ++d) { b.lo[d] = __longlong_as_double(0x7ff0000000000000LL); b.hi[d] = -b.lo[d]; }
+    for (int d = 0; d < 4; ++d) { b.lo[d] = Num<PREC>::inf(); b.hi[d] = -b.lo[d]; }
 }
 template <int PREC>
 __device__ __forceinline__ void box_union(BoxT<PREC> &b, const BoxT<PREC> &x) {
@@ -223,64 +194,24 @@ __device__ __forceinline__ void read_fbox<0>(const MeshDev &m, uint32_t face, Bo
 // Per-thread accumulators of the bounds pass, in the box precision (FP32
 // min/max in the mixed mode: FP64 arithmetic is a scarce pipe on GB300)
 template <int PREC>
-struct BoundAcc;
-template <>
-struct BoundAcc<1> {
-    float lo[4], hi[4], w[4];
+struct BoundAcc {
+    typename Num<PREC>::T lo[4], hi[4], w[4];
     unsigned seen;
     __device__ void init() {
 #pragma unroll
-        for (int d = 0; d < 4; ++d) { lo[d] = __int_as_float(0x7f800000); hi[d] = -lo[d]; w[d] = 0.0f; }
+        for (int d = 0; d < 4; ++d) { lo[d] = Num<PREC>::inf(); hi[d] = -lo[d]; w[d] = 0; }
         seen = 0;
     }
-    __device__ void add(const BoxT<1> &b) {
-        add_bounds(b);
-        add_width(b);
-    }
-    __device__ void add_bounds(const BoxT<1> &b) {
+    __device__ void add(const BoxT<PREC> &raw) {
+        const BoxT<PREC> b = closed<PREC>(raw);
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
-            lo[d] = fminf(lo[d], b.lo[d]);
-            hi[d] = fmaxf(hi[d], b.hi[d]);
+            lo[d] = min(lo[d], b.lo[d]);
+            hi[d] = max(hi[d], b.hi[d]);
+            w[d] = max(w[d], b.hi[d] - b.lo[d]);
         }
         seen = 1;
     }
-    __device__ void add_width(const BoxT<1> &b) {
-#pragma unroll
-        for (int d = 0; d < 4; ++d) w[d] = fmaxf(w[d], b.hi[d] - b.lo[d]);
-    }
-    __device__ double get_lo(int d) const { return (double)lo[d]; }
-    __device__ double get_hi(int d) const { return (double)hi[d]; }
-    __device__ double get_w(int d) const { return (double)w[d]; }
-};
-template <>
-struct BoundAcc<0> {
-    double lo[4], hi[4], w[4];
-    unsigned seen;
-    __device__ void init() {
-#pragma unroll
-        for (int d = 0; d < 4; ++d) { lo[d] = __longlong_as_double(0x7ff0000000000000LL); hi[d] = -lo[d]; w[d] = 0.0; }
-        seen = 0;
-    }
-    __device__ void add(const BoxT<0> &b) {
-        add_bounds(b);
-        add_width(b);
-    }
-    __device__ void add_bounds(const BoxT<0> &b) {
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-            lo[d] = fmin(lo[d], b.lo[d]);
-            hi[d] = fmax(hi[d], b.hi[d]);
-        }
-        seen = 1;
-    }
-    __device__ void add_width(const BoxT<0> &b) {
-#pragma unroll
-        for (int d = 0; d < 4; ++d) w[d] = fmax(w[d], b.hi[d] - b.lo[d]);
-    }
-    __device__ double get_lo(int d) const { return lo[d]; }
-    __device__ double get_hi(int d) const { return hi[d]; }
-    __device__ double get_w(int d) const { return w[d]; }
 };
 
 // ord_enc of the value as a double: FP64 values directly; FP32 values through the
@@ -359,7 +290,7 @@ __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x
 // d = V - c:
 //   |d|_inf <= D = max_i max(pb.hi_i - c_i, c_i - pb.lo_i)   (all V in pb)
 //   hi_i - lo_i <= 2^-23 L + 2^-149                           (adjacent floats)
-//   d~ = fl(hi - c): |d_i - d~_i| <= (hi_i - lo_i) + u |d~_i|, |d~_i| <= D (1 + u)
+//   d~ = fl(lo - c): |d_i - d~_i| <= (hi_i - lo_i) + u |d~_i|, |d~_i| <= D (1 + u)
 //   a~_k = fl(e_k . d~) (4 FMAs, error <= gamma_4 sum_i |e_ki||d~_i|, gamma_4 <
 //   4.0001 u), so |e_k . d - a~_k| <= n_k nu, nu = 2^-23 L + 5.001 u D (+ 2^-149)
 //   and h_k = max |a~_k| + n_k nu (n_k >= |e_k|_1);
@@ -384,10 +315,10 @@ __device__ __forceinline__ void patch_frame(const Vtx<1> *sv, int W, int t, int 
     D *= 1.0001f;
     float t1[4] = {0.0f, 0.0f, 0.0f, 0.0f}, t2[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (patch_lane) {
-        const float4 v00 = *reinterpret_cast<const float4 *>(sv[pr0 * W + p0].hi);
-        const float4 v01 = *reinterpret_cast<const float4 *>(sv[pr0 * W + p0 + cq].hi);
-        const float4 v10 = *reinterpret_cast<const float4 *>(sv[pr1 * W + p0].hi);
-        const float4 v11 = *reinterpret_cast<const float4 *>(sv[pr1 * W + p0 + cq].hi);
+        const float4 v00 = *reinterpret_cast<const float4 *>(sv[pr0 * W + p0].v);
+        const float4 v01 = *reinterpret_cast<const float4 *>(sv[pr0 * W + p0 + cq].v);
+        const float4 v10 = *reinterpret_cast<const float4 *>(sv[pr1 * W + p0].v);
+        const float4 v11 = *reinterpret_cast<const float4 *>(sv[pr1 * W + p0 + cq].v);
         t1[0] = (v01.x - v00.x) + (v11.x - v10.x); t2[0] = (v10.x - v00.x) + (v11.x - v01.x);
         t1[1] = (v01.y - v00.y) + (v11.y - v10.y); t2[1] = (v10.y - v00.y) + (v11.y - v01.y);
         t1[2] = (v01.z - v00.z) + (v11.z - v10.z); t2[2] = (v10.z - v00.z) + (v11.z - v01.z);
@@ -436,7 +367,7 @@ __device__ __forceinline__ void patch_frame(const Vtx<1> *sv, int W, int t, int 
     // maximum keeps NaN
     unsigned am[4] = {0u, 0u, 0u, 0u};
     auto vertex = [&](const Vtx<1> &v) {
-        const float4 hv = *reinterpret_cast<const float4 *>(v.hi);
+        const float4 hv = *reinterpret_cast<const float4 *>(v.v);
         const float d[4] = {hv.x - c[0], hv.y - c[1], hv.z - c[2], hv.w - c[3]};
 #pragma unroll
         for (int k = 0; k < 4; ++k) am[k] = max(am[k], abs_bits(dot4f(E[k], d)));
@@ -532,18 +463,17 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
                 for (int c = 0; c < 4; ++c) x[r][c] = __ldg(m.c[c] + off);
             }
         }
-        // a vertex's split copy is written by the tile that owns it: rows below the
-        // tile's last (the next tile's first) and the mesh's last row
+        // a vertex is written by the tile that owns it: rows below the tile's last
+        // (the next tile's first) and the mesh's last row
         const bool last_rows = kq0 + rows_q == m.nqk;
 #pragma unroll
         for (int r = 0; r <= TK; ++r) {
             if (col_ok && r <= rows_q) {
 #pragma unroll
                 for (int c = 0; c < 4; ++c) nonfinite |= !finite64(x[r][c]);
-                if (r < rows_q || last_rows)
-                    vtx_and_split<PREC>(x[r], sv[r * W + t], m, (size_t)(kq0 + r) * m.N + vi);
-                else
-                    to_vtx(x[r], sv[r * W + t]);
+                const Vtx<PREC> v = to_vtx<PREC>(x[r]);
+                sv[r * W + t] = v;
+                if (r < rows_q || last_rows) write_vlo(m, (size_t)(kq0 + r) * m.N + vi, v);
             }
         }
         // the last vertex column of the tile (wraps to column 0 on a periodic mesh);
@@ -558,9 +488,9 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
                 y[c] = __ldg(m.c[c] + off);
                 nonfinite |= !finite64(y[c]);
             }
-            const bool own_col = !m.periodic && vj == m.N - 1 && (t < rows_q || last_rows);
-            if (own_col) vtx_and_split<PREC>(y, sv[t * W + cols_q], m, off);
-            else to_vtx(y, sv[t * W + cols_q]);
+            const Vtx<PREC> v = to_vtx<PREC>(y);
+            sv[t * W + cols_q] = v;
+            if (!m.periodic && vj == m.N - 1 && (t < rows_q || last_rows)) write_vlo(m, off, v);
         }
     }
     __syncthreads();
@@ -601,9 +531,6 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
                     bq.lo[d] = min(prev.lo[d], next.lo[d]);
                     bq.hi[d] = max(prev.hi[d], next.hi[d]);
                 }
-                const uint32_t q = (uint32_t)(kq0 + r) * (uint32_t)m.N + (uint32_t)i;
-                acc.add_bounds(bq);
-                write_fbox<PREC>(m, q, bq);
                 if ((r % kPatchK) < kPatchK / 2) box_union<PREC>(ptop, bq);
                 else box_union<PREC>(pbot, bq);
                 prev = next;
@@ -619,12 +546,12 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
                                    (uint32_t)(i / kPatchI);
                 if (patch_lane && (t % (kPatchI / 2)) == 0) {
                     const uint32_t half = (uint32_t)((t % kPatchI) / (kPatchI / 2));
-                    write_box<PREC>(m.qbox, 4 * p + half, ptop);
-                    write_box<PREC>(m.qbox, 4 * p + 2 + half, pbot);
+                    write_box<PREC>(m.qbox, 4 * p + half, closed<PREC>(ptop));
+                    write_box<PREC>(m.qbox, 4 * p + 2 + half, closed<PREC>(pbot));
                 }
                 if (patch_lane && (t % kPatchI) == 0) {
-                    write_box<PREC>(m.pbox, p, pb);
-                    acc.add_width(pb);
+                    write_box<PREC>(m.pbox, p, closed<PREC>(pb));
+                    acc.add(pb);
                 }
                 if (r < kPatchK) pb0 = pb;
                 else pb1 = pb;
@@ -637,7 +564,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
         if constexpr (PREC == 1) {
             if (a.frames) {
                 for (int pr = 0; pr * kPatchK < rows_q; ++pr) {
-                    const BoxT<1> pbx = pr == 0 ? pb0 : pb1;
+                    const BoxT<1> pbx = closed<1>(pr == 0 ? pb0 : pb1);
                     const uint32_t p = (uint32_t)(kq0 / kPatchK + pr) * (uint32_t)m.npi + (uint32_t)(i / kPatchI);
                     patch_frame(sv, W, t, cols_q, pr * kPatchK, min(kPatchK, rows_q - pr * kPatchK), pbx,
                                 m.pframe, p, patch_lane);

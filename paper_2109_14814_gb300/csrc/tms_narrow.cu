@@ -113,14 +113,18 @@ __device__ __forceinline__ float split_diff(float hp, float lp, float hq, float 
     return d;
 }
 
+// a triangle's vertices as FP32 splits, made from the FP64 coordinates: the tests that
+// need the low parts see a few per cent of the quads, so keeping them for every vertex
+// (16 bytes each, written by the bounds pass) cost more than splitting here
 __device__ __forceinline__ void gather_split(const MeshDev &m, uint32_t t, float4 v[3][2]) {
-    int ii[3], kk[3];
-    tri_ij(m, t, ii, kk);
+    double x[3][4];
+    gather_tri(m, t, x);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const size_t idx = (size_t)kk[j] * m.N + ii[j];
-        v[j][0] = __ldg(m.split + idx);
-        v[j][1] = __ldg(m.split + (size_t)m.N * m.M + idx);
+        split_f32(x[j][0], v[j][0].x, v[j][1].x);
+        split_f32(x[j][1], v[j][0].y, v[j][1].y);
+        split_f32(x[j][2], v[j][0].z, v[j][1].z);
+        split_f32(x[j][3], v[j][0].w, v[j][1].w);
     }
 }
 
@@ -135,16 +139,30 @@ __device__ __forceinline__ void quad_ik(const MeshDev &m, uint32_t q, int &i, in
     i = (int)(q - kk * (uint32_t)m.N);
 }
 
-// the high halves of the split copies of the quad's vertices (i,k), (i+1,k),
-// (i,k+1), (i+1,k+1) (the FP32 rounding of each coordinate)
-__device__ __forceinline__ void gather_quad_hi(const MeshDev &m, uint32_t q, float4 v[4]) {
+// the quad's vertices (i,k), (i+1,k), (i,k+1), (i+1,k+1), each coordinate rounded
+// down to FP32
+__device__ __forceinline__ void gather_quad_lo(const MeshDev &m, uint32_t q, float4 v[4]) {
     int i, k;
     quad_ik(m, q, i, k);
     const int ip = (i + 1 == m.N) ? 0 : i + 1;
     const size_t idx[4] = {(size_t)k * m.N + i, (size_t)k * m.N + ip, (size_t)(k + 1) * m.N + i,
                            (size_t)(k + 1) * m.N + ip};
 #pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = __ldg(m.split + idx[j]);
+    for (int j = 0; j < 4; ++j) v[j] = __ldg(m.vlo + idx[j]);
+}
+
+// a face's vertices for the quad-level test: a quad's, or a triangle's x2, x1, x3, x3
+template <int FACE>
+__device__ __forceinline__ void gather_face_lo(const MeshDev &m, uint32_t face, float4 v[4]) {
+    if (FACE == 1) {
+        gather_quad_lo(m, face, v);
+    } else {
+        int ii[3], kk[3];
+        tri_ij(m, face, ii, kk);
+        v[1] = __ldg(m.vlo + (size_t)kk[0] * m.N + ii[0]);
+        v[0] = __ldg(m.vlo + (size_t)kk[1] * m.N + ii[1]);
+        v[2] = v[3] = __ldg(m.vlo + (size_t)kk[2] * m.N + ii[2]);
+    }
 }
 
 // Overlap of the two triangles' boxes, as the separating-axis test along each
@@ -363,24 +381,26 @@ __device__ __forceinline__ SplitVec split_vec(const float4 P[2], const float4 Q[
     return r;
 }
 
-// p - q from the FP32 roundings hp = RN32(p), hq = RN32(q) alone: p = hp + dp
-// with |dp| <= u |hp| + 2^-150 (subnormal spacing), so t = fl(hp - hq) has
-// |t - (p - q)| <= u |t| / (1 - u) + u (|hp| + |hq|) + 2^-149, bounded with margin.
-// Looser than split_vec by about |hp| / |p - q|, which the quad-level test
-// absorbs except for near-misses far below a face's size.
-__device__ __forceinline__ SplitVec hi_vec(const float4 &P, const float4 &Q) {
+// p - q from the coordinates rounded down, fp = f32_rd(p), fq = f32_rd(q), alone:
+// |p - fp| <= 2u |fp| + 2^-126 (one FP32 place; 2^-126 below the normal range), so
+// t = fl(fp - fq) has |t - (p - q)| <= u |t| / (1 - u) + 2u (|fp| + |fq|) + 2^-125,
+// bounded with margin; a coordinate of 2^128 or more is rounded down to FLT_MAX or
+// -inf, which says nothing about it.  Looser than split_vec by about |fp| / |p - q|,
+// which the quad-level test absorbs except for near-misses far below a face's size.
+__device__ __forceinline__ SplitVec lo_vec(const float4 &P, const float4 &Q) {
     const float u = 5.9604645e-08f;
     SplitVec r;
     float tm = 0.0f, hm = 0.0f;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const float hp = comp(P, c), hq = comp(Q, c);
-        const float t = hp - hq;
+        const float fp = comp(P, c), fq = comp(Q, c);
+        const float t = fp - fq;
         r.v[c] = t;
         tm = fmaxf(tm, fabsf(t));
-        hm = fmaxf(hm, fabsf(hp) + fabsf(hq));
+        hm = fmaxf(hm, fabsf(fp) + fabsf(fq));
     }
-    r.E = ((1.001f * u) * tm + (1.001f * u) * hm) * 1.001f + 3e-45f;
+    r.E = ((1.001f * u) * tm + (2.001f * u) * hm) * 1.001f + 3e-38f;
+    if (!(hm < 3.4e38f)) r.E = __int_as_float(0x7f800000);
     r.M = tm;
     return r;
 }
@@ -468,6 +488,7 @@ __device__ __forceinline__ bool separated(const float w[4], const SplitVec &e1, 
 // triangle's edges are differences of the quad's vertices (|A_ij| <= 2 max of
 // the edge vectors below), and every offset y2 - x2 is r0 plus at most the
 // vectors to each quad's far vertex.
+// (With triangle faces the fourth vertex repeats the third.)
 // One axis of the quad-level test: A's vertices at 0, a1, a2, a3 and B's at r0,
 // r0 + b1, r0 + b2, r0 + b3 (all relative to A's v0) projected on w, each with
 // its rounding and input error; true when the widened intervals are further
@@ -533,8 +554,8 @@ __device__ __forceinline__ bool quad_sat_vectors(const SplitVec &a1, const Split
     return false;
 }
 
-// The quad-level test from the quads' FP32 vertex roundings alone (hi_vec
-// bounds, half the data of the split copies).  Directions: the mixed ones
+// The quad-level test from the quads' vertices rounded down to FP32 alone (lo_vec
+// bounds).  Directions: the mixed ones
 // MLO..MHI-1 -- 0: orthogonal to A's first-triangle edges a1, a2 and B's b1,
 // 1: to a1, a2, b2, 2: to b1, b2, a1, 3: to b1, b2, a2 (both quads thin along
 // each when their planes share a direction) -- then, with DUALS, the dual axes
@@ -542,12 +563,12 @@ __device__ __forceinline__ bool quad_sat_vectors(const SplitVec &a1, const Split
 // computed), so w is not normalised.  A candidate it cannot clear goes on to
 // the tests on the split copies.
 template <int MLO, int MHI, bool DUALS>
-__device__ __forceinline__ bool quad_reject_hi(const float4 QA[4], const float4 QB[4], float tau) {
-    const SplitVec a1 = hi_vec(QA[1], QA[0]), a2 = hi_vec(QA[2], QA[0]);
-    const SplitVec a3 = hi_vec(QA[3], QA[0]);
-    const SplitVec b1 = hi_vec(QB[1], QB[0]), b2 = hi_vec(QB[2], QB[0]);
-    const SplitVec b3 = hi_vec(QB[3], QB[0]);
-    const SplitVec r0 = hi_vec(QB[0], QA[0]);
+__device__ __forceinline__ bool quad_reject_lo(const float4 QA[4], const float4 QB[4], float tau) {
+    const SplitVec a1 = lo_vec(QA[1], QA[0]), a2 = lo_vec(QA[2], QA[0]);
+    const SplitVec a3 = lo_vec(QA[3], QA[0]);
+    const SplitVec b1 = lo_vec(QB[1], QB[0]), b2 = lo_vec(QB[2], QB[0]);
+    const SplitVec b3 = lo_vec(QB[3], QB[0]);
+    const SplitVec r0 = lo_vec(QB[0], QA[0]);
     const float amax = 2.0f * fmaxf(fmaxf(fmaxf(a1.M + a1.E, a2.M + a2.E), fmaxf(a3.M + a3.E, b1.M + b1.E)),
                                     fmaxf(b2.M + b2.E, b3.M + b3.E));
     const float rmax = (r0.M + r0.E) + (a3.M + a3.E) + (b3.M + b3.E);
@@ -677,8 +698,8 @@ __device__ __forceinline__ bool narrow_fp64(const MeshDev &ma, const MeshDev &mb
 }
 
 // Stage 1b: the triangle pairs the quad-level test (k_quad_filter) leaves, one
-// per lane (with face_level 0, every triangle candidate): the (widened)
-// triangle boxes, the triangle-level separating-axis test, and for the pairs
+// per lane: the (widened) triangle boxes (of a quad candidate's four pairs), the
+// triangle-level separating-axis test, and for the pairs
 // left a per-warp queue feeding the verified solve 32 pairs at a time, so that
 // the solve does not run with most lanes idle; pairs the tests cannot reject go
 // to the survivor list.  With the FP32 filters off, every triangle pair of
@@ -749,48 +770,15 @@ __global__ void __launch_bounds__(256, 2) k_narrow_filter(NarrowArgs a) {
             __syncwarp();
         }
     };
-    if (FACE == 1 && a.fp32_filter) {
-        // the candidates the quad-level test (k_quad_filter) could not clear: each
-        // of their four triangle pairs on a lane of its own (triangle boxes, the
-        // triangle-level separating axes), the pairs left queued for the
-        // verified solve, 32 at a time
-        const unsigned long long ni = 4 * clamp_count(&a.ctr->qkeep, a.cand_cap);
-        for (unsigned long long i0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane; i0 < ni;
-             i0 += stride) {
-            const unsigned long long it = i0 + lane;
-            const bool valid = it < ni;
-            uint32_t g = 0;
-            const int sub = (int)(it & 3);
-            float4 X[3][2], Y[3][2];
-            if (valid) {
-                g = a.qsurv[it >> 2];
-                const Cand cd = a.cand[g];
-                const int2 pr = a.pairs[cd.pair];
-                gather_split(a.meshes[pr.x], 2 * cd.faceA + (sub & 1), X);
-                gather_split(a.meshes[pr.y], 2 * cd.faceB + (sub >> 1), Y);
-            }
-            pair_tests(valid, g, sub, X, Y, true);
-            drain_full();
-        }
-        if (qn) {
-            drain(0, qn);
-            __syncwarp();
-        }
-        if (lane == 0) {
-            if (n_sat) atomicAdd(&a.ctr->sat, n_sat);
-            if (n_full) atomicAdd(&a.ctr->fp32, n_full);
-        }
-        return;
-    }
-    for (unsigned long long g0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane;
-         g0 < n; g0 += stride) {
-        const unsigned long long g = g0 + lane;
-        const bool valid = g < n;
-        Cand cd;
-        cd.faceA = cd.faceB = cd.pair = 0;
-        if (valid) cd = a.cand[g];
-        if (!a.fp32_filter) {
-            // every triangle pair of the candidate to the FP64 solve
+    if (!a.fp32_filter) {
+        // every triangle pair of the candidate to the FP64 solve
+        for (unsigned long long g0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane; g0 < n;
+             g0 += stride) {
+            const unsigned long long g = g0 + lane;
+            const bool valid = g < n;
+            Cand cd;
+            cd.faceA = cd.faceB = cd.pair = 0;
+            if (valid) cd = a.cand[g];
             const int nsub = FACE == 0 ? 1 : 4;
             for (int sub = 0; sub < nsub; ++sub) {
                 const uint32_t ta = FACE == 0 ? cd.faceA : 2 * cd.faceA + (sub & 1);
@@ -805,18 +793,30 @@ __global__ void __launch_bounds__(256, 2) k_narrow_filter(NarrowArgs a) {
                     a.surv[pos] = sv;
                 }
             }
-            continue;
         }
-        const int2 pr = a.pairs[valid ? cd.pair : 0];
-        if (FACE == 0) {
-            float4 X[3][2], Y[3][2];
-            if (valid) {
-                gather_split(a.meshes[pr.x], cd.faceA, X);
-                gather_split(a.meshes[pr.y], cd.faceB, Y);
-            }
-            pair_tests(valid, (uint32_t)g, 0, X, Y, false);
-            drain_full();
+        return;
+    }
+    // the candidates the quad-level test (k_quad_filter) could not clear: each of
+    // their triangle pairs on a lane of its own (a quad candidate's four take the
+    // triangle boxes first; the triangle-level separating axes), the pairs left
+    // queued for the verified solve, 32 at a time
+    const unsigned long long ni = (FACE == 0 ? 1 : 4) * clamp_count(&a.ctr->qkeep, a.cand_cap);
+    for (unsigned long long i0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane; i0 < ni;
+         i0 += stride) {
+        const unsigned long long it = i0 + lane;
+        const bool valid = it < ni;
+        uint32_t g = 0;
+        const int sub = FACE == 0 ? 0 : (int)(it & 3);
+        float4 X[3][2], Y[3][2];
+        if (valid) {
+            g = a.qsurv[FACE == 0 ? it : it >> 2];
+            const Cand cd = a.cand[g];
+            const int2 pr = a.pairs[cd.pair];
+            gather_split(a.meshes[pr.x], FACE == 0 ? cd.faceA : 2 * cd.faceA + (sub & 1), X);
+            gather_split(a.meshes[pr.y], FACE == 0 ? cd.faceB : 2 * cd.faceB + (sub >> 1), Y);
         }
+        pair_tests(valid, g, sub, X, Y, FACE == 1);
+        drain_full();
     }
     if (qn) {
         drain(0, qn);
@@ -828,12 +828,13 @@ __global__ void __launch_bounds__(256, 2) k_narrow_filter(NarrowArgs a) {
     }
 }
 
-// Stage 1a (quad faces): the quad-level separating-axis test of every candidate
-// on the FP32 roundings of its quads' vertices, the first mixed directions
+// Stage 1a: the quad-level separating-axis test of every candidate (quads, or triangles)
+// on its quads' vertices rounded down to FP32, the first mixed directions
 // first; the candidates they leave gather in a per-warp queue, and every 32 of
 // them take the other directions with all lanes busy; those still not cleared
 // are listed for the per-pair path of k_narrow_filter.
 constexpr int kQuadWarps = 8;
+template <int FACE>
 __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a) {
     __shared__ uint32_t s_q[kQuadWarps][64];
     if (a.ctr->cand > a.cand_cap) return;
@@ -853,9 +854,9 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
             const Cand cd = a.cand[g];
             const int2 pr = a.pairs[cd.pair];
             float4 QA[4], QB[4];
-            gather_quad_hi(a.meshes[pr.x], cd.faceA, QA);
-            gather_quad_hi(a.meshes[pr.y], cd.faceB, QB);
-            keep = !quad_reject_hi<kQuadFirstAxes, 4, true>(QA, QB, tauf);
+            gather_face_lo<FACE>(a.meshes[pr.x], cd.faceA, QA);
+            gather_face_lo<FACE>(a.meshes[pr.y], cd.faceB, QB);
+            keep = !quad_reject_lo<kQuadFirstAxes, 4, true>(QA, QB, tauf);
         }
         const unsigned long long pos = warp_append(&a.ctr->qkeep, keep, FULL);
         if (keep && pos < a.cand_cap) a.qsurv[pos] = g;
@@ -869,9 +870,9 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
             const Cand cd = a.cand[g];
             const int2 pr = a.pairs[cd.pair];
             float4 QA[4], QB[4];
-            gather_quad_hi(a.meshes[pr.x], cd.faceA, QA);
-            gather_quad_hi(a.meshes[pr.y], cd.faceB, QB);
-            need = !quad_reject_hi<0, kQuadFirstAxes, false>(QA, QB, tauf);
+            gather_face_lo<FACE>(a.meshes[pr.x], cd.faceA, QA);
+            gather_face_lo<FACE>(a.meshes[pr.y], cd.faceB, QB);
+            need = !quad_reject_lo<0, kQuadFirstAxes, false>(QA, QB, tauf);
         }
         n_quad += __popc(__ballot_sync(FULL, valid));
         const uint32_t want = __ballot_sync(FULL, need);
@@ -1354,9 +1355,10 @@ void configure_narrow() {
 
 void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st) {
     if (face_level == 0) {
+        if (a.fp32_filter) k_quad_filter<0><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
         k_narrow_filter<0><<<sms * filter_resident<0>(), 256, 0, st>>>(a);
     } else {
-        if (a.fp32_filter) k_quad_filter<<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
+        if (a.fp32_filter) k_quad_filter<1><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
         k_narrow_filter<1><<<sms * filter_resident<1>(), 256, 0, st>>>(a);
     }
     k_narrow_fp64<<<sms * 16, kSolveBlock, 0, st>>>(a);

@@ -86,7 +86,7 @@ struct Buffers {
     Grid *grids;
     Counters *ctr;
     unsigned long long *partials;
-    float4 *split[2];
+    float4 *vlo[2];
     unsigned char *fbox[2];
     uint32_t *bmA, *bmH;
     uint64_t *ek;
@@ -116,8 +116,8 @@ size_t carve(unsigned char *base, Buffers &b) {
     b.grids = c.take<Grid>(1);
     b.ctr = c.take<Counters>(1);
     b.partials = c.take<unsigned long long>(5 * kMaxGrid);
-    b.split[0] = c.take<float4>(2 * kMaxViewVertices);
-    b.split[1] = c.take<float4>(2 * kMaxViewVertices);
+    b.vlo[0] = c.take<float4>(kMaxViewVertices);
+    b.vlo[1] = c.take<float4>(kMaxViewVertices);
     b.sort_scratch = c.take<unsigned char>(radix_scratch_size(kRawHitCap, 2 * kMaxTriBits));
     b.cand = c.take<Cand>(kCandCap);
     b.tkey = c.take<unsigned long long>(kTableSize);
@@ -249,8 +249,8 @@ extern "C" tms_status tms_search_noalloc(tms_mesh A, tms_mesh B, const tms_param
     const int rows = p.tile_rows == 8 ? 8 : 4;
     Tables t;
     memset(&t, 0, sizeof(t));
-    ma.split = b.split[0];
-    mb.split = b.split[1];
+    ma.vlo = b.vlo[0];
+    mb.vlo = b.vlo[1];
     ma.fbox = b.fbox[0];
     mb.fbox = b.fbox[1];
     t.meshes[0] = ma;

@@ -411,7 +411,9 @@ void emit_waves(const EmitArgs &a, int face_level, int sms, cudaStream_t st) {
 // ---------------------------------------------------------------------------
 // quad pairs of the patch pairs (patch level)
 // ---------------------------------------------------------------------------
-constexpr int kPatchWarps = 8;
+// warps of a patch-quad block (the plain precision's boxes take twice the shared memory)
+template <int PREC>
+constexpr int kPatchWarps = PREC == 1 ? 8 : 4;
 constexpr unsigned kPatchFlush = 64;   // staged candidates per atomic
 constexpr int kQuarterBlock = 128;     // stage 1: one lane per patch pair
 
@@ -421,8 +423,8 @@ constexpr int kQuarterBlock = 128;     // stage 1: one lane per patch pair
 // and is dropped before any quad box is read; the others are listed with their
 // 16-bit mask (bit 4 i + j: A quarter i meets B quarter j).
 // Stage 2 (k_patch_quads), one warp per listed pair, grid-stride: the pair's
-// quarter boxes and quad boxes are loaded together (neither waits for the
-// other).  Lane l holds quad (row l / kPatchI, column l % kPatchI) of each
+// quarter boxes and the vertices of its quads are loaded together (neither waits
+// for the other), and the quad boxes made from the vertices.  Lane l holds quad (row l / kPatchI, column l % kPatchI) of each
 // patch; a quad that meets none of the other patch's quarter boxes cannot
 // overlap any of its quads (they all lie in those boxes), so each side is cut
 // to its quads that meet one.  The survivors' pairs take the box test of
@@ -606,21 +608,70 @@ __global__ void __launch_bounds__(kQuarterBlock) k_patch_quarters(PatchArgs a) {
     }
 }
 
+// A vertex of a patch in shared memory, and the box of a quad from its four.  The
+// quad boxes are not kept in memory: a patch's 45 vertices are 720 bytes against
+// 1024 of boxes, the vertices rounded down (16 bytes each) stay in L2 where the
+// boxes (32 bytes a quad) did not, and the bounds pass has them to write anyway.
+template <int PREC>
+struct PVert;
+template <>
+struct __align__(16) PVert<1> {
+    float v[4];
+    __device__ void load(const MeshDev &m, size_t idx) {
+        const float4 x = __ldg(m.vlo + idx);
+        v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    }
+    static __device__ __forceinline__ float above(float x) { return f32_above(x); }
+};
+template <>
+struct __align__(16) PVert<0> {
+    double v[4];
+    __device__ void load(const MeshDev &m, size_t idx) {
+#pragma unroll
+        for (int d = 0; d < 4; ++d) v[d] = __ldg(m.c[d] + idx);
+    }
+    static __device__ __forceinline__ double above(double x) { return x; }
+};
+constexpr int kPatchVerts = (kPatchI + 1) * (kPatchK + 1);
+
+// the index of vertex row r, column c of the patch at quad row k0, column i0;
+// past the mesh's end some vertex of it (the quads there are not used)
+__device__ __forceinline__ size_t patch_vertex(int N, int M, int periodic, int k, int i) {
+    k = min(k, M - 1);
+    if (i >= N) i = periodic ? 0 : N - 1;
+    return (size_t)k * N + i;
+}
+
+template <int PREC>
+__device__ __forceinline__ void quad_box(const PVert<PREC> &own, const PVert<PREC> *row, EBox<PREC> &b) {
+    const PVert<PREC> x = row[1], y = row[kPatchI + 1], z = row[kPatchI + 2];
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        b.lo[d] = min(min(own.v[d], x.v[d]), min(y.v[d], z.v[d]));
+        b.hi[d] = PVert<PREC>::above(max(max(own.v[d], x.v[d]), max(y.v[d], z.v[d])));
+    }
+}
+
 template <int PREC, bool MOLLER>
-__global__ void __launch_bounds__(32 * kPatchWarps, (PREC == 1 && !MOLLER) ? 3 : 2) k_patch_quads(PatchArgs a) {
+__global__ void __launch_bounds__(32 * kPatchWarps<PREC>, (PREC == 1 && !MOLLER) ? 3 : 2) k_patch_quads(PatchArgs a) {
+    constexpr int kW = kPatchWarps<PREC>;
     // survivors' boxes as separate low and high halves (16-byte rows for FP32)
-    __shared__ typename EBox<PREC>::Half sLo[kPatchWarps][2][32], sHi[kPatchWarps][2][32];
-    __shared__ uint32_t sQ[kPatchWarps][2][32];     // survivors' quad ids, [0] A, [1] B
-    __shared__ EBox<PREC> sQuart[kPatchWarps][8];   // the pair's quarter boxes, A's then B's
-    __shared__ Cand sOut[kPatchWarps][kPatchFlush + 32];
+    __shared__ typename EBox<PREC>::Half sLo[kW][2][32], sHi[kW][2][32];
+    __shared__ uint32_t sQ[kW][2][32];     // survivors' quad ids, [0] A, [1] B
+    __shared__ PVert<PREC> sVert[kW][2][kPatchVerts];
+    __shared__ EBox<PREC> sQuart[kW][8];   // the pair's quarter boxes, A's then B's
+    __shared__ Cand sOut[kW][kPatchFlush + 32];
     // nothing to do after an overflow of the patch-level grid (the host retries)
     if (a.ctr->entries > a.ent_cap || a.ctr->pair_slots > kMaxPairSlots) return;
     const unsigned long long n = clamp_count(&a.ctr->psurv, a.ppair_cap);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = lanemask_lt();
-    const unsigned long long gw = blockIdx.x * (unsigned long long)kPatchWarps + warp;
-    const unsigned long long nw = (unsigned long long)gridDim.x * kPatchWarps;
+    const unsigned long long gw = blockIdx.x * (unsigned long long)kW + warp;
+    const unsigned long long nw = (unsigned long long)gridDim.x * kW;
     const int r = lane / kPatchI, c = lane % kPatchI;
+    // the closing row and column: lanes 0..7 row kPatchK, lanes 8..12 column kPatchI
+    const bool edge = lane < kPatchVerts - 32;
+    const int re = lane < kPatchI ? kPatchK : lane - kPatchI, ce = lane < kPatchI ? lane : kPatchI;
     Cand *stage = sOut[warp];
     unsigned staged = 0;
     unsigned long long tests = 0;
@@ -630,43 +681,46 @@ __global__ void __launch_bounds__(32 * kPatchWarps, (PREC == 1 && !MOLLER) ? 3 :
         if (pos < cap) cand_out[pos] = rec;
     };
     uint32_t cached_pair = 0xFFFFFFFFu;
-    const void *fbA = nullptr, *fbB = nullptr, *qbA = nullptr, *qbB = nullptr;
-    int NA = 1, nqiA = 0, nqkA = 0, NB = 1, nqiB = 0, nqkB = 0;
-    uint32_t npiA = 1, npiB = 1;
-    unsigned long long mgA = 0, mgB = 0;
+    const MeshDev *ma = nullptr, *mb = nullptr;
     int2 pr = make_int2(0, 0);
     for (unsigned long long j = gw; j < n; j += nw) {
         const Cand pp = a.psurv[j];
         if (pp.pair != cached_pair) {
             pr = a.pairs[pp.pair];
-            const MeshDev &ma = a.meshes[pr.x];
-            const MeshDev &mb = a.meshes[pr.y];
-            fbA = ma.fbox; qbA = ma.qbox; NA = ma.N; nqiA = ma.nqi; nqkA = ma.nqk; npiA = ma.npi;
-            fbB = mb.fbox; qbB = mb.qbox; NB = mb.N; nqiB = mb.nqi; nqkB = mb.nqk; npiB = mb.npi;
-            mgA = ma.pmagic;
-            mgB = mb.pmagic;
+            ma = a.meshes + pr.x;
+            mb = a.meshes + pr.y;
             cached_pair = pp.pair;
         }
         // lanes 0..7 load the quarter boxes (A's then B's) while every lane loads
-        // its two quad boxes below
+        // its vertices below
         EBox<PREC> xq;
-        if (lane < 8) xq.load(lane < 4 ? qbA : qbB, 4 * (lane < 4 ? pp.faceA : pp.faceB) + (lane & 3));
-        uint32_t pka, pia, pkb, pib;
-        patch_rc(pp.faceA, npiA, mgA, pka, pia);
-        patch_rc(pp.faceB, npiB, mgB, pkb, pib);
-        const int kqa = (int)pka * kPatchK + r, iqa = (int)pia * kPatchI + c;
-        const int kqb = (int)pkb * kPatchK + r, iqb = (int)pib * kPatchI + c;
-        const bool va = kqa < nqkA && iqa < nqiA, vb = kqb < nqkB && iqb < nqiB;
-        const uint32_t qa = (uint32_t)kqa * (uint32_t)NA + (uint32_t)iqa;
-        const uint32_t qb = (uint32_t)kqb * (uint32_t)NB + (uint32_t)iqb;
-        EBox<PREC> ba, bb;
-        ba.set_empty();
-        bb.set_empty();
-        if (va) ba.load(fbA, qa);
-        if (vb) bb.load(fbB, qb);
-        __syncwarp();                          // the previous pair's quarter boxes are read
+        if (lane < 8) xq.load(lane < 4 ? ma->qbox : mb->qbox, 4 * (lane < 4 ? pp.faceA : pp.faceB) + (lane & 3));
+        bool valid[2];
+        uint32_t quad[2];
+        PVert<PREC> own[2];
+        __syncwarp();                          // the previous pair's vertices and boxes are read
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+            const MeshDev &m = s ? *mb : *ma;
+            uint32_t pk, pi;
+            patch_rc(s ? pp.faceB : pp.faceA, (uint32_t)m.npi, m.pmagic, pk, pi);
+            const int k0 = (int)pk * kPatchK, i0 = (int)pi * kPatchI;
+            const int N = m.N, M = m.nqk + 1;
+            own[s].load(m, patch_vertex(N, M, m.periodic, k0 + r, i0 + c));
+            PVert<PREC> e;
+            if (edge) e.load(m, patch_vertex(N, M, m.periodic, k0 + re, i0 + ce));
+            valid[s] = k0 + r < m.nqk && i0 + c < m.nqi;
+            quad[s] = (uint32_t)(k0 + r) * (uint32_t)N + (uint32_t)(i0 + c);
+            sVert[warp][s][r * (kPatchI + 1) + c] = own[s];
+            if (edge) sVert[warp][s][re * (kPatchI + 1) + ce] = e;
+        }
+        const bool va = valid[0], vb = valid[1];
+        const uint32_t qa = quad[0], qb = quad[1];
         if (lane < 8) sQuart[warp][lane] = xq;
         __syncwarp();
+        EBox<PREC> ba, bb;
+        quad_box<PREC>(own[0], &sVert[warp][0][r * (kPatchI + 1) + c], ba);
+        quad_box<PREC>(own[1], &sVert[warp][1][r * (kPatchI + 1) + c], bb);
         // survivors: quads meeting some quarter of the other patch
         bool sa = false, sb = false;
 #pragma unroll 1
@@ -738,7 +792,7 @@ int patch_resident() {
     int &res = g_patch_resident[PREC][MOLLER ? 1 : 0];
     if (res == 0) {
         int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_patch_quads<PREC, MOLLER>, 32 * kPatchWarps,
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_patch_quads<PREC, MOLLER>, 32 * kPatchWarps<PREC>,
                                                           0) != cudaSuccess || nb < 1)
             nb = 1;
         res = nb;
@@ -764,7 +818,7 @@ int quarter_resident() {
 template <int PREC, bool MOLLER>
 void patch_waves(const PatchArgs &a, int sms, cudaStream_t st) {
     k_patch_quarters<PREC><<<sms * quarter_resident<PREC>(), kQuarterBlock, 0, st>>>(a);
-    k_patch_quads<PREC, MOLLER><<<sms * patch_resident<PREC, MOLLER>(), 32 * kPatchWarps, 0, st>>>(a);
+    k_patch_quads<PREC, MOLLER><<<sms * patch_resident<PREC, MOLLER>(), 32 * kPatchWarps<PREC>, 0, st>>>(a);
 }
 
 }  // namespace

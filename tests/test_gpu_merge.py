@@ -71,9 +71,11 @@ def test_short_merge_of_a_batch():
             if k != "pair":
                 assert np.array_equal(rec[k][offs[p]:offs[p + 1]], one[k]), (p, k)
         assert (rec["pair"][offs[p]:offs[p + 1]] == p).all()
-    h2 = tms.search_batched(As, Bs, inject=16)
-    _identical(rec, gpu_records(h2))
-    assert np.array_equal(offs, h2.offsets.cpu().numpy())
+    # the first nine pairs by the sort (their raw hits make one sort tile)
+    h2 = tms.search_batched(As[:9], Bs[:9], inject=16)
+    assert tms.last_stats()["raw_hits"] <= 2048
+    _identical({k: v[:offs[9]] for k, v in rec.items()}, gpu_records(h2))
+    assert np.array_equal(offs[:10], h2.offsets.cpu().numpy())
 
 
 def test_more_hits_than_the_short_merge_takes():
