@@ -11,12 +11,15 @@
 // decimation in time from bit-reversed input; inverse: decimation in frequency
 // to bit-reversed output, read back through the same permutation.  All in
 // FP64 in shared memory.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 
 #include <string>
 
 #include "tms_common.cuh"
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -131,55 +134,248 @@ __global__ void __launch_bounds__(kFftThreads) k_theta_fft(const ThetaArgs a) {
     }
 }
 
-// Phase alignment cost: block (x, a) computes cost_a(m) for 128 shifts m; the
-// sum over i runs in order, one thread per shift, through shared tiles of the
-// previous circle and of the matching window of the shifted one.
-constexpr int kPhThreads = 128;
-constexpr int kPhTile = 512;
+// Phase alignment cost.  N^2 distances of C coordinates, each C subtractions, C
+// multiply-adds, a square root and an addition: in FP64 about 19 instructions of a
+// pipe that takes 19 clocks an SM for each of a warp's (9.6 ms for 16 alignments of
+// 4 x 4096 circles), so here the distances are computed on the FP32 pipe, whose rate
+// is some fifty times that, in numbers of two or three floats:
+//   digits      every coordinate, scaled by the alignment's power of two to |y| <= 1,
+//               as y = x1 + x2 + x3 with x1 a multiple of 2^-22, x2 of 2^-45, and x3
+//               the rest rounded to FP32 (2^-70); the differences of the first two
+//               digits are exact FP32 numbers;
+//   distance    the difference as a float pair, its square with the product's error
+//               term, the sum over the coordinates with every addition's error, the
+//               root with one correction: about 2^-47 relative, without bias;
+//   sum         four distances as a pair, then FP64 (two additions every four
+//               distances, which the FP64 pipe takes beside the rest).
+// 1.27 ms for those 16 alignments (1.05 G warp instructions, issue 79%).
+// A distance's error, 3e-15 rms, averages out over the sum, whose own FP64 roundings
+// are a quarter as many as in order of i: against 113-bit costs the relative error is
+// 3.6e-16 rms at N = 200 (4.1e-16 in FP64 in order of i), 1.6e-16 at 1000 (7.4e-16),
+// 1.9e-16 at 4096 (1.8e-15).  The two meet near N = 160: shorter circles, whose time
+// is launches, take the FP64 loop, and so does an alignment whose largest value's
+// exponent leaves no room for the scaling, or that is not finite.
+// Split: a cluster of eight blocks takes 512 shifts, each block an eighth of the i
+// (the same split for every shift and number of alignments: equal terms give equal
+// costs), each thread two neighbouring shifts, whose windows overlap; the even and
+// odd entries of the window are apart in shared memory, so that a warp's loads of
+// every second entry are consecutive.
+constexpr int kPhThreads = 256;
+constexpr int kPhShifts = 2 * kPhThreads;
+constexpr int kPhTile = 128;            // i per shared tile (a multiple of 4)
+constexpr int kPhSplit = 8;             // blocks of a cluster, each an eighth of the i
+constexpr int kPhWin = kPhTile + kPhShifts;
+constexpr int kPhWide = 0x7fffffff;     // no scale: the FP64 loop
+constexpr int kPhLeast = 192;           // shorter circles take the FP64 loop
 
 struct PhaseArgs {
     const double *wr;
     const double *wp;
     double *cost;
+    int *scale;                         // per alignment: the exponent e, |values| < 2^e
     int N, ncoord, nalign;
 };
 
-__global__ void __launch_bounds__(kPhThreads) k_phase_cost(const PhaseArgs a) {
-    extern __shared__ double ps[];
-    const int C = a.ncoord, N = a.N;
-    double *prev = ps;                          // C x kPhTile
-    double *win = ps + C * kPhTile;             // C x (kPhTile + kPhThreads)
-    const int al = blockIdx.y;
-    const int m0 = blockIdx.x * kPhThreads;
-    const int m = m0 + threadIdx.x;
+// The scale of each alignment, left in the shift output, which the minimum's kernel
+// writes last.
+__global__ void __launch_bounds__(1024) k_phase_scale(const PhaseArgs a) {
+    __shared__ unsigned top[32];
+    const long long n = (long long)a.ncoord * a.N, base = n * blockIdx.x;
+    unsigned m = 0;                     // high words of |x|: the largest holds the largest exponent
+    for (long long q = threadIdx.x; q < n; q += 1024) {
+        m = max(m, (unsigned)__double2hiint(a.wr[base + q]) & 0x7fffffffu);
+        m = max(m, (unsigned)__double2hiint(a.wp[base + q]) & 0x7fffffffu);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+        m = __reduce_max_sync(0xffffffffu, top[threadIdx.x]);
+        const int e = (int)(m >> 20);
+        if (threadIdx.x == 0) a.scale[blockIdx.x] = a.N < kPhLeast || e < 100 || e > 1900 ? kPhWide : e - 1022;
+    }
+}
+
+__device__ __forceinline__ double power_of_two(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+
+// a float pair sum: s + e = x + y exactly (Knuth), and for |x| >= |y| or x = 0 (Dekker)
+__device__ __forceinline__ void two_sum(float x, float y, float &s, float &e) {
+    s = __fadd_rn(x, y);
+    const float b = __fsub_rn(s, x);
+    e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, b)), __fsub_rn(y, b));
+}
+__device__ __forceinline__ void fast_sum(float x, float y, float &s, float &e) {
+    s = __fadd_rn(x, y);
+    e = __fsub_rn(y, __fsub_rn(s, x));
+}
+
+// the distance between two points given by their digits, as a float pair; what the
+// pair has no room for (the low halves' squares, the root's second-order terms: 2^-50
+// of the distance, but of one sign) goes to `rest`
+template <int C>
+__device__ __forceinline__ void pair_distance(const float (&x)[3][C], const float (&y)[3][C], float &g, float &lo,
+                                              float &rest) {
+    float S = 0.0f, T = 0.0f, L2 = 0.0f;   // the squares' sum, and the low halves'
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+        float h, e, H, L;
+        // the first two differences are exact; the second is at most 2^-22, the least
+        // nonzero value of the first
+        fast_sum(__fsub_rn(x[0][c], y[0][c]), __fsub_rn(x[1][c], y[1][c]), h, e);
+        fast_sum(h, __fadd_rn(e, __fsub_rn(x[2][c], y[2][c])), H, L);
+        const float p = __fmul_rn(H, H);
+        float q = __fmaf_rn(H, H, -p);
+        q = __fmaf_rn(H, __fadd_rn(L, L), q);
+        L2 = __fmaf_rn(L, L, L2);
+        if (c == 0) {
+            S = p;
+            T = q;
+        } else {
+            float s, r;
+            two_sum(S, p, s, r);
+            S = s;
+            T = __fadd_rn(T, __fadd_rn(r, q));
+        }
+    }
+    // sqrt(S + T): g the root of S to a rounding, then one correction by the residual
+    // (0 for S = 0, where the reciprocal root stays finite)
+    const float r = rsqrtf(fmaxf(S, 1e-37f));
+    const float hr = __fmul_rn(0.5f, r), g0 = __fmul_rn(S, r);
+    g = __fmaf_rn(__fmaf_rn(-g0, g0, S), hr, g0);
+    lo = __fmul_rn(__fadd_rn(__fmaf_rn(-g, g, S), T), hr);
+    // with d = sqrt(S) - g and t = T hr: lo = d - d^2 hr + t and sqrt(S + T) =
+    // g + d + t - t^2 hr + ..., so d^2 - t^2 = lo (lo - 2 t) is missing
+    rest = __fmaf_rn(__fmaf_rn(lo, __fmaf_rn(-T, r, lo), L2), hr, rest);
+}
+
+// the digits of a value scaled to |y| <= 1
+__device__ __forceinline__ void digits(double y, float &x1, float &x2, float &x3) {
+    constexpr double m1 = 1.5 * (double)(1 << 30), m2 = 1.5 * (double)(1 << 7);
+    const double t1 = __dsub_rn(__dadd_rn(y, m1), m1);      // to a multiple of 2^-22
+    const double r1 = __dsub_rn(y, t1);
+    const double t2 = __dsub_rn(__dadd_rn(r1, m2), m2);     // to a multiple of 2^-45
+    x1 = (float)t1;
+    x2 = (float)t2;
+    x3 = (float)__dsub_rn(r1, t2);
+}
+
+template <int C>
+__global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k_phase_cost(const PhaseArgs a) {
+    extern __shared__ __align__(16) float ps[];
+    float(*prev)[3][C] = reinterpret_cast<float(*)[3][C]>(ps);            // [kPhTile], by i
+    float *win = ps + kPhTile * 3 * C;                                    // [odd][digit][C][kPhWin / 2]
+    constexpr int kHalf = kPhWin / 2;
+    double *part = reinterpret_cast<double *>(win + 3 * C * kPhWin);      // [kPhShifts]
+    const int N = a.N, al = blockIdx.y, t = threadIdx.x;
+    const int rank = blockIdx.x % kPhSplit;
+    const int m0 = (int)(blockIdx.x / kPhSplit) * kPhShifts;
     const double *Wr = a.wr + (long long)al * C * N;
     const double *Wp = a.wp + (long long)al * C * N;
-    double acc = 0.0;
-    for (int i0 = 0; i0 < N; i0 += kPhTile) {
-        const int ti = min(kPhTile, N - i0);
-        __syncthreads();
-        for (int q = threadIdx.x; q < C * kPhTile; q += kPhThreads) {
-            const int c = q / kPhTile, u = q % kPhTile;
-            prev[q] = u < ti ? Wp[(long long)c * N + i0 + u] : 0.0;
-        }
-        const int wlen = kPhTile + kPhThreads;
-        for (int q = threadIdx.x; q < C * wlen; q += kPhThreads) {
-            const int c = q / wlen, u = q % wlen;
-            win[q] = Wr[(long long)c * N + (i0 + m0 + u) % N];
-        }
-        __syncthreads();
-        if (m < N) {
-            for (int u = 0; u < ti; ++u) {
-                double d2 = 0.0;
-                for (int c = 0; c < C; ++c) {
-                    const double d = win[c * wlen + u + threadIdx.x] - prev[c * kPhTile + u];
-                    d2 = fma(d, d, d2);
+    const int e = a.scale[al];
+    double acc[2] = {0.0, 0.0};
+    float rest[2] = {0.0f, 0.0f};
+    if (e == kPhWide) {
+        if (rank == 0)
+            for (int k = 0; k < 2; ++k) {
+                const int m = m0 + 2 * t + k;
+                if (m >= N) continue;
+                for (int i = 0; i < N; ++i) {
+                    const int w = i + m < N ? i + m : i + m - N;
+                    double d2 = 0.0;
+                    for (int c = 0; c < C; ++c) {
+                        const double d = Wr[(long long)c * N + w] - Wp[(long long)c * N + i];
+                        d2 = fma(d, d, d2);
+                    }
+                    acc[k] += sqrt(d2);
                 }
-                acc += sqrt(d2);
+                a.cost[(long long)al * N + m] = acc[k];
+            }
+        return;                         // the whole cluster: e is the alignment's
+    }
+    const double down = power_of_two(-e);
+    const int per = ((N + 4 * kPhSplit - 1) / (4 * kPhSplit)) * 4;
+    const int i_end = (int)min((long long)N, (long long)(rank + 1) * per);
+    for (long long i0 = (long long)rank * per; i0 < i_end; i0 += kPhTile) {
+        const int ti = (int)min((long long)kPhTile, i_end - i0);
+        __syncthreads();                // the previous tile is read
+        for (int q = t; q < C * kPhTile; q += kPhThreads) {
+            const int c = q / kPhTile, u = q % kPhTile;
+            if (u < ti) digits(Wp[(long long)c * N + i0 + u] * down, prev[u][0][c], prev[u][1][c], prev[u][2][c]);
+        }
+        const int w0 = (int)((i0 + m0) % N);
+        const int wn = min(kPhWin, ti + kPhShifts + 4);
+        for (int c = 0; c < C; ++c)
+            for (int u = t; u < wn; u += kPhThreads) {
+                float x1, x2, x3;
+                digits(Wr[(long long)c * N + ((unsigned)w0 + (unsigned)u) % (unsigned)N] * down, x1, x2, x3);
+                float *o = win + ((u & 1) * 3 * C + c) * kHalf + (u >> 1);
+                o[0] = x1;
+                o[C * kHalf] = x2;
+                o[2 * C * kHalf] = x3;
+            }
+        __syncthreads();
+        if (m0 + 2 * t >= N) continue;
+        for (int u = 0; u < ti; u += 4) {
+            // window entries u + 2t + j, j = 0..4: shift k at i0 + u + v reads entry v + k
+            float x[2][3][C];
+            auto load = [&](int j, float (&w)[3][C]) {
+                const float *p = win + (j & 1) * 3 * C * kHalf + (u >> 1) + t + (j >> 1);
+#pragma unroll
+                for (int d = 0; d < 3; ++d)
+#pragma unroll
+                    for (int c = 0; c < C; ++c) w[d][c] = p[(d * C + c) * kHalf];
+            };
+            load(0, x[0]);
+            float G[2] = {0.0f, 0.0f}, E[2] = {0.0f, 0.0f};
+#pragma unroll
+            for (int v = 0; v < 4; ++v) {
+                load(v + 1, x[(v + 1) & 1]);
+                if (u + v < ti) {
+                    float y[3][C];
+#pragma unroll
+                    for (int d = 0; d < 3; ++d)
+#pragma unroll
+                        for (int c = 0; c < C; ++c) y[d][c] = prev[u + v][d][c];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        float g, lo, s, r;
+                        pair_distance<C>(x[(v + k) & 1], y, g, lo, rest[k]);
+                        two_sum(G[k], g, s, r);
+                        G[k] = s;
+                        E[k] = __fadd_rn(E[k], __fadd_rn(r, lo));
+                    }
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                acc[k] += (double)G[k];
+                acc[k] += (double)E[k];
             }
         }
     }
-    if (m < N) a.cost[(long long)al * N + m] = acc;
+    // the eight parts, added in order of i by the cluster's first block
+    part[2 * t] = acc[0] + (double)rest[0];
+    part[2 * t + 1] = acc[1] + (double)rest[1];
+    cg::cluster_group cluster = cg::this_cluster();
+    cluster.sync();
+    if (rank == 0) {
+        for (int q = t; q < kPhShifts; q += kPhThreads) {
+            double s = part[q];
+            for (int r = 1; r < kPhSplit; ++r) s += cluster.map_shared_rank(part, r)[q];
+            if (m0 + q < N) a.cost[(long long)al * N + m0 + q] = s * power_of_two(e);
+        }
+    }
+    cluster.sync();                     // the parts are read before their blocks end
+}
+
+template <int C>
+cudaError_t launch_phase_cost(const PhaseArgs &a, cudaStream_t st) {
+    constexpr size_t smem = (size_t)(kPhTile + kPhWin) * 3 * C * sizeof(float) + kPhShifts * sizeof(double);
+    const cudaError_t e = cudaFuncSetAttribute(k_phase_cost<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const dim3 grid((unsigned)((a.N + kPhShifts - 1) / kPhShifts) * kPhSplit, (unsigned)a.nalign);
+    k_phase_cost<C><<<grid, kPhThreads, smem, st>>>(a);
+    return cudaGetLastError();
 }
 
 // Smallest cost per alignment, ties to the smallest shift.
@@ -276,19 +472,20 @@ extern "C" tms_status tms_phase_align(const double *dWr, const double *dWprev, i
         !device_ptr(dCost) || !device_ptr(dShift))
         return fail(TMS_ERR_ARG, "tms_phase_align: arrays must be device pointers");
     if (nAlign > 65535) return fail(TMS_ERR_ARG, "tms_phase_align: nAlign > 65535");
-    const size_t smem = (size_t)nCoord * (2 * kPhTile + kPhThreads) * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(k_phase_cost, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return fail(TMS_ERR_CUDA, cudaGetErrorString(e));
     PhaseArgs a;
     a.wr = dWr;
     a.wp = dWprev;
     a.cost = dCost;
+    a.scale = dShift;
     a.N = N;
     a.ncoord = nCoord;
     a.nalign = nAlign;
-    dim3 grid((N + kPhThreads - 1) / kPhThreads, nAlign);
-    k_phase_cost<<<grid, kPhThreads, smem, (cudaStream_t)stream>>>(a);
+    k_phase_scale<<<nAlign, 1024, 0, (cudaStream_t)stream>>>(a);
+    cudaError_t (*const launch[8])(const PhaseArgs &, cudaStream_t) = {
+        launch_phase_cost<1>, launch_phase_cost<2>, launch_phase_cost<3>, launch_phase_cost<4>,
+        launch_phase_cost<5>, launch_phase_cost<6>, launch_phase_cost<7>, launch_phase_cost<8>};
+    cudaError_t e = launch[nCoord - 1](a, (cudaStream_t)stream);
+    if (e != cudaSuccess) return fail(TMS_ERR_CUDA, std::string("tms_phase_align: ") + cudaGetErrorString(e));
     k_phase_argmin<<<nAlign, 256, 0, (cudaStream_t)stream>>>(dCost, N, dShift);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(TMS_ERR_CUDA, std::string("tms_phase_align: ") +
