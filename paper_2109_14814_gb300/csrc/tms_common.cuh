@@ -352,25 +352,26 @@ __device__ __forceinline__ float f32_special(unsigned long long b, int e32, int 
     if (dir < 0) return neg ? -1.17549435e-38f : 0.0f;
     return neg ? -0.0f : 1.17549435e-38f;
 }
+// (out of line: the compiler would run parts of it for every value, under a predicate)
+static __device__ __noinline__ float f32_rd_special(double x) {
+    return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, -1);
+}
 // round down.  In the FP32 normal range the bits of |x| shifted right by 29, less the
 // exponents' difference, are the truncated FP32 magnitude
 __device__ __forceinline__ float f32_rd(double x) {
     const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
     const unsigned mag = h & 0x7fffffffu;
-    if (mag - (897u << 20) >= (254u << 20))
-        return f32_special((unsigned long long)__double_as_longlong(x), (int)(mag >> 20) - 896, -1);
+    if (mag - (897u << 20) >= (254u << 20)) return f32_rd_special(x);
     unsigned f = __funnelshift_r(l, mag, 29) - (896u << 23);
     if ((int)h < 0 && (l & 0x1FFFFFFFu) != 0u) ++f;                    // negative, inexact
     return __uint_as_float(f | (h & 0x80000000u));
 }
-// an upper bound of every x with f32_rd(x) = f: the next FP32 number; outside the
-// normal range as f32_special rounds (an exact x is over by one place too, so that
-// the value rounded down is all a vertex has to keep)
+// an upper bound of every x with f32_rd(x) = f, one or two FP32 places above f (2^-23 |f|
+// is at least a place; 2^-126 covers what is rounded to 0): two instructions of the FMA
+// pipe, where the next number from the bits takes six of the busier integer pipe.  An
+// exact x is over by that too, so that the value rounded down is all a vertex keeps
 __device__ __forceinline__ float f32_above(float f) {
-    const int b = __float_as_int(f);
-    const float up = __int_as_float(b + (b >= 0 ? 1 : -1));
-    const float least = 1.17549435e-38f;
-    return f <= 0.0f && f >= -least ? (f < 0.0f ? 0.0f : least) : up;
+    return f + fmaf(fabsf(f), 1.1920932e-7f, 1.17549435e-38f);
 }
 __device__ __forceinline__ float f32_rn(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
