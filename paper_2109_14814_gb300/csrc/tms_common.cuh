@@ -56,8 +56,8 @@ struct MeshDev {
                           // precision without the FP32 filters has no use for it)
     void *fbox;           // plan scratch, face level only: per face slot its box,
                           // written by the bounds pass (mixed precision: float4
-                          // lo, float4 hi, rounded outward; plain: 8 doubles
-                          // lo[4], hi[4]);
+                          // lo, float4 hi, rounded outward; plain: 8 ordered
+                          // integers lo[4], hi[4], ord64);
                           // slot = face id (quad k*N + i, or triangle 2(k*N + i) + t)
     int N;                // theta samples
     int M;                // vertex rows in the view
@@ -381,6 +381,16 @@ __device__ __forceinline__ float f32_rn(double x) {
     const unsigned rem = (unsigned)(b & 0x1FFFFFFFULL);
     f += (unsigned)(rem > 0x10000000u) | ((unsigned)(rem == 0x10000000u) & (f & 1u));
     return __uint_as_float(f | ((unsigned)(b >> 63) << 31));
+}
+// A double as an integer of the same order (the plain precision's boxes: GB300's
+// FP64 pipe takes two lanes a clock, its integer pipes at least 64).  -0 lies
+// below +0; the two compare equal as doubles, so a vertex's -0 is kept as +0.
+__device__ __forceinline__ long long ord64(double v) {
+    const long long b = __double_as_longlong(v);
+    return b >= 0 ? b : (b == (long long)0x8000000000000000ULL ? 0 : b ^ 0x7fffffffffffffffLL);
+}
+__device__ __forceinline__ double ord64_value(long long o) {
+    return __longlong_as_double(o >= 0 ? o : o ^ 0x7fffffffffffffffLL);
 }
 // finiteness from the exponent bits (no FP64 compare)
 __device__ __forceinline__ bool finite64(double x) {

@@ -45,7 +45,9 @@ constexpr unsigned FULL = 0xffffffffu;
 // A vertex as the boxes need it: its coordinates rounded down to FP32 (mixed
 // precision; every exact coordinate then lies in [v, f32_above(v)], so the box of a
 // set of vertices is [min v, f32_above(max v)] and one value a coordinate does), or
-// as they are (plain).
+// as integers of the doubles' order (plain; minima, maxima and comparisons of doubles
+// run on the FP64 pipe: the bounds pass of 1019 x 253 and 771 x 331 meshes took 99 us
+// of it, and 22 us as integers).
 template <int PREC>
 struct Num;
 template <>
@@ -57,10 +59,10 @@ struct Num<1> {
 };
 template <>
 struct Num<0> {
-    typedef double T;
-    static __device__ __forceinline__ double of(double x) { return x; }
-    static __device__ __forceinline__ double above(double v) { return v; }
-    static __device__ __forceinline__ double inf() { return __longlong_as_double(0x7ff0000000000000LL); }
+    typedef long long T;
+    static __device__ __forceinline__ long long of(double x) { return ord64(x); }
+    static __device__ __forceinline__ long long above(long long v) { return v; }
+    static __device__ __forceinline__ long long inf() { return 0x7fffffffffffffffLL; }
 };
 
 template <int PREC>
@@ -104,7 +106,9 @@ __device__ __forceinline__ void write_vlo(const MeshDev &m, size_t idx, const Vt
     m.vlo[idx] = make_float4(v.v[0], v.v[1], v.v[2], v.v[3]);
 }
 __device__ __forceinline__ void write_vlo(const MeshDev &m, size_t idx, const Vtx<0> &v) {
-    if (m.vlo) m.vlo[idx] = make_float4(f32_rd(v.v[0]), f32_rd(v.v[1]), f32_rd(v.v[2]), f32_rd(v.v[3]));
+    if (m.vlo)
+        m.vlo[idx] = make_float4(f32_rd(ord64_value(v.v[0])), f32_rd(ord64_value(v.v[1])),
+                                 f32_rd(ord64_value(v.v[2])), f32_rd(ord64_value(v.v[3])));
 }
 
 template <int PREC>
@@ -117,15 +121,20 @@ struct GridView<1> {
 #pragma unroll
         for (int d = 0; d < 4; ++d) { o[d] = g.o32[d]; e[d] = g.e32[d]; inv[d] = g.inv32[d]; n[d] = g.n[d]; }
     }
+    __device__ int cell(float v, int d) const { return cell_of(v, o[d], inv[d], n[d]); }
 };
 template <>
 struct GridView<0> {
-    double o[4], e[4], inv[4];
+    double origin[4], inv[4];
+    long long o[4], e[4];
     int n[4];
     __device__ void load(const Grid &g) {
 #pragma unroll
-        for (int d = 0; d < 4; ++d) { o[d] = g.o64[d]; e[d] = g.e64[d]; inv[d] = g.inv64[d]; n[d] = g.n[d]; }
+        for (int d = 0; d < 4; ++d) {
+            origin[d] = g.o64[d]; o[d] = ord64(g.o64[d]); e[d] = ord64(g.e64[d]); inv[d] = g.inv64[d]; n[d] = g.n[d];
+        }
     }
+    __device__ int cell(long long v, int d) const { return cell_of(ord64_value(v), origin[d], inv[d], n[d]); }
 };
 
 // the (closed) box of a face or patch into slot `face` of a box array
@@ -139,11 +148,11 @@ __device__ __forceinline__ void write_box<1>(void *arr, uint32_t face, const Box
 }
 template <>
 __device__ __forceinline__ void write_box<0>(void *arr, uint32_t face, const BoxT<0> &b) {
-    double2 *p = reinterpret_cast<double2 *>(arr) + 4 * (size_t)face;
-    p[0] = make_double2(b.lo[0], b.lo[1]);
-    p[1] = make_double2(b.lo[2], b.lo[3]);
-    p[2] = make_double2(b.hi[0], b.hi[1]);
-    p[3] = make_double2(b.hi[2], b.hi[3]);
+    longlong2 *p = reinterpret_cast<longlong2 *>(arr) + 4 * (size_t)face;
+    p[0] = make_longlong2(b.lo[0], b.lo[1]);
+    p[1] = make_longlong2(b.lo[2], b.lo[3]);
+    p[2] = make_longlong2(b.hi[0], b.hi[1]);
+    p[3] = make_longlong2(b.hi[2], b.hi[3]);
 }
 template <int PREC>
 __device__ __forceinline__ void write_fbox(const MeshDev &m, uint32_t face, const BoxT<PREC> &b) {
@@ -185,17 +194,21 @@ __device__ __forceinline__ void read_fbox<1>(const MeshDev &m, uint32_t face, Bo
 }
 template <>
 __device__ __forceinline__ void read_fbox<0>(const MeshDev &m, uint32_t face, BoxT<0> &b) {
-    const double2 *p = reinterpret_cast<const double2 *>(m.fbox) + 4 * (size_t)face;
-    const double2 x0 = __ldg(p), x1 = __ldg(p + 1), x2 = __ldg(p + 2), x3 = __ldg(p + 3);
+    const longlong2 *p = reinterpret_cast<const longlong2 *>(m.fbox) + 4 * (size_t)face;
+    const longlong2 x0 = __ldg(p), x1 = __ldg(p + 1), x2 = __ldg(p + 2), x3 = __ldg(p + 3);
     b.lo[0] = x0.x; b.lo[1] = x0.y; b.lo[2] = x1.x; b.lo[3] = x1.y;
     b.hi[0] = x2.x; b.hi[1] = x2.y; b.hi[2] = x3.x; b.hi[3] = x3.y;
 }
 
-// Per-thread accumulators of the bounds pass, in the box precision (FP32
-// min/max in the mixed mode: FP64 arithmetic is a scarce pipe on GB300)
+__device__ __forceinline__ float extent(float lo, float hi) { return hi - lo; }
+__device__ __forceinline__ long long extent(long long lo, long long hi) {
+    return __double_as_longlong(ord64_value(hi) - ord64_value(lo));
+}
+
+// Per-thread accumulators of the bounds pass, in the boxes' numbers
 template <int PREC>
 struct BoundAcc {
-    typename Num<PREC>::T lo[4], hi[4], w[4];
+    typename Num<PREC>::T lo[4], hi[4], w[4];   // w: extents (plain: the bits of doubles >= 0)
     unsigned seen;
     __device__ void init() {
 #pragma unroll
@@ -208,15 +221,17 @@ struct BoundAcc {
         for (int d = 0; d < 4; ++d) {
             lo[d] = min(lo[d], b.lo[d]);
             hi[d] = max(hi[d], b.hi[d]);
-            w[d] = max(w[d], b.hi[d] - b.lo[d]);
+            w[d] = max(w[d], extent(b.lo[d], b.hi[d]));
         }
         seen = 1;
     }
 };
 
-// ord_enc of the value as a double: FP64 values directly; FP32 values through the
+// ord_enc of the value as a double: ordered integers directly; FP32 values through the
 // exact float -> double conversion done on the bits (integer operations only)
-__device__ __forceinline__ unsigned long long ord_enc_any(double v) { return ord_enc(v); }
+__device__ __forceinline__ unsigned long long ord_enc_any(long long v) {
+    return (unsigned long long)v ^ 0x8000000000000000ULL;
+}
 __device__ __forceinline__ unsigned long long ord_enc_any(float v) {
     const unsigned b = __float_as_uint(v);
     const unsigned long long sgn = (unsigned long long)(b >> 31) << 63;
@@ -618,8 +633,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
     }
 
     // block reduction, then one set of atomics per block
-    // in the accumulators' own type: FP32 in the mixed mode (no FP64 instruction
-    // in this kernel: GB300's FP64 pipe is narrow), FP64 in the plain mode
+    // in the accumulators' own type (no FP64 instruction: GB300's FP64 pipe is narrow)
     typedef typename std::remove_reference<decltype(acc.lo[0])>::type AccT;
     __shared__ AccT red[8][12];
     __shared__ unsigned redf[8][2];
@@ -731,8 +745,8 @@ __global__ void __launch_bounds__(32 * kCellWarps) k_cell_pass(FacePassArgs a, i
             count = 1;
 #pragma unroll
             for (int d = 0; d < 4; ++d) {
-                clo[d] = cell_of(b.lo[d], g.o[d], g.inv[d], g.n[d]);
-                const int chi = cell_of(b.hi[d], g.o[d], g.inv[d], g.n[d]);
+                clo[d] = g.cell(b.lo[d], d);
+                const int chi = g.cell(b.hi[d], d);
                 cnt[d] = chi - clo[d] + 1;
                 count *= (unsigned)cnt[d];
             }

@@ -77,8 +77,8 @@ struct __align__(16) EBox<1> {
 };
 template <>
 struct __align__(16) EBox<0> {
-    struct __align__(16) Half { double v[4]; };
-    double lo[4], hi[4];
+    struct __align__(16) Half { long long v[4]; };
+    long long lo[4], hi[4];        // ordered integers (ord64)
     __device__ void store_halves(Half &l, Half &h) const {
 #pragma unroll
         for (int d = 0; d < 4; ++d) { l.v[d] = lo[d]; h.v[d] = hi[d]; }
@@ -91,19 +91,19 @@ struct __align__(16) EBox<0> {
         return ov;
     }
     __device__ void load(const void *fbox, uint32_t face) {
-        const double2 *p = reinterpret_cast<const double2 *>(fbox) + 4 * (size_t)face;
-        const double2 x0 = __ldg(p), x1 = __ldg(p + 1), x2 = __ldg(p + 2), x3 = __ldg(p + 3);
+        const longlong2 *p = reinterpret_cast<const longlong2 *>(fbox) + 4 * (size_t)face;
+        const longlong2 x0 = __ldg(p), x1 = __ldg(p + 1), x2 = __ldg(p + 2), x3 = __ldg(p + 3);
         lo[0] = x0.x; lo[1] = x0.y; lo[2] = x1.x; lo[3] = x1.y;
         hi[0] = x2.x; hi[1] = x2.y; hi[2] = x3.x; hi[3] = x3.y;
     }
     __device__ void set_empty() {
 #pragma unroll
-        for (int d = 0; d < 4; ++d) { lo[d] = __longlong_as_double(0x7ff0000000000000LL); hi[d] = -lo[d]; }
+        for (int d = 0; d < 4; ++d) { lo[d] = 0x7fffffffffffffffLL; hi[d] = -lo[d]; }
     }
     __device__ uint2 low_cell(const Grid &g) const {
         int c[4];
 #pragma unroll
-        for (int d = 0; d < 4; ++d) c[d] = cell_of(lo[d], g.o64[d], g.inv64[d], g.n[d]);
+        for (int d = 0; d < 4; ++d) c[d] = cell_of(ord64_value(lo[d]), g.o64[d], g.inv64[d], g.n[d]);
         return make_uint2((uint32_t)c[0] | ((uint32_t)c[1] << 16), (uint32_t)c[2] | ((uint32_t)c[3] << 16));
     }
 };
@@ -625,12 +625,12 @@ struct __align__(16) PVert<1> {
 };
 template <>
 struct __align__(16) PVert<0> {
-    double v[4];
+    long long v[4];                // ordered integers (ord64)
     __device__ void load(const MeshDev &m, size_t idx) {
 #pragma unroll
-        for (int d = 0; d < 4; ++d) v[d] = __ldg(m.c[d] + idx);
+        for (int d = 0; d < 4; ++d) v[d] = ord64(__ldg(m.c[d] + idx));
     }
-    static __device__ __forceinline__ double above(double x) { return x; }
+    static __device__ __forceinline__ long long above(long long x) { return x; }
 };
 constexpr int kPatchVerts = (kPatchI + 1) * (kPatchK + 1);
 
