@@ -392,11 +392,6 @@ __device__ __forceinline__ long long ord64(double v) {
 __device__ __forceinline__ double ord64_value(long long o) {
     return __longlong_as_double(o >= 0 ? o : o ^ 0x7fffffffffffffffLL);
 }
-// finiteness from the exponent bits (no FP64 compare)
-__device__ __forceinline__ bool finite64(double x) {
-    return (((unsigned long long)__double_as_longlong(x) >> 52) & 0x7ff) != 0x7ff;
-}
-
 // cell index along one coordinate: monotone non-decreasing in v, clamped
 __device__ __forceinline__ int cell_of(float v, float o, float inv, int n) {
     float t = (v - o) * inv;

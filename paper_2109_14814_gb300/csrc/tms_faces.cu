@@ -255,6 +255,30 @@ __device__ __forceinline__ unsigned long long ord_enc_any(float v) {
     return (bb >= 0) ? (db | 0x8000000000000000ULL) : ~db;
 }
 
+// Maxima over a warp, as integers of the values' order: FP32 values by one instruction
+// on their bits (negative ones with the magnitude's bits flipped), ordered 64-bit
+// integers by shuffles.  A minimum is a maximum of the complements (negated).
+__device__ __forceinline__ int ord32(float v) {
+    const int b = __float_as_int(v);
+    return b ^ ((b >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ long long warp_max(float v) { return __reduce_max_sync(FULL, ord32(v)); }
+__device__ __forceinline__ long long warp_max(int v) { return __reduce_max_sync(FULL, v); }
+__device__ __forceinline__ long long warp_max(long long v) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) v = max(v, __shfl_xor_sync(FULL, v, off));
+    return v;
+}
+__device__ __forceinline__ int negated(float v) { return ~ord32(v); }
+__device__ __forceinline__ long long negated(long long v) { return ~v; }
+// the Bounds encoding of a reduced value
+template <int PREC>
+__device__ __forceinline__ unsigned long long encoded(long long v) {
+    if (PREC == 0) return ord_enc_any(v);
+    const int b = (int)v;
+    return ord_enc_any(__int_as_float(b ^ ((b >> 31) & 0x7fffffff)));
+}
+
 // the pass entry (mesh of a pass) holding global index x, by binary search
 __device__ __forceinline__ int find_entry(const FacePassArgs &a, long long x, bool by_face) {
     int lo = 0, hi = a.n_entries - 1;
@@ -291,11 +315,12 @@ __device__ __forceinline__ void cross4(const float a[4], const float b[4], const
 // an integer maximum of |x| keeps a NaN, which fmaxf would drop
 __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
 
-// The frame of a patch, computed by its kPatchI lanes at the close of its patch
-// row and written as kFrameF4 float4 by its first lane.  Every lane of the
-// warp calls it (the shuffles are uniform).  pr0: the patch's first vertex
-// row in the tile's vertex array sv; rq: its quad rows; pb: its box (held by
-// every lane of the patch).
+// The frame of a patch, in three steps over the tile's patches: one thread a patch
+// computes the axes (frame_axes), the patch's kPatchI lanes project its vertices on
+// them (frame_extents), and one thread a patch closes the bounds and writes the record
+// (frame_write).  What is the same for a whole patch runs on as many threads as there
+// are patches (16 of a 128 x 4 tile): computed by all of a patch's lanes it was a third
+// of the kernel's instructions (65.6 M and 87 us at 4096 x 512; 54.5 M and 72 us so).
 // Axes: e_0, e_1 from the patch's two parameter directions (sums of opposite
 // edges, one Gram-Schmidt step), e_2 orthogonal to e_0, e_1 and the coordinate
 // axis farthest from their span, e_3 orthogonal to e_0, e_1, e_2.  A patch
@@ -313,23 +338,33 @@ __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x
 //   G~_ij = fl(delta_ij - sum_k e_ki e_kj) (4 FMAs, error <= gamma_4 (1 + 4 e_max^2)).
 // Sums and products of non-negative terms are rounded up by a factor 1.0001
 // (a handful of roundings of 2^-24 each); absolute terms cover underflow.
-__device__ __forceinline__ void patch_frame(const Vtx<1> *sv, int W, int t, int cols_q, int pr0, int rq,
-                                            const BoxT<1> &pb, float4 *out, uint32_t p, bool patch_lane) {
-    const float u = 5.9604645e-08f;
-    const float inf = __int_as_float(0x7f800000);
-    const int p0 = t & ~(kPatchI - 1), l = t - p0;
-    const int cq = patch_lane ? min(kPatchI, cols_q - p0) : 0;    // the patch's quad columns
-    const int pr1 = pr0 + rq;
-    float c[4], L = 0.0f, D = 0.0f;
+struct PatchScratch {         // of a patch of the tile
+    float4 lo, hi;            // its (closed) box
+    float4 axes[5];           // c, e_0..e_3
+    uint4 top;                // max |e_k . (V - c)| (bits)
+    uint4 flags;              // x: no usable axes
+};
+
+__device__ __forceinline__ void patch_centre(const PatchScratch &P, float c[4], float &L, float &D) {
+    const float lo[4] = {P.lo.x, P.lo.y, P.lo.z, P.lo.w}, hi[4] = {P.hi.x, P.hi.y, P.hi.z, P.hi.w};
+    L = D = 0.0f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        c[i] = 0.5f * (pb.lo[i] + pb.hi[i]);
-        L = fmaxf(L, fmaxf(fabsf(pb.lo[i]), fabsf(pb.hi[i])));
-        D = fmaxf(D, fmaxf(pb.hi[i] - c[i], c[i] - pb.lo[i]));
+        c[i] = 0.5f * (lo[i] + hi[i]);
+        L = fmaxf(L, fmaxf(fabsf(lo[i]), fabsf(hi[i])));
+        D = fmaxf(D, fmaxf(hi[i] - c[i], c[i] - lo[i]));
     }
     D *= 1.0001f;
-    float t1[4] = {0.0f, 0.0f, 0.0f, 0.0f}, t2[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    if (patch_lane) {
+}
+
+// sv: the tile's vertices; p0, cq: the patch's first quad column in the tile and its
+// columns, pr0, rq: its quad rows
+__device__ __forceinline__ void frame_axes(const Vtx<1> *sv, int W, int p0, int cq, int pr0, int rq, PatchScratch &P) {
+    const int pr1 = pr0 + rq;
+    float c[4], L, D;
+    patch_centre(P, c, L, D);
+    float t1[4], t2[4];
+    {
         const float4 v00 = *reinterpret_cast<const float4 *>(sv[pr0 * W + p0].v);
         const float4 v01 = *reinterpret_cast<const float4 *>(sv[pr0 * W + p0 + cq].v);
         const float4 v10 = *reinterpret_cast<const float4 *>(sv[pr1 * W + p0].v);
@@ -352,7 +387,7 @@ __device__ __forceinline__ void patch_frame(const Vtx<1> *sv, int W, int t, int 
 #pragma unroll
     for (int i = 0; i < 4; ++i) E[1][i] = t2[i] * s2;
     // zero or unbounded parameter directions: no frame
-    bool bad = !(n1 > 1e-30f && n1 < 1e30f && n2 > 1e-30f && n2 < 1e30f);
+    const bool bad = !(n1 > 1e-30f && n1 < 1e30f && n2 > 1e-30f && n2 < 1e30f);
     {
         // e_2 from the coordinate axis k farthest from span(e_0, e_1): the one
         // with the least e_0k^2 + e_1k^2 (|cross4(e_0, e_1, axis_k)|^2 is one minus
@@ -377,24 +412,55 @@ __device__ __forceinline__ void patch_frame(const Vtx<1> *sv, int W, int t, int 
 #pragma unroll
         for (int i = 0; i < 4; ++i) E[3][i] = x[i] * s4;
     }
-    // the vertices: lane l takes column p0 + l of the patch (rows pr0..pr1), and
-    // lanes 0..rq the closing column p0 + cq, one vertex each; the integer
-    // maximum keeps NaN
-    unsigned am[4] = {0u, 0u, 0u, 0u};
-    auto vertex = [&](const Vtx<1> &v) {
-        const float4 hv = *reinterpret_cast<const float4 *>(v.v);
-        const float d[4] = {hv.x - c[0], hv.y - c[1], hv.z - c[2], hv.w - c[3]};
+    P.axes[0] = make_float4(c[0], c[1], c[2], c[3]);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) am[k] = max(am[k], abs_bits(dot4f(E[k], d)));
-    };
-    if (l < cq)
-        for (int rr = pr0; rr <= pr1; ++rr) vertex(sv[rr * W + t]);
-    if (cq > 0 && l <= rq) vertex(sv[(pr0 + l) * W + p0 + cq]);
+    for (int k = 0; k < 4; ++k) P.axes[1 + k] = make_float4(E[k][0], E[k][1], E[k][2], E[k][3]);
+    P.flags.x = bad;
+}
+
+// Lane l of a patch takes its vertex column l (rows pr0..pr0 + rq) and, for l <= rq, the
+// vertex of the closing column in row pr0 + l; the integer maximum keeps NaN.  Every
+// lane of the warp calls it (cq = 0: no patch).
+__device__ __forceinline__ void frame_extents(const Vtx<1> *sv, int W, int t, int cq, int pr0, int rq, PatchScratch &P) {
+    const int l = t & (kPatchI - 1), p0 = t - l;
+    unsigned am[4] = {0u, 0u, 0u, 0u};
+    if (cq > 0) {
+        const float4 c = P.axes[0], e0 = P.axes[1], e1 = P.axes[2], e2 = P.axes[3], e3 = P.axes[4];
+        auto vertex = [&](const Vtx<1> &v) {
+            const float4 x = *reinterpret_cast<const float4 *>(v.v);
+            const float d[4] = {x.x - c.x, x.y - c.y, x.z - c.z, x.w - c.w};
+            auto dot = [&](const float4 &e) {
+                return abs_bits(fmaf(e.w, d[3], fmaf(e.z, d[2], fmaf(e.y, d[1], e.x * d[0]))));
+            };
+            am[0] = max(am[0], dot(e0));
+            am[1] = max(am[1], dot(e1));
+            am[2] = max(am[2], dot(e2));
+            am[3] = max(am[3], dot(e3));
+        };
+        if (l < cq)
+            for (int rr = pr0; rr <= pr0 + rq; ++rr) vertex(sv[rr * W + t]);
+        if (l <= rq) vertex(sv[(pr0 + l) * W + p0 + cq]);
+    }
 #pragma unroll
     for (int off = 1; off < kPatchI; off <<= 1)
 #pragma unroll
         for (int k = 0; k < 4; ++k) am[k] = max(am[k], __shfl_xor_sync(0xffffffffu, am[k], off));
-    // per-patch terms (every lane alike)
+    if (cq > 0 && l == 0) P.top = make_uint4(am[0], am[1], am[2], am[3]);
+}
+
+__device__ __forceinline__ void frame_write(const PatchScratch &P, float4 *out, uint32_t p) {
+    const float u = 5.9604645e-08f;
+    const float inf = __int_as_float(0x7f800000);
+    float c[4], L, D;
+    patch_centre(P, c, L, D);
+    float E[4][4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float4 e = P.axes[1 + k];
+        E[k][0] = e.x; E[k][1] = e.y; E[k][2] = e.z; E[k][3] = e.w;
+    }
+    const unsigned am[4] = {P.top.x, P.top.y, P.top.z, P.top.w};
+    bool bad = P.flags.x != 0;
     float nk[4], emax = 0.0f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -432,16 +498,11 @@ __device__ __forceinline__ void patch_frame(const Vtx<1> *sv, int W, int t, int 
         h[0] = h[1] = h[2] = h[3] = inf;
         rho = inf;
     }
-    if (patch_lane && l == 0) {
-        float4 *o = out + (size_t)p * kFrameF4;
-        o[0] = make_float4(c[0], c[1], c[2], c[3]);
-        o[1] = make_float4(E[0][0], E[0][1], E[0][2], E[0][3]);
-        o[2] = make_float4(E[1][0], E[1][1], E[1][2], E[1][3]);
-        o[3] = make_float4(E[2][0], E[2][1], E[2][2], E[2][3]);
-        o[4] = make_float4(E[3][0], E[3][1], E[3][2], E[3][3]);
-        o[5] = make_float4(h[0], h[1], h[2], h[3]);
-        o[6] = make_float4(rho, L, nk[2], nk[3]);
-    }
+    float4 *o = out + (size_t)p * kFrameF4;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) o[k] = P.axes[k];
+    o[5] = make_float4(h[0], h[1], h[2], h[3]);
+    o[6] = make_float4(rho, L, nk[2], nk[3]);
 }
 
 // ---------------------------------------------------------------------------
@@ -453,6 +514,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
     Vtx<PREC> *sv = reinterpret_cast<Vtx<PREC> *>(smem_raw);
     const int TI = blockDim.x;
     const int W = TI + 1;
+    PatchScratch *sp = reinterpret_cast<PatchScratch *>(sv + (TK + 1) * W);   // with frames: the tile's patches
     const long long tile = blockIdx.x;
 
     const PassEntry pe = a.entries[find_entry(a, tile, false)];
@@ -464,7 +526,9 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
     const int rows_q = min(TK, m.nqk - kq0);
 
     // ---- load the tile's vertices: rows kq0..kq0+rows_q, columns i0..i0+cols_q
-    unsigned nonfinite = 0;
+    // the largest high word of |x| tells whether any is not finite (a test of each value
+    // beside its rounding becomes an FP64 comparison)
+    unsigned top = 0;
     {
         const int t = threadIdx.x;
         double x[TK + 1][4];
@@ -485,7 +549,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
         for (int r = 0; r <= TK; ++r) {
             if (col_ok && r <= rows_q) {
 #pragma unroll
-                for (int c = 0; c < 4; ++c) nonfinite |= !finite64(x[r][c]);
+                for (int c = 0; c < 4; ++c) top = max(top, (unsigned)__double2hiint(x[r][c]) & 0x7fffffffu);
                 const Vtx<PREC> v = to_vtx<PREC>(x[r]);
                 sv[r * W + t] = v;
                 if (r < rows_q || last_rows) write_vlo(m, (size_t)(kq0 + r) * m.N + vi, v);
@@ -501,7 +565,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) {
                 y[c] = __ldg(m.c[c] + off);
-                nonfinite |= !finite64(y[c]);
+                top = max(top, (unsigned)__double2hiint(y[c]) & 0x7fffffffu);
             }
             const Vtx<PREC> v = to_vtx<PREC>(y);
             sv[t * W + cols_q] = v;
@@ -523,12 +587,10 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
         // the row loop and its shuffles are uniform).  The widest extent the
         // grid needs is then the widest patch's.
         // this column's boxes over the upper and lower halves of the patch row
-        BoxT<PREC> prev, ptop, pbot, pb0, pb1;   // pb0, pb1: the boxes of the tile's patch rows
+        BoxT<PREC> prev, ptop, pbot;
         box_empty(prev);
         box_empty(ptop);
         box_empty(pbot);
-        box_empty(pb0);
-        box_empty(pb1);
         // the patch exists when its first column is in the tile
         const bool patch_lane = (t & ~(kPatchI - 1)) < cols_q;
         if (col_valid) {
@@ -565,25 +627,40 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
                     write_box<PREC>(m.qbox, 4 * p + 2 + half, closed<PREC>(pbot));
                 }
                 if (patch_lane && (t % kPatchI) == 0) {
-                    write_box<PREC>(m.pbox, p, closed<PREC>(pb));
+                    const BoxT<PREC> cb = closed<PREC>(pb);
+                    write_box<PREC>(m.pbox, p, cb);
                     acc.add(pb);
+                    if constexpr (PREC == 1) {
+                        PatchScratch &P = sp[(r / kPatchK) * (TI / kPatchI) + t / kPatchI];
+                        P.lo = make_float4(cb.lo[0], cb.lo[1], cb.lo[2], cb.lo[3]);
+                        P.hi = make_float4(cb.hi[0], cb.hi[1], cb.hi[2], cb.hi[3]);
+                    }
                 }
-                if (r < kPatchK) pb0 = pb;
-                else pb1 = pb;
                 box_empty(ptop);
                 box_empty(pbot);
             }
         }
-        // the frames of the tile's patches, after its rows (fewer registers live
-        // than at the close of each patch row)
+        // the frames of the tile's patches
         if constexpr (PREC == 1) {
             if (a.frames) {
-                for (int pr = 0; pr * kPatchK < rows_q; ++pr) {
-                    const BoxT<1> pbx = closed<1>(pr == 0 ? pb0 : pb1);
-                    const uint32_t p = (uint32_t)(kq0 / kPatchK + pr) * (uint32_t)m.npi + (uint32_t)(i / kPatchI);
-                    patch_frame(sv, W, t, cols_q, pr * kPatchK, min(kPatchK, rows_q - pr * kPatchK), pbx,
-                                m.pframe, p, patch_lane);
+                const int across = TI / kPatchI, np = across * ((rows_q + kPatchK - 1) / kPatchK);
+                __syncthreads();
+                for (int q = t; q < np; q += TI) {
+                    const int p0 = (q % across) * kPatchI, pr0 = (q / across) * kPatchK;
+                    if (p0 < cols_q)
+                        frame_axes(sv, W, p0, min(kPatchI, cols_q - p0), pr0, min(kPatchK, rows_q - pr0), sp[q]);
                 }
+                __syncthreads();
+                const int cq = patch_lane ? min(kPatchI, cols_q - (t & ~(kPatchI - 1))) : 0;
+                for (int pr0 = 0; pr0 < rows_q; pr0 += kPatchK)
+                    frame_extents(sv, W, t, cq, pr0, min(kPatchK, rows_q - pr0),
+                                  sp[(pr0 / kPatchK) * across + t / kPatchI]);
+                __syncthreads();
+                for (int q = t; q < np; q += TI)
+                    if ((q % across) * kPatchI < cols_q)
+                        frame_write(sp[q], m.pframe,
+                                    (uint32_t)(kq0 / kPatchK + q / across) * (uint32_t)m.npi +
+                                        (uint32_t)(i0 / kPatchI + q % across));
             }
         }
     } else if (FACE == 1 && col_valid) {
@@ -632,52 +709,41 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
         }
     }
 
-    // block reduction, then one set of atomics per block
-    // in the accumulators' own type (no FP64 instruction: GB300's FP64 pipe is narrow)
-    typedef typename std::remove_reference<decltype(acc.lo[0])>::type AccT;
-    __shared__ AccT red[8][12];
+    // block reduction, then one set of atomics per block, each of twelve lanes its own
+    // (lo, hi, extent of every coordinate)
+    __shared__ long long red[8][12];
     __shared__ unsigned redf[8][2];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int d = 0; d < 4; ++d) {
-        for (int off = 16; off > 0; off >>= 1) {
-            acc.lo[d] = min(acc.lo[d], __shfl_xor_sync(FULL, acc.lo[d], off));
-            acc.hi[d] = max(acc.hi[d], __shfl_xor_sync(FULL, acc.hi[d], off));
-            acc.w[d] = max(acc.w[d], __shfl_xor_sync(FULL, acc.w[d], off));
-        }
+        const long long l = ~warp_max(negated(acc.lo[d])), h = warp_max(acc.hi[d]), w = warp_max(acc.w[d]);
+        if (lane == 0) { red[warp][d] = l; red[warp][4 + d] = h; red[warp][8 + d] = w; }
     }
-    unsigned fl = __reduce_or_sync(FULL, nonfinite);
-    unsigned seen = __reduce_or_sync(FULL, acc.seen);
+    const unsigned fl = __any_sync(FULL, top >= 0x7ff00000u) ? 1u : 0u;
+    const unsigned seen = __reduce_or_sync(FULL, acc.seen);
     if (lane == 0) {
-#pragma unroll
-        for (int d = 0; d < 4; ++d) { red[warp][d] = acc.lo[d]; red[warp][4 + d] = acc.hi[d]; red[warp][8 + d] = acc.w[d]; }
         redf[warp][0] = fl;
         redf[warp][1] = seen;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    if (warp == 0) {
         const int nw = blockDim.x >> 5;
         Bounds *B = a.bounds + pe.mesh;
-        unsigned f = 0, s = 0;
-        for (int w = 0; w < nw; ++w) { f |= redf[w][0]; s |= redf[w][1]; }
-        if (s) {
-#pragma unroll
-            for (int d = 0; d < 4; ++d) {
-                AccT l = red[0][d], h = red[0][4 + d], ww = red[0][8 + d];
-                for (int w = 1; w < nw; ++w) {
-                    l = min(l, red[w][d]);
-                    h = max(h, red[w][4 + d]);
-                    ww = max(ww, red[w][8 + d]);
-                }
-                atomicMin(&B->lo[d], ord_enc_any(l));
-                atomicMax(&B->hi[d], ord_enc_any(h));
-                atomicMax(&B->w[d], ord_enc_any(ww));
-            }
-            atomicOr(&B->faces, 1u);
+        const unsigned f = __any_sync(FULL, lane < nw && redf[lane & 7][0]), s = __any_sync(FULL, lane < nw && redf[lane & 7][1]);
+        if (s && lane < 12) {
+            long long v = red[0][lane];
+            for (int w = 1; w < nw; ++w) v = lane < 4 ? min(v, red[w][lane]) : max(v, red[w][lane]);
+            const unsigned long long e = encoded<PREC>(v);
+            if (lane < 4) atomicMin(&B->lo[lane], e);
+            else if (lane < 8) atomicMax(&B->hi[lane - 4], e);
+            else atomicMax(&B->w[lane - 8], e);
         }
-        if (f) {
-            atomicOr(&B->flags, ST_NONFINITE);
-            atomicOr(&a.ctr->status, ST_NONFINITE);
+        if (lane == 0) {
+            if (s) atomicOr(&B->faces, 1u);
+            if (f) {
+                atomicOr(&B->flags, ST_NONFINITE);
+                atomicOr(&a.ctr->status, ST_NONFINITE);
+            }
         }
     }
 }
@@ -928,6 +994,7 @@ __global__ void k_grid_params(const Bounds *b, const int2 *pairs, int n_pairs, G
 template <int PREC, int FACE, int TK>
 void launch_one(const FacePassArgs &a, int block, cudaStream_t st) {
     size_t smem = (size_t)(TK + 1) * (block + 1) * sizeof(Vtx<PREC>);
+    if (PREC == 1 && a.patch) smem += (size_t)(block / kPatchI) * (TK / kPatchK) * sizeof(PatchScratch);
     k_bounds_pass<PREC, FACE, TK><<<(unsigned)a.total_tiles, block, smem, st>>>(a);
 }
 
