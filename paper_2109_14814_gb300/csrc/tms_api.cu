@@ -82,17 +82,23 @@ struct Plan {
     MeshDev *d_meshes = nullptr;
     std::vector<MeshDev> h_meshes;    // host copy of the mesh table
     int2 pair0 = {0, 0};              // pair 0's meshes in it
-    // patch level: the patch views (one "face" per patch, its box in pbox),
-    // which the cell passes and the grid emission read instead of the meshes
+    // patch level: the patch pairs come from the meshes' trees (tms_tree.cu), not
+    // from the grid
     bool patch = false;
     // patch frames (mixed precision with the FP32 filters): the patch-pair
     // test drops pairs that no triangle pair in them can make an FP64 hit
     bool frames = false;
-    MeshDev *d_pmeshes = nullptr;
     // per-pair cell multipliers (size classes tuned by tms_autotune), or empty
     std::vector<float> cm_pair;
     float *d_cm_pair = nullptr;
     unsigned char *pbox = nullptr;    // patch boxes of all meshes
+    unsigned char *tbox = nullptr;    // node boxes of all meshes' trees above the patches
+    MeshTree *d_trees = nullptr;
+    long long *d_top_base = nullptr;
+    long long top_tiles = 0;
+    int top = 0;
+    uint32_t up_blocks[kTreeLevels / 2] = {};
+    Cand *nodes[2] = {nullptr, nullptr};   // node pairs, odd and even levels (ent_cap each)
     unsigned char *qbox = nullptr;    // their quarter boxes
     float4 *pframe = nullptr;         // their frames (kFrameF4 float4 per patch)
     Cand *ppairs = nullptr;
@@ -154,10 +160,10 @@ struct Plan {
     void free_scratch() {
         void *ptrs[] = {bmA, bmH, ek, ev, eslot, erank, grouped, tkey, crec, tcnt, tstart,
                         sort_scratch, cand, surv, hits, hk, hk2, okeys, hv, hv2,
-                        keep, kscan, ppairs, psurv, qsurv};
+                        keep, kscan, ppairs, psurv, qsurv, nodes[0], nodes[1]};
         for (void *p : ptrs)
             if (p) cudaFree(p);
-        ppairs = psurv = nullptr;
+        ppairs = psurv = nodes[0] = nodes[1] = nullptr;
         qsurv = nullptr;
         bmA = bmH = nullptr; ek = nullptr; ev = eslot = erank = grouped = nullptr;
         tkey = nullptr; crec = nullptr; tcnt = nullptr; tstart = nullptr;
@@ -169,8 +175,8 @@ struct Plan {
         if (st) cudaStreamSynchronize(st);
         free_scratch();
         void *ptrs[] = {d_meshes, d_pairs, d_pass_bounds, d_pass_all, d_pass_A, d_pass_B, d_bounds,
-                        d_ctr, partials, vlo, fbox, d_pmeshes, pbox, qbox, pframe, d_cm_pair,
-                        tail, bbase};
+                        d_ctr, partials, vlo, fbox, pbox, qbox, pframe, d_cm_pair,
+                        tail, bbase, tbox, d_trees, d_top_base};
         for (void *p : ptrs)
             if (p) cudaFree(p);
         if (h_ctr) cudaFreeHost(h_ctr);
@@ -183,32 +189,37 @@ struct Plan {
 
     tms_status alloc_scratch() {
         free_scratch();
-        TMS_CK(dalloc(&bmA, (size_t)1 << (bmA_bits)));
-        TMS_CK(dalloc(&bmH, (size_t)1 << (bmH_bits)));
-        TMS_CK(dalloc(&ek, ent_cap));
-        TMS_CK(dalloc(&ev, ent_cap));
-        TMS_CK(dalloc(&eslot, ent_cap));
-        TMS_CK(dalloc(&erank, ent_cap));
-        TMS_CK(dalloc(&grouped, ent_cap));
-        // cell table: a power of two, all slots free (zero); distinct cells are
-        // far fewer than entries, so it starts at a sixteenth of the entry
-        // capacity (L2-resident) and grows when a search finds it over half full
-        tsize = 1024;
-        const unsigned long long want = (prm.inject & 8u) ? 0 : ent_cap / 16;
-        while ((tsize < want || tsize < tsize_min) && tsize < (1ULL << 31)) tsize <<= 1;
-        TMS_CK(dalloc(&tkey, tsize));
-        TMS_CK(dalloc(&tcnt, tsize));
-        TMS_CK(dalloc(&tstart, tsize));
-        TMS_CK(cudaMemset(tkey, 0, tsize * sizeof(unsigned long long)));
-        TMS_CK(cudaMemset(tcnt, 0, tsize * sizeof(uint2)));
-        // per cell: a cell holding both meshes has at least two entries
-        TMS_CK(dalloc(&crec, ent_cap / 2 + 1));
+        if (patch) {
+            TMS_CK(dalloc(&nodes[0], ent_cap));
+            TMS_CK(dalloc(&nodes[1], ent_cap));
+            TMS_CK(dalloc(&ppairs, ppair_cap));
+            TMS_CK(dalloc(&psurv, ppair_cap));
+        } else {
+            TMS_CK(dalloc(&bmA, (size_t)1 << (bmA_bits)));
+            TMS_CK(dalloc(&bmH, (size_t)1 << (bmH_bits)));
+            TMS_CK(dalloc(&ek, ent_cap));
+            TMS_CK(dalloc(&ev, ent_cap));
+            TMS_CK(dalloc(&eslot, ent_cap));
+            TMS_CK(dalloc(&erank, ent_cap));
+            TMS_CK(dalloc(&grouped, ent_cap));
+            // cell table: a power of two, all slots free (zero); distinct cells are
+            // far fewer than entries, so it starts at a sixteenth of the entry
+            // capacity (L2-resident) and grows when a search finds it over half full
+            tsize = 1024;
+            const unsigned long long want = (prm.inject & 8u) ? 0 : ent_cap / 16;
+            while ((tsize < want || tsize < tsize_min) && tsize < (1ULL << 31)) tsize <<= 1;
+            TMS_CK(dalloc(&tkey, tsize));
+            TMS_CK(dalloc(&tcnt, tsize));
+            TMS_CK(dalloc(&tstart, tsize));
+            TMS_CK(cudaMemset(tkey, 0, tsize * sizeof(unsigned long long)));
+            TMS_CK(cudaMemset(tcnt, 0, tsize * sizeof(uint2)));
+            // per cell: a cell holding both meshes has at least two entries
+            TMS_CK(dalloc(&crec, ent_cap / 2 + 1));
+        }
         TMS_CK(dalloc(reinterpret_cast<unsigned char **>(&sort_scratch),
                       radix_scratch_size(hit_cap, 2 * tri_bits + pair_bits)));
         TMS_CK(dalloc(&cand, cand_cap));
         TMS_CK(dalloc(&qsurv, cand_cap));
-        if (patch) TMS_CK(dalloc(&ppairs, ppair_cap));
-        if (patch) TMS_CK(dalloc(&psurv, ppair_cap));
         TMS_CK(dalloc(&surv, surv_cap));
         TMS_CK(dalloc(&hits, hit_cap));
         TMS_CK(dalloc(&hk, hit_cap));
@@ -263,15 +274,50 @@ struct Plan {
         kernels += 5 + (dOffsets ? 1 : 0);
     }
 
-    void enqueue(cudaStream_t s) {
+    // Patch level: bounds pass, trees, patch pairs, quad pairs.
+    void enqueue_patches(cudaStream_t s) {
+        const tms_params &p = prm;
+        const int block = (p.block_faces == 64 || p.block_faces == 256) ? p.block_faces : 128;
+        mark(0, s);
+        mark(1, s);
+        FacePassArgs fa;
+        memset(&fa, 0, sizeof(fa));
+        fa.meshes = d_meshes;
+        fa.tile_rows = p.tile_rows;
+        fa.ctr = d_ctr;
+        fa.entries = d_pass_bounds; fa.n_entries = n_pass_bounds; fa.total_tiles = tiles_all;
+        fa.mode = MODE_BOUNDS;
+        fa.patch = 1;
+        fa.frames = frames ? 1 : 0;
+        fa.nonfinite = tail + kTailBuckets + kTailMax / 32;
+        launch_face_pass(fa, p.precision, 1, block, s);
+        for (int i = 2; i < 10; ++i) mark(i, s);
+        TreeArgs ta;
+        ta.trees = d_trees; ta.n_meshes = n_meshes; ta.pairs = d_pairs; ta.n_pairs = nPairs;
+        ta.top = top; ta.top_base = d_top_base; ta.top_tiles = top_tiles;
+        memcpy(ta.up_blocks, up_blocks, sizeof(up_blocks));
+        ta.list[0] = nodes[0]; ta.list[1] = nodes[1]; ta.cap = ent_cap;
+        ta.ppairs = ppairs; ta.ppair_cap = ppair_cap; ta.ctr = d_ctr; ta.tail = tail;
+        ta.nonfinite = fa.nonfinite; ta.grid0 = d_grids;
+        launch_tree(ta, p.precision, grid / 2, s);
+        mark(10, s);
+        PatchArgs pa;
+        pa.ppairs = ppairs; pa.psurv = psurv; pa.ppair_cap = ppair_cap; pa.meshes = d_meshes;
+        pa.pairs = d_pairs; pa.ctr = d_ctr; pa.cand = cand; pa.cand_cap = cand_cap;
+        pa.moller = p.moller;
+        pa.frames = frames ? 1 : 0;
+        pa.tau = p.tau;
+        launch_patch_quads(pa, p.precision, grid / 2, s);
+        kernels = 1 + tree_launches(top) + 2;
+    }
+
+    // Face level: bounds pass, grid, cells, candidate emission.
+    void enqueue_faces(cudaStream_t s) {
         const tms_params &p = prm;
         const int prec = p.precision, fl = p.face_level;
         const int block = (p.block_faces == 64 || p.block_faces == 256) ? p.block_faces : 128;
-        kernels = 0;
         mark(0, s);
-        // the occupancy filter runs at the face level only: patches are few, and
-        // nearly every patch-cell incidence lies in a cell both meshes occupy
-        const bool filter = p.cell_filter && !patch;
+        const bool filter = p.cell_filter != 0;
         launch_search_init(d_bounds, n_meshes, d_ctr, filter ? bmA : nullptr,
                            (unsigned long long)1 << bmA_bits, filter ? bmH : nullptr,
                            (unsigned long long)1 << bmH_bits, long_tail ? nullptr : tail, grid, s);
@@ -281,7 +327,6 @@ struct Plan {
         ga.tkey = tkey; ga.tcnt = tcnt; ga.tstart = tstart; ga.tsize = tsize;
         ga.cells = crec; ga.grids = d_grids;
         ga.grouped = grouped; ga.partials = partials; ga.ctr = d_ctr;
-        kernels += 1;
         mark(1, s);
 
         FacePassArgs fa;
@@ -301,16 +346,10 @@ struct Plan {
 
         fa.entries = d_pass_bounds; fa.n_entries = n_pass_bounds; fa.total_tiles = tiles_all;
         fa.mode = MODE_BOUNDS;
-        fa.patch = patch ? 1 : 0;
-        fa.frames = frames ? 1 : 0;
         launch_face_pass(fa, prec, fl, block, s);
-        // the cell passes and the grid emission work on the patches (patch level)
-        fa.patch = 0;
-        fa.frames = 0;
-        if (patch) fa.meshes = d_pmeshes;
         mark(2, s);
         launch_grid_params(d_bounds, d_pairs, nPairs, d_grids, p.cell_mult, s, d_cm_pair);
-        kernels += 2;
+        kernels = 3;
         mark(3, s);
 
         if (filter) {
@@ -349,29 +388,16 @@ struct Plan {
         ea.cells = crec; ea.vals = grouped;
         ea.grids = d_grids; ea.meshes = d_meshes; ea.pairs = d_pairs; ea.ctr = d_ctr;
         ea.ent_cap = ent_cap; ea.cand = cand; ea.cand_cap = cand_cap; ea.moller = p.moller;
-        ea.cand_ctr = &d_ctr->cand;
-        ea.waves = 0;
-        if (patch) {
-            // patch pairs with overlapping boxes, each once (owner cell); few
-            // tiles (about one per cell), so one wave of blocks
-            ea.meshes = d_pmeshes; ea.cand = ppairs; ea.cand_cap = ppair_cap;
-            ea.cand_ctr = &d_ctr->ppairs; ea.moller = 0; ea.waves = 1;
-        }
         launch_emit(ea, prec, fl, grid / 2, s);
         kernels += 1;
         mark(10, s);
-        if (patch) {
-            // the quad pairs of the patch pairs
-            PatchArgs pa;
-            pa.ppairs = ppairs; pa.psurv = psurv; pa.ppair_cap = ppair_cap; pa.meshes = d_meshes;
-            pa.pairs = d_pairs;
-            pa.ctr = d_ctr; pa.ent_cap = ent_cap; pa.cand = cand; pa.cand_cap = cand_cap;
-            pa.moller = p.moller;
-            pa.frames = frames ? 1 : 0;
-            pa.tau = p.tau;
-            launch_patch_quads(pa, prec, grid / 2, s);
-            kernels += 2;
-        }
+    }
+
+    void enqueue(cudaStream_t s) {
+        const tms_params &p = prm;
+        const int fl = p.face_level;
+        if (patch) enqueue_patches(s);
+        else enqueue_faces(s);
         mark(11, s);
 
         NarrowArgs na;
@@ -473,10 +499,9 @@ tms_status check_mesh(tms_mesh m, int device) {
     return TMS_OK;
 }
 
-// a mesh in a pass: bounds-pass tiles over its quads; cell-pass slots over its
-// faces, or over its patches (patch level)
+// a mesh in a pass: bounds-pass tiles over its quads; cell-pass slots over its faces
 void fill_pass(std::vector<PassEntry> &v, long long &tiles, long long &fslots, const tms_mesh m,
-               int mesh_index, int pair, int role, int block, int rows, int face_level, bool patch) {
+               int mesh_index, int pair, int role, int block, int rows, int face_level) {
     PassEntry e;
     e.mesh = mesh_index;
     e.pair = pair;
@@ -486,8 +511,7 @@ void fill_pass(std::vector<PassEntry> &v, long long &tiles, long long &fslots, c
     e.tile_base = tiles;
     tiles += (long long)e.tiles_i * tiles_k;
     e.face_base = fslots;
-    e.faces = patch ? (long long)((m->dev.nqi + kPatchI - 1) / kPatchI) * ((m->dev.nqk + kPatchK - 1) / kPatchK)
-                    : (long long)face_slots(m->dev, face_level);
+    e.faces = (long long)face_slots(m->dev, face_level);
     fslots += (e.faces + 31) / 32 * 32;
     v.push_back(e);
 }
@@ -530,29 +554,24 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         meshes.push_back(m->dev);
         row_of[m->id] = r;
         long long unused = 0;
-        fill_pass(pbounds, P->tiles_all, unused, m, r, 0, 0, block, rows, fl, patch);
+        fill_pass(pbounds, P->tiles_all, unused, m, r, 0, 0, block, rows, fl);
         return r;
     };
     for (int i = 0; i < nPairs; ++i) {
         const int ia = row(A[i]), ib = row(B[i]);
         pairs.push_back(make_int2(ia, ib));
         const unsigned long long fpq = prm.face_level == 0 ? 2 : 1;
-        auto cells_of = [&](const MeshDev &d) -> unsigned long long {
-            if (patch)
-                return (unsigned long long)((d.nqi + kPatchI - 1) / kPatchI) * ((d.nqk + kPatchK - 1) / kPatchK);
-            return fpq * (unsigned long long)d.nqi * d.nqk;
-        };
-        P->facesA += cells_of(A[i]->dev);
-        P->facesB += cells_of(B[i]->dev);
+        P->facesA += fpq * (unsigned long long)A[i]->dev.nqi * A[i]->dev.nqk;
+        P->facesB += fpq * (unsigned long long)B[i]->dev.nqi * B[i]->dev.nqk;
         max_tri = std::max(max_tri, 2ULL * A[i]->dev.N * A[i]->dev.nqk);
         max_tri = std::max(max_tri, 2ULL * B[i]->dev.N * B[i]->dev.nqk);
     }
     long long unused = 0;
     for (int i = 0; i < nPairs; ++i) {
-        fill_pass(pall, unused, P->fslots_all, A[i], pairs[i].x, i, 0, block, rows, fl, patch);
-        fill_pass(pall, unused, P->fslots_all, B[i], pairs[i].y, i, 1, block, rows, fl, patch);
-        fill_pass(pa, unused, P->fslots_A, A[i], pairs[i].x, i, 0, block, rows, fl, patch);
-        fill_pass(pb, unused, P->fslots_B, B[i], pairs[i].y, i, 1, block, rows, fl, patch);
+        fill_pass(pall, unused, P->fslots_all, A[i], pairs[i].x, i, 0, block, rows, fl);
+        fill_pass(pall, unused, P->fslots_all, B[i], pairs[i].y, i, 1, block, rows, fl);
+        fill_pass(pa, unused, P->fslots_A, A[i], pairs[i].x, i, 0, block, rows, fl);
+        fill_pass(pb, unused, P->fslots_B, B[i], pairs[i].y, i, 1, block, rows, fl);
     }
     // written by the bounds pass: the vertices rounded down to FP32 (16 bytes each;
     // the plain precision without the FP32 filters reads none) and, at the face
@@ -579,13 +598,49 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         pframe_off.push_back(pframe_total);
         pframe_total += ((unsigned long long)md.npi * md.npk * kFrameF4 + 15) / 16 * 16;
     }
-    std::vector<MeshDev> pmeshes;
+    // the trees: levels above the patches, up to the lowest that leaves few pairs
+    std::vector<MeshTree> trees(patch ? meshes.size() : 0);
+    std::vector<long long> top_base;
+    unsigned long long tbox_total = 0, nodes1 = 0;
+    if (patch) {
+        for (size_t i = 0; i < meshes.size(); ++i) {
+            int ni = meshes[i].npi, nk = meshes[i].npk;
+            for (int l = 0; l < kTreeLevels; ++l, ni = (ni + 3) / 4, nk = (nk + 3) / 4) {
+                TreeLevel &t = trees[i].lev[l];
+                t.ni = ni;
+                t.nk = nk;
+                t.magic = recip64((unsigned long long)ni);
+                t.box = nullptr;
+            }
+            nodes1 += (unsigned long long)trees[i].lev[1].ni * trees[i].lev[1].nk;
+        }
+        auto size = [&](int mesh, int l) { return (long long)trees[mesh].lev[l].ni * trees[mesh].lev[l].nk; };
+        for (P->top = 0; P->top < kTreeTop; ++P->top) {
+            unsigned long long n = 0;
+            for (const int2 &q : pairs) n += (unsigned long long)size(q.x, P->top) * size(q.y, P->top);
+            if (n <= kTreeTopPairs) break;
+        }
+        for (const int2 &q : pairs) {
+            top_base.push_back(P->top_tiles);
+            P->top_tiles += (size(q.x, P->top) + 31) / 32 * ((size(q.y, P->top) + 31) / 32);
+        }
+        for (size_t i = 0; i < meshes.size(); ++i) {
+            for (int l = 0; l < kTreeLevels / 2; ++l) {
+                trees[i].up_base[l] = P->up_blocks[l];
+                if (2 * l + 2 < kTreeLevels) P->up_blocks[l] += (uint32_t)size((int)i, 2 * l + 2);
+            }
+            // k_tree_up makes two levels at a time
+            for (int l = 1; P->top > 0 && l <= (P->top + 1) / 2 * 2; ++l)
+                tbox_total += ((unsigned long long)size((int)i, l) * box_bytes + 255) / 256 * 256;
+        }
+    }
     {
         cudaError_t se = dalloc(&P->vlo, vlo_total);
         if (se == cudaSuccess && !patch) se = dalloc(&P->fbox, fbox_total);
         if (se == cudaSuccess && patch) se = dalloc(&P->pbox, pbox_total);
         if (se == cudaSuccess && patch) se = dalloc(&P->qbox, 4 * pbox_total);
         if (se == cudaSuccess && P->frames) se = dalloc(&P->pframe, pframe_total);
+        if (se == cudaSuccess && patch) se = dalloc(&P->tbox, tbox_total);
         if (se != cudaSuccess) { g_err = cudaGetErrorString(se); delete P; return TMS_ERR_CUDA; }
         for (size_t i = 0; i < meshes.size(); ++i) {
             meshes[i].vlo = keep_vlo ? P->vlo + vlo_off[i] : nullptr;
@@ -596,18 +651,14 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
                 if (P->frames) meshes[i].pframe = P->pframe + pframe_off[i];
             }
         }
-        // a patch view is a mesh of npi x npk quad-like slots, all valid
-        for (const MeshDev &md : meshes) {
-            MeshDev v = md;
-            v.N = md.npi;
-            v.M = md.npk + 1;
-            v.periodic = 1;
-            v.nqi = md.npi;
-            v.nqk = md.npk;
-            v.fbox = md.pbox;
-            v.vlo = nullptr;
-            v.pframe = nullptr;
-            pmeshes.push_back(v);
+        unsigned long long off = 0;
+        for (size_t i = 0; i < trees.size(); ++i) {
+            trees[i].lev[0].box = meshes[i].pbox;
+            for (int l = 1; P->top > 0 && l <= (P->top + 1) / 2 * 2; ++l) {
+                TreeLevel &t = trees[i].lev[l];
+                t.box = P->tbox + off;
+                off += ((unsigned long long)t.ni * t.nk * box_bytes + 255) / 256 * 256;
+            }
         }
     }
     P->n_meshes = (int)meshes.size();
@@ -632,7 +683,12 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     cudaError_t e;
 #define TMS_PCK(call) do { if ((e = (call)) != cudaSuccess) { g_err = cudaGetErrorString(e); delete P; return TMS_ERR_CUDA; } } while (0)
     TMS_PCK(dalloc(&P->d_meshes, meshes.size()));
-    TMS_PCK(dalloc(&P->d_pmeshes, pmeshes.size()));
+    if (patch) {
+        TMS_PCK(dalloc(&P->d_trees, trees.size()));
+        TMS_PCK(dalloc(&P->d_top_base, top_base.size()));
+        TMS_PCK(cudaMemcpy(P->d_trees, trees.data(), trees.size() * sizeof(MeshTree), cudaMemcpyHostToDevice));
+        TMS_PCK(cudaMemcpy(P->d_top_base, top_base.data(), top_base.size() * sizeof(long long), cudaMemcpyHostToDevice));
+    }
     if (!cm_pair.empty()) {
         TMS_PCK(dalloc(&P->d_cm_pair, cm_pair.size()));
         TMS_PCK(cudaMemcpy(P->d_cm_pair, cm_pair.data(), cm_pair.size() * sizeof(float),
@@ -652,7 +708,9 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         P->d_grids = reinterpret_cast<Grid *>(blk + kGridOffset);
     }
     TMS_PCK(dalloc(&P->partials, 5 * 1024));
-    TMS_PCK(dalloc(&P->tail, kTailBuckets + kTailMax / 32));
+    // (and the word the bounds pass leaves a vertex that is not finite in)
+    TMS_PCK(dalloc(&P->tail, kTailBuckets + kTailMax / 32 + 1));
+    TMS_PCK(cudaMemset(P->tail, 0, (kTailBuckets + kTailMax / 32 + 1) * sizeof(uint32_t)));
     TMS_PCK(dalloc(&P->bbase, kTailBuckets + 1));
     // the range of (pair, triA), over which the buckets are spread
     P->bscale = (float)((double)kTailBuckets /
@@ -666,7 +724,6 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         P->h_grid0 = reinterpret_cast<Grid *>(hb + kGridOffset);
     }
     TMS_PCK(cudaMemcpy(P->d_meshes, meshes.data(), meshes.size() * sizeof(MeshDev), cudaMemcpyHostToDevice));
-    TMS_PCK(cudaMemcpy(P->d_pmeshes, pmeshes.data(), pmeshes.size() * sizeof(MeshDev), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pairs, pairs.data(), pairs.size() * sizeof(int2), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pass_bounds, pbounds.data(), pbounds.size() * sizeof(PassEntry), cudaMemcpyHostToDevice));
     TMS_PCK(cudaMemcpy(P->d_pass_all, pall.data(), pall.size() * sizeof(PassEntry), cudaMemcpyHostToDevice));
@@ -681,10 +738,10 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
 
     const unsigned long long faces = P->facesA + P->facesB;
     unsigned long long ent = prm.entry_capacity > 0 ? (unsigned long long)prm.entry_capacity
-                             : patch ? 4 * faces + (1 << 16)
+                             : patch ? std::max<unsigned long long>(1 << 16, 16 * nodes1)
                              : (prm.cell_filter ? std::max<unsigned long long>(1 << 16, faces / 2)
                                                 : 4 * faces + (1 << 16));
-    if (prm.inject & 1u) ent = 1;
+    if ((prm.inject & 1u) || (patch && (prm.inject & 8u))) ent = 1;
     P->ent_cap = std::min<unsigned long long>(ent, 0x7fffffffULL);
     // patch level: candidates are quad pairs, about one per quad of A
     const unsigned long long quadsA = [&] {
@@ -695,7 +752,8 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     P->cand_cap = prm.cand_capacity > 0 ? (unsigned long long)prm.cand_capacity
                   : patch ? std::max<unsigned long long>(1 << 16, quadsA + quadsA / 4)
                           : std::max<unsigned long long>(1 << 16, 2 * P->ent_cap);
-    P->ppair_cap = patch ? std::max<unsigned long long>(1 << 16, 4 * faces) : 0;
+    // (a patch has 32 quads)
+    P->ppair_cap = patch ? std::max<unsigned long long>(1 << 16, faces / 8) : 0;
     P->hit_cap = prm.hit_capacity > 0 ? (unsigned long long)prm.hit_capacity
                                       : std::max<unsigned long long>(1 << 14, P->cand_cap / 16);
     P->surv_cap = std::max<unsigned long long>(1 << 16, P->cand_cap / 8);
@@ -762,6 +820,7 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
         TMS_CK(configure_face_pass());
         configure_emit();
         configure_patch_quads();
+        configure_tree();
         configure_narrow();
         g_configured_mask |= 1 << device;
     }
@@ -796,11 +855,17 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
             return TMS_ERR_TIMEOUT;
         }
         bool grow = false;
-        if ((c.status & ST_TABLE_FULL) || c.claimed > P->tsize / 2) {
+        if (!P->patch && ((c.status & ST_TABLE_FULL) || c.claimed > P->tsize / 2)) {
             P->tsize_min = P->tsize * 4;
             grow = true;
         }
-        if (!grow && c.entries > P->ent_cap) {
+        unsigned long long nodes = 0;
+        for (unsigned long long v : c.nodes) nodes = std::max(nodes, v);
+        if (!grow && P->patch && nodes > P->ent_cap) {
+            P->ent_cap = nodes + nodes / 4 + 1024;
+            grow = true;
+        }
+        if (!grow && !P->patch && c.entries > P->ent_cap) {
             P->ent_cap = std::min<unsigned long long>(0x7fffffffULL, c.entries + c.entries / 4 + 1024);
             P->bmH_bits = std::min(25, std::max(11, ceil_log2(P->ent_cap * 8) - 5));
             P->cand_cap = std::max(P->cand_cap, 2 * P->ent_cap);
@@ -841,6 +906,7 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     tms_stats st;
     memset(&st, 0, sizeof(st));
     st.entries = (long long)c.entries;
+    for (unsigned long long v : c.nodes) st.entries += (long long)v;
     st.cells = (long long)c.cells;
     st.pair_slots = (long long)c.pair_slots;
     st.candidates = (long long)c.cand;
@@ -860,7 +926,9 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     st.kernels = P->kernels;
     g_stats[user] = st;
     if (prm.timing) g_stage_ms[user] = std::vector<float>(P->stage_ms, P->stage_ms + Plan::kStages);
-    if (c.entries > P->ent_cap || c.cand > P->cand_cap || c.fp64 > P->surv_cap ||
+    unsigned long long lists = c.entries;
+    for (unsigned long long v : c.nodes) lists = std::max(lists, v);
+    if (lists > P->ent_cap || c.cand > P->cand_cap || c.fp64 > P->surv_cap ||
         c.raw_hits > P->hit_cap || (P->patch && c.ppairs > P->ppair_cap)) {
         g_err = "scratch capacity still exceeded after retries";
         *nHits = (long long)c.out;

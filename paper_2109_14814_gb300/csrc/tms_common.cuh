@@ -161,6 +161,7 @@ struct Counters {
     unsigned long long psurv;      // patch pairs with an overlapping quarter pair
     unsigned long long raw_hits;
     unsigned long long out;
+    unsigned long long nodes[8];   // patch level: node pairs of each level of the tree
     unsigned int status;
     unsigned int dropped;          // raw hits merged into another record (short tail)
 };
@@ -451,8 +452,9 @@ struct FacePassArgs {
     uint32_t *ent_val;             // face id
     Counters *ctr;
     unsigned long long ent_cap;
-    int patch;                     // bounds pass: also the patch boxes, and the
-                                   // widest patch (not face) extent for the grid
+    int patch;                     // bounds pass: the patch boxes (no face boxes, and
+                                   // no world bounds: the tree needs none)
+    unsigned *nonfinite;           // patch level: set when a vertex is not finite
     int frames;                    // bounds pass, patch level, mixed precision:
                                    // also the patch frames (MeshDev::pframe)
 };
@@ -530,6 +532,42 @@ struct GroupArgs {
 void launch_group_count(const GroupArgs &a, int grid, cudaStream_t st);
 void launch_group_cells(const GroupArgs &a, int grid, cudaStream_t st);
 
+// Patch level: the tree of a mesh's patches.  Level 0 holds the patches, a node of
+// level l + 1 covers 4 x 4 nodes of level l; id = k * ni + i.
+struct TreeLevel {
+    void *box;                     // box per node, in the format of MeshDev::pbox
+    int ni, nk;
+    unsigned long long magic;      // recip64(ni)
+};
+constexpr int kTreeLevels = 8;
+constexpr int kTreeTop = kTreeLevels - 3;             // the highest top level
+constexpr unsigned long long kTreeTopPairs = 1ULL << 22;
+struct MeshTree {
+    TreeLevel lev[kTreeLevels];
+    uint32_t up_base[kTreeLevels / 2];                // first node of level 2, 4, .. over all meshes
+};
+struct TreeArgs {
+    const MeshTree *trees;         // per mesh
+    int n_meshes;
+    const int2 *pairs;
+    int n_pairs;
+    int top;                       // the level whose node pairs are all tested
+    const long long *top_base;     // per pair: its first 32 x 32 tile of them
+    long long top_tiles;
+    uint32_t up_blocks[kTreeLevels / 2];              // nodes of level 2, 4, .. of all meshes
+    Cand *list[2];                 // node pairs of odd and even levels
+    unsigned long long cap;
+    Cand *ppairs;                  // patch pairs with overlapping boxes, each once
+    unsigned long long ppair_cap;
+    Counters *ctr;                 // started here (nothing before it counts)
+    uint32_t *tail;                // the short merge's counts, likewise
+    unsigned *nonfinite;           // the bounds pass's finding, taken over and reset
+    Grid *grid0;                   // pair 0: whether its boxes' overlap is empty
+};
+void launch_tree(const TreeArgs &a, int precision, int sms, cudaStream_t st);
+int tree_launches(int top);
+void configure_tree();
+
 struct EmitArgs {
     const CellRec *cells;          // the cells holding faces of both meshes
     const uint32_t *vals;          // face ids grouped by cell
@@ -540,9 +578,7 @@ struct EmitArgs {
     unsigned long long ent_cap;
     Cand *cand;
     unsigned long long cand_cap;
-    unsigned long long *cand_ctr;  // the output's counter (candidates, or patch pairs)
     int moller;
-    int waves;                     // waves of resident blocks (0: the default, 4)
 };
 // whole waves of resident blocks on `sms` SMs
 void launch_emit(const EmitArgs &a, int precision, int face_level, int sms, cudaStream_t st);
@@ -560,7 +596,6 @@ struct PatchArgs {
     const MeshDev *meshes;         // the meshes (quad and patch boxes)
     const int2 *pairs;
     Counters *ctr;
-    unsigned long long ent_cap;
     Cand *cand;
     unsigned long long cand_cap;
     int moller;

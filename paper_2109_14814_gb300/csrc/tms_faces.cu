@@ -574,7 +574,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
     }
     __syncthreads();
 
-    BoundAcc<PREC> acc;
+    BoundAcc<PREC> acc;                // world bounds and widest face (face level)
     acc.init();
 
     const int t = threadIdx.x;
@@ -584,8 +584,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
         // quad faces with patches: as below, and each column's box over the
         // patch row (kPatchK quad rows; tiles are whole patch rows) united across
         // the kPatchI lanes of the patch (every lane of the block takes part:
-        // the row loop and its shuffles are uniform).  The widest extent the
-        // grid needs is then the widest patch's.
+        // the row loop and its shuffles are uniform)
         // this column's boxes over the upper and lower halves of the patch row
         BoxT<PREC> prev, ptop, pbot;
         box_empty(prev);
@@ -629,7 +628,6 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
                 if (patch_lane && (t % kPatchI) == 0) {
                     const BoxT<PREC> cb = closed<PREC>(pb);
                     write_box<PREC>(m.pbox, p, cb);
-                    acc.add(pb);
                     if constexpr (PREC == 1) {
                         PatchScratch &P = sp[(r / kPatchK) * (TI / kPatchI) + t / kPatchI];
                         P.lo = make_float4(cb.lo[0], cb.lo[1], cb.lo[2], cb.lo[3]);
@@ -709,6 +707,10 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
         }
     }
 
+    if (a.patch) {
+        if (__any_sync(FULL, top >= 0x7ff00000u) && (threadIdx.x & 31) == 0) atomicOr(a.nonfinite, 1u);
+        return;
+    }
     // block reduction, then one set of atomics per block, each of twelve lanes its own
     // (lo, hi, extent of every coordinate)
     __shared__ long long red[8][12];

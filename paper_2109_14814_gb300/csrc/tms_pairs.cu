@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(32 * kEmitWarps, (PREC == 1 && !MOLLER) ? 5 : 
     auto flush = [&]() {
         __syncwarp();
         unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(a.cand_ctr, (unsigned long long)staged);
+        if (lane == 0) base = atomicAdd(&a.ctr->cand, (unsigned long long)staged);
         base = __shfl_sync(FULL, base, 0);
         for (unsigned k = lane; k < staged; k += 32)
             if (base + k < cap) cand_out[base + k] = stage[k];
@@ -365,7 +365,7 @@ __global__ void __launch_bounds__(32 * kEmitWarps, (PREC == 1 && !MOLLER) ? 5 : 
         if (total > kStageCap) {
             // a dense tile: its candidates straight to one reserved range
             unsigned long long base = 0;
-            if (lane == 0) base = atomicAdd(a.cand_ctr, (unsigned long long)total);
+            if (lane == 0) base = atomicAdd(&a.ctr->cand, (unsigned long long)total);
             base = __shfl_sync(FULL, base, 0);
             unsigned long long pos = base + incl - cnt;
             for (uint32_t k = K; k; k &= k - 1, ++pos)
@@ -403,8 +403,7 @@ int emit_resident() {
 
 template <int PREC, bool MOLLER>
 void emit_waves(const EmitArgs &a, int face_level, int sms, cudaStream_t st) {
-    const int waves = a.waves > 0 ? a.waves : kEmitWaves;
-    k_emit<PREC, MOLLER><<<sms * emit_resident<PREC, MOLLER>() * waves, 32 * kEmitWarps, 0, st>>>(
+    k_emit<PREC, MOLLER><<<sms * emit_resident<PREC, MOLLER>() * kEmitWaves, 32 * kEmitWarps, 0, st>>>(
         a, face_level);
 }
 
@@ -560,8 +559,6 @@ __device__ __forceinline__ bool frames_separated(const PFrame &X, const PFrame &
 
 template <int PREC>
 __global__ void __launch_bounds__(kQuarterBlock) k_patch_quarters(PatchArgs a) {
-    // nothing to do after an overflow of the patch-level grid (the host retries)
-    if (a.ctr->entries > a.ent_cap || a.ctr->pair_slots > kMaxPairSlots) return;
     const unsigned long long n = clamp_count(&a.ctr->ppairs, a.ppair_cap);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
     uint32_t cached_pair = 0xFFFFFFFFu;
@@ -661,8 +658,6 @@ __global__ void __launch_bounds__(32 * kPatchWarps<PREC>, (PREC == 1 && !MOLLER)
     __shared__ PVert<PREC> sVert[kW][2][kPatchVerts];
     __shared__ EBox<PREC> sQuart[kW][8];   // the pair's quarter boxes, A's then B's
     __shared__ Cand sOut[kW][kPatchFlush + 32];
-    // nothing to do after an overflow of the patch-level grid (the host retries)
-    if (a.ctr->entries > a.ent_cap || a.ctr->pair_slots > kMaxPairSlots) return;
     const unsigned long long n = clamp_count(&a.ctr->psurv, a.ppair_cap);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t lt = lanemask_lt();
