@@ -130,7 +130,7 @@ struct Plan {
     uint2 *tstart = nullptr;
     void *sort_scratch = nullptr;
     unsigned long long *partials = nullptr;
-    Cand *cand = nullptr, *surv = nullptr;
+    Cand *cand = nullptr;
     uint32_t *qsurv = nullptr;        // candidates left by the quad-level test
     float4 *vlo = nullptr;            // vertices of all meshes rounded down to FP32
     unsigned char *fbox = nullptr;    // face boxes of all meshes (face level)
@@ -159,7 +159,7 @@ struct Plan {
 
     void free_scratch() {
         void *ptrs[] = {bmA, bmH, ek, ev, eslot, erank, grouped, tkey, crec, tcnt, tstart,
-                        sort_scratch, cand, surv, hits, hk, hk2, okeys, hv, hv2,
+                        sort_scratch, cand, hits, hk, hk2, okeys, hv, hv2,
                         keep, kscan, ppairs, psurv, qsurv, nodes[0], nodes[1]};
         for (void *p : ptrs)
             if (p) cudaFree(p);
@@ -167,7 +167,7 @@ struct Plan {
         qsurv = nullptr;
         bmA = bmH = nullptr; ek = nullptr; ev = eslot = erank = grouped = nullptr;
         tkey = nullptr; crec = nullptr; tcnt = nullptr; tstart = nullptr;
-        sort_scratch = nullptr; cand = surv = nullptr; hits = nullptr; hk = hk2 = okeys = nullptr;
+        sort_scratch = nullptr; cand = nullptr; hits = nullptr; hk = hk2 = okeys = nullptr;
         hv = hv2 = keep = kscan = nullptr;
         if (exec) { cudaGraphExecDestroy(exec); exec = nullptr; }
     }
@@ -219,8 +219,7 @@ struct Plan {
         TMS_CK(dalloc(reinterpret_cast<unsigned char **>(&sort_scratch),
                       radix_scratch_size(hit_cap, 2 * tri_bits + pair_bits)));
         TMS_CK(dalloc(&cand, cand_cap));
-        TMS_CK(dalloc(&qsurv, cand_cap));
-        TMS_CK(dalloc(&surv, surv_cap));
+        TMS_CK(dalloc(&qsurv, surv_cap));
         TMS_CK(dalloc(&hits, hit_cap));
         TMS_CK(dalloc(&hk, hit_cap));
         TMS_CK(dalloc(&hk2, hit_cap));
@@ -401,14 +400,14 @@ struct Plan {
         mark(11, s);
 
         NarrowArgs na;
-        na.cand = cand; na.cand_cap = cand_cap; na.surv = surv; na.surv_cap = surv_cap;
-        na.qsurv = qsurv;
+        na.cand = cand; na.cand_cap = cand_cap;
+        na.qsurv = qsurv; na.qsurv_cap = surv_cap;
         na.meshes = d_meshes; na.pairs = d_pairs;
         na.ctr = d_ctr; na.hits = hits; na.hit_key = hk; na.hit_val = hv; na.hit_cap = hit_cap;
         na.tau = p.tau; na.tri_bits = tri_bits; na.fp32_filter = p.narrow_filter;
         na.tail = long_tail ? nullptr : tail; na.hit_slot = kscan; na.bscale = bscale;
         launch_narrow(na, fl, grid / 2, s);
-        kernels += p.narrow_filter ? 3 : 2;
+        kernels += p.narrow_filter ? 2 : 1;
         mark(12, s);
         if (long_tail) enqueue_long_tail(s);
         else enqueue_short_tail(s);
@@ -821,7 +820,6 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
         configure_emit();
         configure_patch_quads();
         configure_tree();
-        configure_narrow();
         g_configured_mask |= 1 << device;
     }
     Plan *P = find_plan(A, B, nPairs, prm, cm_pair, user, dHits, hitCap, dOffsets, device);
@@ -879,8 +877,8 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
             P->cand_cap = c.cand + c.cand / 4 + 1024;
             grow = true;
         }
-        if (!grow && c.fp64 > P->surv_cap) {
-            P->surv_cap = c.fp64 + c.fp64 / 4 + 1024;
+        if (!grow && c.qkeep > P->surv_cap) {
+            P->surv_cap = c.qkeep + c.qkeep / 4 + 1024;
             grow = true;
         }
         if (!grow && c.raw_hits > P->hit_cap) {
@@ -928,7 +926,7 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     if (prm.timing) g_stage_ms[user] = std::vector<float>(P->stage_ms, P->stage_ms + Plan::kStages);
     unsigned long long lists = c.entries;
     for (unsigned long long v : c.nodes) lists = std::max(lists, v);
-    if (lists > P->ent_cap || c.cand > P->cand_cap || c.fp64 > P->surv_cap ||
+    if (lists > P->ent_cap || c.cand > P->cand_cap || c.qkeep > P->surv_cap ||
         c.raw_hits > P->hit_cap || (P->patch && c.ppairs > P->ppair_cap)) {
         g_err = "scratch capacity still exceeded after retries";
         *nHits = (long long)c.out;
@@ -1067,6 +1065,7 @@ tms_status tms_build_mesh(const double *dX, const double *dY, const double *dPx,
     m->dev.nqk = k1 - k0 - 1;
     m->dev.pad = 0;
     m->dev.nmagic = recip64((unsigned long long)N);
+    m->dev.dtheta = 6.283185307179586476925286766559 / N;
     *out = m;
     return TMS_OK;
 }

@@ -79,6 +79,7 @@ struct MeshDev {
                                 // is __umul64hi(id, pmagic) (exact for 32-bit ids)
     unsigned long long nmagic;  // ceil(2^64 / N): a quad id's row is
                                 // __umul64hi(q, nmagic) (N >= 2, exact for 32-bit ids)
+    double dtheta;              // 2 pi / N
     float4 *pframe;       // plan scratch (patch level, mixed precision, FP32
                           // filters on): per patch its frame, kFrameF4 float4
                           // at slot * kFrameF4 (layout at kFrameF4); else NULL
@@ -374,10 +375,13 @@ __device__ __forceinline__ float f32_rd(double x) {
 __device__ __forceinline__ float f32_above(float f) {
     return f + fmaf(fabsf(f), 1.1920932e-7f, 1.17549435e-38f);
 }
+static __device__ __noinline__ float f32_rn_special(double x) {
+    return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, 0);
+}
 __device__ __forceinline__ float f32_rn(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);
     const int e32 = (int)((b >> 52) & 0x7ff) - 896;
-    if (e32 <= 0 || e32 >= 255) return f32_special(b, e32, 0);
+    if (e32 <= 0 || e32 >= 255) return f32_rn_special(x);
     unsigned f = f32_bits_trunc(b, e32) & 0x7fffffffu;
     const unsigned rem = (unsigned)(b & 0x1FFFFFFFULL);
     f += (unsigned)(rem > 0x10000000u) | ((unsigned)(rem == 0x10000000u) & (f & 1u));
@@ -610,9 +614,8 @@ void configure_patch_quads();
 struct NarrowArgs {
     const Cand *cand;
     unsigned long long cand_cap;
-    uint32_t *qsurv;               // [cand_cap] candidates the quad-level test left
-    Cand *surv;                    // triangle pairs left for the FP64 solve
-    unsigned long long surv_cap;
+    uint32_t *qsurv;               // candidates the quad-level test left
+    unsigned long long qsurv_cap;
     const MeshDev *meshes;
     const int2 *pairs;
     Counters *ctr;
@@ -627,32 +630,9 @@ struct NarrowArgs {
     uint32_t *hit_slot;            // [hit_cap] the hit's place in its bucket
     float bscale;                  // tail_bucket's scale
 };
-// the quad-level test over all candidates (quad faces), then the filter on what it
-// left as one wave of resident blocks on `sms` SMs, then the FP64 solve
+// the quad-level test over all candidates, then the triangle pairs of those left and
+// the FP64 solves; with the filters off, the FP64 solves alone
 void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st);
-void configure_narrow();
-
-// FP32 split of a double: hi = RN32(x), lo = RN32(x - hi), integer operations
-// only in the normal range
-__device__ __forceinline__ void split_f32(double x, float &hi, float &lo) {
-    hi = f32_rn(x);
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int e = (int)((b >> 52) & 0x7ff);
-    const int e32 = e - 896;
-    // x = sign * (2^52 + m) * 2^(e - 1075); the low 29 bits of m were rounded away
-    const unsigned long long m = b & 0xFFFFFFFFFFFFFULL;
-    const int rem = (int)(m & 0x1FFFFFFFULL);
-    const unsigned hb = __float_as_uint(hi) & 0x7fffffffu;
-    const unsigned trunc = ((unsigned)e32 << 23) | (unsigned)(m >> 29);
-    // rounded up (|hi| > |x|): x - hi = -(2^29 - rem) ulp, else +rem ulp (ulp = 2^(e-1075))
-    const int r = (hb != trunc) ? rem - (1 << 29) : rem;
-    const int ex = e - 1075 + 127;   // 2^(e - 1075) as an FP32 power of two
-    float l = 0.0f;
-    if (e32 > 0 && e32 < 255 && ex >= 1) l = __int2float_rn(r) * __uint_as_float((unsigned)ex << 23);
-    // outside that range lo is 0 and the caller's error bound carries an absolute
-    // term for coordinates below 2^-74
-    lo = (b >> 63) ? -l : l;
-}
 
 struct DedupArgs {
     const uint64_t *keys;          // sorted hit keys

@@ -5,15 +5,15 @@
 //   [x1-x2 | x3-x2 | y2-y1 | y2-y3] (a, b, c, d)^T = y2 - x2,
 // and the triangles meet iff a, b, c, d >= 0, a + b <= 1, c + d <= 1; the common
 // point is x2 + a(x1-x2) + b(x3-x2).  The paper ran this on the CPU; here it is
-// one thread per triangle pair in FP64 (Gaussian elimination with partial
+// four lanes per triangle pair in FP64 (Gaussian elimination with partial
 // pivoting).  Readings of the paper fixed by this library: the inequalities are
 // closed with tolerance tau (margin = min(a, b, c, d, 1-a-b, 1-c-d) >= -tau),
 // and a singular system (a zero pivot) is not a hit.  The (theta, s) estimates
 // are the interpolation formulas that follow Eq. (precise).
 //
 // Mixed precision (optional): a verified FP32 solve first.  The system is formed
-// in FP32 from a split copy of the vertices (hi + lo per coordinate), with a
-// bound on every entry's error.  Gaussian elimination on [A | I | r] gives z~
+// in FP32 from the rounded entries of the FP64 system, with a bound on every
+// entry's error.  Gaussian elimination on [A | I | r] gives z~
 // and an approximate inverse C; with alpha >= |I - C A|_inf (computed with its
 // rounding and input-error terms), A is nonsingular when alpha < 1 and
 //   |z - z~|_inf <= | |C| |r - A z~| |_inf / (1 - alpha),
@@ -37,13 +37,6 @@ constexpr double kTwoPi = 6.283185307179586476925286766559;
 // ---------------------------------------------------------------------------
 // FP64 Gaussian elimination with partial pivoting, fully unrolled in registers
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ __forceinline__ void swap_(T &a, T &b) {
-    T t = a;
-    a = b;
-    b = t;
-}
-
 template <typename T>
 __device__ __forceinline__ bool solve4_gepp(T A[4][4], T r[4], T z[4], T &det) {
     T sign = 1;
@@ -100,34 +93,6 @@ __device__ __forceinline__ void gather_tri(const MeshDev &m, uint32_t t, double 
     for (int j = 0; j < 3; ++j) load_vertex(m, ii[j], kk[j], v[j]);
 }
 
-// One entry of the FP32 system: the difference p - q of two split coordinates and
-// a bound on its error against the exact difference of the FP64 coordinates.
-__device__ __forceinline__ float split_diff(float hp, float lp, float hq, float lq, float &err) {
-    const float u = 5.9604645e-08f;
-    const float t1 = hp - hq, t2 = lp - lq;
-    const float d = t1 + t2;
-    // relative rounding of the three FP32 operations, the split remainders, and an
-    // absolute term for coordinates below 2^-74 (whose lo part is not kept)
-    err = (u * (fabsf(t1) + fabsf(t2) + fabsf(d))) * 1.0001f + (u * u) * (fabsf(hp) + fabsf(hq)) * 1.01f +
-          1e-29f;
-    return d;
-}
-
-// a triangle's vertices as FP32 splits, made from the FP64 coordinates: the tests that
-// need the low parts see a few per cent of the quads, so keeping them for every vertex
-// (16 bytes each, written by the bounds pass) cost more than splitting here
-__device__ __forceinline__ void gather_split(const MeshDev &m, uint32_t t, float4 v[3][2]) {
-    double x[3][4];
-    gather_tri(m, t, x);
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-        split_f32(x[j][0], v[j][0].x, v[j][1].x);
-        split_f32(x[j][1], v[j][0].y, v[j][1].y);
-        split_f32(x[j][2], v[j][0].z, v[j][1].z);
-        split_f32(x[j][3], v[j][0].w, v[j][1].w);
-    }
-}
-
 __device__ __forceinline__ float comp(const float4 &v, int c) {
     return c == 0 ? v.x : (c == 1 ? v.y : (c == 2 ? v.z : v.w));
 }
@@ -165,57 +130,14 @@ __device__ __forceinline__ void gather_face_lo(const MeshDev &m, uint32_t face, 
     }
 }
 
-// Overlap of the two triangles' boxes, as the separating-axis test along each
-// coordinate axis: each coordinate's interval from the split copies (widened by
-// the split remainder and a relative 1e-6, more than the FP32 rounding of the
-// test), and the pair dropped only when a gap exceeds 3 tau' (D_X + D_Y) plus the
-// FP64 solve's reach (the triangles widened to weights >= -tau', widen3 and
-// fp64_reach, with max|A| at most the largest extent and |r| at most twice the
-// largest coordinate) -- so that no FP64 hit is dropped whatever tau.
-__device__ __forceinline__ bool split_boxes_overlap(const float4 X[3][2], const float4 Y[3][2], float tau) {
-    float xl[4], xh[4], yl[4], yh[4];
-    float dmax = 0.0f, cmax = 0.0f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        xl[c] = 3.4e38f; xh[c] = -3.4e38f; yl[c] = 3.4e38f; yh[c] = -3.4e38f;
-#pragma unroll
-        for (int j = 0; j < 3; ++j) {
-            const float hx = comp(X[j][0], c), lx = comp(X[j][1], c);
-            const float dx = fabsf(lx) + 1e-6f * fabsf(hx) + 1e-29f;
-            xl[c] = fminf(xl[c], hx - dx);
-            xh[c] = fmaxf(xh[c], hx + dx);
-            const float hy = comp(Y[j][0], c), ly = comp(Y[j][1], c);
-            const float dy = fabsf(ly) + 1e-6f * fabsf(hy) + 1e-29f;
-            yl[c] = fminf(yl[c], hy - dy);
-            yh[c] = fmaxf(yh[c], hy + dy);
-        }
-        dmax = fmaxf(dmax, fmaxf(xh[c] - xl[c], yh[c] - yl[c]));
-        cmax = fmaxf(cmax, fmaxf(fmaxf(fabsf(xl[c]), fabsf(xh[c])), fmaxf(fabsf(yl[c]), fabsf(yh[c]))));
-    }
-    const float tp = widen3(tau);
-    const float reach = fp64_reach(dmax * 1.001f, 2.0f * cmax * 1.001f, tau);
-    bool ov = true;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const float need = (tp * ((xh[c] - xl[c]) + (yh[c] - yl[c])) + reach) * 1.001f;
-        ov &= !(yl[c] - xh[c] > need || xl[c] - yh[c] > need);
-    }
-    return ov;
-}
+// The FP32 system of a triangle pair: A and r as the FP64 solve forms them, rounded
+// to nearest, so every entry is within kEntry |entry| + kTiny of the FP64 one (2^-126
+// below the FP32 normal range; the FP64 entry's own rounding is inside the margin).
+constexpr float kEntry = 1.001f * 5.9604645e-08f, kTiny = 1.2e-38f;
 
 // true when the verified FP32 solve proves margin < -2 tau (not a hit)
-__device__ __noinline__ bool fp32_verified_reject(const float4 X[3][2], const float4 Y[3][2],
-                                                  float tau) {
+__device__ __forceinline__ bool fp32_verified_reject(const float (&A)[4][4], const float (&r)[4], float tau) {
     const float u = 5.9604645e-08f;
-    float A[4][4], EA[4][4], r[4], Er[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        A[c][0] = split_diff(comp(X[0][0], c), comp(X[0][1], c), comp(X[1][0], c), comp(X[1][1], c), EA[c][0]);
-        A[c][1] = split_diff(comp(X[2][0], c), comp(X[2][1], c), comp(X[1][0], c), comp(X[1][1], c), EA[c][1]);
-        A[c][2] = split_diff(comp(Y[1][0], c), comp(Y[1][1], c), comp(Y[0][0], c), comp(Y[0][1], c), EA[c][2]);
-        A[c][3] = split_diff(comp(Y[1][0], c), comp(Y[1][1], c), comp(Y[2][0], c), comp(Y[2][1], c), EA[c][3]);
-        r[c] = split_diff(comp(Y[1][0], c), comp(Y[1][1], c), comp(X[1][0], c), comp(X[1][1], c), Er[c]);
-    }
     // Gaussian elimination with partial pivoting on [A | I | r]
     float M[4][9];
 #pragma unroll
@@ -272,13 +194,13 @@ __device__ __noinline__ bool fp32_verified_reject(const float4 X[3][2], const fl
         }
     }
     // alpha >= |I - C A_exact|_inf: computed I - C A, its rounding (6u (1 + |C||A|))
-    // and the input error |C| EA, the last two as one product |C| W with
-    // W = 6u |A| + EA
+    // and the input error |C| E, the last two as one product |C| W with
+    // W = (6u + kEntry) |A| + kTiny
     float W[4][4];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) W[k][j] = fmaf(6.0f * u, fabsf(A[k][j]), EA[k][j]);
+        for (int j = 0; j < 4; ++j) W[k][j] = fmaf(6.0f * u + kEntry, fabsf(A[k][j]), kTiny);
     float alpha = 0.0f, cnorm = 0.0f, anorm = 0.0f;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -302,17 +224,17 @@ __device__ __noinline__ bool fp32_verified_reject(const float4 X[3][2], const fl
     alpha *= 1.0001f;
     if (!(alpha < 0.5f)) return false;
     // |r_exact - A_exact z~| componentwise
+    const float zsum = (fabsf(z[0]) + fabsf(z[1])) + (fabsf(z[2]) + fabsf(z[3]));
     float res[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        float acc = r[i], mag = fabsf(r[i]), pert = Er[i];
+        float acc = r[i], mag = fabsf(r[i]);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             acc = fmaf(-A[i][j], z[j], acc);
             mag = fmaf(fabsf(A[i][j]), fabsf(z[j]), mag);
-            pert = fmaf(EA[i][j], fabsf(z[j]), pert);
         }
-        res[i] = (fabsf(acc) + 6.0f * u * mag + pert) * 1.0001f;
+        res[i] = (fabsf(acc) + (6.0f * u + kEntry) * mag + kTiny * (1.0f + zsum)) * 1.0001f;
     }
     float err = 0.0f, zmax = 0.0f;
 #pragma unroll
@@ -351,8 +273,8 @@ __device__ __noinline__ bool fp32_verified_reject(const float4 X[3][2], const fl
 // coordinates m_ij = e1_i e2_j - e1_j e2_i); any direction is valid, these
 // make the triangle's own interval almost a point.  det A is the pairing of
 // the two planes' Plucker coordinates.  Every FP32 value carries a bound on its
-// rounding and on the error of the split inputs, so the test is rigorous for
-// the FP64 vertices.
+// rounding and on the error of its input, so the test is rigorous for the FP64
+// vertices.
 // ---------------------------------------------------------------------------
 struct SplitVec {
     float v[4];
@@ -360,24 +282,16 @@ struct SplitVec {
     float M;       // max_c |v_c|
 };
 
-// p - q of split vertices: t1 = hp - hq, t2 = lp - lq, v = t1 + t2 with
-// |v - exact| <= 2u(1+u)|t1| + 3u^2 (|hp| + |hq|) (the split remainders and the
-// three roundings; |t2| <= u (1+u)^2 (|hp| + |hq|)), evaluated with margin
-__device__ __forceinline__ SplitVec split_vec(const float4 P[2], const float4 Q[2]) {
-    const float u = 5.9604645e-08f;
+// column j of the FP32 system, or its negative
+__device__ __forceinline__ SplitVec column_vec(const float (&A)[4][4], int j, float sign) {
     SplitVec r;
-    float t1m = 0.0f, hm = 0.0f, vm = 0.0f;
+    r.M = 0.0f;
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-        const float hp = comp(P[0], c), lp = comp(P[1], c), hq = comp(Q[0], c), lq = comp(Q[1], c);
-        const float t1 = hp - hq, t2 = lp - lq;
-        r.v[c] = t1 + t2;
-        t1m = fmaxf(t1m, fabsf(t1));
-        hm = fmaxf(hm, fabsf(hp) + fabsf(hq));
-        vm = fmaxf(vm, fabsf(r.v[c]));
+        r.v[c] = sign * A[c][j];
+        r.M = fmaxf(r.M, fabsf(A[c][j]));
     }
-    r.E = (2.001f * u) * t1m + (3.01f * u * u) * hm + 2e-29f;
-    r.M = vm;
+    r.E = kEntry * r.M + kTiny;
     return r;
 }
 
@@ -385,8 +299,9 @@ __device__ __forceinline__ SplitVec split_vec(const float4 P[2], const float4 Q[
 // |p - fp| <= 2u |fp| + 2^-126 (one FP32 place; 2^-126 below the normal range), so
 // t = fl(fp - fq) has |t - (p - q)| <= u |t| / (1 - u) + 2u (|fp| + |fq|) + 2^-125,
 // bounded with margin; a coordinate of 2^128 or more is rounded down to FLT_MAX or
-// -inf, which says nothing about it.  Looser than split_vec by about |fp| / |p - q|,
-// which the quad-level test absorbs except for near-misses far below a face's size.
+// -inf, which says nothing about it.  Looser than the
+// FP64 difference rounded to FP32 by about |fp| / |p - q|, which the quad-level test
+// absorbs except for near-misses far below a face's size.
 __device__ __forceinline__ SplitVec lo_vec(const float4 &P, const float4 &Q) {
     const float u = 5.9604645e-08f;
     SplitVec r;
@@ -561,7 +476,7 @@ __device__ __forceinline__ bool quad_sat_vectors(const SplitVec &a1, const Split
 // each when their planes share a direction) -- then, with DUALS, the dual axes
 // of quad_sat_vectors.  Any direction serves (the bounds hold for the FP32 w as
 // computed), so w is not normalised.  A candidate it cannot clear goes on to
-// the tests on the split copies.
+// the tests of its triangle pairs.
 template <int MLO, int MHI, bool DUALS>
 __device__ __forceinline__ bool quad_reject_lo(const float4 QA[4], const float4 QB[4], float tau) {
     const SplitVec a1 = lo_vec(QA[1], QA[0]), a2 = lo_vec(QA[2], QA[0]);
@@ -601,14 +516,18 @@ constexpr int kQuadFirstAxes = 2;
 
 // true when the separating-axis test proves that the FP64 solve of the pair
 // reports no hit (fp64_reach)
-__device__ __noinline__ bool fp32_sat_reject(const float4 X[3][2], const float4 Y[3][2],
-                                                float tau) {
-    // vectors relative to x2
-    const SplitVec e1 = split_vec(X[0], X[1]);    // x1 - x2
-    const SplitVec e2 = split_vec(X[2], X[1]);    // x3 - x2
-    const SplitVec f1 = split_vec(Y[0], Y[1]);    // y1 - y2
-    const SplitVec f2 = split_vec(Y[2], Y[1]);    // y3 - y2
-    const SplitVec r = split_vec(Y[1], X[1]);     // y2 - x2
+__device__ __forceinline__ bool fp32_sat_reject(const float (&A)[4][4], const float (&rhs)[4], float tau) {
+    // vectors relative to x2: x1 - x2, x3 - x2, y1 - y2, y3 - y2, y2 - x2
+    const SplitVec e1 = column_vec(A, 0, 1.0f), e2 = column_vec(A, 1, 1.0f);
+    const SplitVec f1 = column_vec(A, 2, -1.0f), f2 = column_vec(A, 3, -1.0f);
+    SplitVec r;
+    r.M = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        r.v[c] = rhs[c];
+        r.M = fmaxf(r.M, fabsf(rhs[c]));
+    }
+    r.E = kEntry * r.M + kTiny;
     const SplitVec s1 = add_vec(r, f1), s3 = add_vec(r, f2);
     float mE[6], mF[6], epsE, epsF;
     plucker(e1, e2, mE, epsE);
@@ -633,206 +552,183 @@ __device__ __noinline__ bool fp32_sat_reject(const float4 X[3][2], const float4 
     return false;
 }
 
-// (theta, s) estimate for weights (u, v) in triangle t (formulas after Eq. (precise))
-__device__ __forceinline__ void tri_params(const MeshDev &m, uint32_t t, double u, double v,
-                                           double &th, double &sv) {
-    uint32_t q = t >> 1;
-    int tau = t & 1;
-    const int k = (int)__umul64hi((unsigned long long)q, m.nmagic), i = (int)(q - (uint32_t)k * (uint32_t)m.N);
-    double dth = kTwoPi / m.N;
-    double th_i = i * dth, th_ip = th_i + dth;
-    double s_k = m.s[k], s_kp = m.s[k + 1];
-    if (tau == 0) {
-        th = (1.0 - u) * th_i + u * th_ip;
-        sv = (1.0 - v) * s_k + v * s_kp;
-    } else {
-        th = u * th_i + (1.0 - u) * th_ip;
-        sv = v * s_k + (1.0 - v) * s_kp;
-    }
-    // fmod(th, 2 pi): the weights of a hit lie in [-1, 2] (tau < 1) and dth <= pi, so
-    // -2 pi < th < 4 pi, where one subtraction is exact
-    if (th >= kTwoPi) th -= kTwoPi;
-    if (th < 0) th += kTwoPi;
+// ---------------------------------------------------------------------------
+// FP64 solve (Eq. (precise)) by four lanes a triangle pair
+// ---------------------------------------------------------------------------
+// A warp's FP64 instruction holds its scheduler's part of the pipe for 64 clocks
+// (measured, whatever its active lanes), so the solve's time is its count of FP64
+// instructions: one lane a pair took 245 of them in a row (7.6 us), four lanes, lane c
+// with row c of the system, take about 105.  Row operations, pivot choices (as
+// integers) and results are those of one lane's elimination with partial pivoting.
+__device__ __forceinline__ double quad_lane(double v, int base, int j) { return __shfl_sync(FULL, v, base + j); }
+
+// the ordered bits of |v| (NaN above everything)
+__device__ __forceinline__ unsigned long long abs64(double v) {
+    return (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffULL;
 }
-
-// FP64 narrow-phase test of one triangle pair (Eq. (precise)); fills h on a hit
-__device__ __forceinline__ bool narrow_fp64(const MeshDev &ma, const MeshDev &mb, uint32_t ta,
-                                            uint32_t tb, double tau, tms_hit &h) {
-    double x[3][4], y[3][4];
-    gather_tri(ma, ta, x);
-    gather_tri(mb, tb, y);
-    double A[4][4], r[4], col0[4], col1[4];
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        A[c][0] = x[0][c] - x[1][c];
-        A[c][1] = x[2][c] - x[1][c];
-        A[c][2] = y[1][c] - y[0][c];
-        A[c][3] = y[1][c] - y[2][c];
-        r[c] = y[1][c] - x[1][c];
-        col0[c] = A[c][0];
-        col1[c] = A[c][1];
+// Triangles ta of ma and tb of mb (every lane of the warp calls it; dead quads solve
+// whatever they are given): true on a quad's four lanes when the pair is a hit, whose
+// record they then write to *out with pair index `pair`; `slot` gives the place.
+template <typename Slot>
+__device__ __forceinline__ void solve_pair(const MeshDev &ma, const MeshDev &mb, uint32_t ta, uint32_t tb,
+                                           uint32_t pair, double tau, bool live, tms_hit *hits, const Slot &slot) {
+    const int lane = threadIdx.x & 31, c = lane & 3, base = lane & ~3;
+    double x1, A[4], r;
+    {
+        int ii[3], kk[3];
+        const double *pa = ma.c[c], *pb = mb.c[c];
+        tri_ij(ma, ta, ii, kk);
+        const double x0 = __ldg(pa + (size_t)kk[0] * ma.N + ii[0]), x2 = __ldg(pa + (size_t)kk[2] * ma.N + ii[2]);
+        x1 = __ldg(pa + (size_t)kk[1] * ma.N + ii[1]);
+        tri_ij(mb, tb, ii, kk);
+        const double y0 = __ldg(pb + (size_t)kk[0] * mb.N + ii[0]), y1 = __ldg(pb + (size_t)kk[1] * mb.N + ii[1]);
+        const double y2 = __ldg(pb + (size_t)kk[2] * mb.N + ii[2]);
+        A[0] = x0 - x1;
+        A[1] = x2 - x1;
+        A[2] = y1 - y0;
+        A[3] = y1 - y2;
+        r = y1 - x1;
     }
-    double n2[4];
+    const double col0 = A[0], col1 = A[1], col2 = A[2], col3 = A[3];
+    // the row's place in the permuted system, and which lane holds each place
+    int place = c, holder[4];
+    bool ok = true, negative = false;
+    double inv[4], diag[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) n2[j] = A[0][j] * A[0][j] + A[1][j] * A[1][j] + A[2][j] * A[2][j] + A[3][j] * A[3][j];
-    double z[4], det;
-    const bool ok = solve4_gepp<double>(A, r, z, det);
-    if (!ok) return false;
-    const double a = z[0], b = z[1], c = z[2], d = z[3];
-    const double m = fmin(fmin(fmin(a, b), fmin(c, d)), fmin(1.0 - a - b, 1.0 - c - d));
-    const bool finite = isfinite(a) && isfinite(b) && isfinite(c) && isfinite(d);
-    if (!(finite && m >= -tau)) return false;
-    const double rho = fabs(det) / (sqrt(n2[0]) * sqrt(n2[1]) * sqrt(n2[2]) * sqrt(n2[3]));
-    if (!(rho > 0.0)) return false;
-    h.triA = ta;
-    h.triB = tb;
-    h.a = a; h.b = b; h.c = c; h.d = d;
+    for (int col = 0; col < 4; ++col) {
+        // the largest |A[.][col]| of the rows not used yet, the first in place among equals
+        unsigned long long best = place >= col ? abs64(A[col]) : 0ULL;
+        int bp = place >= col ? place : 4, bl = c;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) h.P[k] = x[1][k] + a * col0[k] + b * col1[k];
-    tri_params(ma, ta, a, b, h.theta_u, h.s_u);
-    tri_params(mb, tb, c, d, h.theta_s, h.s_s);
-    h.rho = rho;
-    h.margin = m;
-    h.flags = (rho < 1e-12 || fabs(m) < 1e-12) ? 1u : 0u;
-    return true;
-}
-
-// Stage 1b: the triangle pairs the quad-level test (k_quad_filter) leaves, one
-// per lane: the (widened) triangle boxes (of a quad candidate's four pairs), the
-// triangle-level separating-axis test, and for the pairs
-// left a per-warp queue feeding the verified solve 32 pairs at a time, so that
-// the solve does not run with most lanes idle; pairs the tests cannot reject go
-// to the survivor list.  With the FP32 filters off, every triangle pair of
-// every candidate goes to the survivor list.
-template <int FACE>
-__global__ void __launch_bounds__(256, 2) k_narrow_filter(NarrowArgs a) {
-    constexpr int kW = 8, kQ = 32 + 4 * 32;
-    __shared__ uint32_t q_cand[kW][kQ];          // triangle pairs for the verified solve
-    __shared__ uint8_t q_sub[kW][kQ];
-    if (a.ctr->cand > a.cand_cap) return;
-    const unsigned long long n = a.ctr->cand;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t lt = lanemask_lt();
-    // tau rounded up once per thread: the FP32 tests only widen by it
-    const float tauf = __double2float_ru(a.tau);
-    unsigned long long n_sat = 0, n_full = 0;               // tests run, per warp
-    unsigned qn = 0;                                        // queued pairs (warp-uniform)
-
-    // the verified solve of pair-queue items [base, base + cnt)
-    auto drain = [&](unsigned base, unsigned cnt) {
-        bool keep = false;
-        uint32_t ta = 0, tb = 0, pair = 0;
-        if ((unsigned)lane < cnt) {
-            const uint32_t g = q_cand[warp][base + lane];
-            const unsigned sub = q_sub[warp][base + lane];
-            const Cand c2 = a.cand[g];
-            ta = FACE == 0 ? c2.faceA : 2 * c2.faceA + (sub & 1u);
-            tb = FACE == 0 ? c2.faceB : 2 * c2.faceB + (sub >> 1);
-            pair = c2.pair;
-            const int2 pr = a.pairs[pair];
-            float4 X[3][2], Y[3][2];
-            gather_split(a.meshes[pr.x], ta, X);
-            gather_split(a.meshes[pr.y], tb, Y);
-            keep = !fp32_verified_reject(X, Y, tauf);
+        for (int off = 1; off <= 2; off <<= 1) {
+            const unsigned long long ob = __shfl_xor_sync(FULL, best, off);
+            const int op = __shfl_xor_sync(FULL, bp, off), ol = __shfl_xor_sync(FULL, bl, off);
+            if (ob > best || (ob == best && op < bp)) { best = ob; bp = op; bl = ol; }
         }
-        n_full += cnt;
-        const unsigned long long pos = warp_append(&a.ctr->fp64, keep, FULL);
-        if (keep && pos < a.surv_cap) {
-            Cand sv;
-            sv.faceA = ta;
-            sv.faceB = tb;
-            sv.pair = pair;
-            sv.pad = 0;
-            a.surv[pos] = sv;
-        }
-    };
-    // one triangle pair through the box and separating-axis tests; the pairs
-    // they cannot reject join the pair queue (all lanes call it together)
-    auto pair_tests = [&](bool valid, uint32_t g, int sub, const float4 X[3][2], const float4 Y[3][2],
-                          bool boxes) {
-        const bool tested = valid && (!boxes || split_boxes_overlap(X, Y, tauf));
-        const bool need = tested && !fp32_sat_reject(X, Y, tauf);
-        n_sat += __popc(__ballot_sync(FULL, tested));
-        const uint32_t want = __ballot_sync(FULL, need);
-        if (need) {
-            const unsigned slot = qn + __popc(want & lt);
-            q_cand[warp][slot] = g;
-            q_sub[warp][slot] = (uint8_t)sub;
-        }
-        qn += __popc(want);
-    };
-    auto drain_full = [&]() {
-        __syncwarp();
-        while (qn >= 32) {
-            qn -= 32;
-            drain(qn, 32);
-            __syncwarp();
-        }
-    };
-    if (!a.fp32_filter) {
-        // every triangle pair of the candidate to the FP64 solve
-        for (unsigned long long g0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane; g0 < n;
-             g0 += stride) {
-            const unsigned long long g = g0 + lane;
-            const bool valid = g < n;
-            Cand cd;
-            cd.faceA = cd.faceB = cd.pair = 0;
-            if (valid) cd = a.cand[g];
-            const int nsub = FACE == 0 ? 1 : 4;
-            for (int sub = 0; sub < nsub; ++sub) {
-                const uint32_t ta = FACE == 0 ? cd.faceA : 2 * cd.faceA + (sub & 1);
-                const uint32_t tb = FACE == 0 ? cd.faceB : 2 * cd.faceB + (sub >> 1);
-                const unsigned long long pos = warp_append(&a.ctr->fp64, valid, FULL);
-                if (valid && pos < a.surv_cap) {
-                    Cand sv;
-                    sv.faceA = ta;
-                    sv.faceB = tb;
-                    sv.pair = cd.pair;
-                    sv.pad = 0;
-                    a.surv[pos] = sv;
-                }
+        ok &= best != 0ULL;
+        // swap places with the row at place col
+        negative ^= bp != col;
+        place = c == bl ? col : place == col ? bp : place;
+        holder[col] = base + bl;
+        double p[4];
+#pragma unroll
+        for (int j = col; j < 4; ++j) p[j] = __shfl_sync(FULL, A[j], holder[col]);
+        const double pr = __shfl_sync(FULL, r, holder[col]);
+        diag[col] = p[col];
+        inv[col] = 1.0 / p[col];
+        if (col < 3) {
+            const double f = A[col] * inv[col];
+            const bool below = place > col;
+#pragma unroll
+            for (int j = col + 1; j < 4; ++j) {
+                const double v = A[j] - f * p[j];
+                A[j] = below ? v : A[j];
             }
+            const double v = r - f * pr;
+            r = below ? v : r;
         }
-        return;
     }
-    // the candidates the quad-level test (k_quad_filter) could not clear: each of
-    // their triangle pairs on a lane of its own (a quad candidate's four take the
-    // triangle boxes first; the triangle-level separating axes), the pairs left
-    // queued for the verified solve, 32 at a time
-    const unsigned long long ni = (FACE == 0 ? 1 : 4) * clamp_count(&a.ctr->qkeep, a.cand_cap);
-    for (unsigned long long i0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane; i0 < ni;
-         i0 += stride) {
-        const unsigned long long it = i0 + lane;
-        const bool valid = it < ni;
-        uint32_t g = 0;
-        const int sub = FACE == 0 ? 0 : (int)(it & 3);
-        float4 X[3][2], Y[3][2];
-        if (valid) {
-            g = a.qsurv[FACE == 0 ? it : it >> 2];
-            const Cand cd = a.cand[g];
-            const int2 pr = a.pairs[cd.pair];
-            gather_split(a.meshes[pr.x], FACE == 0 ? cd.faceA : 2 * cd.faceA + (sub & 1), X);
-            gather_split(a.meshes[pr.y], FACE == 0 ? cd.faceB : 2 * cd.faceB + (sub >> 1), Y);
+    double z[4];
+#pragma unroll
+    for (int row = 3; row >= 0; --row) {
+        double acc = r;
+#pragma unroll
+        for (int j = row + 1; j < 4; ++j) acc = acc - A[j] * z[j];
+        z[row] = __shfl_sync(FULL, acc * inv[row], holder[row]);
+    }
+    const double rest1 = 1.0 - z[0] - z[1], rest2 = 1.0 - z[2] - z[3];
+    // the margin as an ordered integer
+    long long mo = min(min(min(ord64(z[0]), ord64(z[1])), min(ord64(z[2]), ord64(z[3]))), min(ord64(rest1), ord64(rest2)));
+    bool finite = true;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) finite &= abs64(z[j]) < 0x7ff0000000000000ULL;
+    bool hit = live && ok && finite && mo >= ord64(-tau);
+    if (!__any_sync(FULL, hit)) return;
+    const double det = (negative ? -1.0 : 1.0) * diag[0] * diag[1] * diag[2] * diag[3];
+    // lane c takes column c's norm
+    double n2 = 0.0;
+    {
+        const double cols[4] = {col0, col1, col2, col3};
+        double e[4];
+#pragma unroll
+        for (int row = 0; row < 4; ++row) {
+            double v = 0.0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const double o = __shfl_sync(FULL, cols[j], base + row);
+                v = j == c ? o : v;
+            }
+            e[row] = v;
         }
-        pair_tests(valid, g, sub, X, Y, FACE == 1);
-        drain_full();
+        n2 = e[0] * e[0] + e[1] * e[1] + e[2] * e[2] + e[3] * e[3];
     }
-    if (qn) {
-        drain(0, qn);
-        __syncwarp();
+    const double nc = sqrt(n2);
+    const double norms = quad_lane(nc, base, 0) * quad_lane(nc, base, 1) * quad_lane(nc, base, 2) * quad_lane(nc, base, 3);
+    const double rho = fabs(det) / norms;
+    const double m = ord64_value(mo);
+    hit &= rho > 0.0;
+    // lane c's coordinate of the point, and its estimate: theta_u, s_u, theta_s, s_s
+    // (formulas after Eq. (precise))
+    const double P = x1 + z[0] * col0 + z[1] * col1;
+    double est;
+    {
+        const MeshDev &me = c < 2 ? ma : mb;
+        const uint32_t t = c < 2 ? ta : tb, q = t >> 1;
+        const int k = (int)__umul64hi((unsigned long long)q, me.nmagic), i = (int)(q - (uint32_t)k * (uint32_t)me.N);
+        double v0, v1;
+        if (c & 1) {
+            v0 = me.s[k];
+            v1 = me.s[k + 1];
+        } else {
+            v0 = i * me.dtheta;
+            v1 = v0 + me.dtheta;
+        }
+        const double w = c == 0 ? z[0] : c == 1 ? z[1] : c == 2 ? z[2] : z[3];
+        // T2 measures its weights from the other corner
+        const double w0 = t & 1 ? w : 1.0 - w, w1 = t & 1 ? 1.0 - w : w;
+        est = w0 * v0 + w1 * v1;
+        // theta: fmod(est, 2 pi); the weights of a hit lie in [-1, 2] (tau < 1) and dtheta
+        // <= pi, so -2 pi < theta < 4 pi, where one subtraction is exact
+        if (!(c & 1)) {
+            if (est >= kTwoPi) est -= kTwoPi;
+            if (est < 0) est += kTwoPi;
+        }
     }
-    if (lane == 0) {
-        if (n_sat) atomicAdd(&a.ctr->sat, n_sat);
-        if (n_full) atomicAdd(&a.ctr->fp32, n_full);
+    const unsigned long long pos = slot(hit);
+    if (!hit || pos == ~0ULL) return;
+    double *o = reinterpret_cast<double *>(hits + pos);
+    o[2 + c] = c == 0 ? z[0] : c == 1 ? z[1] : c == 2 ? z[2] : z[3];
+    o[6 + c] = P;
+    o[10 + c] = est;
+    const unsigned band = rho < 1e-12 || fabs(m) < 1e-12 ? 1u : 0u;
+    if (c == 0) reinterpret_cast<uint2 *>(o)[0] = make_uint2(ta, tb);
+    else if (c == 1) reinterpret_cast<uint2 *>(o)[1] = make_uint2(pair, band);
+    else if (c == 2) o[14] = rho;
+    else o[15] = m;
+}
+
+// the place of a new raw hit (its key and bucket written), or ~0 past the capacity;
+// every lane of the warp calls it, a quad's lanes with the same hit
+__device__ __forceinline__ unsigned long long hit_place(const NarrowArgs &a, bool hit, uint32_t ta, uint32_t tb,
+                                                        uint32_t pair) {
+    const int lane = threadIdx.x & 31;
+    unsigned long long pos = warp_append(&a.ctr->raw_hits, hit && (lane & 3) == 0, FULL);
+    pos = __shfl_sync(FULL, pos, lane & ~3);
+    if (!hit || pos >= a.hit_cap) return ~0ULL;
+    if ((lane & 3) == 0) {
+        const uint64_t key = ((uint64_t)pair << (2 * a.tri_bits)) | ((uint64_t)ta << a.tri_bits) | (uint64_t)tb;
+        a.hit_key[pos] = key;
+        if (a.tail) a.hit_slot[pos] = atomicAdd(a.tail + tail_bucket(key, a.tri_bits, a.bscale), 1u);
+        else a.hit_val[pos] = (uint32_t)pos;
     }
+    return pos;
 }
 
 // Stage 1a: the quad-level separating-axis test of every candidate (quads, or triangles)
 // on its quads' vertices rounded down to FP32, the first mixed directions
 // first; the candidates they leave gather in a per-warp queue, and every 32 of
 // them take the other directions with all lanes busy; those still not cleared
-// are listed for the per-pair path of k_narrow_filter.
+// are listed for k_narrow_pairs.
 constexpr int kQuadWarps = 8;
 template <int FACE>
 __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a) {
@@ -859,7 +755,7 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
             keep = !quad_reject_lo<kQuadFirstAxes, 4, true>(QA, QB, tauf);
         }
         const unsigned long long pos = warp_append(&a.ctr->qkeep, keep, FULL);
-        if (keep && pos < a.cand_cap) a.qsurv[pos] = g;
+        if (keep && pos < a.qsurv_cap) a.qsurv[pos] = g;
     };
     for (unsigned long long g0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane;
          g0 < n; g0 += stride) {
@@ -892,38 +788,98 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
     if (lane == 0 && n_quad) atomicAdd(&a.ctr->quad, n_quad);
 }
 
-// Stage 2: the FP64 solve for the survivors, one lane each.  Bound by the FP64
-// pipe, which takes 16 cycles an SM for a warp's instruction (two lanes a clock)
-// and by the solve's dependent chain; blocks of one warp, so that a few thousand
-// solves spread over every SM (in blocks of 256, 12,000 of them sat on 48 SMs).
-constexpr int kSolveBlock = 32;
-__global__ void __launch_bounds__(kSolveBlock) k_narrow_fp64(NarrowArgs a) {
-    if (a.ctr->cand > a.cand_cap || a.ctr->fp64 > a.surv_cap) return;
-    const unsigned long long n = a.ctr->fp64;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+// Stage 2: the triangle pairs of the candidates the quad-level test left, one a lane:
+// the differences of the FP64 system, its FP32 rounding through the triangle-level
+// separating axes and the verified solve, and the few pairs neither can reject, listed
+// by block, through the FP64 solve, four lanes each.  One kernel, because each step waits
+// on a chain of loads and dependent instructions and there is little work in any (54,000
+// pairs, 12,050 solves at 4096 x 512; 740 and 157 at 1024 x 256): 35 us there against 27
+// for a kernel of the FP32 tests and 21 for one of the solves, and the two launches' 33 us
+// at 1024 x 256, with the quad-level test, became 22.  The FP32 system is the FP64
+// differences rounded, not differences of two-part vertices: fewer conversions.  There is
+// no test of the triangles' boxes; a pair that only they would clear takes the verified
+// solve.
+constexpr int kPairBlock = 128;
+template <int FACE>
+__global__ void __launch_bounds__(kPairBlock) k_narrow_pairs(NarrowArgs a) {
+    __shared__ uint4 s_pair[kPairBlock];
+    __shared__ unsigned s_n;
+    if (a.ctr->cand > a.cand_cap || a.ctr->qkeep > a.qsurv_cap) return;
+    const unsigned long long ni = (FACE == 0 ? 1 : 4) * a.ctr->qkeep;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    // tau rounded up: the FP32 tests only widen by it
+    const float tauf = __double2float_ru(a.tau);
+    for (unsigned long long i0 = blockIdx.x * (unsigned long long)kPairBlock; i0 < ni;
+         i0 += gridDim.x * (unsigned long long)kPairBlock) {
+        const unsigned long long it = i0 + threadIdx.x;
+        const bool valid = it < ni;
+        if (threadIdx.x == 0) s_n = 0;
+        bool need = false, full = false;
+        uint4 p = make_uint4(0u, 0u, 0u, 0u);
+        if (valid) {
+            const Cand cd = a.cand[a.qsurv[FACE == 0 ? it : it >> 2]];
+            const int sub = FACE == 0 ? 0 : (int)(it & 3);
+            const int2 pr = a.pairs[cd.pair];
+            p = make_uint4(FACE == 0 ? cd.faceA : 2 * cd.faceA + (sub & 1),
+                           FACE == 0 ? cd.faceB : 2 * cd.faceB + (sub >> 1), cd.pair, 0u);
+            double x[3][4], y[3][4];
+            gather_tri(a.meshes[pr.x], p.x, x);
+            gather_tri(a.meshes[pr.y], p.y, y);
+            float A[4][4], r[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                A[c][0] = f32_rn(x[0][c] - x[1][c]);
+                A[c][1] = f32_rn(x[2][c] - x[1][c]);
+                A[c][2] = f32_rn(y[1][c] - y[0][c]);
+                A[c][3] = f32_rn(y[1][c] - y[2][c]);
+                r[c] = f32_rn(y[1][c] - x[1][c]);
+            }
+            full = !fp32_sat_reject(A, r, tauf);
+            need = full && !fp32_verified_reject(A, r, tauf);
+        }
+        const unsigned tested = __popc(__ballot_sync(FULL, valid)), solved = __popc(__ballot_sync(FULL, full));
+        if (lane == 0) {
+            if (tested) atomicAdd(&a.ctr->sat, (unsigned long long)tested);
+            if (solved) atomicAdd(&a.ctr->fp32, (unsigned long long)solved);
+        }
+        __syncthreads();
+        const uint32_t want = __ballot_sync(FULL, need);
+        unsigned at = 0;
+        if (lane == 0 && want) at = atomicAdd(&s_n, (unsigned)__popc(want));
+        at = __shfl_sync(FULL, at, 0) + __popc(want & lanemask_lt());
+        if (need) s_pair[at] = p;
+        __syncthreads();
+        const unsigned n = s_n;
+        if (threadIdx.x == 0 && n) atomicAdd(&a.ctr->fp64, (unsigned long long)n);
+        for (unsigned k0 = 8 * warp; k0 < n; k0 += kPairBlock / 4) {
+            const unsigned k = k0 + (lane >> 2);
+            const uint4 q = s_pair[k < n ? k : k0];
+            const int2 pr = a.pairs[q.z];
+            solve_pair(a.meshes[pr.x], a.meshes[pr.y], q.x, q.y, q.z, a.tau, k < n, a.hits,
+                       [&](bool hit) { return hit_place(a, hit, q.x, q.y, q.z); });
+        }
+        __syncthreads();
+    }
+}
+
+// The FP32 filters off: every triangle pair of every candidate through the FP64 solve
+template <int FACE>
+__global__ void __launch_bounds__(kPairBlock) k_narrow_all(NarrowArgs a) {
+    if (a.ctr->cand > a.cand_cap) return;
+    const unsigned long long n = (FACE == 0 ? 1 : 4) * a.ctr->cand;
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.ctr->fp64 = n;
     const int lane = threadIdx.x & 31;
-    for (unsigned long long g0 = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x - lane;
-         g0 < n; g0 += stride) {
-        const unsigned long long g = g0 + lane;
-        bool hit = false;
-        tms_hit h;
-        Cand s;
-        s.faceA = s.faceB = s.pair = 0;
-        if (g < n) {
-            s = a.surv[g];
-            const int2 pr = a.pairs[s.pair];
-            hit = narrow_fp64(a.meshes[pr.x], a.meshes[pr.y], s.faceA, s.faceB, a.tau, h);
-        }
-        const unsigned long long pos = warp_append(&a.ctr->raw_hits, hit, FULL);
-        if (hit && pos < a.hit_cap) {
-            h.pair = s.pair;
-            a.hits[pos] = h;
-            const uint64_t key = ((uint64_t)s.pair << (2 * a.tri_bits)) |
-                                 ((uint64_t)s.faceA << a.tri_bits) | (uint64_t)s.faceB;
-            a.hit_key[pos] = key;
-            if (a.tail) a.hit_slot[pos] = atomicAdd(a.tail + tail_bucket(key, a.tri_bits, a.bscale), 1u);
-            else a.hit_val[pos] = (uint32_t)pos;
-        }
+    const unsigned long long gw = blockIdx.x * (unsigned long long)(kPairBlock / 32) + (threadIdx.x >> 5);
+    const unsigned long long nw = gridDim.x * (unsigned long long)(kPairBlock / 32);
+    for (unsigned long long k0 = 8 * gw; k0 < n; k0 += 8 * nw) {
+        const unsigned long long k = k0 + (lane >> 2), kk = k < n ? k : k0;
+        const Cand cd = a.cand[FACE == 0 ? kk : kk >> 2];
+        const int sub = FACE == 0 ? 0 : (int)(kk & 3);
+        const uint32_t ta = FACE == 0 ? cd.faceA : 2 * cd.faceA + (sub & 1);
+        const uint32_t tb = FACE == 0 ? cd.faceB : 2 * cd.faceB + (sub >> 1);
+        const int2 pr = a.pairs[cd.pair];
+        solve_pair(a.meshes[pr.x], a.meshes[pr.y], ta, tb, cd.pair, a.tau, k < n, a.hits,
+                   [&](bool hit) { return hit_place(a, hit, ta, tb, cd.pair); });
     }
 }
 
@@ -1325,43 +1281,19 @@ __global__ void __launch_bounds__(2 * kAdjointHits) k_adjoint(const __grid_const
 
 }  // namespace
 
-// The filter runs as one wave of resident blocks: its warps stride over the
-// candidates and end by draining part-filled queues with idle lanes, so each
-// extra wave adds a round of those tails (4 waves: 0.255 ms, 2: 0.241, 1: 0.232
-// on the 4096 x 512 workload).  Resident blocks per SM, the same on every
-// GB300, looked up by configure_narrow (outside stream capture) or at the first
-// launch.
-namespace {
-int g_filter_resident[2] = {};
-
-template <int FACE>
-int filter_resident() {
-    int &r = g_filter_resident[FACE];
-    if (r == 0) {
-        int nb = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_narrow_filter<FACE>, 256, 0) != cudaSuccess ||
-            nb < 1)
-            nb = 1;
-        r = nb;
-    }
-    return r;
-}
-}  // namespace
-
-void configure_narrow() {
-    filter_resident<0>();
-    filter_resident<1>();
-}
-
 void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st) {
-    if (face_level == 0) {
-        if (a.fp32_filter) k_quad_filter<0><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
-        k_narrow_filter<0><<<sms * filter_resident<0>(), 256, 0, st>>>(a);
-    } else {
-        if (a.fp32_filter) k_quad_filter<1><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
-        k_narrow_filter<1><<<sms * filter_resident<1>(), 256, 0, st>>>(a);
+    if (!a.fp32_filter) {
+        if (face_level == 0) k_narrow_all<0><<<sms * 16, kPairBlock, 0, st>>>(a);
+        else k_narrow_all<1><<<sms * 16, kPairBlock, 0, st>>>(a);
+        return;
     }
-    k_narrow_fp64<<<sms * 16, kSolveBlock, 0, st>>>(a);
+    if (face_level == 0) {
+        k_quad_filter<0><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
+        k_narrow_pairs<0><<<sms * 8, kPairBlock, 0, st>>>(a);
+    } else {
+        k_quad_filter<1><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
+        k_narrow_pairs<1><<<sms * 8, kPairBlock, 0, st>>>(a);
+    }
 }
 
 void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st) {

@@ -96,7 +96,7 @@ struct Buffers {
     uint2 *tcnt;
     uint2 *tstart;
     void *sort_scratch;
-    Cand *cand, *surv;
+    Cand *cand;
     uint32_t *qsurv;
     tms_hit *hits;
     uint64_t *hk, *hk2, *okeys;
@@ -139,7 +139,6 @@ size_t carve(unsigned char *base, Buffers &b) {
     const size_t broad_end = c.off;
     // narrow phase and merge, over the broad phase's bytes
     c.off = phase;
-    b.surv = c.take<Cand>(kSurvCap);
     b.qsurv = c.take<uint32_t>(kCandCap);
     b.hits = c.take<tms_hit>(kRawHitCap);
     b.hk = c.take<uint64_t>(kRawHitCap);
@@ -181,7 +180,6 @@ tms_status setup(int device, unsigned char **base) {
     NA_CK(cudaGetSymbolAddress(&p, g_arena));
     NA_CK(configure_face_pass());
     configure_emit();
-    configure_narrow();
     Buffers probe;
     if (carve(reinterpret_cast<unsigned char *>(p), probe) > kArenaBytes) {
         g_msg = "scratch layout exceeds the static arena";
@@ -335,8 +333,8 @@ extern "C" tms_status tms_search_noalloc(tms_mesh A, tms_mesh B, const tms_param
     ea.ent_cap = kEntCap; ea.cand = b.cand; ea.cand_cap = kCandCap; ea.moller = p.moller;
     launch_emit(ea, p.precision, p.face_level, grid / 2, s);
     NarrowArgs na;
-    na.cand = b.cand; na.cand_cap = kCandCap; na.surv = b.surv; na.surv_cap = kSurvCap;
-    na.qsurv = b.qsurv;
+    na.cand = b.cand; na.cand_cap = kCandCap;
+    na.qsurv = b.qsurv; na.qsurv_cap = kCandCap;
     na.meshes = b.tables->meshes; na.pairs = b.tables->pairs; na.ctr = b.ctr; na.hits = b.hits;
     na.hit_key = b.hk; na.hit_val = b.hv; na.hit_cap = kRawHitCap; na.tau = p.tau;
     na.tri_bits = tri_bits; na.fp32_filter = p.narrow_filter;
