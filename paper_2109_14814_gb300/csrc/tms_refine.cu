@@ -7,12 +7,18 @@
 // Layout: four lanes per seed, lane c owning coordinate c of every 4-vector
 // (W, its partials, the normal frame, one row of Df).  The four sines/cosines
 // and two exponentials an iteration needs are spread over the four lanes and
-// exchanged by shuffles; dot products are butterfly sums over the quad (the
-// same bits on every lane); the 4x4 solve is a partial-pivot elimination whose
-// rows live in the lanes.  Every stop decision is taken on the quad's first
-// lane and broadcast, so the four lanes always agree.  A warp loops while any
-// of its eight seeds is still iterating; the loop is bounded by max_iter + 1
-// evaluations per seed.
+// exchanged by shuffles; dot products are summed over the quad four at a time; the
+// 4x4 solve is a partial-pivot elimination whose rows live in the lanes.  Every stop
+// decision is taken on the quad's first lane and broadcast, so the four lanes always
+// agree.  A warp loops while any of its eight seeds is still iterating; the loop is
+// bounded by max_iter + 1 evaluations per seed.
+//
+// What bounds it: the FP64 pipe, which takes one warp instruction an SM every 19 clocks
+// (measured).  So scalars that all four lanes would compute alike are computed by one of
+// them and shuffled, comparisons and sign changes are integer, and a block is one warp,
+// so that 1500 warps (12,000 seeds) load the 152 SMs evenly (blocks of four put twelve
+// on some and eight on others): 12,000 seeds 1476 -> 866 us, 12,000 branches of 50 steps
+// 31.5 -> 19.4 ms, the results the same but for roundings in a few of 10,000.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -25,7 +31,7 @@ namespace {
 
 constexpr int kH = TMS_SURF_MAX_HARMONICS;
 constexpr int kF = TMS_SURF_MAX_FOLDS;
-constexpr int kThreads = 128;          // 32 seeds per block
+constexpr int kThreads = 32;           // 8 seeds per block
 constexpr int kSeedsPerBlock = kThreads / 4;
 constexpr unsigned kFull = 0xffffffffu;
 constexpr double kPi = 3.141592653589793;
@@ -141,8 +147,41 @@ __device__ __forceinline__ double quad_sum(double v) {
     return v;
 }
 
+// the quad's sums of four values: lane c holds that of the c-th, added in the order
+// quad_sum adds (three additions instead of eight)
+__device__ __forceinline__ double quad_sum4(double v0, double v1, double v2, double v3, int c) {
+    const bool b0 = c & 1, b1 = c & 2;
+    const double u = (b0 ? v1 : v0) + __shfl_xor_sync(kFull, b0 ? v0 : v1, 1);
+    const double w = (b0 ? v3 : v2) + __shfl_xor_sync(kFull, b0 ? v2 : v3, 1);
+    return (b1 ? w : u) + __shfl_xor_sync(kFull, b1 ? u : w, 2);
+}
+
 __device__ __forceinline__ double lane_val(double v, int base, int j) {
     return __shfl_sync(kFull, v, base + j);
+}
+
+// |v|'s bits (ordered as |v|, NaN above everything), and v negated when neg
+__device__ __forceinline__ long long abs_bits(double v) {
+    return __double_as_longlong(v) & 0x7fffffffffffffffLL;
+}
+__device__ __forceinline__ double flip(double v, bool neg) {
+    return __longlong_as_double(__double_as_longlong(v) ^ (neg ? (long long)(1ULL << 63) : 0LL));
+}
+__device__ __forceinline__ int exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
+
+// the corrector's thresholds: tol^2 and switch_below^2 (not negative) as their bits, the
+// limits of s as ordered integers (a zero limit as the zero that no zero passes)
+struct Stop {
+    long long tol2, sw2, lo, hi;
+};
+
+__device__ __forceinline__ Stop make_stop(const tms_refine_params &pr) {
+    Stop t;
+    t.tol2 = __double_as_longlong(pr.tol * pr.tol);
+    t.sw2 = __double_as_longlong(pr.switch_below * pr.switch_below);
+    t.lo = tms::ord64(pr.s_lo == 0.0 ? -0.0 : pr.s_lo);
+    t.hi = tms::ord64(pr.s_hi == 0.0 ? 0.0 : pr.s_hi);
+    return t;
 }
 
 // p = (s - r0)(s - r1)(s - r2) and its first two derivatives.
@@ -166,25 +205,37 @@ struct Eval {
     double r2, cn2, det, dx[4];
 };
 
+// The walking sheet's coefficients of each harmonic at a quad's own parameter (a, b over
+// k; -a; b), lane fastest: filled when the quad starts a step, read by its iterations.
+struct WalkCoef {
+    double v[kH][4][32];
+};
+
 template <int WALK>
-__device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair &sp,
-                                         const tms_refine_params &pr, double lnlam, double x0,
-                                         double x1, double x2, double x3, double aw, int c,
+__device__ __forceinline__ void evaluate(const Coef &cf, const WalkCoef *wc, const tms_surface_pair &sp,
+                                         const Stop &stop, double lnlam, double x0,
+                                         double x1, double x2, double x3, int c,
                                          int base, Eval &E) {
     const int K = sp.n_harmonics;
     const int NF = sp.n_folds;
+    const int lane = threadIdx.x & 31;
+    // B's sheet at the frame's parameter: its sums are the frame's
+    const bool same = WALK != 2 && sp.alpha_s == sp.alpha_ref;
     // ---- stop checks on the iterate (identical on the quad's lanes)
     int pre = -1;
-    if (!(isfinite(x0) && isfinite(x1) && isfinite(x2) && isfinite(x3)))
-        pre = TMS_REFINE_NON_FINITE;
-    else if (x1 < pr.s_lo || x1 > pr.s_hi || x3 < pr.s_lo || x3 > pr.s_hi)
-        pre = TMS_REFINE_ESCAPED;
+    {
+        const long long o1 = tms::ord64(x1), o3 = tms::ord64(x3);
+        if (max(max(exponent(x0), exponent(x1)), max(exponent(x2), exponent(x3))) == 0x7ff)
+            pre = TMS_REFINE_NON_FINITE;
+        else if (o1 < stop.lo || o1 > stop.hi || o3 < stop.lo || o3 > stop.hi)
+            pre = TMS_REFINE_ESCAPED;
+    }
 
-    // ---- sines/cosines and exponentials, one per lane
-    const double arg = c == 0 ? x0
-                     : c == 1 ? x2 + sp.c0
-                     : c == 2 ? sp.P * (x2 - sp.theta0)
-                              : cf.qpi * (x3 - sp.s0);
+    // ---- sines/cosines and exponentials, one per lane: of x0, x2 + c0,
+    //      P (x2 - theta0) and Q pi (x3 - s0)
+    const double arg = (c == 2 ? sp.P : c == 3 ? cf.qpi : 1.0) *
+                       ((c == 0 ? x0 : c == 3 ? x3 : x2) -
+                        (c == 0 ? 0.0 : c == 1 ? -sp.c0 : c == 2 ? sp.theta0 : sp.s0));
     double sn, cs;
     sincos(arg, &sn, &cs);
     const double sA = lane_val(sn, base, 0), cA = lane_val(cs, base, 0);
@@ -232,38 +283,58 @@ __device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair 
     //      T, T', T'' at theta' (alpha_ref).  cos/sin of k theta by angle addition.
     double TA = 0.0, TAt = 0.0, TB = 0.0, TBt = 0.0, TR = 0.0, TRt = 0.0, TRtt = 0.0;
     double ckA = cA, skA = sA, ckB = cB, skB = sB;
+    // lane c advances one of cos, sin of k theta_u, cos, sin of k theta'
+    const double r1 = c == 0 ? cA : c == 1 ? sA : c == 2 ? cB : sB;
+    const double r2 = c == 0 ? -sA : c == 1 ? cA : c == 2 ? -sB : cB;
 #pragma unroll
     for (int h = 0; h < kH; ++h) {
         if (h < K) {
-            double uak = cf.uak[h][c], ubk = cf.ubk[h][c], una = cf.una[h][c], ub = cf.ub[h][c];
-            double sak = cf.sak[h][c], sbk = cf.sbk[h][c], sna = cf.sna[h][c], sb = cf.sb[h][c];
+            double uak, ubk, una, ub, sak, sbk, sna, sb;
             if (WALK == 1) {
-                uak = fma(aw, cf.dak[h][c], uak);
-                ubk = fma(aw, cf.dbk[h][c], ubk);
-                una = fma(aw, cf.dna[h][c], una);
-                ub = fma(aw, cf.db[h][c], ub);
-            } else if (WALK == 2) {
-                sak = fma(aw, cf.dak[h][c], sak);
-                sbk = fma(aw, cf.dbk[h][c], sbk);
-                sna = fma(aw, cf.dna[h][c], sna);
-                sb = fma(aw, cf.db[h][c], sb);
+                uak = wc->v[h][0][lane];
+                ubk = wc->v[h][1][lane];
+                una = wc->v[h][2][lane];
+                ub = wc->v[h][3][lane];
+            } else {
+                uak = cf.uak[h][c];
+                ubk = cf.ubk[h][c];
+                una = cf.una[h][c];
+                ub = cf.ub[h][c];
+            }
+            if (WALK == 2) {
+                sak = wc->v[h][0][lane];
+                sbk = wc->v[h][1][lane];
+                sna = wc->v[h][2][lane];
+                sb = wc->v[h][3][lane];
+            } else {
+                sak = cf.sak[h][c];
+                sbk = cf.sbk[h][c];
+                sna = cf.sna[h][c];
+                sb = cf.sb[h][c];
             }
             TA = fma(uak, ckA, fma(ubk, skA, TA));
             TAt = fma(ub, ckA, fma(una, skA, TAt));
             TB = fma(sak, ckB, fma(sbk, skB, TB));
             TBt = fma(sb, ckB, fma(sna, skB, TBt));
-            TR = fma(cf.ark[h][c], ckB, fma(cf.brk[h][c], skB, TR));
-            TRt = fma(cf.br[h][c], ckB, fma(cf.nar[h][c], skB, TRt));
+            if (!same) {
+                TR = fma(cf.ark[h][c], ckB, fma(cf.brk[h][c], skB, TR));
+                TRt = fma(cf.br[h][c], ckB, fma(cf.nar[h][c], skB, TRt));
+            }
             TRtt = fma(cf.kar[h][c], ckB, fma(cf.kbr[h][c], skB, TRtt));
             if (h + 1 < K) {
-                const double nA = ckA * cA - skA * sA;
-                skA = skA * cA + ckA * sA;
-                ckA = nA;
-                const double nB = ckB * cB - skB * sB;
-                skB = skB * cB + ckB * sB;
-                ckB = nB;
+                // cos: ck c1 - sk s1;  sin: sk c1 + ck s1
+                const double ck = c & 2 ? ckB : ckA, sk = c & 2 ? skB : skA;
+                const double v = fma(ck, r1, sk * r2);
+                ckA = lane_val(v, base, 0);
+                skA = lane_val(v, base, 1);
+                ckB = lane_val(v, base, 2);
+                skB = lane_val(v, base, 3);
             }
         }
+    }
+    if (same) {
+        TR = TB;
+        TRt = TBt;
     }
 
     // ---- W_A and its partials; B's underlying sheet; the frame sheet
@@ -273,41 +344,36 @@ __device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair 
     const double Wtt = gB * TRtt, Wts = gB1 * TRt, Wss = gB2 * TR + FB2;
     const double v1 = cf.v1[c], v2 = cf.v2[c];
 
-    // ---- normal frame (n1, n2) and its theta- and s-partials
-    const double g11 = quad_sum(t1 * t1), g12 = quad_sum(t1 * t2), g22 = quad_sum(t2 * t2);
-    const double j11 = quad_sum(t1 * v1), j21 = quad_sum(t2 * v1);
-    const double j12 = quad_sum(t1 * v2), j22 = quad_sum(t2 * v2);
-    const double P1 = quad_sum(t1 * Wtt), P2 = quad_sum(t1 * Wts), P3 = quad_sum(Wtt * t2);
-    const double P4 = quad_sum(t2 * Wts), P5 = quad_sum(t1 * Wss), P6 = quad_sum(t2 * Wss);
-    const double Lt1 = quad_sum(Wtt * v1), Ls1 = quad_sum(Wts * v1), Ss1 = quad_sum(Wss * v1);
-    const double Lt2 = quad_sum(Wtt * v2), Ls2 = quad_sum(Wts * v2), Ss2 = quad_sum(Wss * v2);
+    // ---- normal frame (n1, n2) and its theta- and s-partials.  G = J^T J + eps I; lane c
+    //      solves for frame vector r = c & 1 and its derivative in theta (d = 0) or s
+    //      (d = 1), where d t1 = Wtt, d t2 = Wts or d t1 = -Wts, d t2 = -Wss
+    const int r = c & 1, d = c >> 1;
+    const double q1 = quad_sum4(t1 * t1, t1 * t2, t2 * t2, t2 * Wts, c);
+    const double q2 = quad_sum4(t1 * v1, t1 * v2, t2 * v1, t2 * v2, c);
+    const double q3 = quad_sum4(t1 * Wtt, t1 * Wts, Wtt * t2, t1 * Wss, c);
+    const double q4 = quad_sum4(Wtt * v1, Wtt * v2, Wts * v1, Wts * v2, c);
+    const double q5 = quad_sum4(Wss * v1, Wss * v2, t2 * Wss, 0.0, c);
+    const double g11 = lane_val(q1, base, 0), g12 = lane_val(q1, base, 1), g22 = lane_val(q1, base, 2);
     const double eps = cf.hreg * (g11 + g22);
     const double G11 = g11 + eps, G12 = g12, G22 = g22 + eps;
     const double idet = 1.0 / (G11 * G22 - G12 * G12);
-    // d/dtheta and d/ds of G (J^T J + eps I)
-    const double tg11 = 2.0 * P1, tg12 = P2 + P3, tg22 = 2.0 * P4;
-    const double te = cf.hreg * (tg11 + tg22);
-    const double tG11 = tg11 + te, tG22 = tg22 + te;
-    const double sg11 = -2.0 * P2, sg12 = -(P5 + P4), sg22 = -2.0 * P6;
-    const double se = cf.hreg * (sg11 + sg22);
-    const double sG11 = sg11 + se, sG22 = sg22 + se;
-
-    // lane c solves for frame vector r = c & 1, then both are shared
-    double yv[6];
+    double yv[4];
     {
-        const int r = c & 1;
-        const double j1 = r ? j12 : j11, j2 = r ? j22 : j21;
-        const double Lt = r ? Lt2 : Lt1, Ls = r ? Ls2 : Ls1, Ss = r ? Ss2 : Ss1;
+        const double P4 = lane_val(q1, base, 3), P6 = lane_val(q5, base, 2), P3 = lane_val(q3, base, 2);
+        const double j1 = lane_val(q2, base, r), j2 = lane_val(q2, base, 2 + r);
+        const double Ls = lane_val(q4, base, 2 + r), Ss = lane_val(q5, base, r);
+        const double e11 = flip(2.0 * lane_val(q3, base, d), d);
+        const double e12 = flip(lane_val(q3, base, 1 + 2 * d) + (d ? P4 : P3), d);
+        const double e22 = flip(2.0 * (d ? P6 : P4), d);
+        const double te = cf.hreg * (e11 + e22);
+        const double E11 = e11 + te, E22 = e22 + te;
         const double y1 = (G22 * j1 - G12 * j2) * idet, y2 = (G11 * j2 - G12 * j1) * idet;
-        // theta: d t1 = Wtt, d t2 = Wts;  s: d t1 = -Wts, d t2 = -Wss
-        const double a1 = Lt - (tG11 * y1 + tg12 * y2), a2 = Ls - (tg12 * y1 + tG22 * y2);
-        const double b1 = -Ls - (sG11 * y1 + sg12 * y2), b2 = -Ss - (sg12 * y1 + sG22 * y2);
+        const double a1 = flip(lane_val(q4, base, r + 2 * d), d) - (E11 * y1 + e12 * y2);
+        const double a2 = flip(d ? Ss : Ls, d) - (e12 * y1 + E22 * y2);
         yv[0] = y1;
         yv[1] = y2;
         yv[2] = (G22 * a1 - G12 * a2) * idet;
         yv[3] = (G11 * a2 - G12 * a1) * idet;
-        yv[4] = (G22 * b1 - G12 * b2) * idet;
-        yv[5] = (G11 * b2 - G12 * b1) * idet;
     }
     double n[2], nt[2], ns[2];
 #pragma unroll
@@ -315,7 +381,7 @@ __device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair 
         const double v = r == 0 ? v1 : v2;
         const double y1 = lane_val(yv[0], base, r), y2 = lane_val(yv[1], base, r);
         const double dt1 = lane_val(yv[2], base, r), dt2 = lane_val(yv[3], base, r);
-        const double ds1 = lane_val(yv[4], base, r), ds2 = lane_val(yv[5], base, r);
+        const double ds1 = lane_val(yv[2], base, 2 + r), ds2 = lane_val(yv[3], base, 2 + r);
         n[r] = v - t1 * y1 - t2 * y2;
         nt[r] = -(Wtt * y1 + Wts * y2) - (t1 * dt1 + t2 * dt2);
         ns[r] = (Wts * y1 + Wss * y2) - (t1 * ds1 + t2 * ds2);
@@ -329,12 +395,11 @@ __device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair 
     const double fc = WA - (SB + H);
     double m[4] = {WAt, WAs, -(SBt + Ht), -(-SBs + Hs)};
 
-    const double r2 = quad_sum(fc * fc);
-    double cn2 = 1.0;   // product of the squared column norms
-#pragma unroll
-    for (int j = 0; j < 4; ++j) cn2 *= quad_sum(m[j] * m[j]);
-    int fin = isfinite(fc) && isfinite(m[0]) && isfinite(m[1]) && isfinite(m[2]) &&
-              isfinite(m[3]);
+    const double f2 = quad_sum(fc * fc);
+    // product of the squared column norms
+    const double qn = quad_sum4(m[0] * m[0], m[1] * m[1], m[2] * m[2], m[3] * m[3], c);
+    const double cn2 = lane_val(qn, base, 0) * lane_val(qn, base, 1) * lane_val(qn, base, 2) * lane_val(qn, base, 3);
+    int fin = max(max(exponent(fc), exponent(m[0])), max(exponent(m[1]), max(exponent(m[2]), exponent(m[3])))) < 0x7ff;
     fin &= __shfl_xor_sync(kFull, fin, 1);
     fin &= __shfl_xor_sync(kFull, fin, 2);
 
@@ -343,11 +408,11 @@ __device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair 
     int used = 0, pl[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        double cand = ((used >> c) & 1) ? -1.0 : fabs(m[j]);
+        long long cand = ((used >> c) & 1) ? -1LL : abs_bits(m[j]);
         int bl = c;
 #pragma unroll
         for (int off = 1; off <= 2; off <<= 1) {
-            const double oc = __shfl_xor_sync(kFull, cand, off);
+            const long long oc = __shfl_xor_sync(kFull, cand, off);
             const int ol = __shfl_xor_sync(kFull, bl, off);
             if (oc > cand || (oc == cand && ol < bl)) {
                 cand = oc;
@@ -361,20 +426,20 @@ __device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair 
         for (int q = j; q < 4; ++q) pj[q] = lane_val(m[q], base, bl);
         const double prr = lane_val(rr, base, bl);
         det *= pj[j];
-        ip[j] = pj[j] != 0.0 ? 1.0 / pj[j] : 0.0;
-        if (!((used >> c) & 1)) {
+        ip[j] = cand != 0 ? 1.0 / pj[j] : 0.0;
+        if (j < 3 && !((used >> c) & 1)) {
             const double fct = m[j] * ip[j];
 #pragma unroll
             for (int q = j + 1; q < 4; ++q) m[q] -= fct * pj[q];
             rr -= fct * prr;
-            m[j] = 0.0;
         }
     }
+    bool odd = false;
 #pragma unroll
     for (int u = 0; u < 4; ++u)
 #pragma unroll
-        for (int w = u + 1; w < 4; ++w)
-            if (pl[u] > pl[w]) det = -det;
+        for (int w = u + 1; w < 4; ++w) odd ^= pl[u] > pl[w];
+    det = flip(det, odd);
     double dx[4];
 #pragma unroll
     for (int j = 3; j >= 0; --j) {
@@ -386,32 +451,46 @@ __device__ __forceinline__ void evaluate(const Coef &cf, const tms_surface_pair 
 
     E.pre = pre;
     E.fin = fin;
-    E.r2 = r2;
+    E.r2 = f2;
     E.cn2 = cn2;
     E.det = det;
 #pragma unroll
     for (int q = 0; q < 4; ++q) E.dx[q] = dx[q];
 }
 
+// |det| >= rho_min sqrt(cn2), out of line: only near the threshold
+__device__ __noinline__ bool above_rho_min(double det, double rho_min, double cn2) {
+    return fabs(det) >= rho_min * sqrt(cn2);
+}
+
 // The decision of Eq. (dampedNewtonEquation)'s iteration k from an evaluation:
 // -1 to update, else the stop status (taken on the quad's first lane).
-__device__ __forceinline__ int decide(const Eval &E, const tms_refine_params &pr, double tol2, int k,
+__device__ __forceinline__ int decide(const Eval &E, const tms_refine_params &pr, const Stop &stop, int k,
                                       int base) {
     // ||f|| <= tol as ||f||^2 <= tol^2; |det| / prod ||col|| >= rho_min as
-    // |det| >= rho_min sqrt(prod ||col||^2)
+    // |det| >= rho_min sqrt(prod ||col||^2), decided by the exponents alone (|det| >=
+    // 2^(ed - 1023), rho_min < 2^(er - 1022), cn2 < 2^(ec - 1022)) where they do
     int dec = E.pre;
     if (dec < 0) {
+        const int ed = exponent(E.det), er = exponent(pr.rho_min), ec = exponent(E.cn2);
+        const bool clear = ed > 0 && ed < 0x7ff && er < 0x7ff && ec < 0x7ff && 2 * ed + 1020 >= 2 * er + ec;
         if (!E.fin) dec = TMS_REFINE_NON_FINITE;
-        else if (E.r2 <= tol2) dec = TMS_REFINE_CONVERGED;
+        else if (__double_as_longlong(E.r2) <= stop.tol2) dec = TMS_REFINE_CONVERGED;
         else if (k == pr.max_iter) dec = TMS_REFINE_MAX_ITER;
-        else if (!(fabs(E.det) >= pr.rho_min * sqrt(E.cn2))) dec = TMS_REFINE_SINGULAR;
+        else if (!clear && !above_rho_min(E.det, pr.rho_min, E.cn2)) dec = TMS_REFINE_SINGULAR;
     }
     return __shfl_sync(kFull, dec, base);
 }
 
-// Applies a decision to a quad that is still iterating.
-__device__ __forceinline__ void apply(const Eval &E, const tms_refine_params &pr, double sw2, int dec,
-                                      int k, Solve &S) {
+// Applies a decision to a quad that is still iterating (every lane of the warp calls
+// it: lane c updates x_c).
+__device__ __forceinline__ void apply(const Eval &E, const tms_refine_params &pr, const Stop &stop, int dec,
+                                      int k, Solve &S, int c, int base) {
+    const double al = __double_as_longlong(E.r2) > stop.sw2 ? pr.alpha0 : pr.alpha1;
+    const double own = c == 0 ? S.x0 : c == 1 ? S.x1 : c == 2 ? S.x2 : S.x3;
+    const double nx = own - al * (c == 0 ? E.dx[0] : c == 1 ? E.dx[1] : c == 2 ? E.dx[2] : E.dx[3]);
+    const double n0 = lane_val(nx, base, 0), n1 = lane_val(nx, base, 1);
+    const double n2 = lane_val(nx, base, 2), n3 = lane_val(nx, base, 3);
     if (S.code >= 0) return;
     if (E.pre < 0) {
         S.fn = E.r2;
@@ -422,11 +501,10 @@ __device__ __forceinline__ void apply(const Eval &E, const tms_refine_params &pr
         S.code = dec;
         S.iters = k;
     } else {
-        const double al = E.r2 > sw2 ? pr.alpha0 : pr.alpha1;
-        S.x0 -= al * E.dx[0];
-        S.x1 -= al * E.dx[1];
-        S.x2 -= al * E.dx[2];
-        S.x3 -= al * E.dx[3];
+        S.x0 = n0;
+        S.x1 = n1;
+        S.x2 = n2;
+        S.x3 = n3;
         S.k = k + 1;
     }
 }
@@ -437,22 +515,34 @@ __device__ __forceinline__ void newton_solve(const Coef &cf, const tms_surface_p
                                              const tms_refine_params &pr, Solve &S, int c,
                                              int base) {
     const double lnlam = sp.stretch ? log(sp.lam) : 0.0;
-    const double tol2 = pr.tol * pr.tol, sw2 = pr.switch_below * pr.switch_below;
+    const Stop stop = make_stop(pr);
     for (int k = 0; __any_sync(kFull, S.code < 0); ++k) {
         Eval E;
-        evaluate<0>(cf, sp, pr, lnlam, S.x0, S.x1, S.x2, S.x3, 0.0, c, base, E);
-        apply(E, pr, sw2, decide(E, pr, tol2, k, base), k, S);
+        evaluate<0>(cf, nullptr, sp, stop, lnlam, S.x0, S.x1, S.x2, S.x3, c, base, E);
+        apply(E, pr, stop, decide(E, pr, stop, k, base), k, S, c, base);
     }
 }
 
 // One iteration for each quad at its own count S.k (the continuation).
 template <int WALK>
-__device__ __forceinline__ void newton_iter(const Coef &cf, const tms_surface_pair &sp,
-                                            const tms_refine_params &pr, double lnlam, double tol2,
-                                            double sw2, Solve &S, double aw, int c, int base) {
+__device__ __forceinline__ void newton_iter(const Coef &cf, const WalkCoef *wc, const tms_surface_pair &sp,
+                                            const tms_refine_params &pr, const Stop &stop, double lnlam,
+                                            Solve &S, int c, int base) {
     Eval E;
-    evaluate<WALK>(cf, sp, pr, lnlam, S.x0, S.x1, S.x2, S.x3, aw, c, base, E);
-    apply(E, pr, sw2, decide(E, pr, tol2, S.k, base), S.k, S);
+    evaluate<WALK>(cf, wc, sp, stop, lnlam, S.x0, S.x1, S.x2, S.x3, c, base, E);
+    apply(E, pr, stop, decide(E, pr, stop, S.k, base), S.k, S, c, base);
+}
+
+// the walking sheet's coefficients at the quad's parameter (lane c its column c)
+template <int WALK>
+__device__ __forceinline__ void fill_walk(const Coef &cf, WalkCoef &wc, int K, double aw, int c) {
+    const int lane = threadIdx.x & 31;
+    for (int h = 0; h < K; ++h) {
+        wc.v[h][0][lane] = fma(aw, cf.dak[h][c], WALK == 1 ? cf.uak[h][c] : cf.sak[h][c]);
+        wc.v[h][1][lane] = fma(aw, cf.dbk[h][c], WALK == 1 ? cf.ubk[h][c] : cf.sbk[h][c]);
+        wc.v[h][2][lane] = fma(aw, cf.dna[h][c], WALK == 1 ? cf.una[h][c] : cf.sna[h][c]);
+        wc.v[h][3][lane] = fma(aw, cf.db[h][c], WALK == 1 ? cf.ub[h][c] : cf.sb[h][c]);
+    }
 }
 
 __device__ __forceinline__ double wrap_angle(double v) {
@@ -520,6 +610,7 @@ __global__ void __launch_bounds__(kThreads) k_refine(const __grid_constant__ Ref
 template <int WALK>
 __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ ContArgs a) {
     __shared__ Coef cf;
+    __shared__ WalkCoef wc;
     const tms_surface_pair &sp = a.sp;
     const tms_continue_params &cp = a.p;
     const int t = threadIdx.x;
@@ -556,10 +647,10 @@ __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ C
     S.rh = S.fn;
     S.rc2 = 1.0;
     const double lnlam = sp.stretch ? log(sp.lam) : 0.0;
-    const double tol2 = cp.corrector.tol * cp.corrector.tol;
-    const double sw2 = cp.corrector.switch_below * cp.corrector.switch_below;
+    const Stop stop = make_stop(cp.corrector);
+    fill_walk<WALK>(cf, wc, sp.n_harmonics, aj, c);
     while (__any_sync(kFull, alive)) {
-        newton_iter<WALK>(cf, sp, cp.corrector, lnlam, tol2, sw2, S, aj, c, base);
+        newton_iter<WALK>(cf, &wc, sp, cp.corrector, stop, lnlam, S, c, base);
         if (!(alive && S.code >= 0)) continue;
         // ---- step j is done (identical on the quad's lanes; no shuffles below)
         const double xs[4] = {wrap_angle(S.x0), S.x1, wrap_angle(S.x2), S.x3};
@@ -610,6 +701,7 @@ __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ C
         am2 = am1;
         am1 = aj;
         aj = a.alphas[j - 1];
+        fill_walk<WALK>(cf, wc, sp.n_harmonics, aj, c);
         if (j == 1) {
 #pragma unroll
             for (int q = 0; q < 4; ++q) g[q] = p1[q];
