@@ -328,8 +328,8 @@ __device__ __forceinline__ void stage_push(Rec *stage, unsigned &n, bool pred, c
 
 // FP64 -> FP32 conversions from the IEEE-754 encodings, with integer operations
 // only (the FP64 pipe, which also carries FP64 conversions, is scarce on GB300).
-// Normal-range results equal round-down / round-up / round-to-nearest-even of
-// the value.  Outside the FP32 normal range the results are still valid bounds:
+// Normal-range results are a lower bound a place or less below / the nearest, ties to
+// even.  Outside the FP32 normal range the results are still valid bounds:
 // |x| < 2^-126 rounds outward to 0 or +-2^-126 (nearest: to +-0), |x| >= 2^128
 // to +-FLT_MAX or +-inf, NaN stays NaN.
 __device__ __forceinline__ unsigned f32_bits_trunc(unsigned long long b, int e32) {
@@ -358,22 +358,28 @@ __device__ __forceinline__ float f32_special(unsigned long long b, int e32, int 
 static __device__ __noinline__ float f32_rd_special(double x) {
     return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, -1);
 }
-// round down.  In the FP32 normal range the bits of |x| shifted right by 29, less the
-// exponents' difference, are the truncated FP32 magnitude
-__device__ __forceinline__ float f32_rd(double x) {
+// A lower bound of x, at most one FP32 place below it: in the FP32 normal range the bits
+// of |x| shifted right by 29, less the exponents' difference, are the truncated FP32
+// magnitude, and every negative one takes a place more (also where x is a float: to tell
+// costs two of the four instructions that the rest takes).  f32_range is below kF32Range
+// in that range.
+constexpr unsigned kF32Range = 254u << 21;
+__device__ __forceinline__ unsigned f32_range(double x) {
+    return 2u * (unsigned)__double2hiint(x) - (897u << 21);
+}
+__device__ __forceinline__ float f32_rd_normal(double x) {
     const unsigned h = (unsigned)__double2hiint(x), l = (unsigned)__double2loint(x);
-    const unsigned mag = h & 0x7fffffffu;
-    if (mag - (897u << 20) >= (254u << 20)) return f32_rd_special(x);
-    unsigned f = __funnelshift_r(l, mag, 29) - (896u << 23);
-    if ((int)h < 0 && (l & 0x1FFFFFFFu) != 0u) ++f;                    // negative, inexact
-    return __uint_as_float(f | (h & 0x80000000u));
+    return __uint_as_float((__funnelshift_r(l, h, 29) - (896u << 23) + (h >> 31)) | (h & 0x80000000u));
+}
+__device__ __forceinline__ float f32_rd(double x) {
+    return f32_range(x) >= kF32Range ? f32_rd_special(x) : f32_rd_normal(x);
 }
 // an upper bound of every x with f32_rd(x) = f, one or two FP32 places above f (2^-23 |f|
-// is at least a place; 2^-126 covers what is rounded to 0): two instructions of the FMA
-// pipe, where the next number from the bits takes six of the busier integer pipe.  An
+// is at least a place; 2^-126 covers what is rounded to 0, and -FLT_MAX what is rounded to
+// -inf, where the sum is a NaN): two instructions of the FMA pipe and a maximum, where the next number from the bits takes six of the busier integer pipe.  An
 // exact x is over by that too, so that the value rounded down is all a vertex keeps
 __device__ __forceinline__ float f32_above(float f) {
-    return f + fmaf(fabsf(f), 1.1920932e-7f, 1.17549435e-38f);
+    return fmaxf(f + fmaf(fabsf(f), 1.1920932e-7f, 1.17549435e-38f), -3.40282347e38f);
 }
 static __device__ __noinline__ float f32_rn_special(double x) {
     return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, 0);

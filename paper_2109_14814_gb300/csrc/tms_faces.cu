@@ -93,11 +93,41 @@ __device__ __forceinline__ BoxT<PREC> closed(BoxT<PREC> b) {
     return b;
 }
 
-template <int PREC>
-__device__ __forceinline__ Vtx<PREC> to_vtx(const double x[4]) {
-    Vtx<PREC> v;
+// a vertex in the boxes' numbers; top takes high words of coordinates (shifted left by
+// one), those of a coordinate that is not finite among them
+static __device__ __noinline__ float4 rd_special4(double x, double y, double z, double w) {
+    return make_float4(f32_rd(x), f32_rd(y), f32_rd(z), f32_rd(w));
+}
+__device__ __forceinline__ unsigned top_word(const double x[4]) {
+    unsigned t = 0;
 #pragma unroll
-    for (int d = 0; d < 4; ++d) v.v[d] = Num<PREC>::of(x[d]);
+    for (int d = 0; d < 4; ++d) t = max(t, 2u * (unsigned)__double2hiint(x[d]));
+    return t;
+}
+template <int PREC>
+__device__ __forceinline__ Vtx<PREC> to_vtx(const double x[4], unsigned &top);
+template <>
+__device__ __forceinline__ Vtx<1> to_vtx<1>(const double x[4], unsigned &top) {
+    Vtx<1> v;
+    unsigned r = 0;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) {
+        r = max(r, f32_range(x[d]));
+        v.v[d] = f32_rd_normal(x[d]);
+    }
+    if (r >= kF32Range) {
+        const float4 s = rd_special4(x[0], x[1], x[2], x[3]);
+        v.v[0] = s.x; v.v[1] = s.y; v.v[2] = s.z; v.v[3] = s.w;
+        top = max(top, top_word(x));
+    }
+    return v;
+}
+template <>
+__device__ __forceinline__ Vtx<0> to_vtx<0>(const double x[4], unsigned &top) {
+    Vtx<0> v;
+#pragma unroll
+    for (int d = 0; d < 4; ++d) v.v[d] = ord64(x[d]);
+    top = max(top, top_word(x));
     return v;
 }
 
@@ -154,34 +184,34 @@ __device__ __forceinline__ void write_box<0>(void *arr, uint32_t face, const Box
     p[2] = make_longlong2(b.hi[0], b.hi[1]);
     p[3] = make_longlong2(b.hi[2], b.hi[3]);
 }
+// one side of a (closed) box: lo (side 0) or hi (side 1) of slot `face`
+__device__ __forceinline__ void write_side(void *arr, uint32_t face, int side, const float v[4]) {
+    reinterpret_cast<float4 *>(arr)[2 * (size_t)face + side] = make_float4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void write_side(void *arr, uint32_t face, int side, const long long v[4]) {
+    longlong2 *p = reinterpret_cast<longlong2 *>(arr) + 4 * (size_t)face + 2 * side;
+    p[0] = make_longlong2(v[0], v[1]);
+    p[1] = make_longlong2(v[2], v[3]);
+}
 template <int PREC>
 __device__ __forceinline__ void write_fbox(const MeshDev &m, uint32_t face, const BoxT<PREC> &b) {
     write_box<PREC>(m.fbox, face, closed<PREC>(b));
 }
 
-// a box that contains nothing (identity of the union)
+// The least and the negated largest of a vertex column's values over some rows (minima
+// only, so that lanes can reduce either alike).
 template <int PREC>
-__device__ __forceinline__ void box_empty(BoxT<PREC> &b) {
+struct ColBox {
+    typename Num<PREC>::T lo[4], nh[4];
+    __device__ __forceinline__ void init() {
 #pragma unroll
-    for (int d = 0; d < 4; ++d) { b.lo[d] = Num<PREC>::inf(); b.hi[d] = -b.lo[d]; }
-}
-template <int PREC>
-__device__ __forceinline__ void box_union(BoxT<PREC> &b, const BoxT<PREC> &x) {
-#pragma unroll
-    for (int d = 0; d < 4; ++d) { b.lo[d] = min(b.lo[d], x.lo[d]); b.hi[d] = max(b.hi[d], x.hi[d]); }
-}
-// union over aligned groups of `lanes` lanes (a quarter's 4 columns, a patch's 8)
-template <int PREC>
-__device__ __forceinline__ void box_reduce_lanes(BoxT<PREC> &b, int from, int lanes) {
-#pragma unroll
-    for (int off = from; off < lanes; off <<= 1) {
-#pragma unroll
-        for (int d = 0; d < 4; ++d) {
-            b.lo[d] = min(b.lo[d], __shfl_xor_sync(0xffffffffu, b.lo[d], off));
-            b.hi[d] = max(b.hi[d], __shfl_xor_sync(0xffffffffu, b.hi[d], off));
-        }
+        for (int d = 0; d < 4; ++d) lo[d] = nh[d] = Num<PREC>::inf();
     }
-}
+    __device__ __forceinline__ void add(const Vtx<PREC> &v) {
+#pragma unroll
+        for (int d = 0; d < 4; ++d) { lo[d] = min(lo[d], v.v[d]); nh[d] = min(nh[d], -v.v[d]); }
+    }
+};
 
 template <int PREC>
 __device__ __forceinline__ void read_fbox(const MeshDev &m, uint32_t face, BoxT<PREC> &b);
@@ -311,16 +341,19 @@ __device__ __forceinline__ void cross4(const float a[4], const float b[4], const
     x[2] = det3(a[0], a[1], a[3], b[0], b[1], b[3], c[0], c[1], c[3]);
     x[3] = -det3(a[0], a[1], a[2], b[0], b[1], b[2], c[0], c[1], c[2]);
 }
-// non-negative floats (and NaN, above +inf) compare as their bit patterns:
-// an integer maximum of |x| keeps a NaN, which fmaxf would drop
-__device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x) & 0x7fffffffu; }
+// the maximum that keeps a NaN (fmaxf would drop it)
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 
 // The frame of a patch, in three steps over the tile's patches: one thread a patch
 // computes the axes (frame_axes), the patch's kPatchI lanes project its vertices on
 // them (frame_extents), and one thread a patch closes the bounds and writes the record
 // (frame_write).  What is the same for a whole patch runs on as many threads as there
 // are patches (16 of a 128 x 4 tile): computed by all of a patch's lanes it was a third
-// of the kernel's instructions (65.6 M and 87 us at 4096 x 512; 54.5 M and 72 us so).
+// of the kernel's instructions (65.6 M and 87 us at 4096 x 512 then, 54.5 M and 72 us so).
 // Axes: e_0, e_1 from the patch's two parameter directions (sums of opposite
 // edges, one Gram-Schmidt step), e_2 orthogonal to e_0, e_1 and the coordinate
 // axis farthest from their span, e_3 orthogonal to e_0, e_1, e_2.  A patch
@@ -341,7 +374,7 @@ __device__ __forceinline__ unsigned abs_bits(float x) { return __float_as_uint(x
 struct PatchScratch {         // of a patch of the tile
     float4 lo, hi;            // its (closed) box
     float4 axes[5];           // c, e_0..e_3
-    uint4 top;                // max |e_k . (V - c)| (bits)
+    float4 top;               // max |e_k . (V - c)|
     uint4 flags;              // x: no usable axes
 };
 
@@ -418,34 +451,38 @@ __device__ __forceinline__ void frame_axes(const Vtx<1> *sv, int W, int p0, int 
     P.flags.x = bad;
 }
 
-// Lane l of a patch takes its vertex column l (rows pr0..pr0 + rq) and, for l <= rq, the
-// vertex of the closing column in row pr0 + l; the integer maximum keeps NaN.  Every
-// lane of the warp calls it (cq = 0: no patch).
-__device__ __forceinline__ void frame_extents(const Vtx<1> *sv, int W, int t, int cq, int pr0, int rq, PatchScratch &P) {
+// Lane l of a patch takes its vertex column l (its own vertices, rows 0..rq of the patch)
+// and, for l <= rq, the vertex of the closing column in row l.  Every lane of the warp
+// calls it (cq = 0: no patch).
+__device__ __forceinline__ void frame_extents(const Vtx<1> *sv, const Vtx<1> *own, int W, int t, int cq, int pr0, int rq,
+                                              PatchScratch &P) {
     const int l = t & (kPatchI - 1), p0 = t - l;
-    unsigned am[4] = {0u, 0u, 0u, 0u};
+    float am[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if (cq > 0) {
         const float4 c = P.axes[0], e0 = P.axes[1], e1 = P.axes[2], e2 = P.axes[3], e3 = P.axes[4];
         auto vertex = [&](const Vtx<1> &v) {
             const float4 x = *reinterpret_cast<const float4 *>(v.v);
             const float d[4] = {x.x - c.x, x.y - c.y, x.z - c.z, x.w - c.w};
             auto dot = [&](const float4 &e) {
-                return abs_bits(fmaf(e.w, d[3], fmaf(e.z, d[2], fmaf(e.y, d[1], e.x * d[0]))));
+                return fabsf(fmaf(e.w, d[3], fmaf(e.z, d[2], fmaf(e.y, d[1], e.x * d[0]))));
             };
-            am[0] = max(am[0], dot(e0));
-            am[1] = max(am[1], dot(e1));
-            am[2] = max(am[2], dot(e2));
-            am[3] = max(am[3], dot(e3));
+            am[0] = max_nan(am[0], dot(e0));
+            am[1] = max_nan(am[1], dot(e1));
+            am[2] = max_nan(am[2], dot(e2));
+            am[3] = max_nan(am[3], dot(e3));
         };
-        if (l < cq)
-            for (int rr = pr0; rr <= pr0 + rq; ++rr) vertex(sv[rr * W + t]);
+        if (l < cq) {
+#pragma unroll
+            for (int rr = 0; rr <= kPatchK; ++rr)
+                if (rr <= rq) vertex(own[rr]);
+        }
         if (l <= rq) vertex(sv[(pr0 + l) * W + p0 + cq]);
     }
 #pragma unroll
     for (int off = 1; off < kPatchI; off <<= 1)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) am[k] = max(am[k], __shfl_xor_sync(0xffffffffu, am[k], off));
-    if (cq > 0 && l == 0) P.top = make_uint4(am[0], am[1], am[2], am[3]);
+        for (int k = 0; k < 4; ++k) am[k] = max_nan(am[k], __shfl_xor_sync(0xffffffffu, am[k], off));
+    if (cq > 0 && l == 0) P.top = make_float4(am[0], am[1], am[2], am[3]);
 }
 
 __device__ __forceinline__ void frame_write(const PatchScratch &P, float4 *out, uint32_t p) {
@@ -459,7 +496,7 @@ __device__ __forceinline__ void frame_write(const PatchScratch &P, float4 *out, 
         const float4 e = P.axes[1 + k];
         E[k][0] = e.x; E[k][1] = e.y; E[k][2] = e.z; E[k][3] = e.w;
     }
-    const unsigned am[4] = {P.top.x, P.top.y, P.top.z, P.top.w};
+    const float am[4] = {P.top.x, P.top.y, P.top.z, P.top.w};
     bool bad = P.flags.x != 0;
     float nk[4], emax = 0.0f;
 #pragma unroll
@@ -486,7 +523,7 @@ __device__ __forceinline__ void frame_write(const PatchScratch &P, float4 *out, 
     float h[4], hs = 0.0f;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        h[k] = fmaf(nk[k], nu, __uint_as_float(am[k])) * 1.0001f + 1e-36f;
+        h[k] = fmaf(nk[k], nu, am[k]) * 1.0001f + 1e-36f;
         hs += h[k];
         bad |= !(h[k] < inf);
     }
@@ -508,8 +545,12 @@ __device__ __forceinline__ void frame_write(const PatchScratch &P, float4 *out, 
 // ---------------------------------------------------------------------------
 // bounds pass
 // ---------------------------------------------------------------------------
+// Registers: 64 a thread for mixed precision (a few of the vertices in flight are
+// spilled) put twice the warps on an SM of the 100 it would take: 64 pairs of
+// meshes from 128 x 32 to 2048 x 512 vertices 960 us a search against 802 (with 80: 840,
+// with 48: 785, but one 4096 x 512 pair is 1-2% slower than with 64).
 template <int PREC, int FACE, int TK>
-__global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
+__global__ void __launch_bounds__(256, PREC == 1 ? 4 : 2) k_bounds_pass(FacePassArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Vtx<PREC> *sv = reinterpret_cast<Vtx<PREC> *>(smem_raw);
     const int TI = blockDim.x;
@@ -529,6 +570,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
     // the largest high word of |x| tells whether any is not finite (a test of each value
     // beside its rounding becomes an FP64 comparison)
     unsigned top = 0;
+    Vtx<PREC> own[TK + 1];             // this thread's vertex column
     {
         const int t = threadIdx.x;
         double x[TK + 1][4];
@@ -548,11 +590,9 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
 #pragma unroll
         for (int r = 0; r <= TK; ++r) {
             if (col_ok && r <= rows_q) {
-#pragma unroll
-                for (int c = 0; c < 4; ++c) top = max(top, (unsigned)__double2hiint(x[r][c]) & 0x7fffffffu);
-                const Vtx<PREC> v = to_vtx<PREC>(x[r]);
-                sv[r * W + t] = v;
-                if (r < rows_q || last_rows) write_vlo(m, (size_t)(kq0 + r) * m.N + vi, v);
+                own[r] = to_vtx<PREC>(x[r], top);
+                sv[r * W + t] = own[r];
+                if (r < rows_q || last_rows) write_vlo(m, (size_t)(kq0 + r) * m.N + vi, own[r]);
             }
         }
         // the last vertex column of the tile (wraps to column 0 on a periodic mesh);
@@ -563,11 +603,8 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
             size_t off = (size_t)(kq0 + t) * m.N + vj;
             double y[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                y[c] = __ldg(m.c[c] + off);
-                top = max(top, (unsigned)__double2hiint(y[c]) & 0x7fffffffu);
-            }
-            const Vtx<PREC> v = to_vtx<PREC>(y);
+            for (int c = 0; c < 4; ++c) y[c] = __ldg(m.c[c] + off);
+            const Vtx<PREC> v = to_vtx<PREC>(y, top);
             sv[t * W + cols_q] = v;
             if (!m.periodic && vj == m.N - 1 && (t < rows_q || last_rows)) write_vlo(m, off, v);
         }
@@ -581,61 +618,73 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
     const bool col_valid = t < cols_q;
     const int i = i0 + t;
     if (FACE == 1 && a.patch) {
-        // quad faces with patches: as below, and each column's box over the
-        // patch row (kPatchK quad rows; tiles are whole patch rows) united across
-        // the kPatchI lanes of the patch (every lane of the block takes part:
-        // the row loop and its shuffles are uniform)
-        // this column's boxes over the upper and lower halves of the patch row
-        BoxT<PREC> prev, ptop, pbot;
-        box_empty(prev);
-        box_empty(ptop);
-        box_empty(pbot);
+        // quad faces with patches.  A quarter (four columns by two rows of quads) is the
+        // union of five vertex columns over three rows: each lane takes its own column,
+        // the four lanes share out the closing column's rows, and exchange so that lane
+        // j ends with one side (j & 1: lo, hi) of one of the two quarters (j & 2: upper,
+        // lower), which it closes and writes; the patch is their union.  (Every lane of
+        // the block takes part: the row loop and its shuffles are uniform.)  With a box
+        // for each quad, every lane reducing whole boxes, and each coordinate's rounding
+        // tested alone the kernel took 48.8 M instructions and 64 us at 4096 x 512; so
+        // 38.4 M (with 64 registers) and 53 us.
+        static_assert(kPatchI == 8 && kPatchK == 4 && TK % kPatchK == 0, "quarters of four columns by two rows");
+        typedef typename Num<PREC>::T T;
+        const int j = t & 3;
         // the patch exists when its first column is in the tile
         const bool patch_lane = (t & ~(kPatchI - 1)) < cols_q;
-        if (col_valid) {
-            box_init(prev, sv[t]);
-            box_add(prev, sv[t + 1]);
-        }
-        for (int r = 0; r < rows_q; ++r) {
-            if (col_valid) {
-                BoxT<PREC> next;
-                box_init(next, sv[(r + 1) * W + t]);
-                box_add(next, sv[(r + 1) * W + t + 1]);
-                BoxT<PREC> bq;
+        const int close = min((t & ~3) + 4, cols_q);      // the quarter's closing column
 #pragma unroll
-                for (int d = 0; d < 4; ++d) {
-                    bq.lo[d] = min(prev.lo[d], next.lo[d]);
-                    bq.hi[d] = max(prev.hi[d], next.hi[d]);
+        for (int pr = 0; pr < TK / kPatchK; ++pr) {
+            const int pr0 = pr * kPatchK, rq = min(kPatchK, rows_q - pr0);
+            if (rq <= 0) break;
+            ColBox<PREC> upper, lower;
+            upper.init();
+            lower.init();
+            if (col_valid) {
+                upper.add(own[pr0]);
+                upper.add(own[pr0 + 1]);
+                if (rq > 1) upper.add(own[pr0 + 2]);
+                if (rq > 2) {
+                    lower.add(own[pr0 + 2]);
+                    lower.add(own[pr0 + 3]);
+                    if (rq > 3) lower.add(own[pr0 + 4]);
                 }
-                if ((r % kPatchK) < kPatchK / 2) box_union<PREC>(ptop, bq);
-                else box_union<PREC>(pbot, bq);
-                prev = next;
             }
-            if ((r % kPatchK) == kPatchK - 1 || r == rows_q - 1) {
-                // quarters over 4 columns, then the patch over both column halves
-                box_reduce_lanes<PREC>(ptop, 1, kPatchI / 2);
-                box_reduce_lanes<PREC>(pbot, 1, kPatchI / 2);
-                BoxT<PREC> pb = ptop;
-                box_union<PREC>(pb, pbot);
-                box_reduce_lanes<PREC>(pb, kPatchI / 2, kPatchI);
-                const uint32_t p = (uint32_t)((kq0 + r) / kPatchK) * (uint32_t)m.npi +
-                                   (uint32_t)(i / kPatchI);
-                if (patch_lane && (t % (kPatchI / 2)) == 0) {
-                    const uint32_t half = (uint32_t)((t % kPatchI) / (kPatchI / 2));
-                    write_box<PREC>(m.qbox, 4 * p + half, closed<PREC>(ptop));
-                    write_box<PREC>(m.qbox, 4 * p + 2 + half, closed<PREC>(pbot));
+            if ((t & ~3) < cols_q) {
+                if (j <= rq) {
+                    const Vtx<PREC> v = sv[(pr0 + j) * W + close];
+                    if (j <= 2) upper.add(v);
+                    if (j >= 2 && rq > 2) lower.add(v);
                 }
-                if (patch_lane && (t % kPatchI) == 0) {
-                    const BoxT<PREC> cb = closed<PREC>(pb);
-                    write_box<PREC>(m.pbox, p, cb);
-                    if constexpr (PREC == 1) {
-                        PatchScratch &P = sp[(r / kPatchK) * (TI / kPatchI) + t / kPatchI];
-                        P.lo = make_float4(cb.lo[0], cb.lo[1], cb.lo[2], cb.lo[3]);
-                        P.hi = make_float4(cb.hi[0], cb.hi[1], cb.hi[2], cb.hi[3]);
-                    }
+                if (j == 0 && rq > 3) lower.add(sv[(pr0 + 4) * W + close]);
+            }
+            T s[4];
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+                const bool odd = t & 1, low = t & 2;
+                const T u = min(odd ? upper.nh[d] : upper.lo[d],
+                                __shfl_xor_sync(FULL, odd ? upper.lo[d] : upper.nh[d], 1));
+                const T w = min(odd ? lower.nh[d] : lower.lo[d],
+                                __shfl_xor_sync(FULL, odd ? lower.lo[d] : lower.nh[d], 1));
+                s[d] = min(low ? w : u, __shfl_xor_sync(FULL, low ? u : w, 2));
+            }
+            const uint32_t p = (uint32_t)(kq0 / kPatchK + pr) * (uint32_t)m.npi + (uint32_t)(i / kPatchI);
+            T out[4];
+#pragma unroll
+            for (int d = 0; d < 4; ++d) out[d] = t & 1 ? Num<PREC>::above(-s[d]) : s[d];
+            if (patch_lane) write_side(m.qbox, 4 * p + (t & 2) + ((t >> 2) & 1), t & 1, out);
+#pragma unroll
+            for (int d = 0; d < 4; ++d) {
+                s[d] = min(s[d], __shfl_xor_sync(FULL, s[d], 2));
+                s[d] = min(s[d], __shfl_xor_sync(FULL, s[d], 4));
+                out[d] = t & 1 ? Num<PREC>::above(-s[d]) : s[d];
+            }
+            if (patch_lane && (t & (kPatchI - 2)) == 0) {
+                write_side(m.pbox, p, t & 1, out);
+                if constexpr (PREC == 1) {
+                    PatchScratch &P = sp[pr * (TI / kPatchI) + t / kPatchI];
+                    (t & 1 ? P.hi : P.lo) = make_float4(out[0], out[1], out[2], out[3]);
                 }
-                box_empty(ptop);
-                box_empty(pbot);
             }
         }
         // the frames of the tile's patches
@@ -650,9 +699,11 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
                 }
                 __syncthreads();
                 const int cq = patch_lane ? min(kPatchI, cols_q - (t & ~(kPatchI - 1))) : 0;
-                for (int pr0 = 0; pr0 < rows_q; pr0 += kPatchK)
-                    frame_extents(sv, W, t, cq, pr0, min(kPatchK, rows_q - pr0),
-                                  sp[(pr0 / kPatchK) * across + t / kPatchI]);
+#pragma unroll
+                for (int pr0 = 0; pr0 < TK; pr0 += kPatchK)
+                    if (pr0 < rows_q)
+                        frame_extents(sv, own + pr0, W, t, cq, pr0, min(kPatchK, rows_q - pr0),
+                                      sp[(pr0 / kPatchK) * across + t / kPatchI]);
                 __syncthreads();
                 for (int q = t; q < np; q += TI)
                     if ((q % across) * kPatchI < cols_q)
@@ -708,7 +759,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
     }
 
     if (a.patch) {
-        if (__any_sync(FULL, top >= 0x7ff00000u) && (threadIdx.x & 31) == 0) atomicOr(a.nonfinite, 1u);
+        if (__any_sync(FULL, top >= 0xffe00000u) && (threadIdx.x & 31) == 0) atomicOr(a.nonfinite, 1u);
         return;
     }
     // block reduction, then one set of atomics per block, each of twelve lanes its own
@@ -721,7 +772,7 @@ __global__ void __launch_bounds__(256) k_bounds_pass(FacePassArgs a) {
         const long long l = ~warp_max(negated(acc.lo[d])), h = warp_max(acc.hi[d]), w = warp_max(acc.w[d]);
         if (lane == 0) { red[warp][d] = l; red[warp][4 + d] = h; red[warp][8 + d] = w; }
     }
-    const unsigned fl = __any_sync(FULL, top >= 0x7ff00000u) ? 1u : 0u;
+    const unsigned fl = __any_sync(FULL, top >= 0xffe00000u) ? 1u : 0u;
     const unsigned seen = __reduce_or_sync(FULL, acc.seen);
     if (lane == 0) {
         redf[warp][0] = fl;
