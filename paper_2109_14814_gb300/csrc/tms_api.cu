@@ -139,7 +139,7 @@ struct Plan {
     uint64_t *hk = nullptr, *hk2 = nullptr, *okeys = nullptr;
     uint32_t *hv = nullptr, *hv2 = nullptr, *keep = nullptr, *kscan = nullptr;
     // short merge: bucket counts and drop bits, each bucket's first place
-    uint32_t *tail = nullptr, *bbase = nullptr;
+    uint32_t *tail = nullptr;
     float bscale = 0.0f;
     // more raw hits than the short merge takes: the radix sort and the scans (as
     // a search of this plan found; the look-back test switch needs that sort too)
@@ -176,7 +176,7 @@ struct Plan {
         free_scratch();
         void *ptrs[] = {d_meshes, d_pairs, d_pass_bounds, d_pass_all, d_pass_A, d_pass_B, d_bounds,
                         d_ctr, partials, vlo, fbox, pbox, qbox, pframe, d_cm_pair,
-                        tail, bbase, tbox, d_trees, d_top_base};
+                        tail, tbox, d_trees, d_top_base};
         for (void *p : ptrs)
             if (p) cudaFree(p);
         if (h_ctr) cudaFreeHost(h_ctr);
@@ -245,13 +245,13 @@ struct Plan {
     void enqueue_short_tail(cudaStream_t s) {
         mark(13, s);
         TailArgs ta;
-        ta.key = hk; ta.slot = kscan; ta.tail = tail; ta.bbase = bbase; ta.bkey = hk2; ta.bidx = hv2;
+        ta.key = hk; ta.slot = kscan; ta.tail = tail; ta.bkey = hk2; ta.bidx = hv2;
         ta.skey = okeys; ta.order = keep; ta.raw = hits; ta.meshes = d_meshes; ta.pairs = d_pairs;
         ta.ctr = d_ctr; ta.raw_cap = hit_cap; ta.out = (tms_hit *)dHits;
         ta.out_cap = (unsigned long long)hitCap; ta.offsets = dOffsets; ta.n_pairs = nPairs;
         ta.tri_bits = tri_bits; ta.tau = prm.tau; ta.bscale = bscale;
-        launch_tail(ta, grid / 2, s);
-        kernels += 3;
+        launch_tail(ta, s);
+        kernels += 1;
     }
 
     // sort and merge of any number of raw hits
@@ -543,7 +543,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     unsigned long long max_tri = 1;
     const int fl = prm.face_level;
     // a mesh that is in several pairs has one row of the mesh table and one bounds
-    // pass (a layer sweep takes every half-layer in four pairs: 387 -> 98 us of its
+    // pass (a layer sweep takes every half-layer in four pairs: 387 -> 117 us of its
     // bounds pass at the paper's shapes)
     std::map<long long, int> row_of;
     auto row = [&](tms_mesh m) {
@@ -710,7 +710,6 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
     // (and the word the bounds pass leaves a vertex that is not finite in)
     TMS_PCK(dalloc(&P->tail, kTailBuckets + kTailMax / 32 + 1));
     TMS_PCK(cudaMemset(P->tail, 0, (kTailBuckets + kTailMax / 32 + 1) * sizeof(uint32_t)));
-    TMS_PCK(dalloc(&P->bbase, kTailBuckets + 1));
     // the range of (pair, triA), over which the buckets are spread
     P->bscale = (float)((double)kTailBuckets /
                         (nPairs == 1 ? 2.0 * A[0]->dev.N * A[0]->dev.nqk
@@ -820,6 +819,7 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
         configure_emit();
         configure_patch_quads();
         configure_tree();
+        TMS_CK(configure_tail());
         g_configured_mask |= 1 << device;
     }
     Plan *P = find_plan(A, B, nPairs, prm, cm_pair, user, dHits, hitCap, dOffsets, device);

@@ -668,7 +668,6 @@ struct TailArgs {
     const uint64_t *key;           // raw hits' keys, in the order they were found
     const uint32_t *slot;          // and their places in their buckets
     uint32_t *tail;                // bucket counts [kTailBuckets], then drop bits [kTailMax / 32]
-    uint32_t *bbase;               // [kTailBuckets + 1] each bucket's first place
     uint64_t *bkey;                // [raw_cap] keys by bucket
     uint32_t *bidx;                // [raw_cap] raw-hit indices by bucket
     uint64_t *skey;                // [raw_cap] sorted keys
@@ -686,7 +685,8 @@ struct TailArgs {
     double tau;
     float bscale;
 };
-void launch_tail(const TailArgs &a, int sms, cudaStream_t st);
+void launch_tail(const TailArgs &a, cudaStream_t st);
+cudaError_t configure_tail();
 
 
 struct AdjointArgs {

@@ -1038,57 +1038,23 @@ __global__ void k_offsets(const uint64_t *out_keys, const unsigned long long *d_
 // ---------------------------------------------------------------------------
 // Latency, not work, bounds the merge of a few thousand hits (a radix pass over
 // six tiles is 7 us of loads, ranking and look-back, and the sort and merge took
-// 15 launches), so it is three launches here.  The FP64 solve counts the hits into
-// buckets of increasing key; k_tail_bucket scans the counts (every block for
-// itself: 32 KB from L2) and lists the hits bucket by bucket; k_tail_rank compares
-// a hit with its bucket (about one at 8192 buckets; however unevenly the hits
-// fall, at most kTailMax compares) and decides whether it is a duplicate;
-// k_tail_out writes the records kept.
+// 15 launches), so it is one launch of one cluster, whose barrier takes the place of
+// the launches between the steps: 16.5 us at 12,045 hits (three launches 10 + 7 + 7; a
+// cluster of eight, with one record a turn, 28), and a search of 1024 x 256 and
+// 771 x 331 vertices (157 hits) 112 -> 100 us.  The FP64 solve counts the hits into
+// buckets of increasing key; each block scans the counts for itself (32 KB from L2) and
+// lists its hits in their buckets; then compares a hit with its bucket (about one at
+// 8192 buckets; however unevenly the hits fall, at most kTailMax compares) and decides
+// whether it is a duplicate; then writes the records kept.
 __device__ __forceinline__ bool tail_count(const TailArgs &a, unsigned &n) {
     const unsigned long long raw = a.ctr->raw_hits;
     n = (unsigned)raw;
     return raw <= a.raw_cap && raw <= kTailMax;
 }
 
-constexpr int kBucketBlock = 1024;
-__global__ void __launch_bounds__(kBucketBlock) k_tail_bucket(TailArgs a) {
-    constexpr int kPer = kTailBuckets / kBucketBlock;
-    static_assert(kPer == 8, "two 16-byte loads a thread");
-    __shared__ uint32_t base[kTailBuckets];
-    __shared__ uint32_t wsum[kBucketBlock / 32];
-    unsigned n;
-    if (!tail_count(a, n)) return;
-    const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const unsigned first = blockIdx.x * kBucketBlock;
-    if (blockIdx.x > 0 && first >= n) return;      // block 0 writes the buckets' places
-    const uint4 lo = reinterpret_cast<const uint4 *>(a.tail)[2 * t], hi = reinterpret_cast<const uint4 *>(a.tail)[2 * t + 1];
-    const uint32_t c[kPer] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-    uint32_t sum = 0;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) sum += c[k];
-    uint32_t incl = sum;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL, incl, off);
-        if (lane >= off) incl += y;
-    }
-    if (lane == 31) wsum[warp] = incl;
-    __syncthreads();
-    uint32_t before = __reduce_add_sync(FULL, lane < warp ? wsum[lane] : 0u) + incl - sum;
-#pragma unroll
-    for (int k = 0; k < kPer; ++k) {
-        base[kPer * t + k] = before;
-        if (blockIdx.x == 0) a.bbase[kPer * t + k] = before;
-        before += c[k];
-    }
-    if (blockIdx.x == 0 && t == kBucketBlock - 1) a.bbase[kTailBuckets] = before;
-    __syncthreads();
-    for (unsigned i = first + t; i < n; i += gridDim.x * kBucketBlock) {
-        const uint64_t key = a.key[i];
-        const unsigned pos = base[tail_bucket(key, a.tri_bits, a.bscale)] + a.slot[i];
-        a.bkey[pos] = key;
-        a.bidx[pos] = i;
-    }
+// what any block of the cluster wrote before is visible to all of them after
+__device__ __forceinline__ void cluster_step() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
 // whether the point with weights (u, v) lies inside its triangle (feature_of's code 0)
@@ -1098,7 +1064,7 @@ __device__ __forceinline__ bool inside(double u, double v, double tau) {
 
 // true when an earlier record of the sorted list finds the same point on the
 // same features (k_dedup_flags' rule)
-__device__ __noinline__ bool tail_duplicate(const TailArgs &a, const tms_hit &h, uint64_t key) {
+__device__ __noinline__ bool tail_duplicate(const TailArgs &a, const uint32_t *base, const tms_hit &h, uint64_t key) {
     const int2 pr = a.pairs[h.pair];
     const MeshDev &ma = a.meshes[pr.x], &mb = a.meshes[pr.y];
     uint32_t incA[6], incB[6], t1[6], t2[6];
@@ -1111,9 +1077,9 @@ __device__ __noinline__ bool tail_duplicate(const TailArgs &a, const tms_hit &h,
                                 (uint64_t)incB[q];
             if (k2 >= key) continue;
             const unsigned b = tail_bucket(k2, a.tri_bits, a.bscale);
-            for (uint32_t e = a.bbase[b]; e < a.bbase[b + 1]; ++e) {
-                if (a.bkey[e] != k2) continue;
-                const tms_hit &o = a.raw[a.bidx[e]];
+            for (uint32_t e = base[b]; e < base[b + 1]; ++e) {
+                if (__ldcg(a.bkey + e) != k2) continue;
+                const tms_hit &o = a.raw[__ldcg(a.bidx + e)];
                 if (feature_of(ma, o.triA, o.a, o.b, a.tau, t1, n1) == fA &&
                     feature_of(mb, o.triB, o.c, o.d, a.tau, t2, n2) == fB)
                     return true;
@@ -1123,52 +1089,105 @@ __device__ __noinline__ bool tail_duplicate(const TailArgs &a, const tms_hit &h,
     return false;
 }
 
-constexpr int kRankBlock = 128;
-__global__ void __launch_bounds__(kRankBlock) k_tail_rank(TailArgs a) {
+constexpr int kTailBlock = 1024, kTailCluster = 16;
+__global__ void __launch_bounds__(kTailBlock) k_tail(TailArgs a) {
+    constexpr int kPer = kTailBuckets / kTailBlock;
+    constexpr unsigned kThreads = kTailBlock * kTailCluster;
+    static_assert(kPer == 8, "two 16-byte loads a thread");
+    __shared__ uint32_t base[kTailBuckets + 1];     // each bucket's first place
+    __shared__ uint32_t wsum[kTailBlock / 32];
     unsigned n;
-    if (!tail_count(a, n)) return;
-    for (unsigned e = blockIdx.x * kRankBlock + threadIdx.x; e < n; e += gridDim.x * kRankBlock) {
-        const uint64_t key = a.bkey[e];
-        const uint32_t idx = a.bidx[e];
+    if (!tail_count(a, n)) return;                  // (every block of the cluster alike)
+    const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const unsigned tid = blockIdx.x * kTailBlock + t;
+    {
+        const uint4 lo = reinterpret_cast<const uint4 *>(a.tail)[2 * t], hi = reinterpret_cast<const uint4 *>(a.tail)[2 * t + 1];
+        const uint32_t c[kPer] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+        uint32_t sum = 0;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) sum += c[k];
+        uint32_t incl = sum;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, incl, off);
+            if (lane >= off) incl += y;
+        }
+        if (lane == 31) wsum[warp] = incl;
+        __syncthreads();
+        uint32_t before = __reduce_add_sync(FULL, lane < warp ? wsum[lane] : 0u) + incl - sum;
+#pragma unroll
+        for (int k = 0; k < kPer; ++k) {
+            base[kPer * t + k] = before;
+            before += c[k];
+        }
+        if (t == kTailBlock - 1) base[kTailBuckets] = before;
+        __syncthreads();
+    }
+    for (unsigned i = tid; i < n; i += kThreads) {
+        const uint64_t key = a.key[i];
+        const unsigned pos = base[tail_bucket(key, a.tri_bits, a.bscale)] + a.slot[i];
+        a.bkey[pos] = key;
+        a.bidx[pos] = i;
+    }
+    cluster_step();
+    for (unsigned e = tid; e < n; e += kThreads) {
+        const uint64_t key = __ldcg(a.bkey + e);
+        const uint32_t idx = __ldcg(a.bidx + e);
         const unsigned b = tail_bucket(key, a.tri_bits, a.bscale);
-        const uint32_t lo = a.bbase[b], hi = a.bbase[b + 1];
+        const uint32_t lo = base[b], hi = base[b + 1];
         uint32_t rank = lo;
-        for (uint32_t j = lo; j < hi; ++j) rank += a.bkey[j] < key;
+        for (uint32_t j = lo; j < hi; ++j) rank += __ldcg(a.bkey + j) < key;
         const tms_hit &h = a.raw[idx];
         const bool shared = !(inside(h.a, h.b, a.tau) && inside(h.c, h.d, a.tau));
-        if (shared && tail_duplicate(a, h, key)) {
+        if (shared && tail_duplicate(a, base, h, key)) {
             atomicOr(a.tail + kTailBuckets + (rank >> 5), 1u << (rank & 31));
             atomicAdd(&a.ctr->dropped, 1u);
         }
         a.skey[rank] = key;
         a.order[rank] = idx | (shared ? 0x80000000u : 0u);
     }
-}
-
-// eight lanes a record, 16 bytes each
-__global__ void __launch_bounds__(256) k_tail_out(TailArgs a) {
-    unsigned n;
-    if (!tail_count(a, n)) return;
+    cluster_step();
+    // eight lanes a record, 16 bytes each
     const uint32_t *drop = a.tail + kTailBuckets;
-    const unsigned dropped = a.ctr->dropped;
-    const unsigned tid = blockIdx.x * 256 + threadIdx.x, l = tid & 7;
+    const unsigned dropped = __ldcg(&a.ctr->dropped), l = tid & 7;
     // records dropped before rank r, counted by the record's eight lanes (every
     // lane of the warp calls it together)
     auto before = [&](unsigned r) {
         if (dropped == 0) return 0u;
         unsigned s = 0;
-        for (unsigned w = l; w < (r >> 5); w += 8) s += __popc(drop[w]);
+        for (unsigned w = l; w < (r >> 5); w += 8) s += __popc(__ldcg(drop + w));
         s += __shfl_xor_sync(FULL, s, 1);
         s += __shfl_xor_sync(FULL, s, 2);
         s += __shfl_xor_sync(FULL, s, 4);
-        return s + ((r & 31) ? __popc(drop[r >> 5] & ((1u << (r & 31)) - 1u)) : 0);
+        return s + ((r & 31) ? __popc(__ldcg(drop + (r >> 5)) & ((1u << (r & 31)) - 1u)) : 0);
     };
-    const unsigned lanes = gridDim.x * 256;
-    for (unsigned g0 = tid & ~31u; g0 < 8 * n; g0 += lanes) {
-        const unsigned r = (g0 + (tid & 31)) >> 3;
+    if (dropped == 0) {
+        // every record is kept, in its rank's place: four of them a turn
+        const unsigned m = (unsigned)(n < a.out_cap ? n : a.out_cap);
+        for (unsigned r0 = tid >> 3; r0 < m; r0 += kThreads / 2) {
+            uint32_t o[4];
+            uint4 v[4];
+#pragma unroll
+            for (unsigned k = 0; k < 4; ++k) {
+                const unsigned r = r0 + k * (kThreads / 8);
+                o[k] = r < m ? __ldcg(a.order + r) : 0u;
+            }
+#pragma unroll
+            for (unsigned k = 0; k < 4; ++k)
+                if (r0 + k * (kThreads / 8) < m) v[k] = reinterpret_cast<const uint4 *>(a.raw + (o[k] & 0x7FFFFFFFu))[l];
+#pragma unroll
+            for (unsigned k = 0; k < 4; ++k) {
+                const unsigned r = r0 + k * (kThreads / 8);
+                if (l == 0 && (o[k] >> 31)) v[k].w |= 2u;        // flags
+                if (r < m) reinterpret_cast<uint4 *>(a.out + r)[l] = v[k];
+            }
+        }
+    }
+    for (unsigned g0 = tid & ~31u; dropped != 0 && g0 < 8 * n; g0 += kThreads) {
+        const unsigned r = (g0 + lane) >> 3;
         const unsigned pos = r - before(r < n ? r : 0);
-        if (r >= n || ((drop[r >> 5] >> (r & 31)) & 1u)) continue;
-        const uint32_t o = a.order[r];
+        if (r >= n || ((__ldcg(drop + (r >> 5)) >> (r & 31)) & 1u)) continue;
+        const uint32_t o = __ldcg(a.order + r);
         uint4 v = reinterpret_cast<const uint4 *>(a.raw + (o & 0x7FFFFFFFu))[l];
         if (l == 0 && (o >> 31)) v.w |= 2u;        // flags
         if (pos < a.out_cap) reinterpret_cast<uint4 *>(a.out + pos)[l] = v;
@@ -1176,14 +1195,14 @@ __global__ void __launch_bounds__(256) k_tail_out(TailArgs a) {
     if (tid == 0) a.ctr->out = n - dropped;
     // offsets: the records kept of earlier pairs, one pair per eight lanes
     if (a.offsets) {
-        for (unsigned g0 = tid & ~31u; g0 < 8u * (a.n_pairs + 1); g0 += lanes) {
-            const unsigned p = (g0 + (tid & 31)) >> 3;
+        for (unsigned g0 = tid & ~31u; g0 < 8u * (a.n_pairs + 1); g0 += kThreads) {
+            const unsigned p = (g0 + lane) >> 3;
             const uint64_t k = (uint64_t)p << (2 * a.tri_bits);
             unsigned lo = 0, hi = n;
             if (p >= (unsigned)a.n_pairs) lo = n;
             while (lo < hi) {
                 const unsigned mid = (lo + hi) >> 1;
-                if (a.skey[mid] < k) lo = mid + 1; else hi = mid;
+                if (__ldcg(a.skey + mid) < k) lo = mid + 1; else hi = mid;
             }
             const unsigned d = before(lo);
             if (l == 0 && p <= (unsigned)a.n_pairs) a.offsets[p] = (long long)(lo - d);
@@ -1305,10 +1324,23 @@ void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st) {
                                                             a.n_pairs, a.tri_bits, a.offsets);
 }
 
-void launch_tail(const TailArgs &a, int sms, cudaStream_t st) {
-    k_tail_bucket<<<kTailMax / kBucketBlock, kBucketBlock, 0, st>>>(a);
-    k_tail_rank<<<kTailMax / kRankBlock, kRankBlock, 0, st>>>(a);
-    k_tail_out<<<2 * sms, 256, 0, st>>>(a);
+// (a cluster of sixteen is above the size that every device has to take)
+cudaError_t configure_tail() {
+    return cudaFuncSetAttribute(k_tail, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+}
+
+void launch_tail(const TailArgs &a, cudaStream_t st) {
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = kTailCluster;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(kTailCluster);
+    c.blockDim = dim3(kTailBlock);
+    c.stream = st;
+    c.attrs = &at;
+    c.numAttrs = 1;
+    cudaLaunchKernelEx(&c, k_tail, a);
 }
 
 void launch_adjoint(const AdjointArgs &a, cudaStream_t st) {
