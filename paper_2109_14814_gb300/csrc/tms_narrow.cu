@@ -295,31 +295,6 @@ __device__ __forceinline__ SplitVec column_vec(const float (&A)[4][4], int j, fl
     return r;
 }
 
-// p - q from the coordinates rounded down, fp = f32_rd(p), fq = f32_rd(q), alone:
-// |p - fp| <= 2u |fp| + 2^-126 (one FP32 place; 2^-126 below the normal range), so
-// t = fl(fp - fq) has |t - (p - q)| <= u |t| / (1 - u) + 2u (|fp| + |fq|) + 2^-125,
-// bounded with margin; a coordinate of 2^128 or more is rounded down to FLT_MAX or
-// -inf, which says nothing about it.  Looser than the
-// FP64 difference rounded to FP32 by about |fp| / |p - q|, which the quad-level test
-// absorbs except for near-misses far below a face's size.
-__device__ __forceinline__ SplitVec lo_vec(const float4 &P, const float4 &Q) {
-    const float u = 5.9604645e-08f;
-    SplitVec r;
-    float tm = 0.0f, hm = 0.0f;
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-        const float fp = comp(P, c), fq = comp(Q, c);
-        const float t = fp - fq;
-        r.v[c] = t;
-        tm = fmaxf(tm, fabsf(t));
-        hm = fmaxf(hm, fabsf(fp) + fabsf(fq));
-    }
-    r.E = ((1.001f * u) * tm + (2.001f * u) * hm) * 1.001f + 3e-38f;
-    if (!(hm < 3.4e38f)) r.E = __int_as_float(0x7f800000);
-    r.M = tm;
-    return r;
-}
-
 // a + b of two vectors with bounds
 __device__ __forceinline__ SplitVec add_vec(const SplitVec &a, const SplitVec &b) {
     const float u = 5.9604645e-08f;
@@ -333,16 +308,6 @@ __device__ __forceinline__ SplitVec add_vec(const SplitVec &a, const SplitVec &b
     r.E = (a.E + b.E + u * vm) * 1.001f;
     r.M = vm;
     return r;
-}
-
-// Plucker coordinates (01, 02, 03, 12, 13, 23) of the plane of u and v, and one
-// bound on the error of every coordinate
-__device__ __forceinline__ void plucker(const SplitVec &a, const SplitVec &b, float m[6], float &eps) {
-    const float u = 5.9604645e-08f;
-    const int I[6] = {0, 0, 0, 1, 1, 2}, J[6] = {1, 2, 3, 2, 3, 3};
-#pragma unroll
-    for (int k = 0; k < 6; ++k) m[k] = fmaf(a.v[I[k]], b.v[J[k]], -(a.v[J[k]] * b.v[I[k]]));
-    eps = ((4.02f * u) * a.M * b.M + 2.0f * (a.E * b.M + b.E * a.M + a.E * b.E)) * 1.001f;
 }
 
 // the dual direction k (orthogonal to the plane and to axis k) from its
@@ -395,124 +360,132 @@ __device__ __forceinline__ bool separated(const float w[4], const SplitVec &e1, 
     return gap > need;
 }
 
-// Quad-level form of the separating-axis test: true when no one of the four
-// triangle pairs of the quad candidate can be an FP64 hit (fp64_reach).  A
-// triangle's vertices are among its quad's, so its projected interval lies
-// inside the quad's, and its widening (3 tau' times its length) is at most the
-// quad's.  Axes: the two longest duals of each quad's first triangle.  Every
-// triangle's edges are differences of the quad's vertices (|A_ij| <= 2 max of
-// the edge vectors below), and every offset y2 - x2 is r0 plus at most the
-// vectors to each quad's far vertex.
+// Quad-level form of the separating-axis test: no one of the four triangle pairs of the
+// quad candidate can be an FP64 hit (fp64_reach).  A triangle's vertices are among its
+// quad's, so its projected interval lies inside the quad's, and its widening (3 tau' times
+// its length) is at most the quad's.  Every triangle's edges are differences of the quad's
+// vertices (|A_ij| <= 2 max of the edge vectors below), and every offset y2 - x2 is r0 plus
+// at most the vectors to each quad's far vertex.
 // (With triangle faces the fourth vertex repeats the third.)
-// One axis of the quad-level test: A's vertices at 0, a1, a2, a3 and B's at r0,
-// r0 + b1, r0 + b2, r0 + b3 (all relative to A's v0) projected on w, each with
-// its rounding and input error; true when the widened intervals are further
-// apart than |w|_1 reach.
-__device__ __forceinline__ bool quad_gap(const float w[4], const SplitVec &a1, const SplitVec &a2,
-                                         const SplitVec &a3, const SplitVec &b1, const SplitVec &b2,
-                                         const SplitVec &b3, const SplitVec &r0, float tp, float reach) {
+//
+// Edge vectors of both quads from their first vertices and the vector between those, from
+// the vertices rounded down to FP32 alone: fp = f32_rd(p) has |p - fp| <= 2u |fp| + 2^-126
+// (one FP32 place; 2^-126 below the normal range), so t = fl(fp - fq) has |t - (p - q)| <=
+// u |t| / (1 - u) + 2u (|fp| + |fq|) + 2^-125.  One bound for all: with the largest |t|
+// among the edges, M, and in r, R, and the largest |fp| of the eight vertices, H; the test
+// is bound by instruction issue, and bounds for each vector of its own were a third of it.
+// Looser than the FP64 difference rounded to FP32 by about H / M, which the test absorbs
+// except for near-misses far below a face's size.
+struct QuadPair {
+    float a[3][4], b[3][4], r[4];
+    float ka, kb;       // error of a projection of A's vectors, and of B's and r, over |w|_1
+    float tp, reach;
+};
+
+__device__ __forceinline__ void quad_pair(const float4 QA[4], const float4 QB[4], float tau, QuadPair &q) {
+    const float u = 5.9604645e-08f;
+    float M = 0.0f, R = 0.0f, H = 0.0f, A3 = 0.0f, B3 = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+        const float a0 = comp(QA[0], c), b0 = comp(QB[0], c);
+        H = fmaxf(H, fmaxf(fabsf(a0), fabsf(b0)));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float ak = comp(QA[k + 1], c), bk = comp(QB[k + 1], c);
+            q.a[k][c] = ak - a0;
+            q.b[k][c] = bk - b0;
+            H = fmaxf(H, fmaxf(fabsf(ak), fabsf(bk)));
+        }
+        M = fmaxf(M, fmaxf(fmaxf(fabsf(q.a[0][c]), fabsf(q.a[1][c])), fmaxf(fabsf(q.b[0][c]), fabsf(q.b[1][c]))));
+        A3 = fmaxf(A3, fabsf(q.a[2][c]));
+        B3 = fmaxf(B3, fabsf(q.b[2][c]));
+        q.r[c] = b0 - a0;
+        R = fmaxf(R, fabsf(q.r[c]));
+    }
+    M = fmaxf(M, fmaxf(A3, B3));
+    // (a coordinate of 2^128 or more is rounded down to FLT_MAX or -inf, which says nothing
+    // about it)
+    const float inf = __int_as_float(0x7f800000);
+    const float h = H < 1.7e38f ? (4.003f * u) * H + 3e-38f : inf;
+    const float E = fmaf(1.002f * u, M, h), Er = fmaf(1.002f * u, R, h);
+    q.ka = fmaf(4.01f * u, M, E) * 1.0001f;
+    q.kb = q.ka + fmaf(4.01f * u, R, Er) * 1.0001f;
+    q.reach = fp64_reach(2.0f * (M + E) * 1.001f, ((R + Er) + (A3 + E) + (B3 + E)) * 1.001f, tau);
+    q.tp = widen3(tau);
+}
+
+// One axis of the quad-level test: A's vertices at 0, a1, a2, a3 and B's at r, r + b1,
+// r + b2, r + b3 (all relative to A's v0) projected on w, each with its rounding and input
+// error (|fl(w.v) - w.v_exact| <= |w|_1 (4.01 u M_v + E_v)); true when the widened intervals
+// are further apart than |w|_1 reach.
+__device__ __forceinline__ float dotv(const float w[4], const float v[4]) {
+    return fmaf(w[3], v[3], fmaf(w[2], v[2], fmaf(w[1], v[1], w[0] * v[0])));
+}
+__device__ __forceinline__ bool quad_gap(const float w[4], const QuadPair &q) {
     const float u = 5.9604645e-08f;
     const float w1 = fabsf(w[0]) + fabsf(w[1]) + fabsf(w[2]) + fabsf(w[3]);
-    const float p1 = dot4(w, a1), p2 = dot4(w, a2), p3 = dot4(w, a3);
-    const float ea = w1 * fmaxf(fmaxf(fmaf(4.01f * u, a1.M, a1.E), fmaf(4.01f * u, a2.M, a2.E)),
-                                fmaf(4.01f * u, a3.M, a3.E));
-    const float q0 = dot4(w, r0);
-    const float s1 = q0 + dot4(w, b1), s2 = q0 + dot4(w, b2), s3 = q0 + dot4(w, b3);
-    const float eb = w1 * (fmaf(4.01f * u, r0.M, r0.E) +
-                           fmaxf(fmaxf(fmaf(4.01f * u, b1.M, b1.E), fmaf(4.01f * u, b2.M, b2.E)),
-                                 fmaf(4.01f * u, b3.M, b3.E))) +
-                     u * fmaxf(fmaxf(fabsf(s1), fabsf(s2)), fabsf(s3));
+    const float p1 = dotv(w, q.a[0]), p2 = dotv(w, q.a[1]), p3 = dotv(w, q.a[2]);
+    const float q0 = dotv(w, q.r);
+    const float s1 = q0 + dotv(w, q.b[0]), s2 = q0 + dotv(w, q.b[1]), s3 = q0 + dotv(w, q.b[2]);
     const float xl = fminf(fminf(0.0f, p1), fminf(p2, p3)), xh = fmaxf(fmaxf(0.0f, p1), fmaxf(p2, p3));
     const float yl = fminf(fminf(q0, s1), fminf(s2, s3)), yh = fmaxf(fmaxf(q0, s1), fmaxf(s2, s3));
-    const float DX = (xh - xl) + 2.0f * ea, DY = (yh - yl) + 2.0f * eb;
-    const float need = (tp * (DX + DY) + w1 * reach + ea + eb) * 1.001f;
+    // u |s| for the sums: at most u times the larger end
+    const float err = fmaf(u, fmaxf(fabsf(yl), fabsf(yh)), w1 * (q.ka + q.kb));
+    const float need = (q.tp * ((xh - xl) + (yh - yl) + 2.0f * err) + w1 * q.reach + err) * 1.001f;
     const float gap = fmaxf(yl - xh, xl - yh) * (1.0f - 4.0f * u);
     return gap > need;
 }
 
-// the vector orthogonal to a, b and c in R^4 (cofactor expansion of the 4 x 4
-// determinant with rows (x, a, b, c))
-__device__ __forceinline__ float det3v(float a0, float a1, float a2, float b0, float b1, float b2,
-                                       float c0, float c1, float c2) {
-    return a0 * (b1 * c2 - b2 * c1) - a1 * (b0 * c2 - b2 * c0) + a2 * (b0 * c1 - b1 * c0);
+// Plucker coordinates (01, 02, 03, 12, 13, 23) of the plane of a and b, and the vector
+// orthogonal to that plane and to v (the cofactors of x in det(x, a, b, v))
+__device__ __forceinline__ void minors(const float a[4], const float b[4], float m[6]) {
+    const int I[6] = {0, 0, 0, 1, 1, 2}, J[6] = {1, 2, 3, 2, 3, 3};
+#pragma unroll
+    for (int k = 0; k < 6; ++k) m[k] = fmaf(a[I[k]], b[J[k]], -(a[J[k]] * b[I[k]]));
 }
-__device__ __forceinline__ void cross4v(const float a[4], const float b[4], const float c[4], float x[4]) {
-    x[0] = det3v(a[1], a[2], a[3], b[1], b[2], b[3], c[1], c[2], c[3]);
-    x[1] = -det3v(a[0], a[2], a[3], b[0], b[2], b[3], c[0], c[2], c[3]);
-    x[2] = det3v(a[0], a[1], a[3], b[0], b[1], b[3], c[0], c[1], c[3]);
-    x[3] = -det3v(a[0], a[1], a[2], b[0], b[1], b[2], c[0], c[1], c[2]);
+__device__ __forceinline__ void orthogonal(const float m[6], const float v[4], float w[4]) {
+    w[0] = fmaf(v[3], m[3], fmaf(v[1], m[5], -(v[2] * m[4])));
+    w[1] = fmaf(-v[3], m[1], fmaf(v[2], m[2], -(v[0] * m[5])));
+    w[2] = fmaf(v[3], m[0], fmaf(v[0], m[4], -(v[1] * m[2])));
+    w[3] = fmaf(-v[2], m[0], fmaf(v[1], m[1], -(v[0] * m[3])));
 }
 
-// the quad-level test on the edge vectors of both quads relative to v0 of A
-__device__ __forceinline__ bool quad_sat_vectors(const SplitVec &a1, const SplitVec &a2, const SplitVec &a3,
-                                                 const SplitVec &b1, const SplitVec &b2, const SplitVec &b3,
-                                                 const SplitVec &r0, float tau) {
-    float mA1[6], mB1[6], epsA1, epsB1;
-    plucker(a1, a2, mA1, epsA1);
-    plucker(b1, b2, mB1, epsB1);
-    const float amax = 2.0f * fmaxf(fmaxf(fmaxf(a1.M + a1.E, a2.M + a2.E), fmaxf(a3.M + a3.E, b1.M + b1.E)),
-                                    fmaxf(b2.M + b2.E, b3.M + b3.E));
-    const float rmax = (r0.M + r0.E) + (a3.M + a3.E) + (b3.M + b3.E);
-    const float reach = fp64_reach(amax * 1.001f, rmax * 1.001f, tau);
-    const float tp = widen3(tau);
+// Directions: FIRST: the mixed ones orthogonal to A's first-triangle edges a1, a2 and B's
+// b1, and to a1, a2, b2; else those to b1, b2, a1 and to b1, b2, a2 (both quads are thin
+// along each when their planes share a direction), then the two longest duals of each
+// quad's first triangle.  Any direction serves (the bounds hold for the FP32 w as
+// computed), so w is not normalised.  A candidate it cannot clear goes on to the tests of
+// its triangle pairs.
+template <bool FIRST>
+__device__ __forceinline__ bool quad_reject(const float4 QA[4], const float4 QB[4], float tau) {
+    QuadPair q;
+    quad_pair(QA, QB, tau, q);
+    float mA[6], mB[6], w[4];
+    minors(q.a[0], q.a[1], mA);
+    if (FIRST) {
+        orthogonal(mA, q.b[0], w);
+        if (quad_gap(w, q)) return true;
+        orthogonal(mA, q.b[1], w);
+        return quad_gap(w, q);
+    }
+    minors(q.b[0], q.b[1], mB);
+    orthogonal(mB, q.a[0], w);
+    if (quad_gap(w, q)) return true;
+    orthogonal(mB, q.a[1], w);
+    if (quad_gap(w, q)) return true;
     int kA1, kA2, kB1, kB2;
-    top2_duals(mA1, kA1, kA2);
-    top2_duals(mB1, kB1, kB2);
+    top2_duals(mA, kA1, kA2);
+    top2_duals(mB, kB1, kB2);
 #pragma unroll 1
     for (int ax = 0; ax < 4; ++ax) {
-        float m[6], w[4];
+        float m[6];
 #pragma unroll
-        for (int k = 0; k < 6; ++k) m[k] = ax < 2 ? mA1[k] : mB1[k];
+        for (int k = 0; k < 6; ++k) m[k] = ax < 2 ? mA[k] : mB[k];
         dual_dir(m, ax == 0 ? kA1 : (ax == 1 ? kA2 : (ax == 2 ? kB1 : kB2)), w);
-        if (quad_gap(w, a1, a2, a3, b1, b2, b3, r0, tp, reach)) return true;
+        if (quad_gap(w, q)) return true;
     }
     return false;
 }
-
-// The quad-level test from the quads' vertices rounded down to FP32 alone (lo_vec
-// bounds).  Directions: the mixed ones
-// MLO..MHI-1 -- 0: orthogonal to A's first-triangle edges a1, a2 and B's b1,
-// 1: to a1, a2, b2, 2: to b1, b2, a1, 3: to b1, b2, a2 (both quads thin along
-// each when their planes share a direction) -- then, with DUALS, the dual axes
-// of quad_sat_vectors.  Any direction serves (the bounds hold for the FP32 w as
-// computed), so w is not normalised.  A candidate it cannot clear goes on to
-// the tests of its triangle pairs.
-template <int MLO, int MHI, bool DUALS>
-__device__ __forceinline__ bool quad_reject_lo(const float4 QA[4], const float4 QB[4], float tau) {
-    const SplitVec a1 = lo_vec(QA[1], QA[0]), a2 = lo_vec(QA[2], QA[0]);
-    const SplitVec a3 = lo_vec(QA[3], QA[0]);
-    const SplitVec b1 = lo_vec(QB[1], QB[0]), b2 = lo_vec(QB[2], QB[0]);
-    const SplitVec b3 = lo_vec(QB[3], QB[0]);
-    const SplitVec r0 = lo_vec(QB[0], QA[0]);
-    const float amax = 2.0f * fmaxf(fmaxf(fmaxf(a1.M + a1.E, a2.M + a2.E), fmaxf(a3.M + a3.E, b1.M + b1.E)),
-                                    fmaxf(b2.M + b2.E, b3.M + b3.E));
-    const float rmax = (r0.M + r0.E) + (a3.M + a3.E) + (b3.M + b3.E);
-    const float reach = fp64_reach(amax * 1.001f, rmax * 1.001f, tau);
-    const float tp = widen3(tau);
-    float w[4];
-    if (MLO <= 0 && 0 < MHI) {
-        cross4v(a1.v, a2.v, b1.v, w);
-        if (quad_gap(w, a1, a2, a3, b1, b2, b3, r0, tp, reach)) return true;
-    }
-    if (MLO <= 1 && 1 < MHI) {
-        cross4v(a1.v, a2.v, b2.v, w);
-        if (quad_gap(w, a1, a2, a3, b1, b2, b3, r0, tp, reach)) return true;
-    }
-    if (MLO <= 2 && 2 < MHI) {
-        cross4v(b1.v, b2.v, a1.v, w);
-        if (quad_gap(w, a1, a2, a3, b1, b2, b3, r0, tp, reach)) return true;
-    }
-    if (MLO <= 3 && 3 < MHI) {
-        cross4v(b1.v, b2.v, a2.v, w);
-        if (quad_gap(w, a1, a2, a3, b1, b2, b3, r0, tp, reach)) return true;
-    }
-    if (DUALS) return quad_sat_vectors(a1, a2, a3, b1, b2, b3, r0, tau);
-    return false;
-}
-
-// the mixed directions every candidate takes in k_quad_filter's first stage; the
-// rest, and the dual axes, only the candidates these leave
-constexpr int kQuadFirstAxes = 2;
 
 // true when the separating-axis test proves that the FP64 solve of the pair
 // reports no hit (fp64_reach)
@@ -529,9 +502,9 @@ __device__ __forceinline__ bool fp32_sat_reject(const float (&A)[4][4], const fl
     }
     r.E = kEntry * r.M + kTiny;
     const SplitVec s1 = add_vec(r, f1), s3 = add_vec(r, f2);
-    float mE[6], mF[6], epsE, epsF;
-    plucker(e1, e2, mE, epsE);
-    plucker(f1, f2, mF, epsF);
+    float mE[6], mF[6];
+    minors(e1.v, e2.v, mE);
+    minors(f1.v, f2.v, mF);
     const float amax = fmaxf(fmaxf(e1.M + e1.E, e2.M + e2.E), fmaxf(f1.M + f1.E, f2.M + f2.E));
     const float reach = fp64_reach(amax * 1.001f, (r.M + r.E) * 1.001f, tau);
     const float tp = widen3(tau);
@@ -727,12 +700,16 @@ __device__ __forceinline__ unsigned long long hit_place(const NarrowArgs &a, boo
 // Stage 1a: the quad-level separating-axis test of every candidate (quads, or triangles)
 // on its quads' vertices rounded down to FP32, the first mixed directions
 // first; the candidates they leave gather in a per-warp queue, and every 32 of
-// them take the other directions with all lanes busy; those still not cleared
-// are listed for k_narrow_pairs.
+// them take the other directions with all lanes busy, what is left of the block's queues
+// at the end together; those still not cleared are listed for k_narrow_pairs.  Bound by
+// instruction issue and the gathers.  One wave of blocks: with four, a warp had one or two
+// turns of 32 candidates and then a queue of about five to work off with 27 lanes idle
+// (4096 x 512, 700,000 candidates: 41.6 us and 19.0 M instructions, so 26.2 and 11.7).
 constexpr int kQuadWarps = 8;
 template <int FACE>
 __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a) {
     __shared__ uint32_t s_q[kQuadWarps][64];
+    __shared__ unsigned s_left[kQuadWarps];
     if (a.ctr->cand > a.cand_cap) return;
     const unsigned long long n = a.ctr->cand;
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
@@ -741,18 +718,18 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
     const float tauf = __double2float_ru(a.tau);
     unsigned long long n_quad = 0;
     unsigned qn = 0;                                 // queued candidates (warp-uniform)
-    // the mixed directions for queue items [base, base + cnt)
-    auto drain = [&](unsigned base, unsigned cnt) {
+    // the other directions for cnt queued candidates
+    auto drain = [&](const uint32_t *q, unsigned cnt) {
         bool keep = false;
         uint32_t g = 0;
         if ((unsigned)lane < cnt) {
-            g = s_q[warp][base + lane];
+            g = q[lane];
             const Cand cd = a.cand[g];
             const int2 pr = a.pairs[cd.pair];
             float4 QA[4], QB[4];
             gather_face_lo<FACE>(a.meshes[pr.x], cd.faceA, QA);
             gather_face_lo<FACE>(a.meshes[pr.y], cd.faceB, QB);
-            keep = !quad_reject_lo<kQuadFirstAxes, 4, true>(QA, QB, tauf);
+            keep = !quad_reject<false>(QA, QB, tauf);
         }
         const unsigned long long pos = warp_append(&a.ctr->qkeep, keep, FULL);
         if (keep && pos < a.qsurv_cap) a.qsurv[pos] = g;
@@ -768,7 +745,7 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
             float4 QA[4], QB[4];
             gather_face_lo<FACE>(a.meshes[pr.x], cd.faceA, QA);
             gather_face_lo<FACE>(a.meshes[pr.y], cd.faceB, QB);
-            need = !quad_reject_lo<0, kQuadFirstAxes, false>(QA, QB, tauf);
+            need = !quad_reject<true>(QA, QB, tauf);
         }
         n_quad += __popc(__ballot_sync(FULL, valid));
         const uint32_t want = __ballot_sync(FULL, need);
@@ -777,14 +754,25 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
         __syncwarp();
         if (qn >= 32) {
             qn -= 32;
-            drain(qn, 32);
+            drain(s_q[warp] + qn, 32);
             __syncwarp();
         }
     }
-    if (qn) {
-        drain(0, qn);
-        __syncwarp();
+    // what the block's warps have left, together
+    if (lane == 0) s_left[warp] = qn;
+    __syncthreads();
+    unsigned first = 0, total = 0;
+#pragma unroll
+    for (int w = 0; w < kQuadWarps; ++w) {
+        first += w < warp ? s_left[w] : 0u;
+        total += s_left[w];
     }
+    const uint32_t mine = (unsigned)lane < qn ? s_q[warp][lane] : 0u;
+    __syncthreads();
+    uint32_t *all = &s_q[0][0];
+    if ((unsigned)lane < qn) all[first + lane] = mine;
+    __syncthreads();
+    for (unsigned k = 32 * warp; k < total; k += 32 * kQuadWarps) drain(all + k, min(32u, total - k));
     if (lane == 0 && n_quad) atomicAdd(&a.ctr->quad, n_quad);
 }
 
@@ -1040,8 +1028,8 @@ __global__ void k_offsets(const uint64_t *out_keys, const unsigned long long *d_
 // six tiles is 7 us of loads, ranking and look-back, and the sort and merge took
 // 15 launches), so it is one launch of one cluster, whose barrier takes the place of
 // the launches between the steps: 16.5 us at 12,045 hits (three launches 10 + 7 + 7; a
-// cluster of eight, with one record a turn, 28), and a search of 1024 x 256 and
-// 771 x 331 vertices (157 hits) 112 -> 100 us.  The FP64 solve counts the hits into
+// cluster of eight, with one record a turn, 28), and a search of 1024 x 256 vertices
+// (157 hits) 112 -> 100 us.  The FP64 solve counts the hits into
 // buckets of increasing key; each block scans the counts for itself (32 KB from L2) and
 // lists its hits in their buckets; then compares a hit with its bucket (about one at
 // 8192 buckets; however unevenly the hits fall, at most kTailMax compares) and decides
@@ -1307,10 +1295,10 @@ void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st
         return;
     }
     if (face_level == 0) {
-        k_quad_filter<0><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
+        k_quad_filter<0><<<sms * 3, 32 * kQuadWarps, 0, st>>>(a);
         k_narrow_pairs<0><<<sms * 8, kPairBlock, 0, st>>>(a);
     } else {
-        k_quad_filter<1><<<sms * 3 * 4, 32 * kQuadWarps, 0, st>>>(a);
+        k_quad_filter<1><<<sms * 3, 32 * kQuadWarps, 0, st>>>(a);
         k_narrow_pairs<1><<<sms * 8, kPairBlock, 0, st>>>(a);
     }
 }
