@@ -250,6 +250,8 @@ struct Plan {
         ta.ctr = d_ctr; ta.raw_cap = hit_cap; ta.out = (tms_hit *)dHits;
         ta.out_cap = (unsigned long long)hitCap; ta.offsets = dOffsets; ta.n_pairs = nPairs;
         ta.tri_bits = tri_bits; ta.tau = prm.tau; ta.bscale = bscale;
+        ta.result = reinterpret_cast<const uint32_t *>(d_ctr); ta.readback = reinterpret_cast<uint32_t *>(h_ctr);
+        ta.words = (int)(kReadback / 4);
         launch_tail(ta, s);
         kernels += 1;
     }
@@ -413,13 +415,19 @@ struct Plan {
         else enqueue_short_tail(s);
         mark(14, s);
 
-        cudaMemcpyAsync(h_ctr, d_ctr, kReadback, cudaMemcpyDeviceToHost, s);
+        // (the short tail's kernel writes them itself)
+        if (long_tail) cudaMemcpyAsync(h_ctr, d_ctr, kReadback, cudaMemcpyDeviceToHost, s);
         mark(15, s);
     }
 
     tms_status run() {
-        TMS_CK(cudaEventRecord(ev_in, user));
-        TMS_CK(cudaStreamWaitEvent(st, ev_in, 0));
+        // a graph runs in the caller's stream; without one, the plan's own stream waits for
+        // the caller's and the caller's for it
+        const cudaStream_t s = prm.use_graph ? user : st;
+        if (!prm.use_graph) {
+            TMS_CK(cudaEventRecord(ev_in, user));
+            TMS_CK(cudaStreamWaitEvent(st, ev_in, 0));
+        }
         if (prm.use_graph) {
             if (!exec) {
                 cudaGraph_t g = nullptr;
@@ -440,16 +448,16 @@ struct Plan {
                     return TMS_ERR_CUDA;
                 }
             }
-            TMS_CK(cudaGraphLaunch(exec, st));
+            TMS_CK(cudaGraphLaunch(exec, s));
         } else {
             enqueue(st);
             TMS_CK(cudaGetLastError());
         }
         if (g_early.host && g_early.n > 0 && dHits)
             TMS_CK(cudaMemcpyAsync(g_early.host, dHits, (size_t)g_early.n * sizeof(tms_hit),
-                                   cudaMemcpyDeviceToHost, st));
-        TMS_CK(cudaEventRecord(ev_out, st));
-        TMS_CK(cudaStreamWaitEvent(user, ev_out, 0));
+                                   cudaMemcpyDeviceToHost, s));
+        TMS_CK(cudaEventRecord(ev_out, s));
+        if (!prm.use_graph) TMS_CK(cudaStreamWaitEvent(user, ev_out, 0));
         TMS_CK(cudaEventSynchronize(ev_out));
         if (prm.timing) {
             for (int i = 0; i < kStages; ++i) {

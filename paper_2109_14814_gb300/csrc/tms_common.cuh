@@ -684,6 +684,9 @@ struct TailArgs {
     int tri_bits;
     double tau;
     float bscale;
+    const uint32_t *result;        // the counters and the first pair's grid, words of them
+    uint32_t *readback;            // and their copy in pinned host memory
+    int words;
 };
 void launch_tail(const TailArgs &a, cudaStream_t st);
 cudaError_t configure_tail();

@@ -1040,6 +1040,12 @@ __device__ __forceinline__ bool tail_count(const TailArgs &a, unsigned &n) {
     return raw <= a.raw_cap && raw <= kTailMax;
 }
 
+// The search's counters to the host, by one block of the last kernel: a copy of their 300
+// bytes as a node of its own took the copy engine about 4 us.
+__device__ __forceinline__ void tail_readback(const TailArgs &a) {
+    for (int k = threadIdx.x; k < a.words; k += blockDim.x) a.readback[k] = __ldcg(a.result + k);
+}
+
 // what any block of the cluster wrote before is visible to all of them after
 __device__ __forceinline__ void cluster_step() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -1085,8 +1091,11 @@ __global__ void __launch_bounds__(kTailBlock) k_tail(TailArgs a) {
     __shared__ uint32_t base[kTailBuckets + 1];     // each bucket's first place
     __shared__ uint32_t wsum[kTailBlock / 32];
     unsigned n;
-    if (!tail_count(a, n)) return;                  // (every block of the cluster alike)
     const unsigned t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    if (!tail_count(a, n)) {                        // (every block of the cluster alike)
+        if (blockIdx.x == 0) tail_readback(a);
+        return;
+    }
     const unsigned tid = blockIdx.x * kTailBlock + t;
     {
         const uint4 lo = reinterpret_cast<const uint4 *>(a.tail)[2 * t], hi = reinterpret_cast<const uint4 *>(a.tail)[2 * t + 1];
@@ -1180,7 +1189,11 @@ __global__ void __launch_bounds__(kTailBlock) k_tail(TailArgs a) {
         if (l == 0 && (o >> 31)) v.w |= 2u;        // flags
         if (pos < a.out_cap) reinterpret_cast<uint4 *>(a.out + pos)[l] = v;
     }
-    if (tid == 0) a.ctr->out = n - dropped;
+    if (blockIdx.x == 0) {
+        if (t == 0) a.ctr->out = n - dropped;
+        __syncthreads();
+        tail_readback(a);
+    }
     // offsets: the records kept of earlier pairs, one pair per eight lanes
     if (a.offsets) {
         for (unsigned g0 = tid & ~31u; g0 < 8u * (a.n_pairs + 1); g0 += kThreads) {
