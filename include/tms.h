@@ -132,7 +132,8 @@ typedef struct {
                              raw-hit buffers at one record (exercises each growth
                              and its retry) */
     int block_faces;      /* bounds-pass tile width in quads (64/128/256; 0 = 128) */
-    int tile_rows;        /* bounds-pass tile height in quad rows (4 or 8; 0 = 4) */
+    int tile_rows;        /* bounds-pass tile height in quad rows (4 or 8; 0 = 4; the patch
+                             level takes 8 in mixed precision where they fill the GPU) */
     int timing;           /* 1 = record CUDA events between stages (in the graph) so
                              that tms_last_stage_ms() reports per-stage device time */
     int patch;            /* broad-phase level: 0 = the grid holds the faces

@@ -545,12 +545,13 @@ __device__ __forceinline__ void frame_write(const PatchScratch &P, float4 *out, 
 // ---------------------------------------------------------------------------
 // bounds pass
 // ---------------------------------------------------------------------------
-// Registers: 64 a thread for mixed precision (a few of the vertices in flight are
-// spilled) put twice the warps on an SM of the 100 it would take: 64 pairs of
-// meshes from 128 x 32 to 2048 x 512 vertices 960 us a search against 802 (with 80: 840,
-// with 48: 785, but one 4096 x 512 pair is 1-2% slower than with 64).
+// Registers, mixed precision: 64 a thread for tiles of 4 rows (a few of the vertices in
+// flight are spilled), 80 for those of 8: 64 pairs of meshes from 128 x 32 to 2048 x 512
+// vertices took 960 us a search with the 100 that 4 rows would take, 840 with 80, 802 with
+// 64; with 8 rows (a patch row at a time) the pass takes 398 us with 80, 411 with 64, and
+// 449 with 128 and the next patch row's loads before the current one's boxes.
 template <int PREC, int FACE, int TK>
-__global__ void __launch_bounds__(256, PREC == 1 ? 4 : 2) k_bounds_pass(FacePassArgs a) {
+__global__ void __launch_bounds__(256, PREC == 1 ? (TK == 4 ? 4 : 3) : 2) k_bounds_pass(FacePassArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     Vtx<PREC> *sv = reinterpret_cast<Vtx<PREC> *>(smem_raw);
     const int TI = blockDim.x;
@@ -570,53 +571,60 @@ __global__ void __launch_bounds__(256, PREC == 1 ? 4 : 2) k_bounds_pass(FacePass
     // the largest high word of |x| tells whether any is not finite (a test of each value
     // beside its rounding becomes an FP64 comparison)
     unsigned top = 0;
-    Vtx<PREC> own[TK + 1];             // this thread's vertex column
-    {
-        const int t = threadIdx.x;
-        double x[TK + 1][4];
-        const bool col_ok = t < cols_q;
-        const int vi = i0 + t;
+    const int t = threadIdx.x;
+    const bool col_valid = t < cols_q;
+    const int i = i0 + t;
+    // a vertex is written by the tile that owns it: rows below the tile's last
+    // (the next tile's first) and the mesh's last row
+    const bool last_rows = kq0 + rows_q == m.nqk;
+    // this thread's vertex column over a patch row: rows r0..r0 + kPatchK of the tile (the
+    // first of them, where r0 > 0, as the last of the patch row before)
+    Vtx<PREC> own[kPatchK + 1];
+    auto load_rows = [&](int r0, bool first) {
+        double x[kPatchK + 1][4];
 #pragma unroll
-        for (int r = 0; r <= TK; ++r) {
-            if (col_ok && r <= rows_q) {
-                size_t off = (size_t)(kq0 + r) * m.N + vi;
+        for (int r = 0; r <= kPatchK; ++r) {
+            if (r == 0 && !first) continue;
+            if (col_valid && r0 + r <= rows_q) {
+                const size_t off = (size_t)(kq0 + r0 + r) * m.N + i;
 #pragma unroll
                 for (int c = 0; c < 4; ++c) x[r][c] = __ldg(m.c[c] + off);
             }
         }
-        // a vertex is written by the tile that owns it: rows below the tile's last
-        // (the next tile's first) and the mesh's last row
-        const bool last_rows = kq0 + rows_q == m.nqk;
+        if (!first) own[0] = own[kPatchK];
 #pragma unroll
-        for (int r = 0; r <= TK; ++r) {
-            if (col_ok && r <= rows_q) {
+        for (int r = 0; r <= kPatchK; ++r) {
+            if (r == 0 && !first) continue;
+            if (col_valid && r0 + r <= rows_q) {
                 own[r] = to_vtx<PREC>(x[r], top);
-                sv[r * W + t] = own[r];
-                if (r < rows_q || last_rows) write_vlo(m, (size_t)(kq0 + r) * m.N + vi, own[r]);
+                sv[(r0 + r) * W + t] = own[r];
+                if (r0 + r < rows_q || last_rows) write_vlo(m, (size_t)(kq0 + r0 + r) * m.N + i, own[r]);
             }
         }
-        // the last vertex column of the tile (wraps to column 0 on a periodic mesh);
-        // it belongs to the next tile, except an open mesh's last column
-        if (t <= rows_q) {
-            int vj = i0 + cols_q;
-            if (vj == m.N) vj = 0;
-            size_t off = (size_t)(kq0 + t) * m.N + vj;
-            double y[4];
+    };
+    load_rows(0, true);
+    // the last vertex column of the tile (wraps to column 0 on a periodic mesh);
+    // it belongs to the next tile, except an open mesh's last column
+    if (t <= rows_q) {
+        int vj = i0 + cols_q;
+        if (vj == m.N) vj = 0;
+        size_t off = (size_t)(kq0 + t) * m.N + vj;
+        double y[4];
 #pragma unroll
-            for (int c = 0; c < 4; ++c) y[c] = __ldg(m.c[c] + off);
-            const Vtx<PREC> v = to_vtx<PREC>(y, top);
-            sv[t * W + cols_q] = v;
-            if (!m.periodic && vj == m.N - 1 && (t < rows_q || last_rows)) write_vlo(m, off, v);
-        }
+        for (int c = 0; c < 4; ++c) y[c] = __ldg(m.c[c] + off);
+        const Vtx<PREC> v = to_vtx<PREC>(y, top);
+        sv[t * W + cols_q] = v;
+        if (!m.periodic && vj == m.N - 1 && (t < rows_q || last_rows)) write_vlo(m, off, v);
+    }
+    if (!(FACE == 1 && a.patch)) {
+#pragma unroll
+        for (int r0 = kPatchK; r0 < TK; r0 += kPatchK) load_rows(r0, false);
     }
     __syncthreads();
 
     BoundAcc<PREC> acc;                // world bounds and widest face (face level)
     acc.init();
 
-    const int t = threadIdx.x;
-    const bool col_valid = t < cols_q;
-    const int i = i0 + t;
     if (FACE == 1 && a.patch) {
         // quad faces with patches.  A quarter (four columns by two rows of quads) is the
         // union of five vertex columns over three rows: each lane takes its own column,
@@ -626,7 +634,7 @@ __global__ void __launch_bounds__(256, PREC == 1 ? 4 : 2) k_bounds_pass(FacePass
         // the block takes part: the row loop and its shuffles are uniform.)  With a box
         // for each quad, every lane reducing whole boxes, and each coordinate's rounding
         // tested alone the kernel took 48.8 M instructions and 64 us at 4096 x 512; so
-        // 38.4 M (with 64 registers) and 53 us.
+        // 38.4 M (with 64 registers, tiles of 4 rows) and 53 us.
         static_assert(kPatchI == 8 && kPatchK == 4 && TK % kPatchK == 0, "quarters of four columns by two rows");
         typedef typename Num<PREC>::T T;
         const int j = t & 3;
@@ -637,17 +645,21 @@ __global__ void __launch_bounds__(256, PREC == 1 ? 4 : 2) k_bounds_pass(FacePass
         for (int pr = 0; pr < TK / kPatchK; ++pr) {
             const int pr0 = pr * kPatchK, rq = min(kPatchK, rows_q - pr0);
             if (rq <= 0) break;
+            if (pr > 0) {
+                load_rows(pr0, false);
+                __syncthreads();
+            }
             ColBox<PREC> upper, lower;
             upper.init();
             lower.init();
             if (col_valid) {
-                upper.add(own[pr0]);
-                upper.add(own[pr0 + 1]);
-                if (rq > 1) upper.add(own[pr0 + 2]);
+                upper.add(own[0]);
+                upper.add(own[1]);
+                if (rq > 1) upper.add(own[2]);
                 if (rq > 2) {
-                    lower.add(own[pr0 + 2]);
-                    lower.add(own[pr0 + 3]);
-                    if (rq > 3) lower.add(own[pr0 + 4]);
+                    lower.add(own[2]);
+                    lower.add(own[3]);
+                    if (rq > 3) lower.add(own[4]);
                 }
             }
             if ((t & ~3) < cols_q) {
@@ -699,11 +711,16 @@ __global__ void __launch_bounds__(256, PREC == 1 ? 4 : 2) k_bounds_pass(FacePass
                 }
                 __syncthreads();
                 const int cq = patch_lane ? min(kPatchI, cols_q - (t & ~(kPatchI - 1))) : 0;
+                // (the last patch row's vertices are still the thread's own)
+                for (int pr0 = (rows_q - 1) / kPatchK * kPatchK;; pr0 -= kPatchK) {
+                    frame_extents(sv, own, W, t, cq, pr0, min(kPatchK, rows_q - pr0),
+                                  sp[(pr0 / kPatchK) * across + t / kPatchI]);
+                    if (pr0 == 0) break;
+                    if (col_valid) {
 #pragma unroll
-                for (int pr0 = 0; pr0 < TK; pr0 += kPatchK)
-                    if (pr0 < rows_q)
-                        frame_extents(sv, own + pr0, W, t, cq, pr0, min(kPatchK, rows_q - pr0),
-                                      sp[(pr0 / kPatchK) * across + t / kPatchI]);
+                        for (int r = 0; r <= kPatchK; ++r) own[r] = sv[(pr0 - kPatchK + r) * W + t];
+                    }
+                }
                 __syncthreads();
                 for (int q = t; q < np; q += TI)
                     if ((q % across) * kPatchI < cols_q)
