@@ -545,10 +545,15 @@ __device__ __forceinline__ void fill_walk(const Coef &cf, WalkCoef &wc, int K, d
     }
 }
 
+__device__ __noinline__ double wrap_far(double v) { return fmod(v, kTwoPi); }
+
+// v modulo 2 pi in [0, 2 pi] (fmod, which leaves |v| < 2 pi as it is)
 __device__ __forceinline__ double wrap_angle(double v) {
-    double w = fmod(v, kTwoPi);
-    if (w < 0.0) w += kTwoPi;
-    else if (w == 0.0) w = 0.0;   // +0 for a -0 remainder
+    double w = v;
+    if (abs_bits(v) >= __double_as_longlong(kTwoPi)) w = wrap_far(v);
+    const long long b = __double_as_longlong(w);
+    if (b == (long long)(1ULL << 63)) w = 0.0;   // +0 for a -0 remainder
+    else if (b < 0) w += kTwoPi;
     return w;
 }
 
@@ -622,13 +627,10 @@ __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ C
     const int base = lane & ~3;
     const long long i = (long long)blockIdx.x * kSeedsPerBlock + (t >> 2);
     const bool live = i < a.n;
-    double g[4] = {0.0, 0.5, 0.0, 0.5};   // the current step's starting point
-    if (live) {
-        const double *s = a.x0 + i * a.ld;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) g[q] = s[q];
-    }
-    double p1[4] = {0.0, 0.0, 0.0, 0.0}, p2[4] = {0.0, 0.0, 0.0, 0.0};   // x_{j-1}, x_{j-2}
+    const bool angle = !(c & 1);
+    double g = angle ? 0.0 : 0.5;         // lane c's coordinate of the current step's start
+    if (live) g = a.x0[i * a.ld + c];
+    double p1 = 0.0, p2 = 0.0;            // of x_{j-1}, x_{j-2}
     bool alive = live;
     int j = 0;
     double rho_prev = nan_value();
@@ -636,10 +638,10 @@ __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ C
     double aj = a0, am1 = a0, am2 = a0;   // alpha_j, alpha_{j-1}, alpha_{j-2}
     const long long K1 = (long long)a.steps + 1;
     Solve S;
-    S.x0 = g[0];
-    S.x1 = g[1];
-    S.x2 = g[2];
-    S.x3 = g[3];
+    S.x0 = lane_val(g, base, 0);
+    S.x1 = lane_val(g, base, 1);
+    S.x2 = lane_val(g, base, 2);
+    S.x3 = lane_val(g, base, 3);
     S.code = alive ? -1 : TMS_REFINE_CONVERGED;
     S.iters = 0;
     S.k = 0;
@@ -652,35 +654,41 @@ __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ C
     while (__any_sync(kFull, alive)) {
         newton_iter<WALK>(cf, &wc, sp, cp.corrector, stop, lnlam, S, c, base);
         if (!(alive && S.code >= 0)) continue;
-        // ---- step j is done (identical on the quad's lanes; no shuffles below)
-        const double xs[4] = {wrap_angle(S.x0), S.x1, wrap_angle(S.x2), S.x3};
-        const double rho = S.rh / sqrt(S.rc2);
+        // ---- step j is done: of one quad, as a rule, with the warp's others waiting, so
+        // lane c takes coordinate c, and the square roots and divisions are taken by
+        // different lanes at once (all four on every lane made a step 250 FP64
+        // instructions, over 8 quads a third of all: 19.4 ms for 12,000 branches of 50
+        // steps; CONT_FIGURES)
+        const unsigned quad = 0xFu << base;
+        const double own = c == 0 ? S.x0 : c == 1 ? S.x1 : c == 2 ? S.x2 : S.x3;
+        const double xs = angle ? wrap_angle(own) : own;
+        const double root = sqrt(c == 3 ? S.rc2 : S.fn);
+        double moved = fabs(xs - g);
+        const double q1 = (c == 3 ? S.rh : moved) / (c == 3 ? root : kTwoPi);
+        const double rho = __shfl_sync(quad, q1, base + 3);
+        if (angle) moved = fabs(moved - kTwoPi * rint(q1));
+        long long jump = abs_bits(moved);
+        jump = max(jump, __shfl_xor_sync(quad, jump, 1));
+        jump = max(jump, __shfl_xor_sync(quad, jump, 2));
         int st = S.code;
         if (st == TMS_REFINE_CONVERGED) {
-            double jump = 0.0;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                double d = fabs(xs[q] - g[q]);
-                if (q == 0 || q == 2) d = fabs(d - kTwoPi * rint(d / kTwoPi));
-                jump = fmax(jump, d);
-            }
-            if (!(jump <= cp.max_jump)) st = TMS_CONT_JUMPED;
-            else if (!(fabs(rho) >= cp.rho_turn)) st = TMS_CONT_TURNING;
-            else if (j > 0 && (rho > 0.0) != (rho_prev > 0.0)) st = TMS_CONT_TURNING;
+            // (the thresholds are not negative, so their bits are ordered as they are)
+            const long long size = abs_bits(rho), inf = 0x7ff0000000000000LL;
+            const bool up = __double_as_longlong(rho) > 0, was_up = __double_as_longlong(rho_prev) > 0;
+            if (jump > __double_as_longlong(cp.max_jump)) st = TMS_CONT_JUMPED;
+            else if (size > inf || size < __double_as_longlong(cp.rho_turn)) st = TMS_CONT_TURNING;
+            else if (j > 0 && up != was_up) st = TMS_CONT_TURNING;
         }
         const long long o = i * K1 + j;
-        a.x[o * 4 + c] = xs[c];
+        a.x[o * 4 + c] = xs;
         if (c == 0) {
             a.status[o] = st;
             if (a.iters) a.iters[o] = S.iters;
             if (a.rho) a.rho[o] = rho;
-            if (a.fnorm) a.fnorm[o] = sqrt(S.fn);
+            if (a.fnorm) a.fnorm[o] = root;
         }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            p2[q] = p1[q];
-            p1[q] = xs[q];
-        }
+        p2 = p1;
+        p1 = xs;
         rho_prev = rho;
         if (st != TMS_REFINE_CONVERGED || j == a.steps) {
             alive = false;
@@ -702,22 +710,18 @@ __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ C
         am1 = aj;
         aj = a.alphas[j - 1];
         fill_walk<WALK>(cf, wc, sp.n_harmonics, aj, c);
-        if (j == 1) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) g[q] = p1[q];
-        } else {
-            const double ratio = (aj - am1) / (am1 - am2);
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                double d = p1[q] - p2[q];
-                if (q == 0 || q == 2) d -= kTwoPi * rint(d / kTwoPi);
-                g[q] = p1[q] + ratio * d;
-            }
+        g = p1;
+        if (j > 1) {
+            double d = p1 - p2;
+            const double q2 = (c == 1 ? aj - am1 : d) / (c == 1 ? am1 - am2 : kTwoPi);
+            const double ratio = __shfl_sync(quad, q2, base + 1);
+            if (angle) d -= kTwoPi * rint(q2);
+            g = p1 + ratio * d;
         }
-        S.x0 = g[0];
-        S.x1 = g[1];
-        S.x2 = g[2];
-        S.x3 = g[3];
+        S.x0 = __shfl_sync(quad, g, base);
+        S.x1 = __shfl_sync(quad, g, base + 1);
+        S.x2 = __shfl_sync(quad, g, base + 2);
+        S.x3 = __shfl_sync(quad, g, base + 3);
         S.code = -1;
         S.iters = 0;
         S.k = 0;
