@@ -18,7 +18,7 @@
 // them and shuffled, comparisons and sign changes are integer, and a block is one warp,
 // so that 1500 warps (12,000 seeds) load the 152 SMs evenly (blocks of four put twelve
 // on some and eight on others): 12,000 seeds 1476 -> 866 us, 12,000 branches of 50 steps
-// 31.5 -> 19.4 ms, the results the same but for roundings in a few of 10,000.
+// 31.5 -> 17.9 ms, the results the same but for roundings in a few of 10,000.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -655,10 +655,9 @@ __global__ void __launch_bounds__(kThreads) k_continue(const __grid_constant__ C
         newton_iter<WALK>(cf, &wc, sp, cp.corrector, stop, lnlam, S, c, base);
         if (!(alive && S.code >= 0)) continue;
         // ---- step j is done: of one quad, as a rule, with the warp's others waiting, so
-        // lane c takes coordinate c, and the square roots and divisions are taken by
-        // different lanes at once (all four on every lane made a step 250 FP64
-        // instructions, over 8 quads a third of all: 19.4 ms for 12,000 branches of 50
-        // steps; CONT_FIGURES)
+        // lane c takes coordinate c, and the square roots and quotients are taken by
+        // different lanes at once (all of them on every lane: 19.4 ms for 12,000 branches
+        // of 50 steps; so 17.9)
         const unsigned quad = 0xFu << base;
         const double own = c == 0 ? S.x0 : c == 1 ? S.x1 : c == 2 ? S.x2 : S.x3;
         const double xs = angle ? wrap_angle(own) : own;
