@@ -69,31 +69,20 @@ FP64_SOLVE_FLOPS = 110
 
 # the broad phase's stages (tms_last_stage_ms labels), and per reported stage the
 # labels it sums and its kernels (the keys of profiles/traffic.json)
-BROAD_STAGES = ("init", "face_bounds", "grid_params", "bitmap_clear", "face_mark_A", "face_probe_B",
-                "face_probe_A", "group_count", "group_cells", "emit", "patch_quads")
+BROAD_STAGES = ("face_bounds", "emit", "patch_quads")
 STAGE_PARTS = {
     "face_bounds": ("face_bounds",),
-    "face_mark": ("face_mark_A",),
-    "face_probe": ("face_probe_B", "face_probe_A"),
-    "group_count": ("group_count",),
-    "group_cells": ("group_cells",),
     "emit": ("emit", "patch_quads"),
     "narrow": ("narrow",),
     "sort_merge": ("sort_hits", "merge_output"),
 }
 STAGE_KERNELS = {
     "face_bounds": "tms::k_bounds_pass",
-    "face_mark": "tms::k_cell_pass<MARK>",
-    "face_probe": "tms::k_cell_pass<EMIT_ALL>",
-    "group_count": "tms::k_group_count",
-    "group_cells": "tms::k_cells_* + k_group_scatter",
-    "emit": "tms::k_emit + k_patch_quarters + k_patch_quads",
-    "narrow": "tms::k_quad_filter + k_narrow_filter + k_narrow_fp64",
-    "sort_merge": "tms::k_radix_* + k_dedup_*",
+    "emit": "tms::k_tree_* + k_patch_quarters + k_patch_quads",
+    "narrow": "tms::k_quad_filter + k_narrow_filter",
+    "sort_merge": "tms::k_tail",
 }
-BROAD_KERNELS = ("k_search_init", "k_bounds_pass", "k_grid_params", "k_cell_pass", "k_group_count",
-                 "k_cells_reduce", "k_cells_partials", "k_cells_down", "k_group_scatter", "k_emit",
-                 "k_patch_quarters", "k_patch_quads")
+BROAD_KERNELS = ("k_bounds_pass", "k_tree_up", "k_tree_top", "k_tree_down", "k_patch_quarters", "k_patch_quads")
 
 
 def dist_env():
@@ -152,21 +141,17 @@ def broad_traffic():
 # the device, inputs larger than L2), after three warm-up searches.  Per kernel:
 # (regex, launches per search, stage label, in the broad phase).
 TRAFFIC_KERNELS = [
-    ("k_search_init", 1, None, True),
     ("k_bounds_pass", 1, "face_bounds", True),
-    ("k_grid_params", 1, None, True),
-    ("k_cell_pass", 1, "face_probe", True),
-    ("k_group_count", 1, "group_count", True),
-    ("k_cells_reduce", 1, "group_cells", True),
-    ("k_cells_partials", 1, "group_cells", True),
-    ("k_cells_down", 1, "group_cells", True),
-    ("k_group_scatter", 1, "group_cells", True),
-    ("k_emit", 1, "emit", True),
+    ("k_tree_up", 1, "emit", True),
+    ("k_tree_top", 1, "emit", True),
+    ("k_tree_down", 2, "emit", True),
     ("k_patch_quarters", 1, "emit", True),
     ("k_patch_quads", 1, "emit", True),
     ("k_quad_filter", 1, "narrow", False),
     ("k_narrow_filter", 1, "narrow", False),
-    ("k_narrow_fp64", 1, "narrow", False),
+    ("k_tail", 1, "sort_merge", False),
+    # face level only (the grid's cell passes)
+    ("k_cell_pass", 3, None, True),
 ]
 TRAFFIC_METRICS = "dram__bytes_read.sum,dram__bytes_write.sum,gpu__time_duration.sum"
 TRAFFIC_BENCH = "python bench.py --steps 1 --warmup 3 --no-e2e --no-cpu --workload-cache {cache}"
@@ -237,7 +222,7 @@ def write_traffic(csv_dir: str) -> dict:
 
 
 # the files that hold the search's kernels and their launch sequence
-SEARCH_SOURCES = ("tms_common.cuh", "tms_faces.cu", "tms_group.cu", "tms_pairs.cu",
+SEARCH_SOURCES = ("tms_common.cuh", "tms_faces.cu", "tms_tree.cu", "tms_pairs.cu",
                   "tms_narrow.cu", "tms_sort.cu", "tms_api.cu")
 
 
@@ -424,24 +409,21 @@ def run_tms(args, ws, rank, local):
     # Roofline of the broad phase (A2-A7: bounds pass through candidate emission),
     # the search's HBM-bound part, as one unit: its algorithmic bytes
     #   B_broad = V * 32 (each mesh's FP64 vertices read once, both meshes)
-    #           + E * 16 (one 8-byte (key, id) entry written and read per
-    #                     face-cell incidence the grid registers)
+    #           + E * 16 (one 8-byte pair of ids written and read per pair of
+    #                     tree nodes listed)
     #           + K * 8  (one 8-byte candidate pair written)
-    # with E and K this search's counts (at the patch level E counts patch-cell
-    # incidences and K quad pairs), divided by the summed device time of the
-    # broad stages; and the ncu DRAM bytes of the same kernels (profiles/
-    # traffic.json, taken on the same sources) over the same time.  Both
+    # with E and K this search's counts (K quad pairs), divided by the summed
+    # device time of the broad stages; and the ncu DRAM bytes of the same kernels
+    # (profiles/traffic.json, taken on the same sources) over the same time.  Both
     # against the measured copy bandwidth.  Per stage, the share of B_broad that
-    # stage moves: the vertex read (bounds pass), the entry writes (cell passes),
-    # the entry reads (cell table), the candidate writes (emission).
+    # stage moves: the vertex read (bounds pass), the rest (trees and patch pairs).
     V2 = pair.A.N * pair.A.M + pair.B.N * pair.B.M
     E, K = stats["entries"], stats["candidates"]
     hbm = peaks.get("hbm_gbs")
     broad_stages = BROAD_STAGES
     broad_ms = sum(stage_ms.get(k, 0.0) for k in broad_stages)
     b_broad = 32 * V2 + 16 * E + 8 * K
-    share = {"face_bounds": 32 * V2, "face_probe": 8 * E, "group_count": 8 * E,
-             "emit": 8 * K}
+    share = {"face_bounds": 32 * V2, "emit": 16 * E + 8 * K}
     kernels = {}
     for st_name, kname in STAGE_KERNELS.items():
         t = sum(stage_ms.get(x, 0.0) for x in STAGE_PARTS[st_name])
@@ -457,8 +439,8 @@ def run_tms(args, ws, rank, local):
                 "frac": ach / hbm if (ach and hbm) else None, "traffic": traffic,
                 "peak_kind": f"{peaks_kind} copy bandwidth",
                 "algorithmic_bytes": b_broad,
-                "algorithmic_formula": "32 V + 16 E + 8 K (V vertices of both meshes, E face-cell "
-                                       "entries, K candidate pairs)",
+                "algorithmic_formula": "32 V + 16 E + 8 K (V vertices of both meshes, E node pairs "
+                                       "of the patch trees, K candidate pairs)",
                 "V": V2, "E": E, "K": K, "ms": broad_ms,
                 "share_of_step": broad_ms / ms_per_step if ms_per_step else None,
                 "ncu_achieved": (traffic / 1e9) / (broad_ms / 1e3) if (traffic and broad_ms) else None,
@@ -598,7 +580,7 @@ def plain_fp64(tms, A, B, out, stream, flush, mixed_hits, fp64_tf=None):
     ach = FP64_SOLVE_FLOPS * st["fp64_solves"] / (t_n * 1e-3) / 1e12 if t_n > 0 else None
     return {"ms_per_search": ms, "hits": len(h), "identical_hit_set_to_mixed": bool(same),
             "fp64_solves": st["fp64_solves"], "narrow_ms": t_n,
-            "fp64": {"kernel": "tms::k_narrow_fp64", "flops_per_solve": FP64_SOLVE_FLOPS,
+            "fp64": {"kernel": "tms::k_narrow_all", "flops_per_solve": FP64_SOLVE_FLOPS,
                      "achieved_tflops": ach, "peak_tflops": fp64_tf,
                      "frac": (ach / fp64_tf) if (ach and fp64_tf) else None,
                      "peak_kind": "measured FP64 FMA-chain probe on this GPU"},

@@ -701,7 +701,7 @@ __device__ __forceinline__ unsigned long long hit_place(const NarrowArgs &a, boo
 // on its quads' vertices rounded down to FP32, the first mixed directions
 // first; the candidates they leave gather in a per-warp queue, and every 32 of
 // them take the other directions with all lanes busy, what is left of the block's queues
-// at the end together; those still not cleared are listed for k_narrow_pairs.  Bound by
+// at the end together; those still not cleared are listed for k_narrow_filter.  Bound by
 // instruction issue and the gathers.  One wave of blocks: with four, a warp had one or two
 // turns of 32 candidates and then a queue of about five to work off with 27 lanes idle
 // (4096 x 512, 700,000 candidates: 41.6 us and 19.0 M instructions, so 26.2 and 11.7).
@@ -789,7 +789,7 @@ __global__ void __launch_bounds__(32 * kQuadWarps, 3) k_quad_filter(NarrowArgs a
 // solve.
 constexpr int kPairBlock = 128;
 template <int FACE>
-__global__ void __launch_bounds__(kPairBlock) k_narrow_pairs(NarrowArgs a) {
+__global__ void __launch_bounds__(kPairBlock) k_narrow_filter(NarrowArgs a) {
     __shared__ uint4 s_pair[kPairBlock];
     __shared__ unsigned s_n;
     if (a.ctr->cand > a.cand_cap || a.ctr->qkeep > a.qsurv_cap) return;
@@ -1309,10 +1309,10 @@ void launch_narrow(const NarrowArgs &a, int face_level, int sms, cudaStream_t st
     }
     if (face_level == 0) {
         k_quad_filter<0><<<sms * 3, 32 * kQuadWarps, 0, st>>>(a);
-        k_narrow_pairs<0><<<sms * 8, kPairBlock, 0, st>>>(a);
+        k_narrow_filter<0><<<sms * 8, kPairBlock, 0, st>>>(a);
     } else {
         k_quad_filter<1><<<sms * 3, 32 * kQuadWarps, 0, st>>>(a);
-        k_narrow_pairs<1><<<sms * 8, kPairBlock, 0, st>>>(a);
+        k_narrow_filter<1><<<sms * 8, kPairBlock, 0, st>>>(a);
     }
 }
 
