@@ -39,23 +39,21 @@ WORKLOAD = dict(workload="mesh-vs-mesh search, 4096x512 vs 4096x512 vertex grids
 ENTRY_BYTES = 8 + 4                   # face-cell entry: u64 key, u32 face id
 NOMINAL_SM_MAX_MHZ = 2070              # GB300 maximum SM clock
 REF_MAX_STEPS = 10                     # timed oracle searches of the reference arm
-# FP32 operations of one verified FP32 solve (an FMA counts 2): 20 system
-# entries with error bounds (12 each), elimination on [A | I | r] (98), back
-# substitution for five right-hand sides (80), the bound matrix W (32),
-# alpha = |I - C A| + |C| W (337), the residual bound (112), the error bound
-# (35) and the margin tests (22)
-FP32_SOLVE_FLOPS = 956
-# FP32 operations of the separating-axis prefilter with all four axes: five
-# split difference vectors with bounds (80), two offset vectors (16), two sets
-# of Plucker coordinates (56), the FP64 solve's reach (12), the two dual
-# choices (28), four interval tests (260)
-SAT_FLOPS = 452
-# FP32 operations of the quad-level test every quad candidate takes: seven split
-# difference vectors (112), the FP64 solve's reach (20), two mixed directions
-# (4D cross products, 56 each) and their interval tests over eight vertices (90
-# each).  The second stage, on the tenth or so of the candidates these leave
-# (two more mixed directions and the dual axes), is not counted.
-QUAD_SAT_FLOPS = 424
+# FP32 operations of one verified FP32 solve (an FMA counts 2; the system is the FP64
+# differences rounded): elimination on [A | I | r] (98), back substitution for five
+# right-hand sides (80), the bound matrix W (32), alpha = |I - C A| + |C| W (337), the
+# residual bound (87), the error bound (35) and the margin tests (22)
+FP32_SOLVE_FLOPS = 691
+# FP32 operations of the separating-axis prefilter with all four axes: the columns'
+# error bounds (10), two offset vectors (16), two sets of Plucker coordinates (36),
+# the FP64 solve's reach (12), the two dual choices (28), four interval tests (260)
+SAT_FLOPS = 362
+# FP32 operations of the quad-level test every quad candidate takes: seven
+# difference vectors and their common bound (40), the FP64 solve's reach (20), the
+# minors of one quad's plane (18), two mixed directions (20 each) and their interval
+# tests over eight vertices (71 each).  The second stage, on the tenth or so of the
+# candidates these leave (two more mixed directions and the dual axes), is not counted.
+QUAD_SAT_FLOPS = 260
 # FP32 lane operations per second of one GB300 (152 SMs x 128 lanes x 2070 MHz,
 # an FMA counted 2)
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.070e9 / 1e12

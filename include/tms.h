@@ -98,16 +98,17 @@ typedef struct {
     int moller;           /* 1 = apply the Moller quick test of Sec. 6.2.3 (FP64,
                              with a rounding guard) to candidates; default 0.
                              Like the boxes, it is not widened by tau. */
-    int cell_filter;      /* 1 = register only faces in grid cells occupied by
-                             both meshes before grouping (default); 0 = emit
+    int cell_filter;      /* patch 0: 1 = register only faces in grid cells occupied
+                             by both meshes before grouping (default); 0 = emit
                              every face-cell incidence (the paper's per-box lists). */
     int narrow_filter;    /* 1 = reject candidates the FP32 tests prove are no
                              FP64 hit: separating axes against the FP64 solve's
                              backward error, and a verified FP32 solve whose
                              error bound certifies margin < -2 tau (default);
                              undecided candidates get the FP64 solve. */
-    float cell_mult;      /* grid cell edge = cell_mult x widest face extent per
-                             coordinate (Sec. 6.2.1 requires > 1 x); default 1.0625 */
+    float cell_mult;      /* patch 0: grid cell edge = cell_mult x widest face extent
+                             per coordinate (Sec. 6.2.1 requires > 1 x); default
+                             1.0625 */
     double tau;           /* margin tolerance of the hit test, default 1e-12; it
                              widens the hit test (weights >= -tau), not the broad
                              phase, whose boxes are the faces' own: meant for
@@ -118,17 +119,18 @@ typedef struct {
     int use_graph;        /* 1 = capture the launch sequence in a CUDA graph on
                              first use and replay it (default 1) */
     unsigned inject;      /* fault injection for tests:
-                             bit0 = force entry capacity 1 (exercises retry),
+                             bit0 = force entry capacity 1 (patch 1: of the lists of
+                             node pairs; exercises retry),
                              bit1 = force a capacity error to be returned,
                              bit2 = report TMS_ERR_TIMEOUT from the host,
                              bit3 = start the cell table at 1024 slots (exercises
-                             its growth),
+                             its growth; patch 1: as bit 0),
                              bit4 = on the device, the hit sort's look-back reads
                              every earlier tile as not yet published, so each of
                              its bounded waits runs out after spin_limit polls
                              (no fault: the kernel records ST_TIMEOUT, keeps its
                              writes in bounds and returns; TMS_ERR_TIMEOUT),
-                             bit5 = start the patch-pair, candidate, survivor and
+                             bit5 = start the patch-pair, candidate, kept-quad and
                              raw-hit buffers at one record (exercises each growth
                              and its retry) */
     int block_faces;      /* bounds-pass tile width in quads (64/128/256; 0 = 128) */
@@ -136,10 +138,11 @@ typedef struct {
                              level takes 8 in mixed precision where they fill the GPU) */
     int timing;           /* 1 = record CUDA events between stages (in the graph) so
                              that tms_last_stage_ms() reports per-stage device time */
-    int patch;            /* broad-phase level: 0 = the grid holds the faces
-                             themselves; 1 = the grid holds patches of 8 x 4 quads
-                             (their boxes the union of the quads'), and the quad
-                             pairs of every patch pair whose boxes overlap are
+    int patch;            /* broad-phase level: 0 = a uniform grid holds the faces;
+                             1 = patches of 8 x 4 quads (their boxes the union of
+                             the quads'), whose overlapping pairs are found down
+                             trees of 4 x 4 nodes over each mesh's own rows and
+                             columns, and the quad pairs of every such patch pair are
                              tested in one warp tile (quad faces only; ignored
                              with face_level 0).  Same candidates either way. */
     int pad0;
@@ -272,15 +275,17 @@ tms_status tms_autotune(const tms_mesh *A, const tms_mesh *B, int nPairs,
 
 /* Per-stage statistics of the last search on `stream` (host copies). */
 typedef struct {
-    long long entries;      /* face-cell entries (grouped by cell) */
-    long long cells;        /* occupied cells holding both meshes */
-    long long pair_slots;   /* sum over cells of nA*nB */
+    long long entries;      /* face-cell entries (grouped by cell); patch level: node
+                               pairs listed, all levels */
+    long long cells;        /* occupied cells holding both meshes (patch level: 0) */
+    long long pair_slots;   /* sum over cells of nA*nB; patch level: patch-box tests */
     long long candidates;   /* candidate face pairs after box and owner tests */
     long long fp64_solves;  /* triangle pairs sent to the FP64 solve */
     long long raw_hits;     /* hits before merging */
     long long hits;         /* output hits */
-    int grid_n[4];          /* cells per coordinate (pair 0) */
-    int empty;              /* trimmed world empty (pair 0) */
+    int grid_n[4];          /* cells per coordinate (pair 0; patch level: 0) */
+    int empty;              /* trimmed world empty (patch level: the meshes' boxes are
+                               apart; pair 0) */
     int retries;            /* capacity retries taken */
     int kernels;            /* kernel launches in one search (graph replay) */
     int pad;
@@ -591,12 +596,11 @@ tms_status tms_phase_align(const double *dWr, const double *dWprev, int N, int n
  *   3 bitmap clear           4 face pass: mark A         5 face pass: probe B
  *   6 face pass: probe A (or emit all)  7 cell table: counts and ranks
  *   8 cells and scatter of the face ids
- *   9 candidate emission (patch level: patch pairs)
+ *   9 candidate emission (patch level: trees and patch pairs)
  *   10 patch level: quad pairs of the patch pairs (0 otherwise)
- *   11 narrow phase          12 sort hits
- *   13 merge + output        14 counter read-back
- * The face passes, cell table and emission work on patches at the patch
- * level.  Writes min(cap, 15) values; *n receives 15. */
+ *   11 narrow phase          12 sort hits (more than 32768 raw hits; else in 13)
+ *   13 merge + output        14 counter read-back (likewise in 13)
+ * At the patch level 0 and 2 to 8 are empty.  Writes min(cap, 15) values; *n receives 15. */
 tms_status tms_last_stage_ms(void *stream, float *ms, int cap, int *n);
 
 /* Frees the scratch and cached plans created for `stream`; NULL frees those of

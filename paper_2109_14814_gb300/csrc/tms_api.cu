@@ -779,7 +779,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
                                       : std::max<unsigned long long>(1 << 14, P->cand_cap / 16);
     P->surv_cap = std::max<unsigned long long>(1 << 16, P->cand_cap / 8);
     if (prm.inject & 32u) {
-        // test switch: the patch-pair, candidate, survivor and raw-hit buffers
+        // test switch: the patch-pair, candidate, kept-quad and raw-hit buffers
         // start at one record, so that each grows in turn
         P->ppair_cap = patch ? 1 : 0;
         P->cand_cap = P->surv_cap = P->hit_cap = 1;

@@ -167,7 +167,7 @@ struct Counters {
     unsigned int dropped;          // raw hits merged into another record (short tail)
 };
 
-// The short merge (k_tail_*, up to kTailMax raw hits): the hits are counted into
+// The short merge (k_tail, up to kTailMax raw hits): the hits are counted into
 // kTailBuckets buckets of increasing key as the FP64 solve lists them.
 constexpr unsigned kTailMax = 32768;
 constexpr unsigned kTailBuckets = 8192;
@@ -661,7 +661,7 @@ struct DedupArgs {
 };
 void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st);
 
-// The merge of at most kTailMax raw hits in three launches, instead of the radix
+// The merge of at most kTailMax raw hits in one launch, instead of the radix
 // sort and launch_dedup (nothing is written when there are more: the host takes
 // that path then).
 struct TailArgs {

@@ -6,8 +6,10 @@
 //                    cell edge > widest face), a finiteness check of every
 //                    vertex, the vertices rounded down to FP32, and the box of
 //                    every face (Sec. 6.2.2; at the patch level the boxes of the
-//                    patches and their quarters);
-//   cell passes      (one read of every face box) the cells each face covers:
+//                    patches and their quarters and the patches' frames instead,
+//                    and no world bounds: tms_tree.cu takes the patch boxes on);
+//   cell passes      (face level; one read of every face box) the cells each face
+//                    covers:
 //     MODE_MARK        occupancy bits of the cells covered by mesh A's faces;
 //     MODE_PROBE_MARK  mesh B: one entry per face-cell incidence in a cell that
 //                      mesh A occupies, and those cells marked "hot";
@@ -22,7 +24,8 @@
 // Bounds pass tiling: a block owns a tile of TI quads along theta x TK quad
 // rows.  All (TI+1) x (TK+1) vertices of the tile are loaded once, coalesced
 // along theta, into shared memory (rounded down to FP32 in the mixed precision
-// mode), then each thread builds the boxes of its quads' faces.
+// mode), then each thread builds the boxes of its quads' faces.  (At the patch level
+// a patch row's vertices at a time.)
 //
 // Cell passes: one thread per face slot; a warp expands its 32 faces' cell
 // ranges into one list of (face, cell) items and works through it 32 items at

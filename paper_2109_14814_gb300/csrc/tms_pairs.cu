@@ -423,15 +423,12 @@ constexpr int kQuarterBlock = 128;     // stage 1: one lane per patch pair
 // 16-bit mask (bit 4 i + j: A quarter i meets B quarter j).
 // Stage 2 (k_patch_quads), one warp per listed pair, grid-stride: the pair's
 // quarter boxes and the vertices of its quads are loaded together (neither waits
-// for the other), and the quad boxes made from the vertices.  Lane l holds quad (row l / kPatchI, column l % kPatchI) of each
-// patch; a quad that meets none of the other patch's quarter boxes cannot
+// for the other), and the quad boxes made from the vertices.  Lane l holds quad
+// (row l / kPatchI, column l % kPatchI) of each patch; a quad that meets none of the other patch's quarter boxes cannot
 // overlap any of its quads (they all lie in those boxes), so each side is cut
 // to its quads that meet one.  The survivors' pairs take the box test of
-// Sec. 6.2.2 (optionally the Moller test of Sec. 6.2.3) and are appended
-// through a per-warp stage: the smaller side's survivors stay in registers, one
-// per lane and repeated in G = 32 / n groups of lanes, while each round reads G
-// of the other side's survivors from shared memory (close to a broadcast), so a
-// round costs two short shared-memory reads and no division.
+// Sec. 6.2.2 (optionally the Moller test of Sec. 6.2.3), 32 of them a turn, and are
+// appended through a per-warp stage.
 // patch id -> (patch row, patch column): the quotient by npi from a 64-bit
 // reciprocal (exact for 32-bit ids, npi >= 2)
 __device__ __forceinline__ void patch_rc(uint32_t patch, uint32_t npi, unsigned long long magic,

@@ -1,7 +1,7 @@
 // Autotuner: picks the parameters the paper leaves to the implementation -- the
-// grid cell size (Sec. 6.2.1 asks only for cells wider than the widest quad),
-// the face level, the broad-phase level (faces or patches in the grid) and the
-// bounds-pass tile shape -- by timing them on the caller's meshes, and keeps the
+// grid cell size (Sec. 6.2.1 asks only for cells wider than the widest quad; the
+// patch level has no grid), the face level, the broad-phase level (faces in a grid or
+// patches in trees) and the bounds-pass tile shape -- by timing them on the caller's meshes, and keeps the
 // choice in a text file read back by later searches (tms_params.autotune_cache).
 //
 // One pair: every setting of a small grid is timed with tms_search.
