@@ -242,7 +242,8 @@ __global__ void __launch_bounds__(256) k_tree_top(TreeArgs a) {
 // Lanes 0-15 hold the children of A's node, lanes 16-31 those of B's.
 template <int PREC>
 __global__ void __launch_bounds__(256) k_tree_down(TreeArgs a, int level) {
-    __shared__ TBox<PREC> sBox[8][32];
+    __shared__ TBox<PREC> sBox[8][32];     // survivors' boxes, A's from 0, B's from 16
+    __shared__ uint32_t sChild[8][32];     // and ids
     __shared__ Cand sOut[8][kPairFlush + 32];
     const unsigned long long n = clamp_count(&a.ctr->nodes[level], a.cap);
     if (256 * n > kMaxPairSlots) {
@@ -293,24 +294,31 @@ __global__ void __launch_bounds__(256) k_tree_down(TreeArgs a, int level) {
         const uint32_t meet = __ballot_sync(FULL, overlap(b, u));
         const uint32_t mA = meet & 0xffffu, mB = meet >> 16;
         if (!mA || !mB) continue;
+        const uint32_t nA = __popc(mA), nB = __popc(mB);
         __syncwarp();                   // the previous pair's boxes are read
-        sBox[warp][lane] = b;
+        if ((meet >> lane) & 1u) {
+            const int at = (lane & 16) + __popc(meet & (lane < 16 ? 0xffffu : 0xffff0000u) & lanemask_lt());
+            sBox[warp][at] = b;
+            sChild[warp][at] = child;
+        }
         __syncwarp();
-        tests += __popc(mA) * __popc(mB);
-        // two of A's children a step, each against all of B's
-        const TBox<PREC> y = sBox[warp][16 + c];
-        const uint32_t childB = __shfl_sync(FULL, child, 16 + c);
-        const bool inB = (mB >> c) & 1u;
-        uint32_t rest = mA;
-        while (rest) {
-            const int j0 = __ffs(rest) - 1;
-            rest &= rest - 1;
-            const int j1 = rest ? __ffs(rest) - 1 : -1;
-            rest &= rest - 1;
-            const int j = lane < 16 ? j0 : j1;
-            const uint32_t childA = __shfl_sync(FULL, child, j & 15);
-            const bool ov = inB && j >= 0 && overlap(sBox[warp][j & 15], y);
-            stage_push<kPairFlush>(stage, staged, ov, node_pair(childA, childB, np.pair), ctr, store);
+        tests += nA * nB;
+        // the nA nB tests one a lane, B's children fastest; test t is child t / nB of A
+        // (below 32 also past the last test) and t % nB of B, from FP32 reciprocals:
+        // (x + 1/2) / nB lies at least 1/32 from an integer for x <= 32.  (Two of A's
+        // children a step against B's sixteen: the leaf level of 64 uneven pairs 71 us, 64 so.)
+        const float rB = __fdividef(1.0f, (float)nB);
+        const uint32_t step_a = (uint32_t)(32.5f * rB), step_b = 32u - step_a * nB;
+        uint32_t ia = (uint32_t)(((float)lane + 0.5f) * rB), ib = (uint32_t)lane - ia * nB;
+        for (uint32_t base = 0; base < nA * nB; base += 32) {
+            const bool ov = base + lane < nA * nB && overlap(sBox[warp][ia], sBox[warp][16 + ib]);
+            stage_push<kPairFlush>(stage, staged, ov, node_pair(sChild[warp][ia], sChild[warp][16 + ib], np.pair), ctr, store);
+            ia += step_a;
+            ib += step_b;
+            if (ib >= nB) {
+                ib -= nB;
+                ++ia;
+            }
         }
     }
     __syncwarp();
