@@ -225,13 +225,15 @@ __global__ void __launch_bounds__(256) k_tree_top(TreeArgs a) {
         TBox<PREC> x, y;
         x.set_empty();
         y.set_empty();
+        // (an unbounded box, of coordinates beyond FP32 on both sides, meets the empty one too)
+        const bool inB = b0 + lane < nB;
         if (a0 + lane < nA) x.load(la.box, (uint32_t)(a0 + lane));
-        if (b0 + lane < nB) y.load(lb.box, (uint32_t)(b0 + lane));
+        if (inB) y.load(lb.box, (uint32_t)(b0 + lane));
         __syncwarp();
         sA[warp][lane] = x;
         __syncwarp();
         for (int j = 0; j < rows; ++j)
-            stage_push<kPairFlush>(stage, staged, overlap(sA[warp][j], y),
+            stage_push<kPairFlush>(stage, staged, inB && overlap(sA[warp][j], y),
                                    node_pair((uint32_t)(a0 + j), (uint32_t)(b0 + lane), (uint32_t)lo), ctr, store);
     }
     __syncwarp();
@@ -290,8 +292,9 @@ __global__ void __launch_bounds__(256) k_tree_down(TreeArgs a, int level) {
         const uint32_t child = (uint32_t)k * (uint32_t)dn.ni + (uint32_t)i;
         TBox<PREC> b;
         b.set_empty();
-        if (i < dn.ni && k < dn.nk) b.load(dn.box, child);
-        const uint32_t meet = __ballot_sync(FULL, overlap(b, u));
+        const bool real = i < dn.ni && k < dn.nk;       // (as in k_tree_top)
+        if (real) b.load(dn.box, child);
+        const uint32_t meet = __ballot_sync(FULL, real && overlap(b, u));
         const uint32_t mA = meet & 0xffffu, mB = meet >> 16;
         if (!mA || !mB) continue;
         const uint32_t nA = __popc(mA), nB = __popc(mB);
