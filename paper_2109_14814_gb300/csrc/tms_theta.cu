@@ -10,7 +10,12 @@
 // real results come back as the real and imaginary parts.  Forward: radix-2
 // decimation in time from bit-reversed input; inverse: decimation in frequency
 // to bit-reversed output, read back through the same permutation.  All in
-// FP64 in shared memory.
+// FP64 in shared memory, the arguments k rho reduced modulo 2 pi as exact
+// numbers: rounded to FP64 ahead of their sine and cosine they were most of the
+// error on rows with high frequencies.  What bounds it: the FP64 pipe (0.89 ms for
+// 4 x 1025 columns of 2048 points, 14 M warp instructions of 19 clocks an SM).  A
+// transform in pairs of floats took 0.16 ms, but holds 2^-48: 8e-15 of a smooth
+// row against 6e-16 here, and 2e-12 of a derivative against 6e-14.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
@@ -42,8 +47,48 @@ __device__ __forceinline__ double2 cmulc(double2 a, double2 b) {   // a * conj(b
     return make_double2(a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y);
 }
 
-__global__ void __launch_bounds__(kFftThreads) k_theta_fft(const ThetaArgs a) {
+__device__ __forceinline__ int exponent(double x) { return (__double2hiint(x) >> 20) & 0x7ff; }
+
+// e^{j x n}: x n as an exact sum of two doubles less the nearest multiple of 2 pi (in
+// three parts), so that its sine and cosine are good to FP64
+__device__ __forceinline__ double2 phase(double x, int n) {
+    constexpr double p1 = 6.283185307179586, p2 = 2.4492935982947064e-16, p3 = -5.989539619436679e-33;
+    const double a = x * n, al = fma(x, (double)n, -a);
+    const double q = rint(a * 0.15915494309189535);
+    double r = fma(-q, p1, a);          // exact: a and q p1 are close
+    const double t = q * p2, tl = fma(q, p2, -t);
+    const double s = r - t;
+    const double sl = ((r - s) - t) - tl + al - q * p3;
+    r = s + sl;
+    double low = (s - r) + sl;          // what r lost: a first-order term
+    if (exponent(a) >= 1023 + 49) {     // no multiple of 2 pi that is exact enough
+        r = a;
+        low = 0.0;
+    }
+    double sn, cs;
+    sincos(r, &sn, &cs);
+    return make_double2(cs - sn * low, sn + cs * low);
+}
+
+// The high word of |x|, with its last bit set for a rest below it: a row's largest tells
+// its size (0: a row of zeros), and the exponent of that size.
+__device__ __forceinline__ unsigned size_word(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7fffffffu) | (__double2loint(x) != 0 ? 1u : 0u);
+}
+__device__ __forceinline__ int size_exponent(unsigned m) {
+    return (m >> 20) ? (int)(m >> 20) - 1023 : 31 - __clz(m) - 1042;
+}
+// 2^e, -1022 <= e <= 1023
+__device__ __forceinline__ double power_of_two(int e) { return __hiloint2double((1023 + e) << 20, 0); }
+// x 2^e, the power of two in halves, which are in range (out of line: the compiler would run
+// it for every value, under a predicate)
+__device__ __noinline__ double scaled(double x, int e) {
+    return x * power_of_two(e / 2) * power_of_two(e - e / 2);
+}
+
+__global__ void __launch_bounds__(kFftThreads, 6) k_theta_fft(const ThetaArgs a) {
     extern __shared__ double2 sm[];
+    __shared__ unsigned top[2][kFftThreads / 32];
     const int N = a.N;
     double2 *z = sm;                 // N values
     double2 *w = sm + N;             // N/2 twiddles e^{-2 pi j m / N}
@@ -57,24 +102,57 @@ __global__ void __launch_bounds__(kFftThreads) k_theta_fft(const ThetaArgs a) {
     const int c0 = 2 * pair, c1 = 2 * pair + 1;
     const bool two = c1 < a.ncoord;
     const double rho = a.rho ? a.rho[col] : a.rho0;
-    if (t < kTab) {
-        double s, c;
-        sincospi(-2.0 * (double)(t * kTab) / (double)N, &s, &c);
-        th[t] = make_double2(c, s);
-        sincospi(-2.0 * (double)t / (double)N, &s, &c);
-        tl[t] = make_double2(c, s);
-        sincos(rho * (double)(t * kTab), &s, &c);
-        hh[t] = make_double2(c, s);
-        sincos(rho * (double)t, &s, &c);
-        hl[t] = make_double2(c, s);
+    // the four tables side by side, as far as they are used
+    static_assert(kFftThreads == 4 * kTab, "64 threads a table");
+    {
+        const int table = t / kTab, e = t % kTab, n = table & 1 ? e : e * kTab;
+        if (n < N / 2) {
+            if (table < 2) {
+                double s, c;
+                sincospi(-2.0 * (double)n / (double)N, &s, &c);
+                (table ? tl : th)[e] = make_double2(c, s);
+            } else {
+                (table == 3 ? hl : hh)[e] = phase(rho, n);
+            }
+        }
     }
     const double *ra = a.in + (long long)c0 * a.ldc + (long long)col * N;
     const double *rb = a.in + (long long)c1 * a.ldc + (long long)col * N;
     const int sh = 32 - a.logN;
-    for (int i = t; i < N; i += kFftThreads)
-        z[__brev((unsigned)i) >> sh] = make_double2(ra[i], two ? rb[i] : 0.0);
+    unsigned ma = 0, mb = 0;
+    for (int i = t; i < N; i += kFftThreads) {
+        const double2 v = make_double2(ra[i], two ? rb[i] : 0.0);
+        z[__brev((unsigned)i) >> sh] = v;
+        ma = max(ma, size_word(v.x));
+        mb = max(mb, size_word(v.y));
+    }
+    ma = __reduce_max_sync(0xffffffffu, ma);
+    mb = __reduce_max_sync(0xffffffffu, mb);
+    if ((t & 31) == 0) {
+        top[0][t >> 5] = ma;
+        top[1][t >> 5] = mb;
+    }
     __syncthreads();
     for (int m = t; m < N / 2; m += kFftThreads) w[m] = cmul(th[m / kTab], tl[m % kTab]);
+#pragma unroll
+    for (int k = 0; k < kFftThreads / 32; ++k) {
+        ma = max(ma, top[0][k]);
+        mb = max(mb, top[1][k]);
+    }
+    // rows of unlike size, whose larger one's rounding would be the smaller one's error, or
+    // of extreme size are brought to about 1 (powers of two: the same digits)
+    int ea = 0, eb = 0;
+    if (max(ma, mb) < 0x7ff00000u) {
+        ea = ma ? size_exponent(ma) : mb ? size_exponent(mb) : 0;
+        eb = mb ? size_exponent(mb) : ea;
+        if (abs(ea - eb) <= 2 && abs(ea) < 900) ea = eb = 0;
+    }
+    if (ea | eb) {
+        for (int i = t; i < N; i += kFftThreads) {
+            double2 &v = z[__brev((unsigned)i) >> sh];
+            v = make_double2(scaled(v.x, -ea), scaled(v.y, -eb));
+        }
+    }
     __syncthreads();
 
     // forward transform (decimation in time)
@@ -95,9 +173,8 @@ __global__ void __launch_bounds__(kFftThreads) k_theta_fft(const ThetaArgs a) {
     for (int i = t; i < N; i += kFftThreads) {
         double2 v = z[i];
         if (i == N / 2) {
-            double s, c;
-            sincos(0.5 * (double)N * rho, &s, &c);
-            const double g = a.derivative ? 0.0 : c;
+            const double2 h = cmul(hh[N / 4 / kTab], hl[N / 4 % kTab]);   // e^{j rho N / 4}
+            const double g = a.derivative ? 0.0 : (h.x - h.y) * (h.x + h.y);
             v = make_double2(v.x * g, v.y * g);
         } else {
             const int k = i < N / 2 ? i : i - N;
@@ -128,9 +205,13 @@ __global__ void __launch_bounds__(kFftThreads) k_theta_fft(const ThetaArgs a) {
     double *oa = a.out + (long long)c0 * a.ldc + (long long)col * N;
     double *ob = a.out + (long long)c1 * a.ldc + (long long)col * N;
     for (int i = t; i < N; i += kFftThreads) {
-        const double2 v = z[__brev((unsigned)i) >> sh];
-        oa[i] = v.x * inv;
-        if (two) ob[i] = v.y * inv;
+        double2 v = z[__brev((unsigned)i) >> sh];
+        v.x *= inv;
+        v.y *= inv;
+        if (ea | eb) v = make_double2(scaled(v.x, ea), scaled(v.y, eb));
+        // (a row of zeros stays one)
+        oa[i] = ma == 0 ? 0.0 : v.x;
+        if (two) ob[i] = mb == 0 ? 0.0 : v.y;
     }
 }
 
@@ -143,416 +224,6 @@ __device__ __forceinline__ void two_sum(float x, float y, float &s, float &e) {
 __device__ __forceinline__ void fast_sum(float x, float y, float &s, float &e) {
     s = __fadd_rn(x, y);
     e = __fsub_rn(y, __fsub_rn(s, x));
-}
-
-// ---------------------------------------------------------------------------
-// translation in float pairs (columns of 1024, 2048 and 4096 points)
-// ---------------------------------------------------------------------------
-// The transform above is bound by the FP64 pipe (0.89 ms for 4 x 1025 columns of 2048
-// points, 14 M warp instructions of 19 clocks an SM).  Most of its error at these sizes
-// is the arguments k rho, rounded to FP64 ahead of their sine and cosine; numbers of two
-// floats (2^-48) with the arguments reduced exactly are nearer the exact result, on a
-// pipe some fifty times as fast (relative error, rms, against 113-bit transforms: 1.1e-14
-// at 1024 points, 2.1e-14 in FP64; 1.2e-14 at 2048, 4.2e-14; 1.3e-14 at 4096, 8.9e-14).
-// At 512 points FP64 is the nearer one (5e-15): those columns and shorter ones keep it,
-// and so do columns of 8192, whose twiddles would not fit beside them.
-// 0.157 ms for those 4 x 1025 columns: 116 M warp instructions, issue 64%; 128 registers
-// a thread, so 16 warps an SM (three blocks at 80 registers: 0.170 ms).
-//
-// One block of N / 8 threads takes a pair of rows at a time, eight points a thread:
-// radix-8 passes in decimation in frequency to digit-reversed order (the first reads
-// the rows themselves), in the last of them, in registers, the rest radix (N / 512),
-// the multiplier and the rest radix of the way back, which mirrors the way there (the
-// inverse is the forward transform of the swapped numbers).  Blocks stay for several
-// rows, whose twiddles and phases they share.  Each row is scaled by a power of two to
-// its largest value, so that neither loses to the other.
-constexpr int kPairLeast = 10, kPairMost = 12;   // log2 N
-
-struct __align__(16) PairC {      // a complex number: float pairs h + l
-    float rh, rl, ih, il;
-};
-
-__device__ __forceinline__ void add_pair(float xh, float xl, float yh, float yl, float &h, float &l) {
-    float s, e;
-    two_sum(xh, yh, s, e);
-    h = s;
-    l = __fadd_rn(e, __fadd_rn(xl, yl));
-}
-__device__ __forceinline__ PairC add_c(const PairC &x, const PairC &y) {
-    PairC z;
-    add_pair(x.rh, x.rl, y.rh, y.rl, z.rh, z.rl);
-    add_pair(x.ih, x.il, y.ih, y.il, z.ih, z.il);
-    return z;
-}
-__device__ __forceinline__ PairC sub_c(const PairC &x, const PairC &y) {
-    PairC z;
-    add_pair(x.rh, x.rl, -y.rh, -y.rl, z.rh, z.rl);
-    add_pair(x.ih, x.il, -y.ih, -y.il, z.ih, z.il);
-    return z;
-}
-// x y with the product's error terms (not normalised)
-__device__ __forceinline__ void mul_pair(float xh, float xl, float yh, float yl, float &h, float &l) {
-    h = __fmul_rn(xh, yh);
-    l = __fmaf_rn(xl, yh, __fmaf_rn(xh, yl, __fmaf_rn(xh, yh, -h)));
-}
-__device__ __forceinline__ void sum_products(float ph, float pl, float qh, float ql, float &h, float &l) {
-    float s, e;
-    two_sum(ph, qh, s, e);
-    fast_sum(s, __fadd_rn(e, __fadd_rn(pl, ql)), h, l);
-}
-__device__ __forceinline__ PairC mul_c(const PairC &x, const PairC &w) {
-    float ah, al, bh, bl;
-    PairC z;
-    mul_pair(x.rh, x.rl, w.rh, w.rl, ah, al);
-    mul_pair(x.ih, x.il, w.ih, w.il, bh, bl);
-    sum_products(ah, al, -bh, -bl, z.rh, z.rl);
-    mul_pair(x.rh, x.rl, w.ih, w.il, ah, al);
-    mul_pair(x.ih, x.il, w.rh, w.rl, bh, bl);
-    sum_products(ah, al, bh, bl, z.ih, z.il);
-    return z;
-}
-__device__ __forceinline__ PairC swapped(const PairC &x) {
-    PairC z = {x.ih, x.il, x.rh, x.rl};
-    return z;
-}
-__device__ __forceinline__ PairC times_minus_i(const PairC &x) {
-    PairC z = {x.ih, x.il, -x.rh, -x.rl};
-    return z;
-}
-__device__ __forceinline__ PairC pair_of(double re, double im) {
-    PairC z;
-    z.rh = (float)re;
-    z.rl = (float)(re - (double)z.rh);
-    z.ih = (float)im;
-    z.il = (float)(im - (double)z.ih);
-    return z;
-}
-
-// transforms of 2, 4 and 8 points, e^{-2 pi j m k / R}, in natural order
-__device__ __forceinline__ void dft2(PairC &a, PairC &b) {
-    const PairC s = add_c(a, b);
-    b = sub_c(a, b);
-    a = s;
-}
-__device__ __forceinline__ void dft4(PairC &x0, PairC &x1, PairC &x2, PairC &x3) {
-    dft2(x0, x2);
-    dft2(x1, x3);
-    x3 = times_minus_i(x3);
-    dft2(x0, x1);                       // X0, X2
-    dft2(x2, x3);                       // X1, X3
-    const PairC t = x1;
-    x1 = x2;
-    x2 = t;
-}
-__device__ __forceinline__ void dft8(PairC (&x)[8]) {
-    constexpr float ch = 0.70710677f, cl = 1.21016175e-8f;     // 1 / sqrt 2
-#pragma unroll
-    for (int m = 0; m < 4; ++m) dft2(x[m], x[m + 4]);
-    {
-        // times (1 - j) / sqrt 2 and (-1 - j) / sqrt 2
-        float ah, al, bh, bl;
-        add_pair(x[5].rh, x[5].rl, x[5].ih, x[5].il, ah, al);
-        add_pair(x[5].ih, x[5].il, -x[5].rh, -x[5].rl, bh, bl);
-        mul_pair(ah, al, ch, cl, x[5].rh, x[5].rl);
-        mul_pair(bh, bl, ch, cl, x[5].ih, x[5].il);
-        add_pair(x[7].ih, x[7].il, -x[7].rh, -x[7].rl, ah, al);
-        add_pair(-x[7].rh, -x[7].rl, -x[7].ih, -x[7].il, bh, bl);
-        mul_pair(ah, al, ch, cl, x[7].rh, x[7].rl);
-        mul_pair(bh, bl, ch, cl, x[7].ih, x[7].il);
-        x[6] = times_minus_i(x[6]);
-    }
-    dft4(x[0], x[1], x[2], x[3]);
-    dft4(x[4], x[5], x[6], x[7]);
-    const PairC t[8] = {x[0], x[4], x[1], x[5], x[2], x[6], x[3], x[7]};
-#pragma unroll
-    for (int m = 0; m < 8; ++m) x[m] = t[m];
-}
-
-// e^{2 pi j q / 4096} over the first octant, as float pairs: made by the compiler from
-// the Taylor series (the angles are at most pi / 4), so that a block's twiddles are
-// loads; a sine and cosine in FP64 for each took 40 us of the kernel's 0.2 ms
-constexpr int kRootBits = kPairMost, kRoots = 1 << kRootBits, kOctant = kRoots / 8;
-struct Roots {
-    float ch[kOctant + 1], cl[kOctant + 1], sh[kOctant + 1], sl[kOctant + 1];
-};
-constexpr Roots octant_roots() {
-    Roots r = {};
-    for (int q = 0; q <= kOctant; ++q) {
-        // cos and sin by Horner from the 20th and 21st powers
-        const double x = 6.283185307179586476925 * q / kRoots, x2 = x * x;
-        double c = 1.0, s = 1.0;
-        for (int k = 20; k >= 2; k -= 2) {
-            c = 1.0 - c * x2 / (k * (k - 1));
-            s = 1.0 - s * x2 / (k * (k + 1));
-        }
-        s *= x;
-        r.ch[q] = (float)c;
-        r.cl[q] = (float)(c - (double)r.ch[q]);
-        r.sh[q] = (float)s;
-        r.sl[q] = (float)(s - (double)r.sh[q]);
-    }
-    return r;
-}
-__device__ const Roots g_roots = octant_roots();
-
-// e^{-2 pi j q / 4096}, 0 <= q < 4096
-__device__ __forceinline__ PairC root(int q) {
-    const int r = q & (kRoots / 4 - 1), quarter = q >> (kRootBits - 2);
-    const bool upper = r > kOctant;
-    const int i = upper ? kRoots / 4 - r : r;
-    const float ch = g_roots.ch[i], cl = g_roots.cl[i], sh = g_roots.sh[i], sl = g_roots.sl[i];
-    const PairC e = upper ? PairC{sh, sl, -ch, -cl} : PairC{ch, cl, -sh, -sl};
-    // times (-j)^quarter
-    const PairC f = quarter & 1 ? times_minus_i(e) : e;
-    return quarter & 2 ? PairC{-f.rh, -f.rl, -f.ih, -f.il} : f;
-}
-
-// x 2^-e as a float pair, for |x| < 2^(e + 1) (truncated, then the rest); values below
-// 2^-126 of that vanish
-__device__ __forceinline__ void scaled_pair(double x, int e, float &h, float &l) {
-    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
-    const int field = (int)((hi >> 20) & 0x7ffu);
-    const int e32 = field ? field - 1023 - e + 127 : 0;
-    const unsigned sign = hi & 0x80000000u;
-    const unsigned mant = __funnelshift_l(lo, hi & 0xfffffu, 3);
-    const float r = __uint2float_rn(lo & 0x1fffffffu) * __uint_as_float((unsigned)max(e32 - 52, 0) << 23);
-    const float a = __uint_as_float(((unsigned)max(e32, 0) << 23) | mant);
-    h = e32 > 0 ? __uint_as_float(__float_as_uint(a) | sign) : 0.0f;
-    l = e32 > 52 ? __uint_as_float(__float_as_uint(r) | sign) : 0.0f;
-}
-// rare cases out of line, or the compiler runs their FP64 instructions every time
-// under a predicate (half of the kernel's time went to them)
-__device__ __noinline__ double lifted(double x) { return x * 0x1p300; }
-__device__ __noinline__ double unscaled_any(float h, float l, int e) { return ldexp((double)h + (double)l, e); }
-// (h + l) 2^e in FP64
-__device__ __forceinline__ double unscaled(float h, float l, int e) {
-    float H, L;
-    fast_sum(h, l, H, L);
-    const unsigned b = __float_as_uint(H);
-    const int e32 = (int)((b >> 23) & 0xffu);
-    // H as a 53-bit integer, L in its last places
-    const float f = __uint_as_float((unsigned)min(306 - e32, 254) << 23);
-    int place = e32 >= 52 ? __float2int_rn(L * f) : 0;
-    if ((int)b < 0) place = -place;
-    long long m = ((long long)(0x800000u | (b & 0x7fffffu)) << 29) + place;
-    int ex = e32 - 127 + 1023 + e;
-    if (m < (1LL << 52)) { m <<= 1; --ex; }
-    if (e32 == 0 || ex < 1 || ex > 2046) return unscaled_any(H, L, e);
-    m = (m & 0xFFFFFFFFFFFFFLL) | ((long long)ex << 52);
-    return __longlong_as_double(m | (long long)((unsigned long long)(b & 0x80000000u) << 32));
-}
-
-// padded so that eight neighbouring points a thread, or any run of points, fall on
-// different banks
-__device__ __forceinline__ int padded(int p) { return p + (p >> 3); }
-
-// e^{j x n} for the phase tables: x n as an exact sum of two doubles less the nearest
-// multiple of 2 pi (in three parts), so that its sine and cosine are good to FP64
-__device__ __forceinline__ PairC phase(double x, int n) {
-    constexpr double p1 = 6.283185307179586, p2 = 2.4492935982947064e-16, p3 = -5.989539619436679e-33;
-    const double a = x * n, al = fma(x, (double)n, -a);
-    double sn, cs;
-    if (!(fabs(a) < 1e15)) {            // no multiple of 2 pi that is exact enough
-        sincos(a, &sn, &cs);
-        return pair_of(cs, sn);
-    }
-    const double q = rint(a * 0.15915494309189535);
-    double r = fma(-q, p1, a);          // exact: a and q p1 are close
-    const double t = q * p2, tl = fma(q, p2, -t);
-    const double s = r - t;
-    const double sl = ((r - s) - t) - tl + al - q * p3;
-    r = s + sl;
-    sincos(r, &sn, &cs);
-    const double low = (s - r) + sl;    // what r lost: a first-order term
-    return pair_of(cs - sn * low, sn + cs * low);
-}
-
-template <int LOG>
-struct PairPlan {
-    static constexpr int N = 1 << LOG, T = N / 8, mid = N / 512;
-    static constexpr int lo_bits = LOG / 2, lo = 1 << lo_bits, hi = N / 2 / lo + 1;
-    // twiddles of the three radix-8 passes, e^{-2 pi j n m / Lp} at [m - 1][n]
-    static constexpr int tw = 7 * (N / 8 + N / 64 + N / 512);
-    static constexpr int data = N + N / 8;
-    static constexpr size_t smem = sizeof(PairC) * (size_t)(data + tw + lo + hi) + 64 * sizeof(unsigned);
-};
-
-template <int LOG>
-__global__ void __launch_bounds__(PairPlan<LOG>::T) k_theta_pairs(const ThetaArgs a, int items) {
-    typedef PairPlan<LOG> P;
-    constexpr int N = P::N, T = P::T;
-    extern __shared__ __align__(16) PairC pc[];
-    PairC *z = pc;
-    PairC *tw = z + P::data;
-    PairC *plo = tw + P::tw, *phi = plo + P::lo;
-    unsigned *top = reinterpret_cast<unsigned *>(phi + P::hi);     // [2][32]
-    const int t = threadIdx.x;
-    {
-        PairC *w = tw;
-        for (int len = N; len >= N / 64; len /= 8) {
-            const int s = len / 8;
-            for (int q = t; q < 7 * s; q += T) {
-                const int m = q / s + 1, n = q % s;
-                w[q] = root(m * n * (kRoots / len));
-            }
-            w += 7 * s;
-        }
-    }
-    const int first = (int)((long long)items * blockIdx.x / gridDim.x);
-    const int last = (int)((long long)items * (blockIdx.x + 1) / gridDim.x);
-    const int pairs = (a.ncoord + 1) / 2;
-    int have = -1;                                     // the column of the phase tables
-    for (int item = first; item < last; ++item) {
-        const int col = item / pairs, c0 = 2 * (item % pairs);
-        const bool two = c0 + 1 < a.ncoord;
-        const double *ra = a.in + (long long)c0 * a.ldc + (long long)col * N;
-        const double *rb = ra + a.ldc;
-        double xa[8], xb[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            xa[m] = ra[t + m * T];
-            xb[m] = two ? rb[t + m * T] : 0.0;
-        }
-        unsigned ma = 0, mb = 0;
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            ma = max(ma, (unsigned)__double2hiint(xa[m]) & 0x7fffffffu);
-            mb = max(mb, (unsigned)__double2hiint(xb[m]) & 0x7fffffffu);
-        }
-        ma = __reduce_max_sync(0xffffffffu, ma);
-        mb = __reduce_max_sync(0xffffffffu, mb);
-        if ((t & 31) == 0) {
-            top[t >> 5] = ma;
-            top[32 + (t >> 5)] = mb;
-        }
-        if (col != have) {
-            const double rho = a.rho ? a.rho[col] : a.rho0;
-            for (int q = t; q < P::lo + P::hi; q += T) {
-                if (q < P::lo) plo[q] = phase(rho, q);
-                else phi[q - P::lo] = phase(rho, (q - P::lo) * P::lo);
-            }
-            have = col;
-        }
-        __syncthreads();
-        ma = mb = 0;
-#pragma unroll 4
-        for (int w = 0; w < T / 32; ++w) {
-            ma = max(ma, top[w]);
-            mb = max(mb, top[32 + w]);
-        }
-        int ea = (int)(ma >> 20) - 1023, eb = (int)(mb >> 20) - 1023;
-        // rows of (nearly) subnormal numbers are lifted first
-        int la = 0, lb = 0;
-        if (min(ma, mb) < (200u << 20)) {
-            if (ma < (200u << 20)) { la = 300; ++ea; }
-            if (mb < (200u << 20)) { lb = 300; ++eb; }
-#pragma unroll
-            for (int m = 0; m < 8; ++m) {
-                if (la) xa[m] = lifted(xa[m]);
-                if (lb) xb[m] = lifted(xb[m]);
-            }
-        }
-        PairC x[8];
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            scaled_pair(xa[m], ea + la, x[m].rh, x[m].rl);
-            scaled_pair(xb[m], eb + lb, x[m].ih, x[m].il);
-        }
-        // ---- there
-        dft8(x);
-#pragma unroll
-        for (int m = 0; m < 8; ++m) z[padded(t + m * T)] = m ? mul_c(x[m], tw[(m - 1) * T + t]) : x[0];
-        __syncthreads();
-        const PairC *w = tw + 7 * T;
-#pragma unroll 1
-        for (int len = N / 8; len > P::mid; len /= 8) {
-            const int s = len / 8, n = t % s, p = (t / s) * len + n;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) x[m] = z[padded(p + m * s)];
-            dft8(x);
-#pragma unroll
-            for (int m = 0; m < 8; ++m) z[padded(p + m * s)] = m ? mul_c(x[m], w[(m - 1) * s + n]) : x[0];
-            w += 7 * s;
-            __syncthreads();
-        }
-        // ---- the middle: eight neighbouring points, 8 / mid groups
-#pragma unroll
-        for (int m = 0; m < 8; ++m) x[m] = z[padded(8 * t + m)];
-        auto rest = [&]() {
-            if (P::mid == 8) dft8(x);
-            else if (P::mid == 4) { dft4(x[0], x[1], x[2], x[3]); dft4(x[4], x[5], x[6], x[7]); }
-            else {
-#pragma unroll
-                for (int m = 0; m < 8; m += 2) dft2(x[m], x[m + 1]);
-            }
-        };
-        rest();
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            // the digits of the group, most significant first: k = d1 + 8 d2 + 64 d3 + 512 d4
-            const int g = (8 * t + m) / P::mid, d4 = m % P::mid;
-            const int k = (g >> 6) + ((g >> 3) & 7) * 8 + (g & 7) * 64 + 512 * d4;
-            const int sk = k < N / 2 ? k : k - N, ak = sk < 0 ? -sk : sk;
-            PairC e = mul_c(phi[ak >> P::lo_bits], plo[ak & (P::lo - 1)]);       // e^{j rho |k|}
-            if (sk < 0) { e.ih = -e.ih; e.il = -e.il; }
-            if (k == N / 2) { e.ih = e.il = 0.0f; }
-            if (a.derivative) {
-                // times j k (0 for the Nyquist frequency)
-                const float f = k == N / 2 ? 0.0f : (float)sk;
-                const float rh = __fmul_rn(f, e.rh), rl = __fmaf_rn(f, e.rl, __fmaf_rn(f, e.rh, -rh));
-                const float ih = __fmul_rn(-f, e.ih), il = __fmaf_rn(-f, e.il, __fmaf_rn(-f, e.ih, -ih));
-                e.rh = ih; e.rl = il; e.ih = rh; e.il = rl;
-            }
-            x[m] = swapped(mul_c(x[m], e));
-        }
-        // ---- and back
-        rest();
-        // the eight points are this thread's own: no wait before they are replaced
-#pragma unroll
-        for (int m = 0; m < 8; ++m) z[padded(8 * t + m)] = x[m];
-        __syncthreads();
-#pragma unroll 1
-        for (int len = P::mid * 8; len < N; len *= 8) {
-            const int s = len / 8, n = t % s, p = (t / s) * len + n;
-            w -= 7 * s;
-#pragma unroll
-            for (int m = 0; m < 8; ++m) x[m] = m ? mul_c(z[padded(p + m * s)], w[(m - 1) * s + n]) : z[padded(p)];
-            dft8(x);
-#pragma unroll
-            for (int m = 0; m < 8; ++m) z[padded(p + m * s)] = x[m];
-            __syncthreads();
-        }
-#pragma unroll
-        for (int m = 0; m < 8; ++m) x[m] = m ? mul_c(z[padded(t + m * T)], tw[(m - 1) * T + t]) : z[padded(t)];
-        dft8(x);
-        // (the next rows' first pass writes z after a barrier behind these reads)
-        double *oa = a.out + (long long)c0 * a.ldc + (long long)col * N;
-        double *ob = oa + a.ldc;
-        // a row with an infinity or a NaN leaves nothing of either; a row of zeros stays one
-        const bool broken = ma >= 0x7ff00000u || mb >= 0x7ff00000u;
-        const double nan = __longlong_as_double(0x7ff8000000000000LL);
-#pragma unroll
-        for (int m = 0; m < 8; ++m) {
-            const double va = unscaled(x[m].ih, x[m].il, ea - LOG), vb = unscaled(x[m].rh, x[m].rl, eb - LOG);
-            oa[t + m * T] = broken ? nan : ma ? va : 0.0;
-            if (two) ob[t + m * T] = broken ? nan : mb ? vb : 0.0;
-        }
-    }
-}
-
-template <int LOG>
-cudaError_t launch_theta_pairs(const ThetaArgs &a, int items, cudaStream_t st) {
-    typedef PairPlan<LOG> P;
-    cudaError_t e = cudaFuncSetAttribute(k_theta_pairs<LOG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P::smem);
-    if (e != cudaSuccess) return e;
-    int device = 0, sms = 0, resident = 0;
-    if ((e = cudaGetDevice(&device)) != cudaSuccess) return e;
-    if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device)) != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&resident, k_theta_pairs<LOG>, P::T, P::smem)) != cudaSuccess)
-        return e;
-    const int grid = items < sms * resident ? items : sms * resident;
-    k_theta_pairs<LOG><<<grid, P::T, P::smem, st>>>(a, items);
-    return cudaGetLastError();
 }
 
 // Phase alignment cost.  N^2 distances of C coordinates, each C subtractions, C
@@ -616,8 +287,6 @@ __global__ void __launch_bounds__(1024) k_phase_scale(const PhaseArgs a) {
         if (threadIdx.x == 0) a.scale[blockIdx.x] = a.N < kPhLeast || e < 100 || e > 1900 ? kPhWide : e - 1022;
     }
 }
-
-__device__ __forceinline__ double power_of_two(int e) { return __hiloint2double((1023 + e) << 20, 0); }
 
 // the distance between two points given by their digits, as a float pair; what the
 // pair has no room for (the low halves' squares, the root's second-order terms: 2^-50
@@ -862,21 +531,11 @@ extern "C" tms_status tms_theta_translate(const double *dIn, double *dOut, int N
     a.derivative = derivative;
     const long long blocks = (long long)nCols * ((nCoord + 1) / 2);
     if (blocks > 0x7fffffffLL) return fail(TMS_ERR_ARG, "tms_theta_translate: too many columns");
-    cudaError_t e;
-    // a common shift so small that its arguments lose little (about 1.2e-17 |rho| N of the
-    // result, against 1.2e-14 in float pairs) is the nearer one in FP64
-    const bool small_shift = !dRho && fabs(rho0) * N < 1000.0;
-    if (logN >= kPairLeast && logN <= kPairMost && !small_shift) {
-        cudaStream_t st = (cudaStream_t)stream;
-        e = logN == 10 ? launch_theta_pairs<10>(a, (int)blocks, st)
-            : logN == 11 ? launch_theta_pairs<11>(a, (int)blocks, st) : launch_theta_pairs<12>(a, (int)blocks, st);
-    } else {
-        const size_t smem = (size_t)(N + N / 2 + 4 * kTab) * sizeof(double2);
-        e = cudaFuncSetAttribute(k_theta_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return fail(TMS_ERR_CUDA, cudaGetErrorString(e));
-        k_theta_fft<<<(unsigned)blocks, kFftThreads, smem, (cudaStream_t)stream>>>(a);
-        e = cudaGetLastError();
-    }
+    const size_t smem = (size_t)(N + N / 2 + 4 * kTab) * sizeof(double2);
+    cudaError_t e = cudaFuncSetAttribute(k_theta_fft, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return fail(TMS_ERR_CUDA, cudaGetErrorString(e));
+    k_theta_fft<<<(unsigned)blocks, kFftThreads, smem, (cudaStream_t)stream>>>(a);
+    e = cudaGetLastError();
     if (e != cudaSuccess) return fail(TMS_ERR_CUDA, std::string("tms_theta_translate: ") +
                                                         cudaGetErrorString(e));
     return TMS_OK;
