@@ -584,8 +584,9 @@ tms_status tms_theta_translate(const double *dIn, double *dOut, int N, int nCols
  *                 a * nCoord * N, coordinate c at + c * N).  1 <= nCoord <= 8.
  *   dCost       : device, nAlign x N doubles out.
  *   dShift      : device, nAlign int32 out: the minimising m.
- * Costs are at least as near the exact ones as FP64 sums in order of i; equal
- * terms give equal costs.  Asynchronous; allocates nothing.
+ * Every distance is within 2^-45 of itself and the sum is taken in FP64 (fewer
+ * than 192 samples: FP64 throughout); equal terms give equal costs.
+ * Asynchronous; allocates nothing.
  */
 tms_status tms_phase_align(const double *dWr, const double *dWprev, int N, int nCoord,
                            int nAlign, double *dCost, int32_t *dShift, void *stream);

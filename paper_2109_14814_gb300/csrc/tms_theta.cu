@@ -231,10 +231,11 @@ __device__ __forceinline__ void fast_sum(float x, float y, float &s, float &e) {
 // pipe that takes 19 clocks an SM for each of a warp's (9.6 ms for 16 alignments of
 // 4 x 4096 circles), so here the distances are computed on the FP32 pipe, whose rate
 // is some fifty times that, in numbers of two or three floats:
-//   digits      every coordinate, scaled by the alignment's power of two to |y| <= 1,
-//               as y = x1 + x2 + x3 with x1 a multiple of 2^-22, x2 of 2^-45, and x3
-//               the rest rounded to FP32 (2^-70); the differences of the first two
-//               digits are exact FP32 numbers;
+//   digits      every coordinate, scaled by the alignment's power of two to |y| <= 1
+//               (times 2^40, so that no square of a difference is subnormal), as
+//               y = x1 + x2 + x3 with x1 a multiple of 2^-22, x2 of 2^-45, and x3 the
+//               rest rounded to FP32 (2^-70); the differences of the first two digits
+//               are exact FP32 numbers;
 //   distance    the difference as a float pair, its square with the product's error
 //               term, the sum over the coordinates with every addition's error, the
 //               root with one correction: about 2^-47 relative, without bias;
@@ -244,9 +245,14 @@ __device__ __forceinline__ void fast_sum(float x, float y, float &s, float &e) {
 // A distance's error, 3e-15 rms, averages out over the sum, whose own FP64 roundings
 // are a quarter as many as in order of i: against 113-bit costs the relative error is
 // 3.6e-16 rms at N = 200 (4.1e-16 in FP64 in order of i), 1.6e-16 at 1000 (7.4e-16),
-// 1.9e-16 at 4096 (1.8e-15).  The two meet near N = 160: shorter circles, whose time
-// is launches, take the FP64 loop, and so does an alignment whose largest value's
-// exponent leaves no room for the scaling, or that is not finite.
+// 1.9e-16 at 4096 (1.8e-15).  The two meet near N = 160: shorter circles take FP64
+// sums, and so does an alignment whose largest value's exponent leaves no room for the
+// scaling, or that is not finite.
+// A value of at least 2^-16 of the alignment's largest is the sum of its digits exactly;
+// each of the others is off by 2^-70 at most, and so is a difference with it by its
+// rounding.  Every value is in one distance of each shift, so `lost` such values cost a
+// shift lost 2^-69: where that could be more than 2^-51 of its cost (a large coordinate
+// that cancels leaves a cost of that size) the shift's cost is made again in FP64.
 // Split: a cluster of eight blocks takes 512 shifts, each block an eighth of the i
 // (the same split for every shift and number of alignments: equal terms give equal
 // costs), each thread two neighbouring shifts, whose windows overlap; the even and
@@ -257,35 +263,120 @@ constexpr int kPhShifts = 2 * kPhThreads;
 constexpr int kPhTile = 128;            // i per shared tile (a multiple of 4)
 constexpr int kPhSplit = 8;             // blocks of a cluster, each an eighth of the i
 constexpr int kPhWin = kPhTile + kPhShifts;
-constexpr int kPhWide = 0x7fffffff;     // no scale: the FP64 loop
-constexpr int kPhLeast = 192;           // shorter circles take the FP64 loop
+constexpr int kPhWide = 0x7fffffff;     // no scale: FP64 sums
+constexpr int kPhLeast = 192;           // shorter circles take FP64 sums
+constexpr int kPhUp = 40;               // the digits' unit is 2^-40 of the scale
 
 struct PhaseArgs {
     const double *wr;
     const double *wp;
     double *cost;
-    int *scale;                         // per alignment: the exponent e, |values| < 2^e
+    int *scale;                         // per alignment (NULL: all kPhWide): the exponent e,
+                                        // |values| < 2^e, + 1024, and from bit 12 l, 2^(l - 1)
+                                        // at least its lost values (l = 0: none)
     int N, ncoord, nalign;
 };
 
 // The scale of each alignment, left in the shift output, which the minimum's kernel
 // writes last.
 __global__ void __launch_bounds__(1024) k_phase_scale(const PhaseArgs a) {
-    __shared__ unsigned top[32];
+    __shared__ unsigned top[32], lost[32];
     const long long n = (long long)a.ncoord * a.N, base = n * blockIdx.x;
+    const int t = threadIdx.x;
     unsigned m = 0;                     // high words of |x|: the largest holds the largest exponent
-    for (long long q = threadIdx.x; q < n; q += 1024) {
+    for (long long q = t; q < n; q += 1024) {
         m = max(m, (unsigned)__double2hiint(a.wr[base + q]) & 0x7fffffffu);
         m = max(m, (unsigned)__double2hiint(a.wp[base + q]) & 0x7fffffffu);
     }
     m = __reduce_max_sync(0xffffffffu, m);
-    if ((threadIdx.x & 31) == 0) top[threadIdx.x >> 5] = m;
+    if ((t & 31) == 0) top[t >> 5] = m;
     __syncthreads();
-    if (threadIdx.x < 32) {
-        m = __reduce_max_sync(0xffffffffu, top[threadIdx.x]);
-        const int e = (int)(m >> 20);
-        if (threadIdx.x == 0) a.scale[blockIdx.x] = a.N < kPhLeast || e < 100 || e > 1900 ? kPhWide : e - 1022;
+    m = __reduce_max_sync(0xffffffffu, top[t & 31]);
+    const int field = (int)(m >> 20);   // 2^(field - 1022) = 2^e
+    if (field < 100 || field > 1900) {
+        if (t == 0) a.scale[blockIdx.x] = kPhWide;
+        return;
     }
+    // values below 2^(e - 16) with a bit below 2^(e - 69)
+    unsigned count = 0;
+    const unsigned small = (unsigned)(field - 15) << 20;
+    auto look = [&](double x) {
+        const unsigned h = (unsigned)__double2hiint(x) & 0x7fffffffu;
+        if (h < small && (h | (unsigned)__double2loint(x)) != 0u) {
+            const int last = __ffs(__double2loint(x)), bit = last ? last - 1 : 31 + __ffs((int)(h | 0x100000u));
+            count += max((int)(h >> 20), 1) - 1075 + bit < field - 1022 - 69;
+        }
+    };
+    for (long long q = t; q < n; q += 1024) {
+        look(a.wr[base + q]);
+        look(a.wp[base + q]);
+    }
+    count = __reduce_add_sync(0xffffffffu, count);
+    if ((t & 31) == 0) lost[t >> 5] = count;
+    __syncthreads();
+    count = __reduce_add_sync(0xffffffffu, lost[t & 31]);
+    const int l = count ? 33 - __clz(count - 1) : 0;
+    int word = (field - 1022 + 1024) | (l << 12);
+    if (4 * (long long)count >= a.N) {
+        // a coordinate's worth of them: where no distance can be large enough (the large
+        // coordinates vary too little), FP64 for all, without the float pairs' sums first.
+        // Ranges from the high words, as integers of the values' order.
+        __shared__ int lo[8], hi[8];
+        if (t < 8) {
+            lo[t] = 0x7fffffff;
+            hi[t] = (int)0x80000000;
+        }
+        __syncthreads();
+        for (int c = 0; c < a.ncoord; ++c) {
+            int least = 0x7fffffff, most = (int)0x80000000;
+            for (int i = t; i < a.N; i += 1024) {
+                const long long q = base + (long long)c * a.N + i;
+                const int r = __double2hiint(a.wr[q]), p = __double2hiint(a.wp[q]);
+                const int ro = r ^ ((r >> 31) & 0x7fffffff), po = p ^ ((p >> 31) & 0x7fffffff);
+                least = min(least, min(ro, po));
+                most = max(most, max(ro, po));
+            }
+            least = __reduce_min_sync(0xffffffffu, least);
+            most = __reduce_max_sync(0xffffffffu, most);
+            if ((t & 31) == 0) {
+                atomicMin(&lo[c], least);
+                atomicMax(&hi[c], most);
+            }
+        }
+        __syncthreads();
+        if (t == 0) {
+            // (the last bits of a high word: outward)
+            double d2 = 0.0;
+            for (int c = 0; c < a.ncoord; ++c) {
+                const int h = hi[c] ^ ((hi[c] >> 31) & 0x7fffffff), g = lo[c] ^ ((lo[c] >> 31) & 0x7fffffff);
+                const double d = (__hiloint2double(h, h < 0 ? 0 : -1) - __hiloint2double(g, g < 0 ? -1 : 0)) *
+                                 power_of_two(1022 - field);
+                d2 = fma(d, d, d2);
+            }
+            if (a.N * sqrt(d2) < power_of_two(51 - 69 + l - 1)) word = kPhWide;
+        }
+    }
+    if (t == 0) a.scale[blockIdx.x] = word;
+}
+
+// the part of shift m's cost at i = first, first + step, ..., in FP64
+template <int C>
+__device__ __forceinline__ double cost_part(const double *Wr, const double *Wp, int N, int m, int first, int step) {
+    double s = 0.0;
+#pragma unroll 1                        // (the float pairs' loop has the registers)
+    for (long long i = first; i < N; i += step) {
+        const long long w = i + m < N ? i + m : i + m - N;
+        double d2 = 0.0;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const double d = Wr[(long long)c * N + w] - Wp[(long long)c * N + i];
+            d2 = fma(d, d, d2);
+        }
+        s += sqrt(d2);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    return s;
 }
 
 // the distance between two points given by their digits, as a float pair; what the
@@ -327,12 +418,12 @@ __device__ __forceinline__ void pair_distance(const float (&x)[3][C], const floa
     rest = __fmaf_rn(__fmaf_rn(lo, __fmaf_rn(-T, r, lo), L2), hr, rest);
 }
 
-// the digits of a value scaled to |y| <= 1
+// the digits of a value scaled to |y| <= 2^kPhUp
 __device__ __forceinline__ void digits(double y, float &x1, float &x2, float &x3) {
-    constexpr double m1 = 1.5 * (double)(1 << 30), m2 = 1.5 * (double)(1 << 7);
-    const double t1 = __dsub_rn(__dadd_rn(y, m1), m1);      // to a multiple of 2^-22
+    constexpr double unit = 1LL << kPhUp, m1 = 1.5 * (1 << 30) * unit, m2 = 1.5 * (1 << 7) * unit;
+    const double t1 = __dsub_rn(__dadd_rn(y, m1), m1);      // to a multiple of 2^(kPhUp - 22)
     const double r1 = __dsub_rn(y, t1);
-    const double t2 = __dsub_rn(__dadd_rn(r1, m2), m2);     // to a multiple of 2^-45
+    const double t2 = __dsub_rn(__dadd_rn(r1, m2), m2);     // to a multiple of 2^(kPhUp - 45)
     x1 = (float)t1;
     x2 = (float)t2;
     x3 = (float)__dsub_rn(r1, t2);
@@ -350,28 +441,20 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
     const int m0 = (int)(blockIdx.x / kPhSplit) * kPhShifts;
     const double *Wr = a.wr + (long long)al * C * N;
     const double *Wp = a.wp + (long long)al * C * N;
-    const int e = a.scale[al];
+    const int word = a.scale ? a.scale[al] : kPhWide;
+    if (word == kPhWide) {              // (the whole cluster: it is the alignment's)
+        // a shift a warp, 64 of them at once in the cluster
+        const int last = min(kPhShifts, N - m0);
+        for (int q = rank * (kPhThreads / 32) + (t >> 5); q < last; q += kPhSplit * (kPhThreads / 32)) {
+            const double s = cost_part<C>(Wr, Wp, N, m0 + q, t & 31, 32);
+            if ((t & 31) == 0) a.cost[(long long)al * N + m0 + q] = s;
+        }
+        return;
+    }
+    const int e = (word & 0xfff) - 1024, lost = word >> 12;
     double acc[2] = {0.0, 0.0};
     float rest[2] = {0.0f, 0.0f};
-    if (e == kPhWide) {
-        if (rank == 0)
-            for (int k = 0; k < 2; ++k) {
-                const int m = m0 + 2 * t + k;
-                if (m >= N) continue;
-                for (int i = 0; i < N; ++i) {
-                    const int w = i + m < N ? i + m : i + m - N;
-                    double d2 = 0.0;
-                    for (int c = 0; c < C; ++c) {
-                        const double d = Wr[(long long)c * N + w] - Wp[(long long)c * N + i];
-                        d2 = fma(d, d, d2);
-                    }
-                    acc[k] += sqrt(d2);
-                }
-                a.cost[(long long)al * N + m] = acc[k];
-            }
-        return;                         // the whole cluster: e is the alignment's
-    }
-    const double down = power_of_two(-e);
+    const double down = power_of_two(kPhUp - e);
     const int per = ((N + 4 * kPhSplit - 1) / (4 * kPhSplit)) * 4;
     const int i_end = (int)min((long long)N, (long long)(rank + 1) * per);
     for (long long i0 = (long long)rank * per; i0 < i_end; i0 += kPhTile) {
@@ -436,15 +519,37 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
     part[2 * t] = acc[0] + (double)rest[0];
     part[2 * t + 1] = acc[1] + (double)rest[1];
     cg::cluster_group cluster = cg::this_cluster();
+    // shifts to be made again (the first block's), costs below which they are
+    __shared__ unsigned short again[kPhShifts];
+    __shared__ int n_again;
+    if (t == 0) n_again = 0;
+    const double least = lost ? power_of_two(kPhUp - 69 + 51 + lost - 1) : 0.0;
     cluster.sync();
     if (rank == 0) {
         for (int q = t; q < kPhShifts; q += kPhThreads) {
             double s = part[q];
             for (int r = 1; r < kPhSplit; ++r) s += cluster.map_shared_rank(part, r)[q];
-            if (m0 + q < N) a.cost[(long long)al * N + m0 + q] = s * power_of_two(e);
+            if (m0 + q >= N) continue;
+            if (s < least) again[atomicAdd(&n_again, 1)] = (unsigned short)q;
+            else a.cost[(long long)al * N + m0 + q] = s * power_of_two(e - kPhUp);
         }
     }
     cluster.sync();                     // the parts are read before their blocks end
+    if (lost == 0) return;
+    const int n = *cluster.map_shared_rank(&n_again, 0);
+    for (int k = rank; k < n; k += kPhSplit) {
+        const int m = m0 + cluster.map_shared_rank(again, 0)[k];
+        const double s = cost_part<C>(Wr, Wp, N, m, t, kPhThreads);
+        __syncthreads();                // (the previous shift's sums are read)
+        if ((t & 31) == 0) part[t >> 5] = s;
+        __syncthreads();
+        if (t == 0) {
+            double sum = part[0];
+            for (int w = 1; w < kPhThreads / 32; ++w) sum += part[w];
+            a.cost[(long long)al * N + m] = sum;
+        }
+    }
+    cluster.sync();                     // the list is read before the first block ends
 }
 
 template <int C>
@@ -554,11 +659,11 @@ extern "C" tms_status tms_phase_align(const double *dWr, const double *dWprev, i
     a.wr = dWr;
     a.wp = dWprev;
     a.cost = dCost;
-    a.scale = dShift;
+    a.scale = N < kPhLeast ? nullptr : dShift;
     a.N = N;
     a.ncoord = nCoord;
     a.nalign = nAlign;
-    k_phase_scale<<<nAlign, 1024, 0, (cudaStream_t)stream>>>(a);
+    if (a.scale) k_phase_scale<<<nAlign, 1024, 0, (cudaStream_t)stream>>>(a);
     cudaError_t (*const launch[8])(const PhaseArgs &, cudaStream_t) = {
         launch_phase_cost<1>, launch_phase_cost<2>, launch_phase_cost<3>, launch_phase_cost<4>,
         launch_phase_cost<5>, launch_phase_cost<6>, launch_phase_cost<7>, launch_phase_cost<8>};
