@@ -332,6 +332,12 @@ __device__ __forceinline__ void top2_duals(const float m[6], int &k1, int &k2) {
     for (int k = 0; k < 4; ++k) k2 = (k != k1 && n[k] > n[k2]) ? k : k2;
 }
 
+// What the relative bounds of the gap tests leave out: below 2^-126 an operation is off by up
+// to 2^-150, and a bound that is a product may vanish.  A projection is three or four
+// factors of an edge's size, so edges of 1e-11 come there; a test has some forty such
+// operations, 700 times fewer than this.
+constexpr float kUnder = 1e-42f;
+
 __device__ __forceinline__ float dot4(const float w[4], const SplitVec &v) {
     return fmaf(w[3], v.v[3], fmaf(w[2], v.v[2], fmaf(w[1], v.v[1], w[0] * v.v[0])));
 }
@@ -355,7 +361,7 @@ __device__ __forceinline__ bool separated(const float w[4], const SplitVec &e1, 
     const float xl = fminf(0.0f, fminf(a1, a3)), xh = fmaxf(0.0f, fmaxf(a1, a3));
     const float yl = fminf(b2, fminf(b1, b3)), yh = fmaxf(b2, fmaxf(b1, b3));
     const float DX = (xh - xl) + 2.0f * ex, DY = (yh - yl) + 2.0f * ey;
-    const float need = (tp * (DX + DY) + w1 * reach + ex + ey) * 1.001f;
+    const float need = fmaf(tp * (DX + DY) + w1 * reach + ex + ey, 1.001f, kUnder);
     const float gap = fmaxf(yl - xh, xl - yh) * (1.0f - 4.0f * u);
     return gap > need;
 }
@@ -431,7 +437,7 @@ __device__ __forceinline__ bool quad_gap(const float w[4], const QuadPair &q) {
     const float yl = fminf(fminf(q0, s1), fminf(s2, s3)), yh = fmaxf(fmaxf(q0, s1), fmaxf(s2, s3));
     // u |s| for the sums: at most u times the larger end
     const float err = fmaf(u, fmaxf(fabsf(yl), fabsf(yh)), w1 * (q.ka + q.kb));
-    const float need = (q.tp * ((xh - xl) + (yh - yl) + 2.0f * err) + w1 * q.reach + err) * 1.001f;
+    const float need = fmaf(q.tp * ((xh - xl) + (yh - yl) + 2.0f * err) + w1 * q.reach + err, 1.001f, kUnder);
     const float gap = fmaxf(yl - xh, xl - yh) * (1.0f - 4.0f * u);
     return gap > need;
 }
