@@ -859,7 +859,11 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     }
     P->last_use = ++g_clock;
     P->retries = 0;
-    for (int attempt = 0; attempt < 8; ++attempt) {
+    // Each list's count is complete only once those before it fit, so each may cost a run of
+    // its own (node pairs of every level, patch pairs, candidates, kept quads, raw hits; a
+    // cell table from 1024 slots up to 2^31 eleven), and the last of them must fit.
+    bool grow = true;
+    for (int run = 0; grow && run < kTreeLevels + 16; ++run) {
         s = P->run();
         if (s != TMS_OK) return s;
         const Counters &c = *P->h_ctr;
@@ -875,7 +879,7 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
             g_err = "a device-side wait gave up (sort look-back)";
             return TMS_ERR_TIMEOUT;
         }
-        bool grow = false;
+        grow = false;
         if (!P->patch && ((c.status & ST_TABLE_FULL) || c.claimed > P->tsize / 2)) {
             P->tsize_min = P->tsize * 4;
             grow = true;
@@ -919,11 +923,6 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
         if (s != TMS_OK) return s;
     }
     const Counters &c = *P->h_ctr;
-    if (c.status & ST_TABLE_FULL) {
-        g_err = "cell table still full after retries";
-        *nHits = (long long)c.out;
-        return TMS_ERR_CAPACITY;
-    }
     tms_stats st;
     memset(&st, 0, sizeof(st));
     st.entries = (long long)c.entries;
@@ -947,10 +946,8 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     st.kernels = P->kernels;
     g_stats[user] = st;
     if (prm.timing) g_stage_ms[user] = std::vector<float>(P->stage_ms, P->stage_ms + Plan::kStages);
-    unsigned long long lists = c.entries;
-    for (unsigned long long v : c.nodes) lists = std::max(lists, v);
-    if (lists > P->ent_cap || c.cand > P->cand_cap || c.qkeep > P->surv_cap ||
-        c.raw_hits > P->hit_cap || (P->patch && c.ppairs > P->ppair_cap)) {
+    // (not from the counts: the last run's lists have grown since)
+    if (grow) {
         g_err = "scratch capacity still exceeded after retries";
         *nHits = (long long)c.out;
         return TMS_ERR_CAPACITY;
