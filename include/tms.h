@@ -132,7 +132,9 @@ typedef struct {
                              writes in bounds and returns; TMS_ERR_TIMEOUT),
                              bit5 = start the patch-pair, candidate, kept-quad and
                              raw-hit buffers at one record (exercises each growth
-                             and its retry) */
+                             and its retry),
+                             bit6 = the allocation of a larger list fails (on the
+                             host, TMS_ERR_CUDA) */
     int block_faces;      /* bounds-pass tile width in quads (64/128/256; 0 = 128) */
     int tile_rows;        /* bounds-pass tile height in quad rows (4 or 8; 0 = 4; the patch
                              level takes 8 in mixed precision where they fill the GPU) */

@@ -919,8 +919,14 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
         if (!grow) break;
         ++P->retries;
         TMS_CK(cudaStreamSynchronize(P->st));
-        s = P->alloc_scratch();
-        if (s != TMS_OK) return s;
+        s = prm.inject & 64u ? TMS_ERR_CUDA : P->alloc_scratch();
+        if (s != TMS_OK) {
+            // its lists are given back or in part missing: a later search makes the plan anew
+            if (prm.inject & 64u) g_err = "injected failure of a larger list's allocation";
+            g_plans.erase(std::find(g_plans.begin(), g_plans.end(), P));
+            delete P;
+            return s;
+        }
     }
     const Counters &c = *P->h_ctr;
     tms_stats st;
