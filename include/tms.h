@@ -134,6 +134,8 @@ typedef struct {
                              raw-hit buffers at one record (exercises each growth
                              and its retry),
                              bit6 = the allocation of a larger list fails (on the
+                             host, TMS_ERR_CUDA),
+                             bit7 = the launch of the hit merge fails (on the
                              host, TMS_ERR_CUDA) */
     int block_faces;      /* bounds-pass tile width in quads (64/128/256; 0 = 128) */
     int tile_rows;        /* bounds-pass tile height in quad rows (4 or 8; 0 = 4; the patch

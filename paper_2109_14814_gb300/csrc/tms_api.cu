@@ -145,6 +145,9 @@ struct Plan {
     // more raw hits than the short merge takes: the radix sort and the scans (as
     // a search of this plan found; the look-back test switch needs that sort too)
     bool long_tail = false;
+    // of the merge's launch, which asks for more than every device has to take: a capture
+    // without it would run, and leave the counters as they were
+    cudaError_t launch_error = cudaSuccess;
     int grid = 304;
     int sort_grid = 608;
     // execution
@@ -253,7 +256,7 @@ struct Plan {
         ta.tri_bits = tri_bits; ta.tau = prm.tau; ta.bscale = bscale;
         ta.result = reinterpret_cast<const uint32_t *>(d_ctr); ta.readback = reinterpret_cast<uint32_t *>(h_ctr);
         ta.words = (int)(kReadback / 4);
-        launch_tail(ta, s);
+        launch_error = (prm.inject & 128u) ? cudaErrorInvalidConfiguration : launch_tail(ta, s);
         kernels += 1;
     }
 
@@ -398,6 +401,7 @@ struct Plan {
     void enqueue(cudaStream_t s) {
         const tms_params &p = prm;
         const int fl = p.face_level;
+        launch_error = cudaSuccess;
         if (patch) enqueue_patches(s);
         else enqueue_faces(s);
         mark(11, s);
@@ -421,6 +425,12 @@ struct Plan {
         mark(15, s);
     }
 
+    tms_status launch_failed() {
+        cudaGetLastError();
+        g_err = std::string("hit merge launch: ") + cudaGetErrorString(launch_error);
+        return TMS_ERR_CUDA;
+    }
+
     tms_status run() {
         // a graph runs in the caller's stream; without one, the plan's own stream waits for
         // the caller's and the caller's for it
@@ -437,6 +447,10 @@ struct Plan {
                 enqueue(st);
                 capturing = false;
                 cudaError_t e = cudaStreamEndCapture(st, &g);
+                if (launch_error != cudaSuccess) {
+                    if (e == cudaSuccess) cudaGraphDestroy(g);
+                    return launch_failed();
+                }
                 if (e != cudaSuccess) {
                     g_err = std::string("graph capture: ") + cudaGetErrorString(e);
                     return TMS_ERR_CUDA;
@@ -452,6 +466,10 @@ struct Plan {
             TMS_CK(cudaGraphLaunch(exec, s));
         } else {
             enqueue(st);
+            if (launch_error != cudaSuccess) {
+                cudaStreamSynchronize(st);     // (the kernels before it read the caller's buffers)
+                return launch_failed();
+            }
             TMS_CK(cudaGetLastError());
         }
         if (g_early.host && g_early.n > 0 && dHits)

@@ -688,7 +688,7 @@ struct TailArgs {
     uint32_t *readback;            // and their copy in pinned host memory
     int words;
 };
-void launch_tail(const TailArgs &a, cudaStream_t st);
+cudaError_t launch_tail(const TailArgs &a, cudaStream_t st);
 cudaError_t configure_tail();
 
 

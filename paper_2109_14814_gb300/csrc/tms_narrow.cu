@@ -1336,7 +1336,7 @@ cudaError_t configure_tail() {
     return cudaFuncSetAttribute(k_tail, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
 }
 
-void launch_tail(const TailArgs &a, cudaStream_t st) {
+cudaError_t launch_tail(const TailArgs &a, cudaStream_t st) {
     cudaLaunchAttribute at;
     at.id = cudaLaunchAttributeClusterDimension;
     at.val.clusterDim.x = kTailCluster;
@@ -1347,7 +1347,7 @@ void launch_tail(const TailArgs &a, cudaStream_t st) {
     c.stream = st;
     c.attrs = &at;
     c.numAttrs = 1;
-    cudaLaunchKernelEx(&c, k_tail, a);
+    return cudaLaunchKernelEx(&c, k_tail, a);
 }
 
 void launch_adjoint(const AdjointArgs &a, cudaStream_t st) {
