@@ -254,9 +254,10 @@ tms_status tms_backward(tms_mesh A, tms_mesh B, const tms_hit *dHits, long long 
 /*
  * tms_autotune -- picks, for these meshes, the search parameters the paper
  * leaves to the implementation (Sec. 6.2.1 grid cell size; Sec. 6.3 launch
- * shape): face level (quads or triangles), cell_mult in {1.0625, 1.5, 2.5},
- * block_faces in {64, 128} and tile_rows in {4, 8}, by timing each of the 24
- * settings (one warm-up and three timed runs, median) with tms_search (nPairs == 1) or
+ * shape): face level (quads or triangles) and broad-phase level (patch),
+ * block_faces and tile_rows (128 x 4, 64 x 4, 128 x 8), and, where the level has a
+ * grid, cell_mult in {1.0625, 1.5, 2.5}, by timing each setting that runs
+ * differently (one warm-up and three timed runs, median) with tms_search (nPairs == 1) or
  * tms_search_batched (nPairs > 1) on `stream`.  The other fields (precision,
  * filters, tau, capacities, use_graph) come from `base` (NULL = defaults) and
  * are kept.  Results are unchanged by the choice: every setting finds the same

@@ -525,6 +525,21 @@ tms_status check_mesh(tms_mesh m, int device) {
     return TMS_OK;
 }
 
+// Quad rows of a bounds-pass tile.  Patch level, mixed precision: tiles of 8 rows read a
+// vertex 9/8 times instead of 5/4 and make the frames of two patch rows at once (64 uneven
+// pairs 396 us against 416, 14 layers 49 against 51, 4096 x 512 54 against 57, 1024 x 256
+// 13.2 against 13.7), where they are two for every SM; with fewer, the longer block is not
+// hidden (64 x 32: 10.5 against 9.3).
+int bounds_tile_rows(const std::vector<tms_mesh> &taken, const tms_params &prm, int grid) {
+    if (prm.tile_rows == 8) return 8;
+    if (prm.patch != 1 || prm.face_level != 1 || prm.precision != 1) return 4;
+    const int block = (prm.block_faces == 64 || prm.block_faces == 256) ? prm.block_faces : 128;
+    long long tall = 0;
+    for (tms_mesh m : taken)
+        tall += (long long)((m->dev.nqi + block - 1) / block) * ((m->dev.nqk + 7) / 8);
+    return tall >= grid ? 8 : 4;
+}
+
 // a mesh in a pass: bounds-pass tiles over its quads; cell-pass slots over its faces
 void fill_pass(std::vector<PassEntry> &v, long long &tiles, long long &fslots, const tms_mesh m,
                int mesh_index, int pair, int role, int block, int rows, int face_level) {
@@ -597,18 +612,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         max_tri = std::max(max_tri, 2ULL * B[i]->dev.N * B[i]->dev.nqk);
     }
     long long unused = 0;
-    // Patch level, mixed precision: tiles of 8 rows read a vertex 9/8 times instead of 5/4
-    // and make the frames of two patch rows at once (64 uneven pairs 396 us against 416,
-    // 14 layers 49 against 51, 4096 x 512 54 against 57, 1024 x 256 13.2 against 13.7),
-    // where they are two for every SM; with fewer, the longer block is not hidden (64 x 32:
-    // 10.5 against 9.3).
-    P->bounds_rows = rows;
-    if (patch && prm.precision == 1 && rows == 4) {
-        long long tall = 0;
-        for (tms_mesh m : taken)
-            tall += (long long)((m->dev.nqi + block - 1) / block) * ((m->dev.nqk + 7) / 8);
-        if (tall >= P->grid) P->bounds_rows = 8;
-    }
+    P->bounds_rows = bounds_tile_rows(taken, prm, P->grid);
     for (size_t r = 0; r < taken.size(); ++r)
         fill_pass(pbounds, P->tiles_all, unused, taken[r], (int)r, 0, 0, block, P->bounds_rows, fl);
     for (int i = 0; i < nPairs; ++i) {
@@ -1117,6 +1121,19 @@ tms_status tms_build_mesh(const double *dX, const double *dY, const double *dPx,
 }  // extern "C"
 
 void tms::set_last_error(const std::string &msg) { g_err = msg; }
+
+int tms::bounds_rows(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms_params &params) {
+    std::map<long long, tms_mesh> seen;
+    for (int i = 0; i < nPairs; ++i) {
+        seen[A[i]->id] = A[i];
+        seen[B[i]->id] = B[i];
+    }
+    std::vector<tms_mesh> taken;
+    for (auto &m : seen) taken.push_back(m.second);
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, A[0]->device);
+    return bounds_tile_rows(taken, params, std::min(1024, 2 * sms));
+}
 
 tms_status tms::mesh_view(tms_mesh m, MeshDev *view, int *device) {
     if (!m || m->magic != kMagic) return TMS_ERR_STATE;

@@ -708,6 +708,9 @@ void launch_adjoint(const AdjointArgs &a, cudaStream_t st);
 // device view of a mesh handle (TMS_ERR_STATE for an invalid handle)
 tms_status mesh_view(tms_mesh m, MeshDev *view, int *device);
 
+// quad rows of a bounds-pass tile of a search of these (live) meshes
+int bounds_rows(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms_params &params);
+
 // The search with per-pair cell multipliers (empty: params->cell_mult for all);
 // tms_search and tms_search_batched after resolving params->autotune_cache.
 tms_status search_with_cm(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms_params &params,

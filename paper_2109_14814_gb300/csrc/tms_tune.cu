@@ -4,10 +4,12 @@
 // patches in trees) and the bounds-pass tile shape -- by timing them on the caller's meshes, and keeps the
 // choice in a text file read back by later searches (tms_params.autotune_cache).
 //
-// One pair: every setting of a small grid is timed with tms_search.
+// One pair: every setting of a small grid is timed with tms_search (at the patch level,
+// which has no cells, one multiplier).
 // A batch of uneven pairs (the continuation sweep): the settings that shape
 // the whole launch sequence (face level, patch level, bounds-pass tile) are
-// timed on the whole batch; then the cell multiplier is chosen per size class
+// timed on the whole batch; then, unless the patch level won, the cell multiplier is
+// chosen per size class
 // -- pairs grouped by their quad count, a class per factor of four -- by
 // coordinate descent, each class's candidates timed on the whole batch with
 // the other classes at their current choice, since the batch runs as one
@@ -287,20 +289,24 @@ extern "C" tms_status tms_autotune(const tms_mesh *A, const tms_mesh *B, int nPa
     tms_params bp = p0;
     for (auto &lv : levels)
         for (auto &sh : shapes)
-            for (int m = 0; m < (nPairs == 1 ? 3 : 1); ++m) {
+            // (a multiplier each at the levels that have a grid)
+            for (int m = 0; m < (nPairs == 1 && !lv[1] ? 3 : 1); ++m) {
                 tms_params p = p0;
                 p.face_level = lv[0];
                 p.patch = lv[1];
                 p.block_faces = sh[0];
-                p.tile_rows = sh[1];
                 p.cell_mult = nPairs == 1 ? mults[m] : p0.cell_mult;
+                p.tile_rows = 4;
+                // where tiles of 8 rows run anyway they have been timed
+                if (sh[1] == 8 && tms::bounds_rows(A, B, nPairs, p) == 8) continue;
+                p.tile_rows = sh[1];
                 const double t = timed(p, none);
                 if (t < bestt) {
                     bestt = t;
                     bp = p;
                 }
             }
-    // per size class: the cell multiplier, by coordinate descent (batches)
+    // per size class: the cell multiplier, by coordinate descent (batches in a grid)
     std::vector<float> cm;
     std::map<int, float> class_best;
     if (nPairs > 1 && bestt < 1e300) {
@@ -319,7 +325,7 @@ extern "C" tms_status tms_autotune(const tms_mesh *A, const tms_mesh *B, int nPa
             const int c = o.second;
             float keep = bp.cell_mult;
             for (float v : cands) {
-                if (v == keep) continue;
+                if (v == keep || bp.patch == 1) continue;
                 std::vector<float> trial = cm;
                 for (int i = 0; i < nPairs; ++i)
                     if (cls[i] == c) trial[i] = v;
@@ -346,7 +352,11 @@ extern "C" tms_status tms_autotune(const tms_mesh *A, const tms_mesh *B, int nPa
         snprintf(buf, sizeof(buf), " %d %d %d %d %.6g %.6g", bp.face_level, bp.patch, bp.block_faces,
                  bp.tile_rows, (double)bp.cell_mult, bestt);
         lines.push_back(batch_key(A, B, nPairs, p0) + buf);
+        std::map<std::string, std::string> known;
+        for (auto &kv : read_cache(cache_path)) known[kv.first] = kv.second;
         for (auto &cb : class_best) {
+            // without a grid nothing was learnt of a class that has a line
+            if (bp.patch == 1 && known.count(class_key(cb.first, p0))) continue;
             snprintf(buf, sizeof(buf), " %.6g", (double)cb.second);
             lines.push_back(class_key(cb.first, p0) + buf);
         }
