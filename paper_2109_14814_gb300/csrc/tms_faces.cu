@@ -32,6 +32,7 @@
 // a time, so its loop runs ceil(sum of cells / 32) times instead of 32 x the
 // largest count.  An entry is (key = pair << 32 | cell << 1 | role, face id).
 #include <cuda_runtime.h>
+#include <float.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -1026,7 +1027,8 @@ __global__ void k_grid_params(const Bounds *b, const int2 *pairs, int n_pairs, G
     double step = (double)cm * fmax(ord_dec(A.w[d]), ord_dec(B.w[d]));
     const double range = empty ? 0.0 : e - o;
     int n;
-    if (!(range > 0.0) || !(step > 0.0)) {
+    // (one cell where a face is unbounded: range / step is no number)
+    if (!(range > 0.0) || !(step > 0.0) || step > DBL_MAX) {
         n = 1;
         step = 0.0;
     } else {

@@ -333,7 +333,9 @@ __global__ void __launch_bounds__(32 * kEmitWarps, (PREC == 1 && !MOLLER) ? 5 : 
             for (int u = 0; u < 4; ++u)
                 K |= (boxes_overlap(abox, sBox[warp][j + u]) ? 1u : 0u) << (j + u);
         }
-        K &= rows;
+        // (an unbounded box, of coordinates beyond FP32 on both sides, meets the empty ones
+        // of the rows and lanes past the tile too)
+        K &= lane < nAt ? rows & (0xFFFFFFFFu >> (32 - nBt)) : 0u;
         if (MOLLER) {
             for (uint32_t k = K; k; k &= k - 1) {
                 const int j = __ffs(k) - 1;
