@@ -666,7 +666,9 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
         for (P->top = 0; P->top < kTreeTop; ++P->top) {
             unsigned long long n = 0;
             for (const int2 &q : pairs) n += (unsigned long long)size(q.x, P->top) * size(q.y, P->top);
-            if (n <= kTreeTopPairs) break;
+            long long most = 0;
+            for (size_t i = 0; i < meshes.size(); ++i) most = std::max(most, size((int)i, P->top));
+            if (n <= kTreeTopPairs && most <= kTreeTopNodes) break;
         }
         for (const int2 &q : pairs) {
             top_base.push_back(P->top_tiles);

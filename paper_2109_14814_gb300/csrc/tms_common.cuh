@@ -552,6 +552,7 @@ struct TreeLevel {
 constexpr int kTreeLevels = 8;
 constexpr int kTreeTop = kTreeLevels - 3;             // the highest top level
 constexpr unsigned long long kTreeTopPairs = 1ULL << 22;
+constexpr long long kTreeTopNodes = 16384;
 struct MeshTree {
     TreeLevel lev[kTreeLevels];
     uint32_t up_base[kTreeLevels / 2];                // first node of level 2, 4, .. over all meshes
