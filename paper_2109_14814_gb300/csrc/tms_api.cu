@@ -142,8 +142,9 @@ struct Plan {
     // short merge: bucket counts and drop bits, each bucket's first place
     uint32_t *tail = nullptr;
     float bscale = 0.0f;
-    // more raw hits than the short merge takes: the radix sort and the scans (as
-    // a search of this plan found; the look-back test switch needs that sort too)
+    // more raw hits than the short merge takes, or too many of a few triangles: the radix
+    // sort and the scans (as a search of this plan found; the look-back test switch needs
+    // that sort too)
     bool long_tail = false;
     // of the merge's launch, which asks for more than every device has to take: a capture
     // without it would run, and leave the counters as they were
@@ -936,7 +937,7 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
             P->hit_cap = c.raw_hits + c.raw_hits / 4 + 1024;
             grow = true;
         }
-        if (!P->long_tail && c.raw_hits > kTailMax) {
+        if (!P->long_tail && (c.raw_hits > kTailMax || (c.status & ST_TAIL_UNEVEN))) {
             P->long_tail = true;
             grow = true;
         }

@@ -41,6 +41,7 @@ enum StatusBits : unsigned int {
     ST_TIMEOUT = 1u << 1,
     ST_PAIR_LIMIT = 1u << 2,
     ST_TABLE_FULL = 1u << 3,
+    ST_TAIL_UNEVEN = 1u << 4,   // a bucket of the short merge holds more than kTailUneven hits
 };
 
 // ---------------------------------------------------------------------------
@@ -171,6 +172,7 @@ struct Counters {
 // kTailBuckets buckets of increasing key as the FP64 solve lists them.
 constexpr unsigned kTailMax = 32768;
 constexpr unsigned kTailBuckets = 8192;
+constexpr unsigned kTailUneven = 1024;
 
 // The bucket of a hit: its (pair, triA) scaled to the buckets, monotone in the
 // key (the conversion and the product round monotonically).
@@ -663,8 +665,8 @@ struct DedupArgs {
 void launch_dedup(const DedupArgs &a, int grid, cudaStream_t st);
 
 // The merge of at most kTailMax raw hits in one launch, instead of the radix
-// sort and launch_dedup (nothing is written when there are more: the host takes
-// that path then).
+// sort and launch_dedup (nothing is written when there are more, or a bucket holds more
+// than kTailUneven: the host takes that path then).
 struct TailArgs {
     const uint64_t *key;           // raw hits' keys, in the order they were found
     const uint32_t *slot;          // and their places in their buckets

@@ -1038,8 +1038,10 @@ __global__ void k_offsets(const uint64_t *out_keys, const unsigned long long *d_
 // (157 hits) 112 -> 100 us.  The FP64 solve counts the hits into
 // buckets of increasing key; each block scans the counts for itself (32 KB from L2) and
 // lists its hits in their buckets; then compares a hit with its bucket (about one at
-// 8192 buckets; however unevenly the hits fall, at most kTailMax compares) and decides
-// whether it is a duplicate; then writes the records kept.
+// 8192 buckets, at most kTailUneven) and decides whether it is a duplicate; then writes the
+// records kept.  Hits that crowd a few buckets (a mesh of few triangles, a small pair of a
+// batch beside large ones) go to the radix sort: a search with 14,000 hits of two triangles
+// took 583 us here and takes 143 so; the two meet near a thousand in a bucket.
 __device__ __forceinline__ bool tail_count(const TailArgs &a, unsigned &n) {
     const unsigned long long raw = a.ctr->raw_hits;
     n = (unsigned)raw;
@@ -1106,9 +1108,12 @@ __global__ void __launch_bounds__(kTailBlock) k_tail(TailArgs a) {
     {
         const uint4 lo = reinterpret_cast<const uint4 *>(a.tail)[2 * t], hi = reinterpret_cast<const uint4 *>(a.tail)[2 * t + 1];
         const uint32_t c[kPer] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
-        uint32_t sum = 0;
+        uint32_t sum = 0, most = 0;
 #pragma unroll
-        for (int k = 0; k < kPer; ++k) sum += c[k];
+        for (int k = 0; k < kPer; ++k) {
+            sum += c[k];
+            most = max(most, c[k]);
+        }
         uint32_t incl = sum;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
@@ -1116,7 +1121,14 @@ __global__ void __launch_bounds__(kTailBlock) k_tail(TailArgs a) {
             if (lane >= off) incl += y;
         }
         if (lane == 31) wsum[warp] = incl;
-        __syncthreads();
+        if (__syncthreads_or(most > kTailUneven)) {  // (every block of the cluster alike)
+            if (blockIdx.x == 0) {
+                if (t == 0) a.ctr->status |= ST_TAIL_UNEVEN;
+                __syncthreads();
+                tail_readback(a);
+            }
+            return;
+        }
         uint32_t before = __reduce_add_sync(FULL, lane < warp ? wsum[lane] : 0u) + incl - sum;
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
