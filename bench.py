@@ -452,7 +452,7 @@ def run_tms(args, ws, rank, local):
         flops = float(FP64_SOLVE_FLOPS) * stats["fp64_solves"]
         t_narrow = stage_ms.get("narrow", 0.0)
         ach = flops / (t_narrow / 1e3) / 1e12 if t_narrow > 0 else None
-        fp64 = {"kernel": "tms::k_narrow", "solves_fp64": stats["fp64_solves"],
+        fp64 = {"kernel": "tms::k_narrow_filter", "solves_fp64": stats["fp64_solves"],
                 "candidates": stats["candidates"], "flops_per_solve": FP64_SOLVE_FLOPS,
                 "achieved_tflops": ach, "peak_tflops": peak64,
                 "frac": (ach / peak64) if (ach and peak64) else None,

@@ -330,35 +330,28 @@ __device__ __forceinline__ void stage_push(Rec *stage, unsigned &n, bool pred, c
 
 // FP64 -> FP32 conversions from the IEEE-754 encodings, with integer operations
 // only (the FP64 pipe, which also carries FP64 conversions, is scarce on GB300).
-// Normal-range results are a lower bound a place or less below / the nearest, ties to
-// even.  Outside the FP32 normal range the results are still valid bounds:
-// |x| < 2^-126 rounds outward to 0 or +-2^-126 (nearest: to +-0), |x| >= 2^128
-// to +-FLT_MAX or +-inf, NaN stays NaN.
+// Normal-range results are a lower bound a place or less below (f32_rd) / the nearest, ties
+// to even (f32_rn).  Outside the FP32 normal range they are a lower bound / nearest still:
+// |x| < 2^-126 goes to +0 or -2^-126 / to +-0, |x| >= 2^128 to FLT_MAX or -inf / to +-inf;
+// NaN stays NaN.
 __device__ __forceinline__ unsigned f32_bits_trunc(unsigned long long b, int e32) {
     return ((unsigned)(b >> 63) << 31) | ((unsigned)e32 << 23) |
            (unsigned)((b & 0xFFFFFFFFFFFFFULL) >> 29);
 }
-__device__ __forceinline__ float f32_special(unsigned long long b, int e32, int dir) {
-    // dir: -1 down, +1 up, 0 nearest
+__device__ __forceinline__ float f32_special(unsigned long long b, int e32, bool down) {
     const unsigned sign = (unsigned)(b >> 63) << 31;
     const bool is_nan = ((b >> 52) & 0x7ff) == 0x7ff && (b & 0xFFFFFFFFFFFFFULL) != 0;
     if (is_nan) return __uint_as_float(0x7fc00000u);
     if (e32 >= 255) {                       // |x| >= 2^128 or inf
-        const bool neg = sign != 0;
-        if (dir == 0) return __uint_as_float(sign | 0x7f800000u);
-        if (dir < 0) return __uint_as_float(neg ? 0xff800000u : 0x7f7fffffu);
-        return __uint_as_float(neg ? 0xff7fffffu : 0x7f800000u);
+        return __uint_as_float(down && !sign ? 0x7f7fffffu : sign | 0x7f800000u);
     }
     // |x| < 2^-126
     const bool nonzero = (b & 0x7FFFFFFFFFFFFFFFULL) != 0;
-    if (dir == 0 || !nonzero) return __uint_as_float(sign);
-    const bool neg = sign != 0;
-    if (dir < 0) return neg ? -1.17549435e-38f : 0.0f;
-    return neg ? -0.0f : 1.17549435e-38f;
+    return down && nonzero ? (sign ? -1.17549435e-38f : 0.0f) : __uint_as_float(sign);
 }
 // (out of line: the compiler would run parts of it for every value, under a predicate)
 static __device__ __noinline__ float f32_rd_special(double x) {
-    return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, -1);
+    return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, true);
 }
 // A lower bound of x, at most one FP32 place below it: in the FP32 normal range the bits
 // of |x| shifted right by 29, less the exponents' difference, are the truncated FP32
@@ -384,7 +377,7 @@ __device__ __forceinline__ float f32_above(float f) {
     return fmaxf(f + fmaf(fabsf(f), 1.1920932e-7f, 1.17549435e-38f), -3.40282347e38f);
 }
 static __device__ __noinline__ float f32_rn_special(double x) {
-    return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, 0);
+    return f32_special((unsigned long long)__double_as_longlong(x), (int)((__double2hiint(x) >> 20) & 0x7ff) - 896, false);
 }
 __device__ __forceinline__ float f32_rn(double x) {
     const unsigned long long b = (unsigned long long)__double_as_longlong(x);

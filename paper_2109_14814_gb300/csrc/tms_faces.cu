@@ -762,20 +762,13 @@ __global__ void __launch_bounds__(256, PREC == 1 ? (TK == 4 ? 4 : 3) : 2) k_boun
             const Vtx<PREC> vc = sv[(r + 1) * W + t];       // (i, k+1)
             const Vtx<PREC> vd = sv[(r + 1) * W + t + 1];   // (i+1, k+1)
             const uint32_t q = (uint32_t)k * (uint32_t)m.N + (uint32_t)i;
-            if (FACE == 0) {
-                BoxT<PREC> b1, b2;
-                box_init(b1, vb); box_add(b1, va); box_add(b1, vc);   // T1: x1=(i+1,k) x2=(i,k) x3=(i,k+1)
-                box_init(b2, vc); box_add(b2, vd); box_add(b2, vb);   // T2: x1=(i,k+1) x2=(i+1,k+1) x3=(i+1,k)
-                acc.add(b1);
-                acc.add(b2);
-                write_fbox<PREC>(m, 2 * q, b1);
-                write_fbox<PREC>(m, 2 * q + 1, b2);
-            } else {
-                BoxT<PREC> bq;
-                box_init(bq, va); box_add(bq, vb); box_add(bq, vc); box_add(bq, vd);
-                acc.add(bq);
-                write_fbox<PREC>(m, q, bq);
-            }
+            BoxT<PREC> b1, b2;
+            box_init(b1, vb); box_add(b1, va); box_add(b1, vc);   // T1: x1=(i+1,k) x2=(i,k) x3=(i,k+1)
+            box_init(b2, vc); box_add(b2, vd); box_add(b2, vb);   // T2: x1=(i,k+1) x2=(i+1,k+1) x3=(i+1,k)
+            acc.add(b1);
+            acc.add(b2);
+            write_fbox<PREC>(m, 2 * q, b1);
+            write_fbox<PREC>(m, 2 * q + 1, b2);
         }
     }
 

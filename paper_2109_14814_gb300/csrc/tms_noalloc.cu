@@ -371,6 +371,7 @@ extern "C" tms_status tms_search_noalloc(tms_mesh A, tms_mesh B, const tms_param
         g_msg = "cell table full";
         return TMS_ERR_STATE;
     }
+    // (kSurvCap bounds a call's work; no list has that length)
     if (c.entries > kEntCap || c.cand > kCandCap || c.fp64 > kSurvCap || c.raw_hits > kRawHitCap) {
         g_msg = "a search stage exceeded the static scratch limits";
         *nHits = -1;
