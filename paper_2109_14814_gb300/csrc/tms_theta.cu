@@ -253,6 +253,9 @@ __device__ __forceinline__ void fast_sum(float x, float y, float &s, float &e) {
 // rounding.  Every value is in one distance of each shift, so `lost` such values cost a
 // shift lost 2^-69: where that could be more than 2^-51 of its cost (a large coordinate
 // that cancels leaves a cost of that size) the shift's cost is made again in FP64.
+// So is one that few distances make, whose errors do not average out: 2.4e-15 of the root of
+// the distances' squares is more than the 1.9e-17 N^(1/2) of the cost that a sum in FP64
+// loses where those squares are more than N / 16384 of the cost's (evenly spread: N < 130).
 // Split: a cluster of eight blocks takes 512 shifts, each block an eighth of the i
 // (the same split for every shift and number of alignments: equal terms give equal
 // costs), each thread two neighbouring shifts, whose windows overlap; the even and
@@ -266,6 +269,7 @@ constexpr int kPhWin = kPhTile + kPhShifts;
 constexpr int kPhWide = 0x7fffffff;     // no scale: FP64 sums
 constexpr int kPhLeast = 192;           // shorter circles take FP64 sums
 constexpr int kPhUp = 40;               // the digits' unit is 2^-40 of the scale
+constexpr double kPhFew = 16384.0;      // N / kPhFew: the share of the squares that few distances pass
 
 struct PhaseArgs {
     const double *wr;
@@ -436,6 +440,7 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
     float *win = ps + kPhTile * 3 * C;                                    // [odd][digit][C][kPhWin / 2]
     constexpr int kHalf = kPhWin / 2;
     double *part = reinterpret_cast<double *>(win + 3 * C * kPhWin);      // [kPhShifts]
+    float *sq = reinterpret_cast<float *>(part + kPhShifts);              // [kPhShifts]
     const int N = a.N, al = blockIdx.y, t = threadIdx.x;
     const int rank = blockIdx.x % kPhSplit;
     const int m0 = (int)(blockIdx.x / kPhSplit) * kPhShifts;
@@ -453,7 +458,7 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
     }
     const int e = (word & 0xfff) - 1024, lost = word >> 12;
     double acc[2] = {0.0, 0.0};
-    float rest[2] = {0.0f, 0.0f};
+    float rest[2] = {0.0f, 0.0f}, squares[2] = {0.0f, 0.0f};
     const double down = power_of_two(kPhUp - e);
     const int per = ((N + 4 * kPhSplit - 1) / (4 * kPhSplit)) * 4;
     const int i_end = (int)min((long long)N, (long long)(rank + 1) * per);
@@ -502,6 +507,7 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
                     for (int k = 0; k < 2; ++k) {
                         float g, lo, s, r;
                         pair_distance<C>(x[(v + k) & 1], y, g, lo, rest[k]);
+                        squares[k] = __fmaf_rn(g, g, squares[k]);
                         two_sum(G[k], g, s, r);
                         G[k] = s;
                         E[k] = __fadd_rn(E[k], __fadd_rn(r, lo));
@@ -518,6 +524,8 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
     // the eight parts, added in order of i by the cluster's first block
     part[2 * t] = acc[0] + (double)rest[0];
     part[2 * t + 1] = acc[1] + (double)rest[1];
+    sq[2 * t] = squares[0];
+    sq[2 * t + 1] = squares[1];
     cg::cluster_group cluster = cg::this_cluster();
     // shifts to be made again (the first block's), costs below which they are
     __shared__ unsigned short again[kPhShifts];
@@ -528,14 +536,17 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
     if (rank == 0) {
         for (int q = t; q < kPhShifts; q += kPhThreads) {
             double s = part[q];
-            for (int r = 1; r < kPhSplit; ++r) s += cluster.map_shared_rank(part, r)[q];
+            float d2 = sq[q];
+            for (int r = 1; r < kPhSplit; ++r) {
+                s += cluster.map_shared_rank(part, r)[q];
+                d2 += cluster.map_shared_rank(sq, r)[q];
+            }
             if (m0 + q >= N) continue;
-            if (s < least) again[atomicAdd(&n_again, 1)] = (unsigned short)q;
+            if (s < least || kPhFew * (double)d2 > N * (s * s)) again[atomicAdd(&n_again, 1)] = (unsigned short)q;
             else a.cost[(long long)al * N + m0 + q] = s * power_of_two(e - kPhUp);
         }
     }
     cluster.sync();                     // the parts are read before their blocks end
-    if (lost == 0) return;
     const int n = *cluster.map_shared_rank(&n_again, 0);
     for (int k = rank; k < n; k += kPhSplit) {
         const int m = m0 + cluster.map_shared_rank(again, 0)[k];
@@ -554,7 +565,7 @@ __global__ void __cluster_dims__(kPhSplit, 1, 1) __launch_bounds__(kPhThreads) k
 
 template <int C>
 cudaError_t launch_phase_cost(const PhaseArgs &a, cudaStream_t st) {
-    constexpr size_t smem = (size_t)(kPhTile + kPhWin) * 3 * C * sizeof(float) + kPhShifts * sizeof(double);
+    constexpr size_t smem = (size_t)(kPhTile + kPhWin) * 3 * C * sizeof(float) + kPhShifts * (sizeof(double) + sizeof(float));
     const cudaError_t e = cudaFuncSetAttribute(k_phase_cost<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)((a.N + kPhShifts - 1) / kPhShifts) * kPhSplit, (unsigned)a.nalign);
