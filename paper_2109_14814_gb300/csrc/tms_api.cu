@@ -30,6 +30,8 @@ struct tms_mesh_s {
 namespace {
 
 constexpr unsigned kMagic = 0x746d7331u;  // "tms1"
+constexpr unsigned long long kTableMost = 1ULL << 31;       // slots of the cell table
+constexpr unsigned long long kEntriesMost = 0x7fffffffULL;  // face-cell entries
 std::mutex g_mu;
 // tms_search_host: the first n output records copied to host memory right
 // after the search on its stream, before the synchronisation that reads the count
@@ -212,7 +214,7 @@ struct Plan {
             // capacity (L2-resident) and grows when a search finds it over half full
             tsize = 1024;
             const unsigned long long want = (prm.inject & 8u) ? 0 : ent_cap / 16;
-            while ((tsize < want || tsize < tsize_min) && tsize < (1ULL << 31)) tsize <<= 1;
+            while ((tsize < want || tsize < tsize_min) && tsize < kTableMost) tsize <<= 1;
             TMS_CK(dalloc(&tkey, tsize));
             TMS_CK(dalloc(&tcnt, tsize));
             TMS_CK(dalloc(&tstart, tsize));
@@ -788,7 +790,7 @@ tms_status make_plan(const tms_mesh *A, const tms_mesh *B, int nPairs, const tms
                              : (prm.cell_filter ? std::max<unsigned long long>(1 << 16, faces / 2)
                                                 : 4 * faces + (1 << 16));
     if ((prm.inject & 1u) || (patch && (prm.inject & 8u))) ent = 1;
-    P->ent_cap = std::min<unsigned long long>(ent, 0x7fffffffULL);
+    P->ent_cap = std::min(ent, kEntriesMost);
     // patch level: candidates are quad pairs, about one per quad of A
     const unsigned long long quadsA = [&] {
         unsigned long long q = 0;
@@ -886,7 +888,8 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
     P->retries = 0;
     // Each list's count is complete only once those before it fit, so each may cost a run of
     // its own (node pairs of every level, patch pairs, candidates, kept quads, raw hits; a
-    // cell table from 1024 slots up to 2^31 eleven), and the last of them must fit.
+    // cell table from 1024 slots up to 2^31 eleven), and the last of them must fit.  A list
+    // that is at its limit ends them.
     bool grow = true;
     for (int run = 0; grow && run < kTreeLevels + 16; ++run) {
         s = P->run();
@@ -905,9 +908,11 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
             return TMS_ERR_TIMEOUT;
         }
         grow = false;
-        if (!P->patch && ((c.status & ST_TABLE_FULL) || c.claimed > P->tsize / 2)) {
-            P->tsize_min = P->tsize * 4;
+        // (the largest table may be over half full)
+        if (!P->patch && ((c.status & ST_TABLE_FULL) || (c.claimed > P->tsize / 2 && P->tsize < kTableMost))) {
             grow = true;
+            if (P->tsize >= kTableMost) break;
+            P->tsize_min = P->tsize * 4;
         }
         unsigned long long nodes = 0;
         for (unsigned long long v : c.nodes) nodes = std::max(nodes, v);
@@ -916,7 +921,11 @@ tms_status search_core(const tms_mesh *A, const tms_mesh *B, int nPairs, const t
             grow = true;
         }
         if (!grow && !P->patch && c.entries > P->ent_cap) {
-            P->ent_cap = std::min<unsigned long long>(0x7fffffffULL, c.entries + c.entries / 4 + 1024);
+            if (P->ent_cap >= kEntriesMost) {
+                grow = true;
+                break;
+            }
+            P->ent_cap = std::min(kEntriesMost, c.entries + c.entries / 4 + 1024);
             P->bmH_bits = std::min(25, std::max(11, ceil_log2(P->ent_cap * 8) - 5));
             P->cand_cap = std::max(P->cand_cap, 2 * P->ent_cap);
             grow = true;
